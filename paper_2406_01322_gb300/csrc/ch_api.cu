@@ -806,35 +806,26 @@ int ch_set_chebyshev(ch_grid* G, int method) {
     if (!G->cf) {
       const GridDev& g = G->g;
       std::vector<uint16_t> dig[2];
-      std::vector<int> fe[2];
       chf::ChebTc t[2];
       for (int dir = 0; dir < 2; ++dir) {
-        int NT, nNt, Kp;
-        if (chf::cheb_tc_tables(g.N, dir, dig[dir], fe[dir], NT, nNt, Kp) != 0) return CH_ERR_SIZE;
-        t[dir].NT = NT;
-        t[dir].nNt = nNt;
-        t[dir].Kp = Kp;
-        t[dir].dir = dir;
+        if (chf::cheb_tc_tables(g.N, dir, dig[dir], &t[dir]) != 0) return CH_ERR_SIZE;
         void* dd = galloc(G, dig[dir].size() * sizeof(uint16_t));
-        void* df = galloc(G, fe[dir].size() * sizeof(int));
-        if (!dd || !df) return CH_ERR_ALLOC;
+        if (!dd) return CH_ERR_ALLOC;
         CK(cudaMemcpy(dd, dig[dir].data(), dig[dir].size() * sizeof(uint16_t),
                       cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(df, fe[dir].data(), fe[dir].size() * sizeof(int), cudaMemcpyHostToDevice));
         t[dir].dig = (const uint16_t*)dd;
-        t[dir].fexp = (const int*)df;
-        CK(chf::cheb_tc_prepare(NT));
       }
+      CK(chf::cheb_tc_prepare());
       CK(chf::zline_coef_prepare(g));
-      // one persistent CTA per SM, each with a plane cache for one tile of rows
+      // one persistent CTA per SM, each with room for one tile's fixed-point rows
       int dev = 0, nsm = 0;
       CK(cudaGetDevice(&dev));
       CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
       if (nsm < 1) nsm = 1;
-      void* cache = galloc(G, (size_t)nsm * chf::cheb_tc_cache_bytes(t[0].Kp));
-      if (!cache) return CH_ERR_ALLOC;
+      void* keep = galloc(G, (size_t)nsm * chf::cheb_tc_keep_bytes(g.N));
+      if (!keep) return CH_ERR_ALLOC;
       for (int dir = 0; dir < 2; ++dir) {
-        t[dir].cache = (uint32_t*)cache;
+        t[dir].keep = (char*)keep;
         t[dir].ctas = nsm;
       }
       int* err = (int*)galloc(G, sizeof(int));

@@ -277,25 +277,24 @@ cudaError_t launch_diag(const GridDev& g, const double* phys7, long long fs,
                         const double* qint, double* part, double* out, cudaStream_t s);
 
 // Chebyshev transform along z as an exact-split (Ozaki) bf16 matrix product on the tensor cores
-// (ch_tc.cu).  Tables of one direction (dir 0 forward: samples -> coefficients; 1 backward):
-// nNt output slices of NT columns covering the outputs n < N (the kernel sums n = N exactly),
-// K padded to Kp (a multiple of 16, < 512).
+// (ch_tc.cu).  Plan of one direction (dir 0 forward: samples -> coefficients; 1 backward) for
+// lines of N + 1 points, N even: the outputs n < N of each parity in nsl slices of NT columns, the
+// N / 2 folded inputs in nst stages of 16, cut into kc groups of gst stages.
 struct ChebTc {
-  const uint16_t* dig = nullptr;   // device: per slice, per K chunk, eight NT x KC digit planes
-  const int* fexp = nullptr;       // device: output-row scale exponents F_n (nNt NT entries)
-  uint32_t* cache = nullptr;       // device: A digit planes of one tile per persistent CTA
-  int NT = 0, nNt = 0, Kp = 0;
+  const uint16_t* dig = nullptr;   // device: matrix digits (cheb_tc_tables)
+  char* keep = nullptr;            // device: fixed-point values of one tile per persistent CTA
+  int NT = 0, nsl = 0, nst = 0, kc = 0, gst = 0;
   int dir = 0;                     // 0 forward (samples -> coefficients), 1 backward
-  int ctas = 0;                    // persistent CTAs (the cache holds ctas cheb_tc_cache_bytes)
+  int q = 0;                       // log2 of the matrix scale
+  long long ymid = 0;              // weight of the middle element, times 2^q
+  int ctas = 0;                    // persistent CTAs (keep holds ctas cheb_tc_keep_bytes)
 };
-// bytes of plane cache one persistent CTA needs for rows of padded length Kp
-size_t cheb_tc_cache_bytes(int Kp);
-// host tables; 0 or -1 (size not supported)
-int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, std::vector<int>& fexp, int& NT,
-                   int& nNt, int& Kp);
-size_t cheb_tc_smem(int NT);
-// raise the shared-memory limit of every instantiation for slice width NT (before any capture)
-cudaError_t cheb_tc_prepare(int NT);
+// bytes of `keep` one persistent CTA needs
+size_t cheb_tc_keep_bytes(int N);
+// plan and host table of the digits; 0 or -1 (size not supported)
+int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t);
+// raise the shared-memory limit of every instantiation (before any capture)
+cudaError_t cheb_tc_prepare();
 // nf fields of complex lines, element type tin / tout (0 float64, 1 float32, 2 double-float; the
 // pairs float64 -> float64, float32 -> float64, double-float -> float64 and float64 -> float32 /
 // double-float), field strides

@@ -1,6 +1,6 @@
 // Chebyshev transforms along z (Sec. 3.2.1) as float64-accurate matrix products on the tensor
 // cores: tcgen05 MMAs with bf16 operands staged in shared memory and fp32 accumulators in tensor
-// memory.
+// memory (the exact split of ch_tc.cuh).
 //
 // The transform of one line is a product with a fixed Nz x Nz matrix B (rows = outputs):
 //   forward (samples at z_k = cos(pi k / N) -> coefficients)
@@ -9,35 +9,28 @@
 //   backward (coefficients -> samples)  f_j = sum_n cos(pi n j / N) a_n.
 // Real and imaginary parts are separate rows of the left operand.
 //
-// Exact split (Ozaki scheme).  A row x with max |x_k| < 2^E becomes the integer vector
-// X_k = round(x_k 2^(54-E)), |X_k| < 2^54 (53 significant bits for the largest element, as in
-// float64), written with signed base-128 digits
-//   X_k = sum_{i=0..7} a_ik 128^(7-i),  a_ik in [-64, 63]
-// (X + bias, bias = 64 sum_t 128^t, stays inside eight 7-bit groups for |X| < 2^54)
-// (bf16 holds these exactly); each output row n of B likewise with its own scale 2^F_n and
-// digits b_jnk.  A digit product C_ij = sum_k a_ik b_jnk is an integer with |C_ij| <= 64*64*K,
-// and the eight products with the same i + j = d share one fp32 accumulator G_d:
-// |G_d| <= 8*64*64*K < 2^24 for K < 512, so every accumulation is exact.  Keeping d <= 7 (36
-// products) drops terms of order 2^-54 of the row-max x column-max scale; with the 2^-55
-// quantisation of both operands and the final rounding the error stays at a few units of 2^-53
-// of max|x| x max_n sum_k |B_nk|, the accuracy of a float64 transform.  The result
-//   sum_k x_k B_nk = 2^(E + F_n - 108) sum_{d<=7} 128^(14-d) G_d
-// is recombined in 64-bit integers and rounded once to float64 (or float32) with integer
-// operations only (the float64 pipe is the scarce resource on this part).
+// Folding.  cos(pi n (N-k) / N) = (-1)^n cos(pi n k / N) and e_k = e_{N-k}, so with H = N / 2
+//   even outputs need only s_k = x_k + x_{N-k}, odd ones only d_k = x_k - x_{N-k}, k < H
+// (both matrices are symmetric in this way), plus (-1)^m x_H for output n = 2m.  The sums and
+// differences are exact in fixed point, the middle element is added to the recombined integer
+// (it is the row's value times one weight), and the last output n = N, sum_k w_k (-1)^k x_k, is
+// summed exactly by the producers; the MMAs then do two H x H products of K = H instead of one
+// (N+1) x (N+1) product of K = N + 1.  All weights share one power-of-two scale 2^q.
 //
-// Tiles and data flow.  A tile is 128 rows (re and im of 64 lines of one field) by all Nz
-// outputs, computed as nNt output slices of NT (48 or 64) columns; the eight accumulators
-// G_0..G_7 of a slice (8 NT fp32 columns) live in tensor memory.  The eight B digit planes of a
-// slice are stacked into one 8 NT-row operand, so A plane i needs a single MMA chain over rows
-// 0 .. (8-i) NT with its accumulator starting at column i NT: product (i, j) lands on diagonal
-// i + j.  (The MMA issue rate, about one instruction per 50..128 cycles, is what limits the
-// kernel; merging the pairs this way cuts 36 small MMAs per k-step to 8..12 large ones.)
-// Persistent CTAs (one per SM) walk the tiles with 16 producer warps and one issuer warp: the
-// producers convert their rows to fixed point once per tile, write the digit planes of the first
-// slice into rotating shared buffers and their 7-bit groups (one byte each) into a per-CTA plane
-// cache in global memory, and rebuild the later slices' planes from that cache; the issuer copies
-// the digits of B and issues the MMAs.  Rows are split into K chunks of 96 that accumulate into
-// the same tensor memory.
+// Tiles and data flow.  A tile is 128 rows (re and im of 64 lines of one field).  Its passes are
+// (output slice of NT columns, parity, K group): the accumulators of a pass live in tensor memory.
+// Persistent CTAs (one per SM) have three kinds of warps, so conversion, MMAs and the epilogue of
+// different passes overlap:
+//   producers (8 warps): per K stage of 16 (one MMA k-step) a thread converts four pairs
+//     (x_k, x_{N-k}) of the real and imaginary rows of one line to fixed point, writes the seven
+//     digit planes of the sums to the stage's shared buffer and keeps the differences (and, with
+//     several slices, the sums) in a per-CTA buffer in global memory (L2), read back by the same
+//     thread for the later passes; thread 0 also issues the bulk copy of the stage's matrix digits;
+//   issuer (1 thread): the MMAs of each stage as it fills;
+//   epilogue (8 warps): drains a pass's accumulators, recombines and stores.
+// What bounds it: integer issue (about 45 instructions per element converted and 25 per output)
+// and the shared-memory bandwidth of the MMA operands; the tensor pipe itself needs 0.93 of the
+// 16-wide stage's time at NT = 64.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -46,674 +39,396 @@
 #include <vector>
 
 #include "ch_internal.h"
+#include "ch_tc.cuh"
 
 namespace chf {
 
 namespace {
 
-constexpr int TCT = 512;          // threads per CTA
-constexpr int TCM = 128;          // rows per tile = tensor-memory lanes
-constexpr int TCKC = 96;          // K per chunk
-constexpr int TCG = TCKC / 8;     // 8-element core-matrix groups per chunk
-constexpr int kNA = 4;            // shared buffers of A digit planes (kNA - 1 copied ahead)
-constexpr int kNB = 1;            // shared buffers of B digit planes
-constexpr int kSmallK = 144;      // K up to which every accumulator stays below 2^22 in magnitude
-// 32-bit words of one cached plane (four 7-bit groups per word, TCM x TCKC groups)
-constexpr int kCacheWords = TCM * TCKC / 4;
-constexpr unsigned long long kBias = 0x0081020408102040ull;   // 64 * sum_{t<8} 128^t
-constexpr uint64_t kWaitNs = 1000000000ull;                   // bound of every device wait
+using namespace tc;
 
-// ---- PTX wrappers -----------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t su32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-// shared-memory matrix descriptor, no swizzle: lbo = byte stride between core matrices along K,
-// sbo = byte stride between 8-row core-matrix groups along M (or N); version 1 at bit 46
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-__device__ __forceinline__ uint64_t gtime() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// bounded wait for the phase with the given parity; false if it did not complete in time
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.b32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-// wait for the phase with the given parity until the global timer passes `deadline`
-__device__ __forceinline__ bool mbar_wait_until(uint32_t bar, uint32_t parity,
-                                                uint64_t deadline) {
-  while (true) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (gtime() > deadline) return false;
-  }
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try(bar, parity)) return true;   // the common case: no clock read
-  return mbar_wait_until(bar, parity, gtime() + kWaitNs);
-}
-// The waits of one thread.  The first wait that runs out clears `ok`; every later wait returns
-// false at once, so a thread spends at most one bound waiting in vain however many waits follow
-// (the transform kernel's issuer then stops issuing and drains, its producers skip their waits).
-struct Waiter {
-  bool ok = true;
-  __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) {
-    ok = ok && mbar_wait(bar, parity);
-    return ok;
-  }
-};
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-      : "memory");
-}
-// L2 policy that keeps lines resident (the per-CTA digit-plane cache and the matrix digits,
-// re-read for every output slice) ahead of the streamed rows and outputs
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-// bulk copy global -> shared with completion on an mbarrier, read under the L2 policy `pol`
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes,
-                                          uint32_t bar, uint64_t pol) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
-      "[%1], %2, [%3], %4;" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "l"(pol)
-      : "memory");
-}
-// a 32-bit store to global memory under the L2 policy `pol`
-__device__ __forceinline__ void st_hint(uint32_t* p, uint32_t v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol)
-               : "memory");
-}
-// streamed (evict-first) loads of the rows' second read and stores of the outputs
-__device__ __forceinline__ double ld_stream(const double* p) { return __ldcs(p); }
-__device__ __forceinline__ float ld_stream(const float* p) { return __ldcs(p); }
-__device__ __forceinline__ df ld_stream(const df* p) {
-  const float2 v = __ldcs(reinterpret_cast<const float2*>(p));
-  return df(v.x, v.y);
-}
-__device__ __forceinline__ void st_stream(double* p, double v) { __stcs(p, v); }
-__device__ __forceinline__ void st_stream(float* p, float v) { __stcs(p, v); }
-__device__ __forceinline__ void st_stream(df* p, df v) {
-  __stcs(reinterpret_cast<float2*>(p), make_float2(v.h, v.l));
-}
-// eight 4-column loads of this warp's 32 lanes, then one wait that the values depend on
-__device__ __forceinline__ void tmem_ld8x4(uint32_t addr, int stride, uint32_t (&v)[8][4]) {
-#pragma unroll
-  for (int d = 0; d < 8; ++d)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3])
-                 : "r"(addr + (uint32_t)(d * stride)));
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]),
-                 "+r"(v[1][1]), "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]),
-                 "+r"(v[2][2]), "+r"(v[2][3]), "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]),
-                 "+r"(v[3][3]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[4][2]), "+r"(v[4][3]),
-                 "+r"(v[5][0]), "+r"(v[5][1]), "+r"(v[5][2]), "+r"(v[5][3]), "+r"(v[6][0]),
-                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3]), "+r"(v[7][0]), "+r"(v[7][1]),
-                 "+r"(v[7][2]), "+r"(v[7][3])
-               :
-               : "memory");
-}
-// ---- float bits -> biased fixed point, digits, and back ---------------------------------------
-template <typename T> struct FBits;
-template <> struct FBits<double> {
-  typedef unsigned long long U;
-  static constexpr int MB = 52, EMAX = 0x7FF, SH0 = 1, EOFF = 1022;
-  __device__ static U bits(double x) { return (U)__double_as_longlong(x); }
-  __device__ static int expo(U b) { return (int)((b >> 52) & 0x7FFull); }
-};
-template <> struct FBits<float> {
-  typedef unsigned int U;
-  static constexpr int MB = 23, EMAX = 0xFF, SH0 = 30, EOFF = 126;
-  __device__ static U bits(float x) { return __float_as_uint(x); }
-  __device__ static int expo(U b) { return (int)((b >> 23) & 0xFFu); }
-};
-// double-float h + l: the bits of h in the low word, of l in the high word; the row scale comes
-// from h (|h + l| < 2^E whenever |h| < 2^E, since |l| <= ulp(h) / 2)
-template <> struct FBits<df> {
-  typedef unsigned long long U;
-  static constexpr int EMAX = 0xFF, EOFF = 126;
-  __device__ static U bits(df x) {
-    return (U)__float_as_uint(x.h) | ((U)__float_as_uint(x.l) << 32);
-  }
-  __device__ static int expo(U b) { return (int)((b >> 23) & 0xFFull); }
-};
+constexpr int kPW = 8, kEW = 8;                   // producer and epilogue warps
+constexpr int kThreads = 32 * (kPW + kEW + 1);    // epilogue 0..7, producers 8..15, issuer 16
+constexpr int kStages = 5;                        // K stages in flight
+constexpr int kStageBytes = kABytes + b_stage_bytes(kNTMax);
+// per stage full, bfull, empty; accfull, accfree, rowfull[2], rowfree[2], fin
+constexpr int kBars = 3 * kStages + 7;
+// stages, row scales and middle terms (two tiles), barriers, the tensor-memory address
+constexpr size_t kSmem = (size_t)kStages * kStageBytes + 2 * kRows * (sizeof(long long) + sizeof(int)) +
+                         (size_t)(kBars + 1) * 8;
+// one pass's stage block kept in global memory: four fixed-point values of two rows per thread
+constexpr size_t kKeepStage = (size_t)kPW * 32 * 8 * sizeof(long long);
 
-// X + bias for an element with bit pattern b in a row whose largest exponent field is maxe
-// (X = round(x 2^(54-E)), E = maxe - EOFF; |X| < 2^54 so X + bias has eight 7-bit groups,
-// group i holding digit a_i + 64)
-template <typename T>
-__device__ __forceinline__ unsigned long long to_biased(typename FBits<T>::U b, int maxe) {
-  typedef FBits<T> F;
-  if (maxe >= F::EMAX) return kBias;
-  const int ef = (int)((b >> F::MB) & (typename F::U)F::EMAX);
-  unsigned long long mant = (unsigned long long)(b & ((((typename F::U)1) << F::MB) - 1));
-  if (ef) mant |= 1ull << F::MB;
-  const int s = (ef ? ef : 1) - maxe + F::SH0;
-  unsigned long long X;
-  if (s >= 0) {
-    X = mant << s;
-  } else {
-    const int sh = -s;
-    X = sh >= 64 ? 0ull : (mant + (1ull << (sh - 1))) >> sh;
-  }
-  const bool neg = (b >> (8 * sizeof(typename F::U) - 1)) & 1;
-  return neg ? kBias - X : kBias + X;
-}
+template <typename TO> __device__ __forceinline__ TO times(TO v, double f) { return v; }
+template <> __device__ __forceinline__ double times<double>(double v, double f) { return v * f; }
 
-// round(f 2^(54-E)) of a float with bit pattern b, E = maxe - 126, as a signed integer
-__device__ __forceinline__ long long fixed_f32(unsigned b, int maxe) {
-  const int ef = (int)((b >> 23) & 0xFFu);
-  unsigned long long mant = b & 0x7FFFFFu;
-  if (ef) mant |= 1ull << 23;
-  const int s = (ef ? ef : 1) - maxe + 30;
-  unsigned long long X;
-  if (s >= 0) {
-    X = mant << s;
-  } else {
-    const int sh = -s;
-    X = sh >= 64 ? 0ull : (mant + (1ull << (sh - 1))) >> sh;
-  }
-  return (b >> 31) ? -(long long)X : (long long)X;
-}
-// X + bias of a double-float: round(h 2^(54-E)) + round(l 2^(54-E)) (one extra unit of error
-// at most, 2^-54 of the row scale)
-template <>
-__device__ __forceinline__ unsigned long long to_biased<df>(unsigned long long b, int maxe) {
-  if (maxe >= 0xFF) return kBias;
-  return kBias + (unsigned long long)(fixed_f32((unsigned)b, maxe) +
-                                      fixed_f32((unsigned)(b >> 32), maxe));
-}
-
-// digits at bit offset sh (< 28) of two elements' 28-bit halves, as two bf16 packed in one word
-// (first in the low half): u = 7-bit group, value u - 64 through the float 2^23 + u
-__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int sh) {
-  const float f0 = __uint_as_float(0x4B000000u | ((w0 >> sh) & 127u)) - 8388672.0f;
-  const float f1 = __uint_as_float(0x4B000000u | ((w1 >> sh) & 127u)) - 8388672.0f;
-  return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-}
-
-// the 7-bit groups at bit offset sh of four elements' 28-bit halves as four bytes (first in the
-// lowest byte): the plane cache's format, half the size of the bf16 digits
-__device__ __forceinline__ uint32_t pack_groups(uint32_t w0, uint32_t w1, uint32_t w2,
-                                                uint32_t w3, int sh) {
-  return ((w0 >> sh) & 127u) | (((w1 >> sh) & 127u) << 8) | (((w2 >> sh) & 127u) << 16) |
-         (((w3 >> sh) & 127u) << 24);
-}
-// two bytes of the plane cache (7-bit groups u, digit u - 64) as two bf16 digits in one word
-__device__ __forceinline__ uint32_t group_pair(uint32_t b2) {
-  const float f0 = __uint_as_float(0x4B000000u | (b2 & 127u)) - 8388672.0f;
-  const float f1 = __uint_as_float(0x4B000000u | ((b2 >> 8) & 127u)) - 8388672.0f;
-  return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-}
-// a 32-bit load under the L2 policy `pol`
-__device__ __forceinline__ uint32_t ld_keep(const uint32_t* p, uint64_t pol) {
-  uint32_t v;
-  asm volatile("ld.global.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
-  return v;
-}
-
-// integer value of an fp32 accumulator: exact for integer values of magnitude <= 2^22 through
-// the float 1.5 2^23 + v (small K) ...
-__device__ __forceinline__ int acc_int_small(uint32_t b) {
-  return __float_as_int(__uint_as_float(b) + 12582912.0f) - 0x4B400000;
-}
-// ... and by one float-to-integer conversion for any integer value below 2^24 (larger K; the
-// accumulator holds an exact integer, so the conversion does not round)
-__device__ __forceinline__ int acc_int(uint32_t b) { return __float2int_rz(__uint_as_float(b)); }
-
-// T 2^e rounded to nearest even, by integer operations (ldexp fallback outside the normal range)
-template <typename TO> __device__ TO scaled(long long T, int e);
-template <> __device__ __forceinline__ double scaled<double>(long long T, int e) {
-  if (T == 0) return 0.0;
-  const unsigned long long sg = (unsigned long long)T & 0x8000000000000000ull;
-  unsigned long long a = sg ? 0ull - (unsigned long long)T : (unsigned long long)T;
-  const int lz = __clzll((long long)a);
-  a <<= lz;                                     // leading one at bit 63
-  unsigned long long mant = a >> 11;            // 53 bits
-  const unsigned rem = (unsigned)(a & 0x7FFull);
-  mant += (rem + (unsigned)(mant & 1ull)) > 0x400u ? 1ull : 0ull;   // to nearest, ties to even
-  const int be = 63 - lz + e + 1023 + (int)(mant >> 53);
-  if (be <= 0 || be >= 2047) return ldexp((double)T, e);
-  return __longlong_as_double((long long)(sg | ((unsigned long long)be << 52) |
-                                          (mant & 0xFFFFFFFFFFFFFull)));
-}
-template <> __device__ __forceinline__ float scaled<float>(long long T, int e) {
-  if (T == 0) return 0.0f;
-  const unsigned long long sg = (unsigned long long)T & 0x8000000000000000ull;
-  unsigned long long a = sg ? 0ull - (unsigned long long)T : (unsigned long long)T;
-  const int lz = __clzll((long long)a);
-  a <<= lz;
-  unsigned long long mant = a >> 40;            // 24 bits
-  const unsigned long long rem = a & 0xFFFFFFFFFFull;
-  mant += (rem + (mant & 1ull)) > (1ull << 39) ? 1ull : 0ull;
-  const int be = 63 - lz + e + 127 + (int)(mant >> 24);
-  if (be <= 0 || be >= 255) return ldexpf((float)T, e);
-  return __uint_as_float((unsigned)(sg >> 32) | ((unsigned)be << 23) |
-                         (unsigned)(mant & 0x7FFFFFull));
-}
-// double-float result: the high part rounded to float from the integer, the low part from the
-// exact integer remainder
-template <> __device__ __forceinline__ df scaled<df>(long long T, int e) {
-  if (T == 0) return df(0.0f, 0.0f);
-  const bool neg = T < 0;
-  unsigned long long a = neg ? 0ull - (unsigned long long)T : (unsigned long long)T;
-  const int lz = __clzll((long long)a);   // |T| < 2^62.3: lz >= 1
-  const unsigned long long n = a << lz;
-  unsigned long long mant = n >> 40;
-  const unsigned long long rem = n & 0xFFFFFFFFFFull;
-  mant += (rem + (mant & 1ull)) > (1ull << 39) ? 1ull : 0ull;
-  // |T| rounded to 24 significant bits; mant may have rounded up to 2^24, so shift by 39 first
-  const unsigned long long ahi = (mant << 39) >> (lz - 1);
-  const long long Thi = neg ? -(long long)ahi : (long long)ahi;
-  return df(scaled<float>(Thi, e), scaled<float>(T - Thi, e));
-}
-// the forward transform's last output carries the factor 1 / (2N) (forward outputs are float64)
-template <typename TO> __device__ __forceinline__ TO last_scale(TO v, double f) { return v; }
-template <> __device__ __forceinline__ double last_scale<double>(double v, double f) {
-  return v * f;
-}
-template <typename TO> __device__ __forceinline__ TO qnan();
-template <> __device__ __forceinline__ double qnan<double>() {
-  return __longlong_as_double(0x7FF8000000000000ll);
-}
-template <> __device__ __forceinline__ float qnan<float>() { return __uint_as_float(0x7FC00000u); }
-template <> __device__ __forceinline__ df qnan<df>() {
-  return df(__uint_as_float(0x7FC00000u), __uint_as_float(0x7FC00000u));
-}
-
-constexpr int kBars = 2 * kNB + 2 * kNA + 3;   // barriers (see the kernel)
-__host__ __device__ constexpr size_t tc_smem_bytes(int NT) {
-  // B planes (kNB chunks), A planes (kNA buffers), row exponents, the barriers and the
-  // tensor-memory address, output-column exponents (at most 512)
-  return (size_t)kNB * 8 * NT * TCKC * 2 + (size_t)kNA * TCM * TCKC * 2 + TCM * sizeof(int) +
-         (size_t)(kBars + 1) * 8 + 512 * sizeof(int);
-}
-
-// ---- the transform kernel ---------------------------------------------------------------------
 // in / out: nf fields of complex lines (re, im interleaved), field stride fsi / fso complex
-// elements, line stride Nz; bdig: nNt output slices of 8 NT Kp bf16 digits (per slice and chunk
-// of K: the eight digit planes stacked as one 8 NT x KC matrix in the canonical no-swizzle
-// K-major core-matrix layout, plane j in rows j NT ..); fexp: F_n; cache: per CTA, nchunk x 8
-// A digit planes of one tile as 7-bit groups, four per 32-bit word (kCacheWords words each).
-//
-// Persistent CTAs (17 warps) walk the tiles of 128 rows; per tile they loop over the nNt output
-// slices.  Warps 0..15 turn the rows into fixed-point values and, for the first slice, write the
-// eight digit planes into kNA rotating shared buffers and their groups into the CTA's plane cache
-// (each thread reads back only what it wrote, so program order orders the two); for each later
-// slice they rebuild its first kNA planes as soon as the previous slice's MMAs are done, drain
-// the previous slice's accumulators, then rebuild the rest as the MMAs free the buffers.  Lane 0
-// of warp 16 allocates the tensor memory and issues the bulk copies of B and the MMAs.  Plane t
-// (counted over tiles, slices and chunks) uses shared buffer t % kNA: its producers wait for
-// `empty` of that buffer (the MMAs of plane t - kNA completed, signalled by tcgen05.commit) and
-// announce it on `full` (one arrival per producer warp).  The digits of B of chunk u (counted
-// over tiles, slices and chunks) go to buffer u % kNB once `bfree` of that buffer says the MMAs
-// of chunk u - kNB are done.  A slice's MMAs start once every producer warp has arrived on
-// `drained` for the previous slice.
-template <typename TI, typename TO, int NT>
-__global__ void __launch_bounds__(TCT + 32, 1)
+// elements, line stride Nz = N + 1; dig: the matrix digits, stage blocks of 7 NT rows x 16 K in
+// the order slice, parity, stage; keep: keep_bytes per CTA; nst stages per parity in kc groups of
+// gst; q: log2 of the matrix scale; ymid: middle weight times 2^q; lastf: factor of output N
+// (forward).
+template <typename TI, typename TO>
+__global__ void __launch_bounds__(kThreads, 1)
     cheb_tc_kernel(const TI* __restrict__ in, long long fsi, TO* __restrict__ out, long long fso,
-                   int nlines, int Nz, int Kp, int tpf, int ntiles, int nNt,
-                   const uint16_t* __restrict__ bdig, const int* __restrict__ fexp,
-                   uint32_t* __restrict__ cache, int fwd, double lastf, int* __restrict__ err) {
+                   int nlines, int Nz, int tpf, int ntiles, int NT, int nsl, int nst, int kc,
+                   int gst, const uint16_t* __restrict__ dig, char* __restrict__ keep,
+                   long long keep_bytes, int fwd, int q, long long ymid, double lastf,
+                   int* __restrict__ err) {
   typedef FBits<TI> F;
   typedef typename F::U U;
   extern __shared__ __align__(1024) unsigned char tsm[];
-  unsigned char* sB = tsm;
-  constexpr uint32_t kBBytes = 8 * NT * TCKC * 2;   // one chunk of B planes
-  unsigned char* sA = sB + (size_t)kNB * kBBytes;
-  int* sE = reinterpret_cast<int*>(sA + (size_t)kNA * TCM * TCKC * 2);
-  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + TCM);
+  unsigned char* stages = tsm;
+  long long* sC = reinterpret_cast<long long*>(tsm + (size_t)kStages * kStageBytes);
+  int* sE = reinterpret_cast<int*>(sC + 2 * kRows);
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + 2 * kRows);
   uint32_t* sT = reinterpret_cast<uint32_t*>(bars + kBars);
-  int* sF = reinterpret_cast<int*>(bars + kBars + 1);   // F_n of every output column (<= 512)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nchunk = (Kp + TCKC - 1) / TCKC;
-  constexpr uint32_t kPlaneBytes = TCM * TCKC * 2;
-  // barriers (8 bytes each, buffer b of a kind at + 8 b): bload[kNB] (B chunk copied),
-  // bfree[kNB] (MMAs of the chunk done); full[kNA] (16 producer warps); empty[kNA] (MMAs of the
-  // plane done); drained (16 producer warps read the accumulators); sliced (every MMA of a slice
-  // done: one phase per slice, so the producers' epilogue waits never alias a buffer's phases);
-  // fin (the issuer's MMAs in flight, after a wait ran out)
-  const uint32_t barB = su32(&bars[0]), barBfree = su32(&bars[kNB]);
-  const uint32_t barFull = su32(&bars[2 * kNB]);
-  const uint32_t barEmpty = su32(&bars[2 * kNB + kNA]);
-  const uint32_t barDrain = su32(&bars[2 * kNB + 2 * kNA]);
-  const uint32_t barSlice = barDrain + 8, barFin = barDrain + 16;
-  const size_t bslice = (size_t)8 * NT * Kp;
-  uint32_t* ccta = cache + (size_t)blockIdx.x * nchunk * 8 * kCacheWords;
-  const bool issuer_warp = (warp == TCT / 32);
-  const bool issuer = issuer_warp && lane == 0;
-  if (issuer) {
-    for (int b = 0; b < kNB; ++b) {
+  const int N = Nz - 1, H = N / 2;
+  const uint32_t barFull = su32(bars), barB = barFull + 8 * kStages;
+  const uint32_t barEmpty = barFull + 16 * kStages, barAccFull = barFull + 24 * kStages;
+  const uint32_t barAccFree = barAccFull + 8, barRow = barAccFull + 16, barRowFree = barAccFull + 32;
+  const uint32_t barFin = barAccFull + 48;
+  if (tid == 0) {
+    for (int b = 0; b < kStages; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barFull + 8 * b), "r"(kPW));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barB + 8 * b));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barBfree + 8 * b));
-    }
-    for (int b = 0; b < kNA; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;" ::"r"(barFull + 8 * b));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barEmpty + 8 * b));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;" ::"r"(barDrain));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barSlice));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barAccFull));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barAccFree), "r"(kEW));
+    for (int b = 0; b < 2; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRow + 8 * b), "r"(kPW));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRowFree + 8 * b), "r"(kEW));
+    }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barFin));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  const bool issuer_warp = warp == kPW + kEW;
   if (issuer_warp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      su32(sT)),
                  "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  if (tid < TCT)
-    for (int c = tid; c < nNt * NT; c += TCT) sF[c] = fexp[c];
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();   // barriers, tensor-memory address and sF visible to every warp
+  __syncthreads();   // barriers and tensor-memory address visible to every warp
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *sT;
-  const uint32_t sA0 = su32(sA), sB0 = su32(sB);
-  const uint64_t keep = policy_evict_last();
+  const uint32_t sBase = su32(stages);
+  const uint32_t bbytes = (uint32_t)b_stage_bytes(NT);
+  char* kcta = keep + (long long)blockIdx.x * keep_bytes;
   Waiter W;
 
   if (issuer_warp) {
     if (lane == 0) {
-      // bf16 x bf16 -> fp32, both K-major, M = 128 (N added per MMA)
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TCM >> 4) << 24);
-      int t = 0, u = 0, S = 0;           // plane, B chunk and slice counters (all tiles)
-      int nfull[kNA] = {};
-      int nbl[kNB] = {}, ibl[kNB] = {};  // B chunks waited for / issued per buffer
-      bool any_mma = false;
-      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        for (int sl = 0; sl < nNt; ++sl, ++S) {
-          for (int ch = 0; ch < nchunk; ++ch, ++u) {
-            const int KCc = min(TCKC, Kp - ch * TCKC);
-            const int bb = u % kNB;
-            // B buffer bb: the MMAs of chunk u - kNB read it
-            if (u >= kNB && !W.wait(barBfree + 8 * bb, ((u - kNB) / kNB) & 1)) goto drain;
-            bulk_load(sB0 + (uint32_t)(bb * kBBytes),
-                      bdig + (size_t)sl * bslice + (size_t)ch * 8 * NT * TCKC,
-                      (uint32_t)(8 * NT * KCc * 2), barB + 8 * bb, keep);
-            ++ibl[bb];
-            if (!W.wait(barB + 8 * bb, nbl[bb] & 1)) goto drain;
-            ++nbl[bb];
-            if (ch == 0 && S > 0 && !W.wait(barDrain, (S - 1) & 1)) goto drain;
-            for (int i = 0; i < 8; ++i, ++t) {
-              const int bf = t % kNA;
-              if (!W.wait(barFull + 8 * bf, nfull[bf] & 1)) goto drain;
-              ++nfull[bf];
+      uint32_t slot = 0, use = 0;   // stage slot and how often it was used
+      uint32_t pass = 0;
+      bool any = false;
+      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+        for (int pp = 0; pp < 2 * nsl; ++pp)
+          for (int c = 0; c < kc; ++c, ++pass) {
+            if (pass > 0 && !W.wait(barAccFree, (pass - 1) & 1)) goto drain;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int s0 = c * gst, s1 = min(nst, s0 + gst);
+            for (int st = s0; st < s1; ++st) {
+              if (!W.wait(barFull + 8 * slot, use & 1) || !W.wait(barB + 8 * slot, use & 1))
+                goto drain;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              // A plane i times B planes 0 .. 7-i at once: the stacked B rows j NT + n land in
-              // accumulator columns i NT + j NT + n = (i + j) NT + n, the diagonal of (i, j).
-              // N = (8 - i) NT is issued in pieces of at most 256.  A k-step adds 2 core-matrix
-              // groups to both start addresses (4096 bytes of A, 2 NT 128 bytes of B).
-              const uint64_t ad = sdesc(sA0 + (uint32_t)(bf * kPlaneBytes), 2048, 128);
-              const uint32_t sBb = sB0 + (uint32_t)(bb * kBBytes);
-              const int ntot = (8 - i) * NT;
-              for (int s = 0; s < KCc / 16; ++s)
-                for (int n0 = 0; n0 < ntot; n0 += 256) {
-                  const int nlen = min(256, ntot - n0);
-                  const uint64_t bd = sdesc(sBb + (uint32_t)(n0 / 8 * 128), NT * 128, 128);
-                  mma_bf16(tmem + (uint32_t)(i * NT + n0), ad + (uint64_t)(s * 256),
-                           bd + (uint64_t)(s * 16 * NT), idesc0 | ((uint32_t)(nlen >> 3) << 17),
-                           (uint32_t)((ch | i | s) != 0));
-                }
-              any_mma = true;
-              mma_commit(barEmpty + 8 * bf);
-              if (i == 7) mma_commit(barBfree + 8 * bb);
-              if (i == 7 && ch == nchunk - 1) mma_commit(barSlice);
+              const uint32_t sA = sBase + slot * (uint32_t)kStageBytes;
+              issue_stage(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
+              any = true;
+              mma_commit(barEmpty + 8 * slot);
+              if (++slot == kStages) {
+                slot = 0;
+                ++use;
+              }
             }
+            mma_commit(barAccFull);
           }
-        }
-      }
     drain:
-      if (!W.ok) {
-        // A wait ran out: nothing more is issued.  Before the tensor memory is released and the
-        // CTA ends, wait (one shared bound for all of them) for the MMAs and the bulk copies
-        // still in flight: the MMAs through one last commit, each copy on its own barrier phase.
-        const uint64_t dl = gtime() + kWaitNs;
-        if (any_mma) {
-          mma_commit(barFin);
-          mbar_wait_until(barFin, 0, dl);
-        }
-        for (int b = 0; b < kNB; ++b)
-          if (ibl[b] > nbl[b]) mbar_wait_until(barB + 8 * b, nbl[b] & 1, dl);
+      if (!W.ok && any) {
+        // a wait ran out: nothing more is issued; wait (bounded) for the MMAs in flight before
+        // the tensor memory is released
+        mma_commit(barFin);
+        mbar_wait_until(barFin, 0, gtime() + kWaitNs);
       }
     }
     __syncwarp();
-  } else {
-    // producers: warp = 8-row core-matrix group, lane = (row in the group, pair of k)
-    const int r = lane >> 2, q = lane & 3;
-    const int m = warp * 8 + r;
-    constexpr int CW = NT / 4;
-    const int qd = warp & 3, cg = warp >> 2;
-    const int mm = qd * 32 + lane;
-    const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cg * CW);
-    // the largest exponent field of this thread's row of tile `tl` over all of K (the row's
-    // first, cold read)
-    auto row_exponent = [&](int tl) {
-      const int fld = tl / tpf;
-      const int line = (tl - fld * tpf) * (TCM / 2) + (m >> 1);
-      const bool rowok = line < nlines;
-      const TI* src = in + ((size_t)fld * fsi + (size_t)(rowok ? line : 0) * Nz) * 2 + (m & 1);
-      int mx = 1;
-      for (int ch = 0; ch < nchunk; ++ch) {
-        const int ngc = min(TCKC, Kp - ch * TCKC) / 8;
+  } else if (warp >= kEW) {
+    // ---- producers: thread = (line l of the tile, g): K positions 4 g .. 4 g + 3 of a stage,
+    // position 4 g + e holding k = 16 st + g + 4 e (so the four threads of a line read
+    // consecutive elements).  Rows 2 l (re) and 2 l + 1 (im); threads g >= 2 take the im row
+    // first, so that a half-warp's 8-byte stores fall on different banks.
+    const int p = tid - 32 * kEW, pw = warp - kEW;
+    const int l = pw * 8 + (lane >> 2), g = lane & 3, sw = g >> 1;
+    const int ra = 2 * l + sw, rb = 2 * l + 1 - sw;
+    const uint32_t oa = (uint32_t)(sw * (int)kALbo + ra * 16 + (g & 1) * 8);
+    const uint32_t ob = (uint32_t)(sw * (int)kALbo + rb * 16 + (g & 1) * 8);
+    const uint64_t pol = policy_evict_last();
+    longlong2* kp = reinterpret_cast<longlong2*>(kcta) + p;
+    uint32_t slot = 0, use = 0;
+    int ti = 0;
+    // the stage's digit planes of v (0..3 row a, 4..7 row b) and, by one thread, the copy of its
+    // matrix digits; false after a wait ran out
+    auto put = [&](const long long (&v)[8], const uint16_t* bsrc) {
+      if (use > 0 && !W.wait_warp(barEmpty + 8 * slot, (use & 1) ^ 1)) return false;
+      unsigned char* sA = stages + (size_t)slot * kStageBytes;
+      if (p == 0) bulk_load(su32(sA) + (uint32_t)kABytes, bsrc, bbytes, barB + 8 * slot, pol);
+      uint32_t lo[8], hi[8];
 #pragma unroll
-        for (int gl = 0; gl < TCG; ++gl)
+      for (int e = 0; e < 8; ++e) {
+        const unsigned long long y = (unsigned long long)v[e] + kBias;
+        lo[e] = (uint32_t)y;
+        hi[e] = (uint32_t)(y >> 32);
+      }
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int k = ch * TCKC + 8 * gl + 2 * q + e;
-            if (gl < ngc && rowok && k < Nz) mx = max(mx, F::expo(F::bits(src[2 * (size_t)k])));
-          }
+      for (int i = 0; i < kPlanes; ++i) {
+        const int b = 6 - i;
+        const uint32_t* w = b < 4 ? lo : hi;
+        *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + oa) =
+            make_uint2(digit_pair(w[0], w[1], b & 3), digit_pair(w[2], w[3], b & 3));
+        *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + ob) =
+            make_uint2(digit_pair(w[4], w[5], b & 3), digit_pair(w[6], w[7], b & 3));
       }
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      return max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    };
-    // L2 prefetch (evict-last) of the row elements of chunk ch of tile tl that this thread
-    // converts: issued one chunk ahead, so the conversion's loads, which the registers allow only
-    // a few at a time, find the rows in L2 instead of DRAM
-    auto prefetch_rows = [&](int tl, int ch) {
-      const int fld = tl / tpf;
-      const int line = (tl - fld * tpf) * (TCM / 2) + (m >> 1);
-      if (line >= nlines) return;
-      const TI* src = in + ((size_t)fld * fsi + (size_t)line * Nz) * 2 + (m & 1);
-      const int ngp = min(TCKC, Kp - ch * TCKC) / 8;
-      for (int gl = 0; gl < ngp; ++gl) {
-        const int k = ch * TCKC + 8 * gl + 2 * q;
-        if (k < Nz)
-          asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(src + 2 * (size_t)k));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barFull + 8 * slot)
+                     : "memory");
+      if (++slot == kStages) {
+        slot = 0;
+        ++use;
       }
+      return true;
     };
-    int t = 0, S = 0;
-    int ahead = -1;   // the next tile's row exponent, read during this tile's last slice
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    auto keep_at = [&](int par, int st) { return kp + (size_t)(par * nst + st) * (4 * kPW * 32); };
+    auto store_keep = [&](longlong2* d, const long long (&v)[8]) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) __stcg(d + i * kPW * 32, make_longlong2(v[2 * i], v[2 * i + 1]));
+    };
+    const size_t bstride = (size_t)bbytes / 2;   // elements of a stage block
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
       const int fld = tile / tpf;
-      const int line0 = (tile - fld * tpf) * (TCM / 2);
-      const int line = line0 + (m >> 1);
+      const int line = (tile - fld * tpf) * (kRows / 2) + l;
       const bool rowok = line < nlines;
-      const TI* src = in + ((size_t)fld * fsi + (size_t)(rowok ? line : 0) * Nz) * 2 + (m & 1);
-      const int maxe = ahead >= 0 ? ahead : row_exponent(tile);
-      ahead = -1;
-      // sE: every producer warp has read the previous tile's entries (before its slice loop)
-      asm volatile("bar.sync 1, %0;" ::"r"(TCT) : "memory");
-      if (q == 0) sE[m] = maxe;
-      asm volatile("bar.sync 1, %0;" ::"r"(TCT) : "memory");
-      const int me = sE[mm];
-      // first slice: generate the planes of every chunk (cached for the later slices); the last
-      // output n = N, sum_k w_k X_k with w_k = e_k (-1)^k (forward) or (-1)^k (backward), is
-      // summed exactly here as S_hi 2^27 + S_lo
-      long long s_hi = 0, s_lo = 0;
-      for (int ch = 0; ch < nchunk; ++ch) {
-        const int ngr = min(TCKC, Kp - ch * TCKC) / 8;
-        uint32_t yh[2 * TCG], yl[2 * TCG];   // bits 28..55 and 0..27 of X + bias
-#pragma unroll
-        for (int gl = 0; gl < TCG; ++gl)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int k = ch * TCKC + 8 * gl + 2 * q + e;
-            U b = 0;
-            if (gl < ngr && rowok && k < Nz) b = F::bits(ld_stream(src + 2 * (size_t)k));
-            const unsigned long long y = to_biased<TI>(b, maxe);
-            yh[2 * gl + e] = (uint32_t)(y >> 28);
-            yl[2 * gl + e] = (uint32_t)y & 0xFFFFFFFu;
-            if (gl < ngr && k < Nz) {
-              const long long xs = (long long)(y - kBias);
-              const int w = ((k & 1) ? -1 : 1) * ((fwd && k != 0 && k != Nz - 1) ? 2 : 1);
-              s_hi += w * (xs >> 27);
-              s_lo += w * (xs & 0x7FFFFFFll);
-            }
-          }
-        if (ch + 1 < nchunk) prefetch_rows(tile, ch + 1);
-        for (int i = 0; i < 8; ++i, ++t) {
-          const int bf = t % kNA;
-          if (t >= kNA) W.wait(barEmpty + 8 * bf, ((t - kNA) / kNA) & 1);
-          uint32_t* dst = reinterpret_cast<uint32_t*>(sA + (size_t)bf * kPlaneBytes);
-          uint32_t* gdst = ccta + (size_t)(ch * 8 + i) * kCacheWords;
-          const int sh = 7 * (3 - (i & 3));
-#pragma unroll
-          for (int g2 = 0; g2 < TCG / 2; ++g2)
-            if (2 * g2 < ngr) {
-              const int gl = 2 * g2;
-              const uint32_t* yy = i < 4 ? yh : yl;
-              dst[(gl * 16 + warp) * 32 + lane] = digit_pair(yy[2 * gl], yy[2 * gl + 1], sh);
-              dst[((gl + 1) * 16 + warp) * 32 + lane] =
-                  digit_pair(yy[2 * gl + 2], yy[2 * gl + 3], sh);
-              // the four 7-bit groups as bytes, read back by this same thread for the later
-              // slices (program order: no fence)
-              st_hint(gdst + (g2 * 16 + warp) * 32 + lane,
-                      pack_groups(yy[2 * gl], yy[2 * gl + 1], yy[2 * gl + 2], yy[2 * gl + 3], sh),
-                      keep);
-            }
-          // the shared-memory plane for the MMAs (async proxy)
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barFull + 8 * bf)
-                         : "memory");
+      const TI* src = in + ((size_t)fld * fsi + (size_t)(rowok ? line : 0) * Nz) * 2;
+      // the rows' scales (their first, cold read)
+      unsigned ka = 0, kb = 0;
+      if (rowok) {
+#pragma unroll 8
+        for (int k = g; k < Nz; k += 4) {
+          ka = max(ka, F::key(F::bits(src[2 * k + sw])));
+          kb = max(kb, F::key(F::bits(src[2 * k + 1 - sw])));
         }
       }
-      s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 1);
-      s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 1);
-      s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
-      s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
-      if (q == 0 && rowok && W.ok) {
-        // sum_k w_k x_k = 2^(E - 54) (S_hi 2^27 + S_lo) = T 2^(E - 51), T = S_hi 2^24 + S_lo / 8
-        // (|sum w X| < 2 Kp 2^54 < 2^64, so three low bits are dropped: 2^-51 of the row scale)
-        const long long T = s_hi * 16777216ll + (s_lo >> 3);
-        TO v = maxe >= F::EMAX ? qnan<TO>() : scaled<TO>(T, maxe - F::EOFF - 51);
-        if (fwd) v = last_scale<TO>(v, lastf);
-        st_stream(out + ((size_t)fld * fso + (size_t)line * Nz) * 2 + (m & 1) + 2 * (size_t)(Nz - 1),
-                  v);
+      // threads g >= 2 hold the rows the other way round
+      unsigned kre = sw ? kb : ka, kim = sw ? ka : kb;
+#pragma unroll
+      for (int off = 1; off < 4; off <<= 1) {
+        kre = max(kre, __shfl_xor_sync(0xffffffffu, kre, off));
+        kim = max(kim, __shfl_xor_sync(0xffffffffu, kim, off));
       }
-      const int oline = line0 + (mm >> 1);
-      TO* dstp =
-          out + ((size_t)fld * fso + (size_t)(oline < nlines ? oline : 0) * Nz) * 2 + (mm & 1);
-      // the later slices' planes, rebuilt from the packed groups of the first slice: plane c
-      // (chunk c / 8, plane c % 8) of the slice that starts at plane number t0s
-      const int tplanes = 8 * nchunk;
-      int tnext = t;                     // next plane to rebuild (the slice after the current)
-      auto rebuild = [&](int upto) {
-        for (; tnext < upto; ++tnext) {
-          const int c = tnext % tplanes;   // planes of a tile are numbered slice by slice
-          const int chc = c >> 3;
-          const int ngc = min(TCKC, Kp - chc * TCKC) / 8;
-          const int bf = tnext % kNA;
-          const uint32_t* gsrc = ccta + (size_t)c * kCacheWords;
-          uint32_t wv[TCG / 2];
+      const int ere = row_scale<TI>(kre), eim = row_scale<TI>(kim);
+      const int ea = sw ? eim : ere, eb = sw ? ere : eim;
+      // the middle element, its integer term for the even outputs, and the row scales
+      long long xmr = 0, xmi = 0;
+      if (g == 0) {
+        if (rowok) {
+          xmr = to_fixed<TI>(F::bits(src[2 * H]), ere);
+          xmi = to_fixed<TI>(F::bits(src[2 * H + 1]), eim);
+        }
+      }
+      if (ti >= 2 && !W.wait_warp(barRowFree + 8 * (ti & 1), ((ti >> 1) - 1) & 1)) break;
+      if (g == 0) {
+        // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
+        sC[(ti & 1) * kRows + 2 * l] = __mul64hi(xmr * 256, ymid * 4);
+        sC[(ti & 1) * kRows + 2 * l + 1] = __mul64hi(xmi * 256, ymid * 4);
+        sE[(ti & 1) * kRows + 2 * l] = ere;
+        sE[(ti & 1) * kRows + 2 * l + 1] = eim;
+      }
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRow + 8 * (ti & 1))
+                     : "memory");
+      // first pass: convert, fold, write the sums' planes, keep the differences
+      long long suma = 0, sumb = 0, s0a = 0, s0b = 0;
+      U xa[4], ya[4], xb[4], yb[4];
+      auto load = [&](int st) {
 #pragma unroll
-          for (int g2 = 0; g2 < TCG / 2; ++g2)
-            wv[g2] = (2 * g2 < ngc) ? ld_keep(gsrc + (g2 * 16 + warp) * 32 + lane, keep) : 0u;
-          if (tnext >= kNA) W.wait(barEmpty + 8 * bf, ((tnext - kNA) / kNA) & 1);
-          uint32_t* dst = reinterpret_cast<uint32_t*>(sA + (size_t)bf * kPlaneBytes);
-#pragma unroll
-          for (int g2 = 0; g2 < TCG / 2; ++g2)
-            if (2 * g2 < ngc) {
-              const int gl = 2 * g2;
-              dst[(gl * 16 + warp) * 32 + lane] = group_pair(wv[g2] & 0xFFFFu);
-              dst[((gl + 1) * 16 + warp) * 32 + lane] = group_pair(wv[g2] >> 16);
-            }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barFull + 8 * bf)
-                         : "memory");
+        for (int e = 0; e < 4; ++e) {
+          const int k = 16 * st + g + 4 * e;
+          const bool ok = rowok && k < H;
+          xa[e] = xb[e] = ya[e] = yb[e] = 0;
+          if (ok) {
+            xa[e] = F::bits(src[2 * k + sw]);
+            xb[e] = F::bits(src[2 * k + 1 - sw]);
+            ya[e] = F::bits(src[2 * (N - k) + sw]);
+            yb[e] = F::bits(src[2 * (N - k) + 1 - sw]);
+          }
         }
       };
-      for (int sl = 0; sl < nNt; ++sl, ++S) {
-        if (sl == nNt - 1 && tile + (int)gridDim.x < ntiles) prefetch_rows(tile + gridDim.x, 0);
-        // every MMA of the slice done
-        W.wait(barSlice, S & 1);
-        // the next slice's first planes into the buffers its MMAs start with (free now)
-        if (sl + 1 < nNt) rebuild(t + min(kNA, tplanes));
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
-        // (w / 4) NT/4 .. + NT/4 - 1 of each of the eight accumulators, 4 at a time (after a
-        // failed wait the producers keep their loop structure, which their named barrier
-        // needs, but wait no more and store nothing)
-        const bool orow = W.ok && oline < nlines;
-        for (int c0 = 0; c0 < CW; c0 += 4) {
-          uint32_t v[8][4];
-          tmem_ld8x4(tb + (uint32_t)c0, NT, v);
+      load(0);
+      bool ok = true;
+      for (int st = 0; st < nst && ok; ++st) {
+        long long s[8], d[8];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int n = sl * NT + cg * CW + c0 + e;
-            if (orow && n < Nz - 1) {
-              int g[8];
-              if (Kp <= kSmallK) {
+        for (int e = 0; e < 4; ++e) {
+          const long long x = to_fixed<TI>(xa[e], ea), y = to_fixed<TI>(ya[e], ea);
+          const long long z = to_fixed<TI>(xb[e], eb), w = to_fixed<TI>(yb[e], eb);
+          s[e] = x + y;
+          d[e] = x - y;
+          s[4 + e] = z + w;
+          d[4 + e] = z - w;
+          suma += s[e];       // at most 62 values below 2^55 per thread
+          sumb += s[4 + e];
+        }
+        if (st == 0) {
+          s0a = s[0];
+          s0b = s[4];
+        }
+        store_keep(keep_at(1, st), d);
+        if (nsl > 1) store_keep(keep_at(0, st), s);
+        if (st + 1 < nst) load(st + 1);
+        ok = put(s, dig + (size_t)st * bstride);
+      }
+      if (!ok) break;
+      // the last output n = N: sum_k w_k (-1)^k x_k, (-1)^k = (-1)^g for this thread's k; weights
+      // e_k = 2 except k = 0, N (forward) or 1
+      {
+        long long tre = sw ? sumb : suma, tim = sw ? suma : sumb;
+        if (g & 1) {
+          tre = -tre;
+          tim = -tim;
+        }
+        const int m2 = (H & 1) ? -1 : 1;
+        // |partial| < 2^61 here; halves of 27 low bits keep the sums over threads in range
+        long long hr = tre >> 27, lr = tre & 0x7FFFFFF, hi_ = tim >> 27, li = tim & 0x7FFFFFF;
+        if (fwd) {
+          hr *= 2; lr *= 2; hi_ *= 2; li *= 2;
+        }
+        if (g == 0) {
+          const int wm = fwd ? 2 * m2 : m2;
+          hr += wm * (xmr >> 27); lr += wm * (xmr & 0x7FFFFFF);
+          hi_ += wm * (xmi >> 27); li += wm * (xmi & 0x7FFFFFF);
+          if (fwd) {   // s_0 counted twice (g = 0: rows in order)
+            hr -= s0a >> 27; lr -= s0a & 0x7FFFFFF;
+            hi_ -= s0b >> 27; li -= s0b & 0x7FFFFFF;
+          }
+        }
 #pragma unroll
-                for (int d = 0; d < 8; ++d) g[d] = acc_int_small(v[d][e]);
-              } else {
+        for (int off = 1; off < 4; off <<= 1) {
+          hr += __shfl_xor_sync(0xffffffffu, hr, off);
+          lr += __shfl_xor_sync(0xffffffffu, lr, off);
+          hi_ += __shfl_xor_sync(0xffffffffu, hi_, off);
+          li += __shfl_xor_sync(0xffffffffu, li, off);
+        }
+        if (g == 0 && rowok) {
+          // sum = 2^(E - 54) (h 2^27 + l) = T 2^(E - 51), T = h 2^24 + l / 8
+          TO vr = ere == kNanRow ? qnan<TO>()
+                                 : scaled<TO>(hr * 16777216ll + ((lr + 4) >> 3), ere - F::EOFF - 51);
+          TO vi = eim == kNanRow ? qnan<TO>()
+                                 : scaled<TO>(hi_ * 16777216ll + ((li + 4) >> 3), eim - F::EOFF - 51);
+          if (fwd) {
+            vr = times<TO>(vr, lastf);
+            vi = times<TO>(vi, lastf);
+          }
+          TO* o = out + ((size_t)fld * fso + (size_t)line * Nz + N) * 2;
+          o[0] = vr;
+          o[1] = vi;
+        }
+      }
+      // the later passes: slice 0 odd, then even and odd of each further slice, from the kept values
+      for (int pp = 1; pp < 2 * nsl && ok; ++pp) {
+        const int par = pp & 1;
+        longlong2 nx[4];
+        auto fetch = [&](int st) {
+          const longlong2* s = keep_at(par, st);
 #pragma unroll
-                for (int d = 0; d < 8; ++d) g[d] = acc_int(v[d][e]);
+          for (int i = 0; i < 4; ++i) nx[i] = __ldcg(s + i * kPW * 32);
+        };
+        fetch(0);
+        for (int st = 0; st < nst && ok; ++st) {
+          long long v[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            v[2 * i] = nx[i].x;
+            v[2 * i + 1] = nx[i].y;
+          }
+          if (st + 1 < nst) fetch(st + 1);
+          ok = put(v, dig + ((size_t)pp * nst + st) * bstride);
+        }
+      }
+      if (!ok) break;
+    }
+    // after a failed wait the copies still in flight finish (bounded) before the CTA ends
+    if (!W.ok && p == 0) {
+      const uint64_t dl = gtime() + kWaitNs;
+      for (int b = 0; b < kStages; ++b) {
+        const uint32_t n = use + (b < (int)slot ? 1u : 0u);   // copies issued to slot b
+        if (n > 0) mbar_wait_until(barB + 8 * b, (n - 1) & 1, dl);
+      }
+    }
+  } else {
+    // ---- epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
+    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators, four at a time
+    const int qd = warp & 3, cg = warp >> 2, CW = NT / 2;
+    const int row = qd * 32 + lane;
+    const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cg * CW);
+    // sums over several K groups are kept here between the groups
+    long long* part = reinterpret_cast<long long*>(kcta + (size_t)2 * nst * kKeepStage) + tid;
+    uint32_t pass = 0;
+    int ti = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
+      const int fld = tile / tpf;
+      const int line = (tile - fld * tpf) * (kRows / 2) + (row >> 1);
+      if (!W.wait_warp(barRow + 8 * (ti & 1), (ti >> 1) & 1)) break;
+      const int me = sE[(ti & 1) * kRows + row];
+      const long long mid = sC[(ti & 1) * kRows + row];
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * (ti & 1))
+                     : "memory");
+      const bool rowok = line < nlines, nan = me == kNanRow;
+      const int ex = me - F::EOFF - q;   // result = T 2^(E - q)
+      TO* dst = out + ((size_t)fld * fso + (size_t)(rowok ? line : 0) * Nz) * 2 + (row & 1);
+      bool ok = true;
+      for (int pp = 0; pp < 2 * nsl && ok; ++pp) {
+        const int par = pp & 1, m0 = (pp >> 1) * NT + cg * CW;
+        for (int c = 0; c < kc; ++c, ++pass) {
+          if (!(ok = W.wait_warp(barAccFull, pass & 1))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          for (int c0 = 0; c0 < CW; c0 += 4) {
+            uint32_t v[7][4];
+            tmem_ld7x4(tb + (uint32_t)c0, NT, v);
+            if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
+              asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+              __syncwarp();
+              if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barAccFree)
+                             : "memory");
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int m = m0 + c0 + e;
+              if (m < H && rowok) {
+                long long T = recombine(v, e);
+                if (c > 0) T += part[(c0 + e) * kEW * 32];
+                if (c + 1 < kc) {
+                  part[(c0 + e) * kEW * 32] = T;
+                  continue;
+                }
+                if (par == 0) {
+                  // (-1)^m x_H Y; the forward weight of n = 0 is half the others'
+                  const long long t = (fwd && m == 0) ? mid / 2 : mid;
+                  T += (m & 1) ? -t : t;
+                }
+                dst[2 * (size_t)(2 * m + par)] = nan ? qnan<TO>() : scaled<TO>(T, ex);
               }
-              const long long H = ((long long)(g[0] * 128 + g[1]) * 128 + g[2]) * 128 + g[3];
-              const long long L = ((long long)(g[4] * 128 + g[5]) * 128 + g[6]) * 128 + g[7];
-              const long long T = H * 262144ll + (L >> 10);   // (H 2^28 + L) / 2^10
-              // sum = 2^(E + F - 108) 2^49 (H 2^28 + L) = T 2^(E + F - 49)
-              st_stream(dstp + 2 * (size_t)n,
-                        me >= F::EMAX ? qnan<TO>() : scaled<TO>(T, me - F::EOFF - 49 + sF[n]));
             }
           }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barDrain) : "memory");
-        // the rest of the next slice's planes, as its MMAs free the buffers
-        if (sl + 1 < nNt) {
-          rebuild(t + tplanes);
-          t += tplanes;
-        }
-        // while the last slice's MMAs run: the next tile's cold row read
-        if (sl == nNt - 2 && tile + (int)gridDim.x < ntiles) ahead = row_exponent(tile + gridDim.x);
       }
+      if (!ok) break;
     }
   }
   if (!W.ok) atomicOr(err, 1);
@@ -723,129 +438,88 @@ __global__ void __launch_bounds__(TCT + 32, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-template <typename TI, typename TO, int NT>
+template <typename TI, typename TO>
 cudaError_t launch_t(const void* in, long long fsi, void* out, long long fso, int nf, int nlines,
                      int Nz, const ChebTc& t, int* err, cudaStream_t s) {
-  const size_t smem = tc_smem_bytes(NT);
-  const int tpf = (nlines + TCM / 2 - 1) / (TCM / 2);
+  const int tpf = (nlines + kRows / 2 - 1) / (kRows / 2);
   const long long ntiles = (long long)nf * tpf;
   if (ntiles <= 0) return cudaSuccess;
   const int grid = (int)std::min<long long>(ntiles, t.ctas);
-  cheb_tc_kernel<TI, TO, NT><<<grid, TCT + 32, smem, s>>>(
-      (const TI*)in, fsi, (TO*)out, fso, nlines, Nz, t.Kp, tpf, (int)ntiles, t.nNt, t.dig,
-      t.fexp, t.cache, t.dir == 0 ? 1 : 0, t.dir == 0 ? 0.5 / (double)(Nz - 1) : 1.0, err);
+  cheb_tc_kernel<TI, TO><<<grid, kThreads, kSmem, s>>>(
+      (const TI*)in, fsi, (TO*)out, fso, nlines, Nz, tpf, (int)ntiles, t.NT, t.nsl, t.nst, t.kc,
+      t.gst, t.dig, t.keep, (long long)cheb_tc_keep_bytes(Nz - 1), t.dir == 0 ? 1 : 0, t.q, t.ymid,
+      t.dir == 0 ? 0.5 / (double)(Nz - 1) : 1.0, err);
   return cudaGetLastError();
-}
-
-template <typename TI, typename TO>
-cudaError_t launch_nt(const void* in, long long fsi, void* out, long long fso, int nf,
-                      int nlines, int Nz, const ChebTc& t, int* err, cudaStream_t s) {
-  return t.NT == 48 ? launch_t<TI, TO, 48>(in, fsi, out, fso, nf, nlines, Nz, t, err, s)
-                    : launch_t<TI, TO, 64>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
 }
 
 uint16_t bf16_bits(float f) {
   uint32_t u;
   memcpy(&u, &f, sizeof u);
-  return (uint16_t)(u >> 16);   // exact: the digits have at most 7 significant bits
+  return (uint16_t)(u >> 16);   // exact: a digit has at most eight significant bits
+}
+
+// weight of input k in output n < N, times 2^q; cs[a] = cos(pi a / N)
+long long weight(const std::vector<long double>& cs, int N, int dir, int q, int n, int k) {
+  long double v = cs[((long long)n * k) % (2 * N)];
+  if (dir == 0) v *= (k == 0 ? 1.0L : 2.0L) / ((n == 0 ? 2.0L : 1.0L) * (long double)N);
+  return (long long)llroundl(ldexpl(v, q));
 }
 
 }  // namespace
 
-int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, std::vector<int>& fexp, int& NT,
-                   int& nNt, int& Kp) {
-  const int Nz = N + 1;
-  Kp = (Nz + 15) / 16 * 16;
-  if (N < 2 || Kp >= 512) return -1;
-  // the MMAs produce outputs n < N (the last one, n = N, has the weights +-1, +-2 and is summed
-  // exactly by the kernel's producers); output slice width 48 or 64, whichever pads less after
-  // weighting 48-wide slices by 5/4 (more MMA instructions per column)
-  const int c48 = (N + 47) / 48 * 48, c64 = (N + 63) / 64 * 64;
-  NT = (5 * c48 <= 4 * c64) ? 48 : 64;
-  nNt = (N + NT - 1) / NT;
-  if (nNt * NT > 512) return -1;   // the kernel keeps F_n of at most 512 columns
-  dig.assign((size_t)nNt * 8 * NT * Kp, 0);
-  fexp.assign((size_t)nNt * NT, 0);
+int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
+  if (N < 2 || N % 2 || (N + 16) / 16 * 16 >= 512) return -1;
+  const int H = N / 2;
+  t->dir = dir;
+  t->nsl = (H + kNTMax - 1) / kNTMax;
+  t->NT = ((H + t->nsl - 1) / t->nsl + 15) / 16 * 16;
+  t->nst = (H + kKS - 1) / kKS;
+  t->kc = (t->nst * kKS + kMaxK - 1) / kMaxK;
+  t->gst = (t->nst + t->kc - 1) / t->kc;
+  // one scale for the whole matrix, its largest weight (1 backward, 2 / N forward) at most 2^54
+  t->q = 54;
+  if (dir == 0)
+    for (int h = H; h > 1; h >>= 1) ++t->q;
   const long double pi = 3.141592653589793238462643383279502884L;
-  std::vector<long double> row(Nz);
-  std::vector<long long> Y(Nz);
-  for (int n = 0; n < N; ++n) {
-    long double mx = 0.0L;
-    for (int k = 0; k < Nz; ++k) {
-      int a = (int)(((long long)n * k) % (2 * N));
-      if (a > N) a = 2 * N - a;   // cos(pi a / N) = cos(pi (2N - a) / N)
-      long double c;
-      if (2 * a == N) c = 0.0L;
-      else if (2 * a < N) c = cosl(pi * (long double)a / (long double)N);
-      else c = -cosl(pi * (long double)(N - a) / (long double)N);
-      long double v = c;
-      if (dir == 0) {
-        const long double ek = (k == 0 || k == N) ? 1.0L : 2.0L;
-        const long double cb = (n == 0 || n == N) ? 2.0L : 1.0L;
-        v = ek * c / (cb * (long double)N);
-      }
-      row[k] = v;
-      if (fabsl(v) > mx) mx = fabsl(v);
-    }
-    int F = 0;
-    if (mx > 0.0L) {
-      F = ilogbl(mx) + 1;
-      for (;;) {
-        bool fit = true;
-        for (int k = 0; k < Nz; ++k) {
-          Y[k] = llroundl(ldexpl(row[k], 54 - F));
-          if (Y[k] >= (1ll << 54) || Y[k] <= -(1ll << 54)) fit = false;
-        }
-        if (fit) break;
-        ++F;
-      }
-    } else {
-      for (int k = 0; k < Nz; ++k) Y[k] = 0;
-    }
-    fexp[n] = F;
-    const int nt = n / NT, nl = n % NT;
-    for (int k = 0; k < Nz; ++k) {
-      const unsigned long long yb = (unsigned long long)Y[k] + kBias;
-      const int ch = k / TCKC, kl = k % TCKC;
-      const int KCc = std::min(TCKC, Kp - ch * TCKC);
-      const size_t base = (size_t)nt * 8 * NT * Kp + (size_t)ch * 8 * NT * TCKC;
-      (void)KCc;
-      for (int j = 0; j < 8; ++j) {
-        // plane j occupies rows j NT .. j NT + NT - 1 of one 8 NT-row K-major matrix
-        const int row = j * NT + nl;
-        const size_t off = ((size_t)(kl / 8) * NT + row / 8) * 64 + (row % 8) * 8 + kl % 8;
-        const int d = (int)((yb >> (7 * (7 - j))) & 127ull) - 64;
-        dig[base + off] = bf16_bits((float)d);
-      }
-    }
+  std::vector<long double> cs(2 * N);   // cos(pi a / N)
+  for (int a = 0; a <= N; ++a) {
+    if (2 * a == N) cs[a] = 0.0L;
+    else if (2 * a < N) cs[a] = cosl(pi * (long double)a / (long double)N);
+    else cs[a] = -cosl(pi * (long double)(N - a) / (long double)N);
   }
+  for (int a = N + 1; a < 2 * N; ++a) cs[a] = cs[2 * N - a];
+  t->ymid = dir == 0 ? (long long)llroundl(ldexpl(2.0L / (long double)N, t->q)) : 1ll << 54;
+  const int NT = t->NT;
+  const size_t block = (size_t)kPlanes * NT * kKS;
+  dig.assign((size_t)2 * t->nsl * t->nst * block, 0);
+  for (int m = 0; m < H; ++m)
+    for (int par = 0; par < 2; ++par)
+      for (int k = 0; k < H; ++k) {
+        const int st = k / kKS, kk = k % kKS;
+        const int pos = 4 * (kk & 3) + (kk >> 2);   // k = 16 st + g + 4 e sits at position 4 g + e
+        const unsigned long long y = (unsigned long long)weight(cs, N, dir, t->q, 2 * m + par, k) + kBias;
+        uint16_t* b = dig.data() + ((size_t)(2 * (m / NT) + par) * t->nst + st) * block;
+        for (int j = 0; j < kPlanes; ++j) {
+          const int row = j * NT + m % NT;
+          b[((size_t)(pos >> 3) * kPlanes * NT + row) * 8 + (pos & 7)] =
+              bf16_bits((float)((int)((y >> (8 * (6 - j))) & 255ull) - 128));
+        }
+      }
   return 0;
 }
 
-size_t cheb_tc_smem(int NT) { return tc_smem_bytes(NT); }
-
-size_t cheb_tc_cache_bytes(int Kp) {
-  return (size_t)((Kp + TCKC - 1) / TCKC) * 8 * kCacheWords * sizeof(uint32_t);
+size_t cheb_tc_keep_bytes(int N) {
+  const size_t nst = (N / 2 + kKS - 1) / kKS;
+  return 2 * nst * kKeepStage + (size_t)(kNTMax / 2) * kEW * 32 * sizeof(long long);
 }
 
-cudaError_t cheb_tc_prepare(int NT) {
-  const size_t smem = tc_smem_bytes(NT);
-  cudaError_t e = cudaSuccess;
-  if (NT == 48) {
-    static SmemLimit c0, c1, c2, c3, c4;
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, double, 48>, smem, &c0);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<float, double, 48>, smem, &c1);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, float, 48>, smem, &c2);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<df, double, 48>, smem, &c3);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, df, 48>, smem, &c4);
-  } else {
-    static SmemLimit c0, c1, c2, c3, c4;
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, double, 64>, smem, &c0);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<float, double, 64>, smem, &c1);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, float, 64>, smem, &c2);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<df, double, 64>, smem, &c3);
-    if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, df, 64>, smem, &c4);
-  }
+cudaError_t cheb_tc_prepare() {
+  static SmemLimit c0, c1, c2, c3, c4;
+  cudaError_t e = ensure_smem(cheb_tc_kernel<double, double>, kSmem, &c0);
+  if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<float, double>, kSmem, &c1);
+  if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, float>, kSmem, &c2);
+  if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<df, double>, kSmem, &c3);
+  if (e == cudaSuccess) e = ensure_smem(cheb_tc_kernel<double, df>, kSmem, &c4);
   return e;
 }
 
@@ -853,15 +527,15 @@ cudaError_t launch_cheb_tc(int tin, int tout, const void* in, long long fsi, voi
                            long long fso, int nf, int nlines, int Nz, const ChebTc& t, int* err,
                            cudaStream_t s) {
   if (tin == 0 && tout == 0)
-    return launch_nt<double, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
+    return launch_t<double, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
   if (tin == 1 && tout == 0)
-    return launch_nt<float, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
+    return launch_t<float, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
   if (tin == 0 && tout == 1)
-    return launch_nt<double, float>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
+    return launch_t<double, float>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
   if (tin == 2 && tout == 0)
-    return launch_nt<df, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
+    return launch_t<df, double>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
   if (tin == 0 && tout == 2)
-    return launch_nt<double, df>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
+    return launch_t<double, df>(in, fsi, out, fso, nf, nlines, Nz, t, err, s);
   return cudaErrorInvalidValue;
 }
 

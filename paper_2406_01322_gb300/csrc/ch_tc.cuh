@@ -1,0 +1,309 @@
+// Building blocks of the exact-split (Ozaki) matrix products on the tensor cores: PTX wrappers,
+// bounded waits, float <-> fixed point, the digit planes, and the issue of one K stage's MMAs.
+//
+// A product of a float64 row x with a fixed matrix B is made exact up to the rounding of the two
+// operands: x becomes the integers X_k = round(x_k 2^(54-E)) (|x_k| < 0.98 2^E over the row), B
+// the integers Y_nk = round(B_nk 2^q), both written with seven signed base-256 digits,
+//   X_k = sum_{i=0..6} a_ik 256^(6-i),  a_ik in [-128, 127],
+// which bf16 holds exactly.  A digit product sum_k a_ik b_jnk is an integer, and the products with
+// the same i + j = d share one fp32 accumulator G_d: |G_d| <= 7 2^14 K < 2^24 for K <= 144, so
+// every accumulation is exact.  d <= 6 is kept (28 products; the dropped ones are random-signed
+// and of order 2^-53 of max|x| max|B|), and
+//   sum_k X_k Y_nk = 256^6 U,  U = sum_{d<=6} 256^(6-d) G_d
+// is recombined in 64-bit integers.  Eight-bit digits need 28 products where seven-bit ones
+// (eight planes, K < 512) need 36; transforms with longer sums are cut into K groups of at most
+// 144 whose recombined integers are added.
+//
+// The seven B digit planes of an output slice are stacked into one 7 NT-row operand, so A plane i
+// needs one MMA chain over rows 0 .. (7-i) NT with its accumulator at column i NT: product (i, j)
+// lands on diagonal i + j.
+#pragma once
+
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "ch_common.cuh"
+
+namespace chf {
+namespace tc {
+
+constexpr int kRows = 128;        // rows per tile = tensor-memory lanes
+constexpr int kPlanes = 7;        // base-256 digits of an operand
+constexpr int kKS = 16;           // K per pipeline stage (one MMA k-step)
+constexpr int kMaxK = 144;        // K up to which the fp32 accumulators stay exact
+constexpr int kNTMax = 64;        // columns of an output slice (7 x 64 tensor-memory columns)
+constexpr int kPlaneBytes = kRows * kKS * 2;             // one A digit plane of a stage
+constexpr int kABytes = kPlanes * kPlaneBytes;           // the A planes of a stage
+constexpr uint32_t kALbo = kRows * 16;                   // A: bytes between 8-element K groups
+__host__ __device__ constexpr int b_stage_bytes(int NT) { return kPlanes * NT * kKS * 2; }
+constexpr unsigned long long kBias = 0x0080808080808080ull;   // 128 sum_{t<7} 256^t
+constexpr uint64_t kWaitNs = 1000000000ull;                   // bound of every device wait
+
+// ---- PTX wrappers -----------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t su32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// shared-memory matrix descriptor, no swizzle: lbo = byte stride between core matrices along K,
+// sbo = byte stride between 8-row core-matrix groups along M (or N); version 1 at bit 46
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
+         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+}
+__device__ __forceinline__ uint64_t gtime() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// bounded wait for the phase with the given parity; false if it did not complete in time
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.b32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// wait for the phase with the given parity until the global timer passes `deadline`
+__device__ __forceinline__ bool mbar_wait_until(uint32_t bar, uint32_t parity,
+                                                uint64_t deadline) {
+  while (true) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (gtime() > deadline) return false;
+  }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  if (mbar_try(bar, parity)) return true;   // the common case: no clock read
+  return mbar_wait_until(bar, parity, gtime() + kWaitNs);
+}
+// The waits of one thread.  The first wait that runs out clears `ok`; every later wait returns
+// false at once, so a thread spends at most one bound waiting in vain however many waits follow
+// (the transform kernels' warps then leave their loops, the issuer after draining its MMAs).
+struct Waiter {
+  bool ok = true;
+  __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) {
+    ok = ok && mbar_wait(bar, parity);
+    return ok;
+  }
+  // the same for a whole warp: false for all lanes if it ran out for any
+  __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity) {
+    ok = __all_sync(0xffffffffu, ok && mbar_wait(bar, parity)) != 0;
+    return ok;
+  }
+};
+__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                         uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+      : "memory");
+}
+// L2 policy that keeps lines resident (the matrix digits, re-read by every tile) ahead of
+// the streamed rows and outputs
+__device__ __forceinline__ uint64_t policy_evict_last() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+// bulk copy global -> shared with completion on an mbarrier, read under the L2 policy `pol`
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes,
+                                          uint32_t bar, uint64_t pol) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+               : "memory");
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+      "[%1], %2, [%3], %4;" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar), "l"(pol)
+      : "memory");
+}
+// seven 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32
+// lanes, then one wait that the values depend on
+__device__ __forceinline__ void tmem_ld7x4(uint32_t addr, int stride, uint32_t (&v)[7][4]) {
+#pragma unroll
+  for (int d = 0; d < 7; ++d)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3])
+                 : "r"(addr + (uint32_t)(d * stride)));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]),
+                 "+r"(v[1][1]), "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]),
+                 "+r"(v[2][2]), "+r"(v[2][3]), "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]),
+                 "+r"(v[3][3]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[4][2]), "+r"(v[4][3]),
+                 "+r"(v[5][0]), "+r"(v[5][1]), "+r"(v[5][2]), "+r"(v[5][3]), "+r"(v[6][0]),
+                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3])
+               :
+               : "memory");
+}
+
+// ---- float <-> fixed point --------------------------------------------------------------------
+// Storage types of a row's elements: the bit pattern, its magnitude bits (an unsigned key that
+// orders |x|; infinities and NaNs are the largest) and the exponent field of the row scale.
+// maxe = row_scale(largest key) is the exponent field of the row's largest element, plus one when
+// that element is above 0.975 of the next power of two: |x| < 0.976 2^E with E = maxe - EOFF, so
+// the sum or difference of two elements stays inside the seven signed base-256 digits (0.996 2^55).
+template <typename T> struct FBits;
+template <> struct FBits<double> {
+  static constexpr int EMAX = 0x7FF, EOFF = 1022, KEY_MB = 20;
+  typedef unsigned long long U;
+  __device__ static U bits(double x) { return (U)__double_as_longlong(x); }
+  __device__ static unsigned key(U b) { return (unsigned)(b >> 32) & 0x7FFFFFFFu; }
+};
+template <> struct FBits<float> {
+  static constexpr int EMAX = 0xFF, EOFF = 126, KEY_MB = 23;
+  typedef unsigned int U;
+  __device__ static U bits(float x) { return __float_as_uint(x); }
+  __device__ static unsigned key(U b) { return b & 0x7FFFFFFFu; }
+};
+// double-float h + l: the bits of h in the low word, of l in the high word; the row scale comes
+// from h (|l| <= ulp(h) / 2)
+template <> struct FBits<df> {
+  static constexpr int EMAX = 0xFF, EOFF = 126, KEY_MB = 23;
+  typedef unsigned long long U;
+  __device__ static U bits(df x) {
+    return (U)__float_as_uint(x.h) | ((U)__float_as_uint(x.l) << 32);
+  }
+  __device__ static unsigned key(U b) { return (unsigned)b & 0x7FFFFFFFu; }
+};
+constexpr int kNanRow = 1 << 14;   // scale of a row that holds an infinity or NaN
+template <typename T> __device__ __forceinline__ int row_scale(unsigned key) {
+  typedef FBits<T> F;
+  const int e = (int)(key >> F::KEY_MB);
+  if (e >= F::EMAX) return kNanRow;
+  const unsigned frac = key & ((1u << F::KEY_MB) - 1u);
+  return max(e, 1) + (frac > (unsigned)(0.95 * (1 << F::KEY_MB)) ? 1 : 0);
+}
+
+// round(x 2^(54-E)) of the element with bit pattern b in a row of scale maxe (E = maxe - EOFF);
+// zero in a row that holds an infinity or NaN (kNanRow), whose results are NaN
+__device__ __forceinline__ long long fixed_f32(unsigned b, int maxe) {
+  int ef = (int)((b >> 23) & 0xFFu);
+  unsigned m = b & 0x7FFFFFu;
+  if (ef) m |= 0x800000u;
+  else ef = 1;
+  const int sh = min(maxe - ef, 63);
+  const unsigned long long r = (((unsigned long long)m << 31 >> sh) + 1ull) >> 1;
+  const long long s = (long long)((int)b >> 31);
+  return ((long long)r ^ s) - s;
+}
+template <typename T> __device__ long long to_fixed(typename FBits<T>::U b, int maxe);
+template <> __device__ __forceinline__ long long to_fixed<double>(unsigned long long b, int maxe) {
+  const unsigned hi = (unsigned)(b >> 32);
+  int ef = (int)((hi >> 20) & 0x7FFu);
+  unsigned mh = hi & 0xFFFFFu;
+  if (ef) mh |= 0x100000u;
+  else ef = 1;
+  const int sh = min(maxe - ef, 63);
+  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)b) << 2;
+  const unsigned long long r = ((m >> sh) + 1ull) >> 1;
+  const long long s = (long long)((int)hi >> 31);
+  return ((long long)r ^ s) - s;
+}
+template <> __device__ __forceinline__ long long to_fixed<float>(unsigned b, int maxe) {
+  return fixed_f32(b, maxe);
+}
+// double-float: both parts converted and added (one extra unit of rounding at most)
+template <> __device__ __forceinline__ long long to_fixed<df>(unsigned long long b, int maxe) {
+  return fixed_f32((unsigned)b, maxe) + fixed_f32((unsigned)(b >> 32), maxe);
+}
+
+// Digit plane i (0 = most significant) of two values, as two bf16 in one word (first in the low
+// half): byte 6 - i of the biased integers, u, stands for the digit u - 128.  With l = u mod 128,
+// the bf16 128 + l is 0x4300 | l, and the digit is (128 + l) - 256 or (128 + l) - 128 (bit 7 of u
+// clear or set; the bf16 -256 and -128 differ in exactly that bit of 0xC380), one exact bf16 add.
+__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byte) {
+  const uint32_t w = __byte_perm(w0, w1, (uint32_t)(byte | (byte << 4) | ((4 + byte) << 8) |
+                                                    ((4 + byte) << 12)));
+  const uint32_t a = (w & 0x007F007Fu) | 0x43004300u;
+  const uint32_t c = (w & 0x00800080u) ^ 0xC380C380u;
+  __nv_bfloat162 r = __hadd2(*reinterpret_cast<const __nv_bfloat162*>(&a),
+                             *reinterpret_cast<const __nv_bfloat162*>(&c));
+  return *reinterpret_cast<uint32_t*>(&r);
+}
+
+// round(U / 64) of the seven diagonal accumulators (exact integers below 2^24 held as fp32):
+// U = sum_d 256^(6-d) G_d.  Sums are formed modulo 2^64; |U| / 64 < 2^63 for sums of at most 496
+// terms per row (|sum_k x_k B_nk| < 496 max|x| max|B|).
+__device__ __forceinline__ long long recombine(const uint32_t (&v)[7][4], int e) {
+  int g[7];
+#pragma unroll
+  for (int d = 0; d < 7; ++d) g[d] = __float2int_rz(__uint_as_float(v[d][e]));
+  const int h = g[0] * 256 + g[1], m = g[2] * 256 + g[3];
+  const long long l = (long long)g[4] * 65536 + ((long long)g[5] * 256 + (long long)g[6]);
+  return (long long)((unsigned long long)(unsigned)h << 34) + (long long)m * 262144 +
+         ((l + 32) >> 6);
+}
+
+// T 2^e rounded once to the output type.  The integer converts in one instruction, the power of
+// two is added to the exponent field; ldexp outside the normal range.
+template <typename TO> __device__ TO scaled(long long T, int e);
+template <> __device__ __forceinline__ double scaled<double>(long long T, int e) {
+  const double v = __ll2double_rn(T);
+  const int hi = __double2hiint(v);
+  const int be = ((hi >> 20) & 0x7FF) + e;
+  if (T == 0) return 0.0;
+  if (be <= 0 || be >= 2047) return ldexp(v, e);
+  return __hiloint2double(hi + (e << 20), __double2loint(v));
+}
+template <> __device__ __forceinline__ float scaled<float>(long long T, int e) {
+  const float v = __ll2float_rn(T);
+  const int b = __float_as_int(v);
+  const int be = ((b >> 23) & 0xFF) + e;
+  if (T == 0) return 0.0f;
+  if (be <= 0 || be >= 255) return ldexpf(v, e);
+  return __int_as_float(b + (e << 23));
+}
+// double-float result: the high part rounded to float, the low part from the exact remainder
+template <> __device__ __forceinline__ df scaled<df>(long long T, int e) {
+  const long long hi = __float2ll_rn(__ll2float_rn(T));   // |T| < 2^62.93: no overflow
+  return df(scaled<float>(hi, e), scaled<float>(T - hi, e));
+}
+template <typename TO> __device__ __forceinline__ TO qnan();
+template <> __device__ __forceinline__ double qnan<double>() {
+  return __longlong_as_double(0x7FF8000000000000ll);
+}
+template <> __device__ __forceinline__ float qnan<float>() { return __uint_as_float(0x7FC00000u); }
+template <> __device__ __forceinline__ df qnan<df>() {
+  return df(__uint_as_float(0x7FC00000u), __uint_as_float(0x7FC00000u));
+}
+
+// ---- one K stage's MMAs -----------------------------------------------------------------------
+// A planes at shared address sA, the stacked B planes (7 NT rows) at sB, both 16 K wide in the
+// canonical no-swizzle K-major core-matrix layout; accumulators from tensor-memory column tmem.
+// A plane i times B rows 0 .. (7-i) NT, in pieces of at most 256 columns of about equal width (an
+// MMA of M = 128 takes N / 2 cycles, but not less than about 50).  init: the accumulators start
+// from zero (plane 0 covers all their columns).
+__device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t sA, uint32_t sB, int NT,
+                                            bool init) {
+  // bf16 x bf16 -> fp32, both K-major, M = 128 (N added per MMA)
+  const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 4) << 24);
+  const uint32_t lbo_b = (uint32_t)(kPlanes * NT * 16);
+#pragma unroll
+  for (int i = 0; i < kPlanes; ++i) {
+    const uint64_t ad = sdesc(sA + (uint32_t)(i * kPlaneBytes), kALbo, 128);
+    const int ntot = (kPlanes - i) * NT;
+    const int np = (ntot + 255) >> 8;
+    const int len = ((ntot / np) + 15) & ~15;
+    for (int n0 = 0; n0 < ntot; n0 += len) {
+      const int nlen = min(len, ntot - n0);
+      mma_bf16(tmem + (uint32_t)(i * NT + n0), ad, sdesc(sB + (uint32_t)(n0 * 16), lbo_b, 128),
+               idesc0 | ((uint32_t)(nlen >> 3) << 17), (uint32_t)!(init && i == 0));
+    }
+  }
+}
+
+}  // namespace tc
+}  // namespace chf
