@@ -19,8 +19,10 @@
 //
 // Tiles and data flow.  A tile is 128 rows (re and im of 64 lines of one field).  Its passes are
 // (output slice of NT columns, parity, K group): the accumulators of a pass live in tensor memory.
-// Persistent CTAs (one per SM) have three kinds of warps, so conversion, MMAs and the epilogue of
-// different passes overlap:
+// Persistent CTAs (one per SM) have four kinds of warps, so the scan, the conversion, the MMAs and
+// the epilogue of different passes and tiles overlap:
+//   scan (3 warps): the rows' scales of the next tile (the rows' first, cold read, after an L2
+//     prefetch of the tile one further ahead) and the middle elements' terms;
 //   producers (8 warps): per K stage of 16 (one MMA k-step) a thread converts four pairs
 //     (x_k, x_{N-k}) of the real and imaginary rows of one line to fixed point, writes the seven
 //     digit planes of the sums to the stage's shared buffer and keeps the differences (and, with
@@ -28,11 +30,10 @@
 //     thread for the later passes; thread 0 also issues the bulk copy of the stage's matrix digits;
 //   issuer (1 thread): the MMAs of each stage as it fills;
 //   epilogue (8 warps): drains a pass's accumulators, recombines and stores.
-// What bounds it: integer issue (about 45 instructions per element converted and 25 per output)
-// and the shared-memory bandwidth of the MMA operands; the tensor pipe itself needs 0.93 of the
-// 16-wide stage's time at NT = 64.
+// Twenty warps keep 96 registers each (seventeen would not allow more: five on one sub-partition).
 #include <math.h>
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
@@ -47,47 +48,117 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPW = 8, kEW = 8;                   // producer and epilogue warps
-constexpr int kThreads = 32 * (kPW + kEW + 1);    // epilogue 0..7, producers 8..15, issuer 16
+constexpr int kPW = 8, kEW = 8, kSW = 3;          // producer, epilogue and scan warps
+constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
 constexpr int kStages = 5;                        // K stages in flight
+constexpr int kRB = 3;                            // tiles whose row scales are held
 constexpr int kStageBytes = kABytes + b_stage_bytes(kNTMax);
-// per stage full, bfull, empty; accfull, accfree, rowfull[2], rowfree[2], fin
-constexpr int kBars = 3 * kStages + 7;
-// stages, row scales and middle terms (two tiles), barriers, the tensor-memory address
-constexpr size_t kSmem = (size_t)kStages * kStageBytes + 2 * kRows * (sizeof(long long) + sizeof(int)) +
-                         (size_t)(kBars + 1) * 8;
+// per stage full, bfull, empty; accfull, accfree, rowfull[kRB], rowfree[kRB], fin
+constexpr int kBars = 3 * kStages + 3 + 2 * kRB;
+// stages, row scales and middle terms, barriers, the tensor-memory address
+constexpr size_t kSmem = (size_t)kStages * kStageBytes +
+                         kRB * kRows * (sizeof(long long) + sizeof(int)) + (size_t)(kBars + 1) * 8;
 // one pass's stage block kept in global memory: four fixed-point values of two rows per thread
 constexpr size_t kKeepStage = (size_t)kPW * 32 * 8 * sizeof(long long);
 
 template <typename TO> __device__ __forceinline__ TO times(TO v, double f) { return v; }
 template <> __device__ __forceinline__ double times<double>(double v, double f) { return v * f; }
 
+// Row of a tile: lines in blocks of eight, the real parts of a block in rows 16 b .. + 7, the
+// imaginary ones in 16 b + 8 .. + 15 (a producer half-warp, eight lines x two K groups of four,
+// then stores 128 contiguous bytes).
+__device__ __forceinline__ int tile_row(int l, int part) { return (l >> 3) * 16 + part * 8 + (l & 7); }
+
+// the bit patterns of one complex element
+template <typename T> struct CBits { typename FBits<T>::U re, im; };
+__device__ __forceinline__ CBits<double> ld_cplx(const double* p) {
+  const double2 v = *reinterpret_cast<const double2*>(p);
+  return {FBits<double>::bits(v.x), FBits<double>::bits(v.y)};
+}
+__device__ __forceinline__ CBits<float> ld_cplx(const float* p) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
+  return {FBits<float>::bits(v.x), FBits<float>::bits(v.y)};
+}
+__device__ __forceinline__ CBits<df> ld_cplx(const df* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return {FBits<df>::bits(df(v.x, v.y)), FBits<df>::bits(df(v.z, v.w))};
+}
+
+// One pass's outputs of one thread: columns m0 .. m0 + CW - 1 of its row, four at a time, from the
+// seven accumulators at tensor-memory address tb; dst: output column m0 (columns 4 scalars apart).
+// Arguments as in the kernel.
+template <typename TO, int NMAG>
+__device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m0, int H, int c,
+                                              int kc, int par, bool rowok, bool nan, bool safe,
+                                              int ex, long long mid, bool halve0, long long* part,
+                                              TO* dst, uint32_t barAccFree, int lane) {
+  for (int c0 = 0; c0 < CW; c0 += 4) {
+    uint32_t v[7][4];
+    tmem_ld7x4(tb + (uint32_t)c0, NT, v);
+    if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barAccFree) : "memory");
+    }
+    long long T[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG>(v, e);
+    if (kc > 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (c > 0) T[e] += part[(c0 + e) * kEW * 32];
+        if (c + 1 < kc) part[(c0 + e) * kEW * 32] = T[e];
+      }
+      if (c + 1 < kc) continue;
+    }
+    if (par == 0) {
+      // (-1)^m x_H Y (m0 + c0 is a multiple of four); the forward weight of n = 0 is half
+      const long long t0 = (halve0 && m0 + c0 == 0) ? mid / 2 : mid;
+      T[0] += t0;
+      T[1] -= mid;
+      T[2] += mid;
+      T[3] -= mid;
+    }
+    TO r[4];
+    if (safe) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r[e] = scaled<TO>(T[e], ex);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r[e] = nan ? qnan<TO>() : scaled_any<TO>(T[e], ex);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (rowok && m0 + c0 + e < H) dst[4 * (c0 + e)] = r[e];
+  }
+}
+
 // in / out: nf fields of complex lines (re, im interleaved), field stride fsi / fso complex
 // elements, line stride Nz = N + 1; dig: the matrix digits, stage blocks of 7 NT rows x 16 K in
 // the order slice, parity, stage; keep: keep_bytes per CTA; nst stages per parity in kc groups of
-// gst; q: log2 of the matrix scale; ymid: middle weight times 2^q; lastf: factor of output N
-// (forward).
+// gst; nmag: accumulators known to stay within 2^22 (7, 3 or 0); q: log2 of the matrix scale;
+// ymid: middle weight times 2^q; lastf: factor of output N (forward).
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kThreads, 1)
     cheb_tc_kernel(const TI* __restrict__ in, long long fsi, TO* __restrict__ out, long long fso,
                    int nlines, int Nz, int tpf, int ntiles, int NT, int nsl, int nst, int kc,
-                   int gst, const uint16_t* __restrict__ dig, char* __restrict__ keep,
+                   int gst, int nmag, const uint16_t* __restrict__ dig, char* __restrict__ keep,
                    long long keep_bytes, int fwd, int q, long long ymid, double lastf,
                    int* __restrict__ err) {
   typedef FBits<TI> F;
-  typedef typename F::U U;
   extern __shared__ __align__(1024) unsigned char tsm[];
   unsigned char* stages = tsm;
   long long* sC = reinterpret_cast<long long*>(tsm + (size_t)kStages * kStageBytes);
-  int* sE = reinterpret_cast<int*>(sC + 2 * kRows);
-  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + 2 * kRows);
+  int* sE = reinterpret_cast<int*>(sC + kRB * kRows);
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + kRB * kRows);
   uint32_t* sT = reinterpret_cast<uint32_t*>(bars + kBars);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int N = Nz - 1, H = N / 2;
   const uint32_t barFull = su32(bars), barB = barFull + 8 * kStages;
   const uint32_t barEmpty = barFull + 16 * kStages, barAccFull = barFull + 24 * kStages;
-  const uint32_t barAccFree = barAccFull + 8, barRow = barAccFull + 16, barRowFree = barAccFull + 32;
-  const uint32_t barFin = barAccFull + 48;
+  const uint32_t barAccFree = barAccFull + 8, barRow = barAccFull + 16;
+  const uint32_t barRowFree = barRow + 8 * kRB, barFin = barRowFree + 8 * kRB;
   if (tid == 0) {
     for (int b = 0; b < kStages; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barFull + 8 * b), "r"(kPW));
@@ -96,9 +167,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barAccFull));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barAccFree), "r"(kEW));
-    for (int b = 0; b < 2; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRow + 8 * b), "r"(kPW));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRowFree + 8 * b), "r"(kEW));
+    for (int b = 0; b < kRB; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRow + 8 * b), "r"(kSW));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRowFree + 8 * b),
+                   "r"(kEW + kPW));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barFin));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -154,40 +226,96 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
+  } else if (warp > kPW + kEW) {
+    // ---- scan: four lines at a time, a warp's lanes along the line
+    const int sw = warp - (kPW + kEW + 1);
+    int ti = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
+      const int fld = tile / tpf;
+      const int line0 = (tile - fld * tpf) * (kRows / 2);
+      const int nl = min(kRows / 2, nlines - line0);
+      const TI* src = in + ((size_t)fld * fsi + (size_t)line0 * Nz) * 2;
+      if (sw == 0 && lane == 0 && tile + (int)gridDim.x < ntiles) {
+        const int tn = tile + gridDim.x, fn = tn / tpf, ln = (tn - fn * tpf) * (kRows / 2);
+        const char* a = reinterpret_cast<const char*>(in + ((size_t)fn * fsi + (size_t)ln * Nz) * 2);
+        const char* z = a + (size_t)min(kRows / 2, nlines - ln) * Nz * 2 * sizeof(TI);
+        const uintptr_t a16 = ((uintptr_t)a + 15) & ~(uintptr_t)15;
+        const uintptr_t z16 = (uintptr_t)z & ~(uintptr_t)15;
+        if (z16 > a16)
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a16),
+                       "r"((uint32_t)(z16 - a16))
+                       : "memory");
+      }
+      const int b = ti % kRB;
+      if (ti >= kRB && !W.wait_warp(barRowFree + 8 * b, (ti / kRB - 1) & 1)) break;
+      for (int l0 = 4 * sw; l0 < kRows / 2; l0 += 4 * kSW) {
+        unsigned kr[4] = {0, 0, 0, 0}, ki[4] = {0, 0, 0, 0};
+#pragma unroll 2
+        for (int k = lane; k < Nz; k += 32) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (l0 + i < nl) {
+              const CBits<TI> x = ld_cplx(src + ((size_t)(l0 + i) * Nz + k) * 2);
+              kr[i] = max(kr[i], F::key(x.re));
+              ki[i] = max(ki[i], F::key(x.im));
+            }
+        }
+        unsigned mr = 0, mi = 0;   // lane i < 4: the keys of line l0 + i
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const unsigned a = __reduce_max_sync(0xffffffffu, kr[i]);
+          const unsigned c = __reduce_max_sync(0xffffffffu, ki[i]);
+          if (lane == i) {
+            mr = a;
+            mi = c;
+          }
+        }
+        if (lane < 4 && l0 + lane < kRows / 2) {
+          const int l = l0 + lane, er = row_scale<TI>(mr), ei = row_scale<TI>(mi);
+          long long xr = 0, xi = 0;
+          if (l < nl) {
+            const CBits<TI> x = ld_cplx(src + ((size_t)l * Nz + H) * 2);
+            xr = Fixed<TI, true>::of(x.re, er);
+            xi = Fixed<TI, true>::of(x.im, ei);
+          }
+          const int ro = b * kRows + tile_row(l, 0);
+          sE[ro] = er;
+          sE[ro + 8] = ei;
+          // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
+          sC[ro] = __mul64hi(xr * 256, ymid * 4);
+          sC[ro + 8] = __mul64hi(xi * 256, ymid * 4);
+        }
+      }
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRow + 8 * b) : "memory");
+    }
   } else if (warp >= kEW) {
     // ---- producers: thread = (line l of the tile, g): K positions 4 g .. 4 g + 3 of a stage,
-    // position 4 g + e holding k = 16 st + g + 4 e (so the four threads of a line read
-    // consecutive elements).  Rows 2 l (re) and 2 l + 1 (im); threads g >= 2 take the im row
-    // first, so that a half-warp's 8-byte stores fall on different banks.
+    // position 4 g + e holding k = 16 st + g + 4 e
     const int p = tid - 32 * kEW, pw = warp - kEW;
-    const int l = pw * 8 + (lane >> 2), g = lane & 3, sw = g >> 1;
-    const int ra = 2 * l + sw, rb = 2 * l + 1 - sw;
-    const uint32_t oa = (uint32_t)(sw * (int)kALbo + ra * 16 + (g & 1) * 8);
-    const uint32_t ob = (uint32_t)(sw * (int)kALbo + rb * 16 + (g & 1) * 8);
+    const int l = pw * 8 + ((lane >> 1) & 7), g = (lane >> 4) * 2 + (lane & 1);
+    const int row = tile_row(l, 0);
+    const uint32_t oa = (uint32_t)((g >> 1) * (int)kALbo + row * 16 + (g & 1) * 8);
     const uint64_t pol = policy_evict_last();
     longlong2* kp = reinterpret_cast<longlong2*>(kcta) + p;
     uint32_t slot = 0, use = 0;
     int ti = 0;
-    // the stage's digit planes of v (0..3 row a, 4..7 row b) and, by one thread, the copy of its
-    // matrix digits; false after a wait ran out
-    auto put = [&](const long long (&v)[8], const uint16_t* bsrc) {
+    // the stage's digit planes of v (biased; 0..3 the real row, 4..7 the imaginary one) and, by
+    // one thread, the copy of its matrix digits; false after a wait ran out
+    auto put = [&](const unsigned long long (&v)[8], const uint16_t* bsrc) {
       if (use > 0 && !W.wait_warp(barEmpty + 8 * slot, (use & 1) ^ 1)) return false;
       unsigned char* sA = stages + (size_t)slot * kStageBytes;
       if (p == 0) bulk_load(su32(sA) + (uint32_t)kABytes, bsrc, bbytes, barB + 8 * slot, pol);
-      uint32_t lo[8], hi[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const unsigned long long y = (unsigned long long)v[e] + kBias;
-        lo[e] = (uint32_t)y;
-        hi[e] = (uint32_t)(y >> 32);
-      }
 #pragma unroll
       for (int i = 0; i < kPlanes; ++i) {
-        const int b = 6 - i;
-        const uint32_t* w = b < 4 ? lo : hi;
+        const int b = 6 - i, sh = b < 4 ? 0 : 32;
+        uint32_t w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = (uint32_t)(v[e] >> sh);
         *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + oa) =
             make_uint2(digit_pair(w[0], w[1], b & 3), digit_pair(w[2], w[3], b & 3));
-        *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + ob) =
+        *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + oa + 128) =
             make_uint2(digit_pair(w[4], w[5], b & 3), digit_pair(w[6], w[7], b & 3));
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -202,9 +330,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       return true;
     };
     auto keep_at = [&](int par, int st) { return kp + (size_t)(par * nst + st) * (4 * kPW * 32); };
-    auto store_keep = [&](longlong2* d, const long long (&v)[8]) {
+    auto store_keep = [&](longlong2* d, const unsigned long long (&v)[8]) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) __stcg(d + i * kPW * 32, make_longlong2(v[2 * i], v[2 * i + 1]));
+      for (int i = 0; i < 4; ++i)
+        __stcg(d + i * kPW * 32, make_longlong2((long long)v[2 * i], (long long)v[2 * i + 1]));
     };
     const size_t bstride = (size_t)bbytes / 2;   // elements of a stage block
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
@@ -212,122 +341,115 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int line = (tile - fld * tpf) * (kRows / 2) + l;
       const bool rowok = line < nlines;
       const TI* src = in + ((size_t)fld * fsi + (size_t)(rowok ? line : 0) * Nz) * 2;
-      // the rows' scales (their first, cold read)
-      unsigned ka = 0, kb = 0;
-      if (rowok) {
-#pragma unroll 8
-        for (int k = g; k < Nz; k += 4) {
-          ka = max(ka, F::key(F::bits(src[2 * k + sw])));
-          kb = max(kb, F::key(F::bits(src[2 * k + 1 - sw])));
-        }
-      }
-      // threads g >= 2 hold the rows the other way round
-      unsigned kre = sw ? kb : ka, kim = sw ? ka : kb;
-#pragma unroll
-      for (int off = 1; off < 4; off <<= 1) {
-        kre = max(kre, __shfl_xor_sync(0xffffffffu, kre, off));
-        kim = max(kim, __shfl_xor_sync(0xffffffffu, kim, off));
-      }
-      const int ere = row_scale<TI>(kre), eim = row_scale<TI>(kim);
-      const int ea = sw ? eim : ere, eb = sw ? ere : eim;
-      // the middle element, its integer term for the even outputs, and the row scales
-      long long xmr = 0, xmi = 0;
-      if (g == 0) {
-        if (rowok) {
-          xmr = to_fixed<TI>(F::bits(src[2 * H]), ere);
-          xmi = to_fixed<TI>(F::bits(src[2 * H + 1]), eim);
-        }
-      }
-      if (ti >= 2 && !W.wait_warp(barRowFree + 8 * (ti & 1), ((ti >> 1) - 1) & 1)) break;
-      if (g == 0) {
-        // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
-        sC[(ti & 1) * kRows + 2 * l] = __mul64hi(xmr * 256, ymid * 4);
-        sC[(ti & 1) * kRows + 2 * l + 1] = __mul64hi(xmi * 256, ymid * 4);
-        sE[(ti & 1) * kRows + 2 * l] = ere;
-        sE[(ti & 1) * kRows + 2 * l + 1] = eim;
-      }
-      __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRow + 8 * (ti & 1))
-                     : "memory");
-      // first pass: convert, fold, write the sums' planes, keep the differences
-      long long suma = 0, sumb = 0, s0a = 0, s0b = 0;
-      U xa[4], ya[4], xb[4], yb[4];
+      const TI *lo = src + 2 * g, *hi = src + 2 * (N - g);
+      CBits<TI> xa[4], xb[4];
       auto load = [&](int st) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int k = 16 * st + g + 4 * e;
-          const bool ok = rowok && k < H;
-          xa[e] = xb[e] = ya[e] = yb[e] = 0;
-          if (ok) {
-            xa[e] = F::bits(src[2 * k + sw]);
-            xb[e] = F::bits(src[2 * k + 1 - sw]);
-            ya[e] = F::bits(src[2 * (N - k) + sw]);
-            yb[e] = F::bits(src[2 * (N - k) + 1 - sw]);
+          const int k = 16 * st + 4 * e;
+          xa[e] = {0, 0};
+          xb[e] = {0, 0};
+          if (rowok && k + g < H) {
+            xa[e] = ld_cplx(lo + 2 * k);
+            xb[e] = ld_cplx(hi - 2 * k);
           }
         }
       };
       load(0);
+      const int rbuf = ti % kRB;
+      if (!W.wait_warp(barRow + 8 * rbuf, (ti / kRB) & 1)) break;
+      const int ere = sE[rbuf * kRows + row], eim = sE[rbuf * kRows + row + 8];
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
+                     : "memory");
+      const bool tiny = __any_sync(0xffffffffu, min(ere, eim) < kTinyScale) != 0;
+      // first pass: convert, fold, write the sums' planes, keep the differences (all biased)
+      unsigned long long sumr = 0, sumi = 0, s0r = 0, s0i = 0;
       bool ok = true;
       for (int st = 0; st < nst && ok; ++st) {
-        long long s[8], d[8];
+        unsigned long long s[8], d[8];
+        if (!tiny) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const long long x = to_fixed<TI>(xa[e], ea), y = to_fixed<TI>(ya[e], ea);
-          const long long z = to_fixed<TI>(xb[e], eb), w = to_fixed<TI>(yb[e], eb);
-          s[e] = x + y;
-          d[e] = x - y;
-          s[4 + e] = z + w;
-          d[4 + e] = z - w;
-          suma += s[e];       // at most 62 values below 2^55 per thread
-          sumb += s[4 + e];
+          for (int e = 0; e < 4; ++e) {
+            const long long x = Fixed<TI, false>::of(xa[e].re, ere), y = Fixed<TI, false>::of(xb[e].re, ere);
+            const long long z = Fixed<TI, false>::of(xa[e].im, eim), w = Fixed<TI, false>::of(xb[e].im, eim);
+            s[e] = x + y + kBias;
+            d[e] = x - y + kBias;
+            s[4 + e] = z + w + kBias;
+            d[4 + e] = z - w + kBias;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const long long x = Fixed<TI, true>::of(xa[e].re, ere), y = Fixed<TI, true>::of(xb[e].re, ere);
+            const long long z = Fixed<TI, true>::of(xa[e].im, eim), w = Fixed<TI, true>::of(xb[e].im, eim);
+            s[e] = x + y + kBias;
+            d[e] = x - y + kBias;
+            s[4 + e] = z + w + kBias;
+            d[4 + e] = z - w + kBias;
+          }
         }
-        if (st == 0) {
-          s0a = s[0];
-          s0b = s[4];
-        }
+        if (st + 1 < nst) load(st + 1);
         store_keep(keep_at(1, st), d);
         if (nsl > 1) store_keep(keep_at(0, st), s);
-        if (st + 1 < nst) load(st + 1);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {   // at most 64 values below 2^56
+          sumr += s[e];
+          sumi += s[4 + e];
+        }
+        if (st == 0) {
+          s0r = s[0];
+          s0i = s[4];
+        }
         ok = put(s, dig + (size_t)st * bstride);
       }
       if (!ok) break;
       // the last output n = N: sum_k w_k (-1)^k x_k, (-1)^k = (-1)^g for this thread's k; weights
-      // e_k = 2 except k = 0, N (forward) or 1
+      // e_k = 2 except k = 0, N (forward) or 1.  High and low parts (27 bits) are added apart.
       {
-        long long tre = sw ? sumb : suma, tim = sw ? suma : sumb;
+        const unsigned long long nb = (unsigned long long)(4 * nst) * kBias;
+        long long tr = (long long)(sumr - nb), tm = (long long)(sumi - nb);
         if (g & 1) {
-          tre = -tre;
-          tim = -tim;
+          tr = -tr;
+          tm = -tm;
         }
-        const int m2 = (H & 1) ? -1 : 1;
-        // |partial| < 2^61 here; halves of 27 low bits keep the sums over threads in range
-        long long hr = tre >> 27, lr = tre & 0x7FFFFFF, hi_ = tim >> 27, li = tim & 0x7FFFFFF;
-        if (fwd) {
-          hr *= 2; lr *= 2; hi_ *= 2; li *= 2;
-        }
+        const int f2 = fwd ? 2 : 1;
+        long long hr = f2 * (tr >> 27), lr = f2 * (tr & 0x7FFFFFF);
+        long long hm = f2 * (tm >> 27), lm = f2 * (tm & 0x7FFFFFF);
         if (g == 0) {
-          const int wm = fwd ? 2 * m2 : m2;
-          hr += wm * (xmr >> 27); lr += wm * (xmr & 0x7FFFFFF);
-          hi_ += wm * (xmi >> 27); li += wm * (xmi & 0x7FFFFFF);
-          if (fwd) {   // s_0 counted twice (g = 0: rows in order)
-            hr -= s0a >> 27; lr -= s0a & 0x7FFFFFF;
-            hi_ -= s0b >> 27; li -= s0b & 0x7FFFFFF;
+          const int wm = (H & 1) ? -f2 : f2;
+          long long xr = 0, xi = 0;
+          if (rowok) {
+            const CBits<TI> x = ld_cplx(src + 2 * H);
+            xr = Fixed<TI, true>::of(x.re, ere);
+            xi = Fixed<TI, true>::of(x.im, eim);
+          }
+          hr += wm * (xr >> 27);
+          lr += wm * (xr & 0x7FFFFFF);
+          hm += wm * (xi >> 27);
+          lm += wm * (xi & 0x7FFFFFF);
+          if (fwd) {   // s_0 was counted twice
+            const long long a = (long long)(s0r - kBias), c = (long long)(s0i - kBias);
+            hr -= a >> 27;
+            lr -= a & 0x7FFFFFF;
+            hm -= c >> 27;
+            lm -= c & 0x7FFFFFF;
           }
         }
 #pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
+        for (int off = 1; off <= 16; off <<= 4) {   // the four threads of the line
           hr += __shfl_xor_sync(0xffffffffu, hr, off);
           lr += __shfl_xor_sync(0xffffffffu, lr, off);
-          hi_ += __shfl_xor_sync(0xffffffffu, hi_, off);
-          li += __shfl_xor_sync(0xffffffffu, li, off);
+          hm += __shfl_xor_sync(0xffffffffu, hm, off);
+          lm += __shfl_xor_sync(0xffffffffu, lm, off);
         }
         if (g == 0 && rowok) {
           // sum = 2^(E - 54) (h 2^27 + l) = T 2^(E - 51), T = h 2^24 + l / 8
           TO vr = ere == kNanRow ? qnan<TO>()
-                                 : scaled<TO>(hr * 16777216ll + ((lr + 4) >> 3), ere - F::EOFF - 51);
+                                 : scaled_any<TO>(hr * 16777216ll + ((lr + 4) >> 3), ere - F::EOFF - 51);
           TO vi = eim == kNanRow ? qnan<TO>()
-                                 : scaled<TO>(hi_ * 16777216ll + ((li + 4) >> 3), eim - F::EOFF - 51);
+                                 : scaled_any<TO>(hm * 16777216ll + ((lm + 4) >> 3), eim - F::EOFF - 51);
           if (fwd) {
             vr = times<TO>(vr, lastf);
             vi = times<TO>(vi, lastf);
@@ -348,11 +470,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         };
         fetch(0);
         for (int st = 0; st < nst && ok; ++st) {
-          long long v[8];
+          unsigned long long v[8];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            v[2 * i] = nx[i].x;
-            v[2 * i + 1] = nx[i].y;
+            v[2 * i] = (unsigned long long)nx[i].x;
+            v[2 * i + 1] = (unsigned long long)nx[i].y;
           }
           if (st + 1 < nst) fetch(st + 1);
           ok = put(v, dig + ((size_t)pp * nst + st) * bstride);
@@ -370,62 +492,46 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ---- epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
-    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators, four at a time
+    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators
     const int qd = warp & 3, cg = warp >> 2, CW = NT / 2;
     const int row = qd * 32 + lane;
+    const int l = (row >> 4) * 8 + (row & 7), part_c = (row >> 3) & 1;
     const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cg * CW);
     // sums over several K groups are kept here between the groups
     long long* part = reinterpret_cast<long long*>(kcta + (size_t)2 * nst * kKeepStage) + tid;
     uint32_t pass = 0;
     int ti = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
-      const int fld = tile / tpf;
-      const int line = (tile - fld * tpf) * (kRows / 2) + (row >> 1);
-      if (!W.wait_warp(barRow + 8 * (ti & 1), (ti >> 1) & 1)) break;
-      const int me = sE[(ti & 1) * kRows + row];
-      const long long mid = sC[(ti & 1) * kRows + row];
+      const int fld = tile / tpf, rbuf = ti % kRB;
+      const int line = (tile - fld * tpf) * (kRows / 2) + l;
+      if (!W.wait_warp(barRow + 8 * rbuf, (ti / kRB) & 1)) break;
+      const int me = sE[rbuf * kRows + row];
+      const long long mid = sC[rbuf * kRows + row];
       __syncwarp();
       if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * (ti & 1))
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
                      : "memory");
       const bool rowok = line < nlines, nan = me == kNanRow;
       const int ex = me - F::EOFF - q;   // result = T 2^(E - q)
-      TO* dst = out + ((size_t)fld * fso + (size_t)(rowok ? line : 0) * Nz) * 2 + (row & 1);
+      const bool safe =
+          __all_sync(0xffffffffu, !rowok || (!nan && safe_exp<TO>(ex))) != 0;
+      TO* dst = out + ((size_t)fld * fso + (size_t)(rowok ? line : 0) * Nz) * 2 + part_c;
       bool ok = true;
       for (int pp = 0; pp < 2 * nsl && ok; ++pp) {
         const int par = pp & 1, m0 = (pp >> 1) * NT + cg * CW;
+        TO* d = dst + 2 * (size_t)(2 * m0 + par);
         for (int c = 0; c < kc; ++c, ++pass) {
           if (!(ok = W.wait_warp(barAccFull, pass & 1))) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          for (int c0 = 0; c0 < CW; c0 += 4) {
-            uint32_t v[7][4];
-            tmem_ld7x4(tb + (uint32_t)c0, NT, v);
-            if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
-              asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-              __syncwarp();
-              if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barAccFree)
-                             : "memory");
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int m = m0 + c0 + e;
-              if (m < H && rowok) {
-                long long T = recombine(v, e);
-                if (c > 0) T += part[(c0 + e) * kEW * 32];
-                if (c + 1 < kc) {
-                  part[(c0 + e) * kEW * 32] = T;
-                  continue;
-                }
-                if (par == 0) {
-                  // (-1)^m x_H Y; the forward weight of n = 0 is half the others'
-                  const long long t = (fwd && m == 0) ? mid / 2 : mid;
-                  T += (m & 1) ? -t : t;
-                }
-                dst[2 * (size_t)(2 * m + par)] = nan ? qnan<TO>() : scaled<TO>(T, ex);
-              }
-            }
-          }
+          if (nmag == 7)
+            epilogue_pass<TO, 7>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
+                                 d, barAccFree, lane);
+          else if (nmag == 3)
+            epilogue_pass<TO, 3>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
+                                 d, barAccFree, lane);
+          else
+            epilogue_pass<TO, 0>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
+                                 d, barAccFree, lane);
         }
       }
       if (!ok) break;
@@ -447,7 +553,7 @@ cudaError_t launch_t(const void* in, long long fsi, void* out, long long fso, in
   const int grid = (int)std::min<long long>(ntiles, t.ctas);
   cheb_tc_kernel<TI, TO><<<grid, kThreads, kSmem, s>>>(
       (const TI*)in, fsi, (TO*)out, fso, nlines, Nz, tpf, (int)ntiles, t.NT, t.nsl, t.nst, t.kc,
-      t.gst, t.dig, t.keep, (long long)cheb_tc_keep_bytes(Nz - 1), t.dir == 0 ? 1 : 0, t.q, t.ymid,
+      t.gst, t.nmag, t.dig, t.keep, (long long)cheb_tc_keep_bytes(Nz - 1), t.dir == 0 ? 1 : 0, t.q, t.ymid,
       t.dir == 0 ? 0.5 / (double)(Nz - 1) : 1.0, err);
   return cudaGetLastError();
 }
@@ -490,21 +596,33 @@ int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
   for (int a = N + 1; a < 2 * N; ++a) cs[a] = cs[2 * N - a];
   t->ymid = dir == 0 ? (long long)llroundl(ldexpl(2.0L / (long double)N, t->q)) : 1ll << 54;
   const int NT = t->NT;
+  double bound = 0.0, bound3 = 0.0;   // of all accumulators and of the first three
   const size_t block = (size_t)kPlanes * NT * kKS;
   dig.assign((size_t)2 * t->nsl * t->nst * block, 0);
   for (int m = 0; m < H; ++m)
-    for (int par = 0; par < 2; ++par)
+    for (int par = 0; par < 2; ++par) {
+      double sum[kPlanes] = {};          // sum_k |digit j|
       for (int k = 0; k < H; ++k) {
         const int st = k / kKS, kk = k % kKS;
         const int pos = 4 * (kk & 3) + (kk >> 2);   // k = 16 st + g + 4 e sits at position 4 g + e
-        const unsigned long long y = (unsigned long long)weight(cs, N, dir, t->q, 2 * m + par, k) + kBias;
+        const unsigned long long y =
+            (unsigned long long)weight(cs, N, dir, t->q, 2 * m + par, k) + kBias;
         uint16_t* b = dig.data() + ((size_t)(2 * (m / NT) + par) * t->nst + st) * block;
         for (int j = 0; j < kPlanes; ++j) {
-          const int row = j * NT + m % NT;
-          b[((size_t)(pos >> 3) * kPlanes * NT + row) * 8 + (pos & 7)] =
-              bf16_bits((float)((int)((y >> (8 * (6 - j))) & 255ull) - 128));
+          const int row = j * NT + m % NT, d = (int)((y >> (8 * (6 - j))) & 255ull) - 128;
+          b[((size_t)(pos >> 3) * kPlanes * NT + row) * 8 + (pos & 7)] = bf16_bits((float)d);
+          sum[j] += abs(d);
         }
       }
+      // |G_d| <= 128 sum_{j <= d} sum_k |b_jk|
+      double acc = 0.0;
+      for (int j = 0; j < kPlanes; ++j) {
+        acc += 128.0 * sum[j];
+        if (j == 2) bound3 = std::max(bound3, acc);
+      }
+      bound = std::max(bound, acc);
+    }
+  t->nmag = bound <= 4194304.0 ? 7 : (bound3 <= 4194304.0 ? 3 : 0);
   return 0;
 }
 

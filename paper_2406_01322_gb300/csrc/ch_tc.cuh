@@ -160,7 +160,10 @@ template <> struct FBits<double> {
   static constexpr int EMAX = 0x7FF, EOFF = 1022, KEY_MB = 20;
   typedef unsigned long long U;
   __device__ static U bits(double x) { return (U)__double_as_longlong(x); }
-  __device__ static unsigned key(U b) { return (unsigned)(b >> 32) & 0x7FFFFFFFu; }
+  // (the low word only tells the smallest subnormals from zero)
+  __device__ static unsigned key(U b) {
+    return max((unsigned)(b >> 32) & 0x7FFFFFFFu, (unsigned)((unsigned)b != 0));
+  }
 };
 template <> struct FBits<float> {
   static constexpr int EMAX = 0xFF, EOFF = 126, KEY_MB = 23;
@@ -178,47 +181,62 @@ template <> struct FBits<df> {
   }
   __device__ static unsigned key(U b) { return (unsigned)b & 0x7FFFFFFFu; }
 };
+// A row of zeros takes the scale kTinyScale.
 constexpr int kNanRow = 1 << 14;   // scale of a row that holds an infinity or NaN
+constexpr int kTinyScale = 64;     // row scales below it need care with subnormals (Fixed)
 template <typename T> __device__ __forceinline__ int row_scale(unsigned key) {
   typedef FBits<T> F;
   const int e = (int)(key >> F::KEY_MB);
   if (e >= F::EMAX) return kNanRow;
+  if (key == 0) return kTinyScale;
   const unsigned frac = key & ((1u << F::KEY_MB) - 1u);
   return max(e, 1) + (frac > (unsigned)(0.95 * (1 << F::KEY_MB)) ? 1 : 0);
 }
 
 // round(x 2^(54-E)) of the element with bit pattern b in a row of scale maxe (E = maxe - EOFF);
-// zero in a row that holds an infinity or NaN (kNanRow), whose results are NaN
-__device__ __forceinline__ long long fixed_f32(unsigned b, int maxe) {
+// zero in a row that holds an infinity or NaN (kNanRow), whose results are NaN.  TINY = false: the
+// implicit mantissa bit is set whatever the exponent field, which is right for normal numbers and
+// harmless for zeros and subnormals once the row scale is at least kTinyScale (they shift out).
+template <bool TINY> __device__ __forceinline__ long long fixed_f32(unsigned b, int maxe) {
   int ef = (int)((b >> 23) & 0xFFu);
-  unsigned m = b & 0x7FFFFFu;
-  if (ef) m |= 0x800000u;
-  else ef = 1;
+  unsigned m = (b & 0x7FFFFFu) | 0x800000u;
+  if (TINY && ef == 0) {
+    m = b & 0x7FFFFFu;
+    ef = 1;
+  }
   const int sh = min(maxe - ef, 63);
   const unsigned long long r = (((unsigned long long)m << 31 >> sh) + 1ull) >> 1;
   const long long s = (long long)((int)b >> 31);
   return ((long long)r ^ s) - s;
 }
-template <typename T> __device__ long long to_fixed(typename FBits<T>::U b, int maxe);
-template <> __device__ __forceinline__ long long to_fixed<double>(unsigned long long b, int maxe) {
-  const unsigned hi = (unsigned)(b >> 32);
-  int ef = (int)((hi >> 20) & 0x7FFu);
-  unsigned mh = hi & 0xFFFFFu;
-  if (ef) mh |= 0x100000u;
-  else ef = 1;
-  const int sh = min(maxe - ef, 63);
-  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)b) << 2;
-  const unsigned long long r = ((m >> sh) + 1ull) >> 1;
-  const long long s = (long long)((int)hi >> 31);
-  return ((long long)r ^ s) - s;
-}
-template <> __device__ __forceinline__ long long to_fixed<float>(unsigned b, int maxe) {
-  return fixed_f32(b, maxe);
-}
+template <typename T, bool TINY> struct Fixed;
+template <bool TINY> struct Fixed<double, TINY> {
+  __device__ __forceinline__ static long long of(unsigned long long b, int maxe) {
+    const unsigned hi = (unsigned)(b >> 32);
+    int ef = (int)((hi >> 20) & 0x7FFu);
+    unsigned mh = (hi & 0xFFFFFu) | 0x100000u;
+    if (TINY && ef == 0) {
+      mh = hi & 0xFFFFFu;
+      ef = 1;
+    }
+    const int sh = min(maxe - ef, 63);
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)b) << 2;
+    const unsigned long long r = ((m >> sh) + 1ull) >> 1;
+    const long long s = (long long)((int)hi >> 31);
+    return ((long long)r ^ s) - s;
+  }
+};
+template <bool TINY> struct Fixed<float, TINY> {
+  __device__ __forceinline__ static long long of(unsigned b, int maxe) {
+    return fixed_f32<TINY>(b, maxe);
+  }
+};
 // double-float: both parts converted and added (one extra unit of rounding at most)
-template <> __device__ __forceinline__ long long to_fixed<df>(unsigned long long b, int maxe) {
-  return fixed_f32((unsigned)b, maxe) + fixed_f32((unsigned)(b >> 32), maxe);
-}
+template <bool TINY> struct Fixed<df, TINY> {
+  __device__ __forceinline__ static long long of(unsigned long long b, int maxe) {
+    return fixed_f32<TINY>((unsigned)b, maxe) + fixed_f32<true>((unsigned)(b >> 32), maxe);
+  }
+};
 
 // Digit plane i (0 = most significant) of two values, as two bf16 in one word (first in the low
 // half): byte 6 - i of the biased integers, u, stands for the digit u - 128.  With l = u mod 128,
@@ -234,42 +252,54 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byt
   return *reinterpret_cast<uint32_t*>(&r);
 }
 
-// round(U / 64) of the seven diagonal accumulators (exact integers below 2^24 held as fp32):
-// U = sum_d 256^(6-d) G_d.  Sums are formed modulo 2^64; |U| / 64 < 2^63 for sums of at most 496
-// terms per row (|sum_k x_k B_nk| < 496 max|x| max|B|).
+// round(U / 64) of column e of the seven diagonal accumulators (exact integers below 2^24 held as
+// fp32), U = sum_d 256^(6-d) G_d.  Sums are formed modulo 2^64; |U| / 64 < 2^63 for sums of at most
+// 496 terms per row (|sum_k x_k B_nk| < 496 max|x| max|B|).  The first NMAG accumulators are known
+// to stay within 2^22 and convert by one float addition (the low bits of 1.5 2^23 + G are G), the
+// others by the conversion instruction (a quarter of the rate).
+template <int NMAG>
 __device__ __forceinline__ long long recombine(const uint32_t (&v)[7][4], int e) {
   int g[7];
 #pragma unroll
-  for (int d = 0; d < 7; ++d) g[d] = __float2int_rz(__uint_as_float(v[d][e]));
+  for (int d = 0; d < 7; ++d)
+    g[d] = d < NMAG ? __float_as_int(__uint_as_float(v[d][e]) + 12582912.0f) - 0x4B400000
+                    : __float2int_rz(__uint_as_float(v[d][e]));
   const int h = g[0] * 256 + g[1], m = g[2] * 256 + g[3];
   const long long l = (long long)g[4] * 65536 + ((long long)g[5] * 256 + (long long)g[6]);
   return (long long)((unsigned long long)(unsigned)h << 34) + (long long)m * 262144 +
          ((l + 32) >> 6);
 }
 
-// T 2^e rounded once to the output type.  The integer converts in one instruction, the power of
-// two is added to the exponent field; ldexp outside the normal range.
+// T 2^e rounded once to the output type: the integer converts in one instruction and the power of
+// two is added to the exponent field, right when safe_exp(e) (the result of every |T| in
+// 1 .. 2^63 is a normal number).
+template <typename TO> __device__ __forceinline__ bool safe_exp(int e) {
+  return FBits<TO>::EMAX == 0xFF ? e > -120 && e < 60 : e > -1000 && e < 950;
+}
 template <typename TO> __device__ TO scaled(long long T, int e);
 template <> __device__ __forceinline__ double scaled<double>(long long T, int e) {
   const double v = __ll2double_rn(T);
-  const int hi = __double2hiint(v);
-  const int be = ((hi >> 20) & 0x7FF) + e;
-  if (T == 0) return 0.0;
-  if (be <= 0 || be >= 2047) return ldexp(v, e);
-  return __hiloint2double(hi + (e << 20), __double2loint(v));
+  return __hiloint2double(__double2hiint(v) + (T != 0 ? e << 20 : 0), __double2loint(v));
 }
 template <> __device__ __forceinline__ float scaled<float>(long long T, int e) {
-  const float v = __ll2float_rn(T);
-  const int b = __float_as_int(v);
-  const int be = ((b >> 23) & 0xFF) + e;
-  if (T == 0) return 0.0f;
-  if (be <= 0 || be >= 255) return ldexpf(v, e);
-  return __int_as_float(b + (e << 23));
+  return __int_as_float(__float_as_int(__ll2float_rn(T)) + (T != 0 ? e << 23 : 0));
 }
 // double-float result: the high part rounded to float, the low part from the exact remainder
 template <> __device__ __forceinline__ df scaled<df>(long long T, int e) {
   const long long hi = __float2ll_rn(__ll2float_rn(T));   // |T| < 2^62.93: no overflow
   return df(scaled<float>(hi, e), scaled<float>(T - hi, e));
+}
+// the same outside the safe exponents
+template <typename TO> __device__ TO scaled_any(long long T, int e);
+template <> __device__ __forceinline__ double scaled_any<double>(long long T, int e) {
+  return ldexp(__ll2double_rn(T), e);
+}
+template <> __device__ __forceinline__ float scaled_any<float>(long long T, int e) {
+  return ldexpf(__ll2float_rn(T), e);
+}
+template <> __device__ __forceinline__ df scaled_any<df>(long long T, int e) {
+  const long long hi = __float2ll_rn(__ll2float_rn(T));
+  return df(ldexpf(__ll2float_rn(hi), e), ldexpf(__ll2float_rn(T - hi), e));
 }
 template <typename TO> __device__ __forceinline__ TO qnan();
 template <> __device__ __forceinline__ double qnan<double>() {
@@ -283,25 +313,37 @@ template <> __device__ __forceinline__ df qnan<df>() {
 // ---- one K stage's MMAs -----------------------------------------------------------------------
 // A planes at shared address sA, the stacked B planes (7 NT rows) at sB, both 16 K wide in the
 // canonical no-swizzle K-major core-matrix layout; accumulators from tensor-memory column tmem.
-// A plane i times B rows 0 .. (7-i) NT, in pieces of at most 256 columns of about equal width (an
-// MMA of M = 128 takes N / 2 cycles, but not less than about 50).  init: the accumulators start
-// from zero (plane 0 covers all their columns).
-__device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t sA, uint32_t sB, int NT,
-                                            bool init) {
+// A plane i times B rows 0 .. (7-i) NT, in pieces of at most 256 columns of equal width (an MMA of
+// M = 128 takes N / 2 cycles, but not less than about 50).  init: the accumulators start from zero
+// (plane 0 covers all their columns).  NT is a template argument because the single issuing thread
+// is what limits the rate otherwise (NT = 64: 912 cycles of MMAs per stage; with the pieces worked
+// out at run time the issue took 2040).
+template <int NT>
+__device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint32_t sB, bool init) {
   // bf16 x bf16 -> fp32, both K-major, M = 128 (N added per MMA)
-  const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 4) << 24);
-  const uint32_t lbo_b = (uint32_t)(kPlanes * NT * 16);
+  constexpr uint32_t idesc0 =
+      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 4) << 24);
+  const uint64_t a0 = sdesc(sA, kALbo, 128), b0 = sdesc(sB, (uint32_t)(kPlanes * NT * 16), 128);
 #pragma unroll
   for (int i = 0; i < kPlanes; ++i) {
-    const uint64_t ad = sdesc(sA + (uint32_t)(i * kPlaneBytes), kALbo, 128);
-    const int ntot = (kPlanes - i) * NT;
-    const int np = (ntot + 255) >> 8;
-    const int len = ((ntot / np) + 15) & ~15;
+    const int ntot = (kPlanes - i) * NT, np = (ntot + 255) / 256;
+    const int len = (ntot / np + 15) / 16 * 16;
+#pragma unroll
     for (int n0 = 0; n0 < ntot; n0 += len) {
-      const int nlen = min(len, ntot - n0);
-      mma_bf16(tmem + (uint32_t)(i * NT + n0), ad, sdesc(sB + (uint32_t)(n0 * 16), lbo_b, 128),
-               idesc0 | ((uint32_t)(nlen >> 3) << 17), (uint32_t)!(init && i == 0));
+      const int nlen = len < ntot - n0 ? len : ntot - n0;
+      mma_bf16(tmem + (uint32_t)(i * NT + n0), a0 + (uint64_t)(i * (kPlaneBytes / 16)),
+               b0 + (uint64_t)n0, idesc0 | ((uint32_t)(nlen >> 3) << 17),
+               (uint32_t)!(init && i == 0));
     }
+  }
+}
+__device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t sA, uint32_t sB, int NT,
+                                            bool init) {
+  switch (NT) {
+    case 16: issue_stage_nt<16>(tmem, sA, sB, init); break;
+    case 32: issue_stage_nt<32>(tmem, sA, sB, init); break;
+    case 48: issue_stage_nt<48>(tmem, sA, sB, init); break;
+    default: issue_stage_nt<64>(tmem, sA, sB, init); break;
   }
 }
 
