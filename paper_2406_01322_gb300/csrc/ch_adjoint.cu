@@ -88,6 +88,8 @@ int ch_adjoint_begin(ch_grid* G, double* J) {
   // float64, no-slip walls, FFT Chebyshev transforms only
   if (G->prec != CH_PREC_FP64 || G->g.bc != 0 || G->cheb != CH_CHEB_FFT) return CH_ERR_ARG;
   if (chf::adj_xline_smem(G->g.Px) > (size_t)chf::kMaxSmem) return CH_ERR_SIZE;
+  const int pr = ch_adjoint_plan(G);
+  if (pr != CH_OK) return pr;
   if (!G->adj_block) {
     const size_t sb = (size_t)G->fs * sizeof(double2);
     const size_t nb = (size_t)G->g.Mx * G->g.ny * 6;  // wall-value adjoints
@@ -131,11 +133,11 @@ int reverse_core(ch_grid* G, const double2* ya, int first, cudaEvent_t* ev) {
   e[1] = chf::launch_adj_zrhs(g, G->a_Rb, G->a_L, G->a_mu, G->a_lam, G->a_mu2, G->a_nlb, G->fs,
                               first, G->a_bb, G->pz, s);
   if (ev) cudaEventRecord(ev[2], s);
-  e[2] = chf::launch_ypass(1, 0, g, g.Py, G->a_nlb, G->yb, kNl, G->fs, G->fsy, 1.0, G->py[0], s);
+  e[2] = ch_launch_y_adj(G, 1, G->a_nlb, (double2*)G->yb, kNl, s);
   if (ev) cudaEventRecord(ev[3], s);
   e[3] = chf::launch_adj_xline(g, ya, (const double2*)G->yb, G->a_x6, G->fsy, G->px[0], s);
   if (ev) cudaEventRecord(ev[4], s);
-  e[4] = chf::launch_ypass(0, 0, g, g.Py, G->a_x6, G->auxA, kYa, G->fsy, G->fs, 1.0, G->py[0], s);
+  e[4] = ch_launch_y_adj(G, 0, G->a_x6, G->auxA, kYa, s);
   if (ev) cudaEventRecord(ev[5], s);
   e[5] = chf::launch_fold_dy(g, G->auxA, G->fs, s);
   if (ev) cudaEventRecord(ev[6], s);
@@ -177,13 +179,11 @@ int adjoint_step_impl(ch_grid* G, const void* state, cudaEvent_t* ev) {
   G->nstep = h.nstep;
   G->t = h.t;
   G->nl_stale = 1;
-  const chf::YMap ym = chf::step_ymap();
   if (ev) cudaEventRecord(ev[0], s);
   // forward fields of s_n on the y-padded grid (the x line's linearisation point)
   cudaError_t e0 = chf::launch_zbwd(0, 0, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s);
   if (ev) cudaEventRecord(ev[1], s);
-  cudaError_t e1 = chf::launch_ypass(1, 0, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0,
-                                     G->py[0], s, &ym);
+  cudaError_t e1 = ch_launch_xy(G, 3, s);
   if (ev) cudaEventRecord(ev[2], s);
   if (e0 != cudaSuccess || e1 != cudaSuccess) {
     cudaGetLastError();

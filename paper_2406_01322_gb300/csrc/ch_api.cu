@@ -18,6 +18,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -187,21 +188,18 @@ thread_local cudaError_t t_last_cuda = cudaSuccess;
 int eval_products(ch_grid* G) {
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  const chf::YMap ym = step_ymap();
   CK(chf::launch_zbwd(0, G->prec, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s));
-  CK(chf::launch_ypass(1, G->prec, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0, G->py[G->prec], s, &ym));
-  CK(chf::launch_xline(G->prec, g, G->ya, G->yb, G->fsy, 1.0, G->px[G->prec], s));
+  CK(ch_launch_xy(G, 3, s));
+  CK(ch_launch_xy(G, 4, s));
   return CH_OK;
 }
 
 // non-linear terms of the current state: the products, then nl <- the seven combined lines of
 // the forward y pass (normalised)
 int eval_nonlinear_impl(ch_grid* G) {
-  const GridDev& g = G->g;
   const int r = eval_products(G);
   if (r != CH_OK) return r;
-  CK(chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs,
-                       1.0 / ((double)g.Px * (double)g.Py), G->py[G->prec], G->stream));
+  CK(ch_launch_xy(G, 5, G->stream));
   return CH_OK;
 }
 
@@ -211,7 +209,6 @@ int eval_nonlinear_impl(ch_grid* G) {
 // CH_STEP_KERNELS events: ev[p] is recorded after position p (right away for an empty position).
 int launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev = nullptr) {
   const GridDev& g = G->g;
-  const chf::YMap ym = step_ymap();
   const bool tc = G->cheb == CH_CHEB_TC;
   const int nlines = g.Mx * g.ny;
   cudaError_t e[CH_STEP_KERNELS];
@@ -250,17 +247,15 @@ int launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev = nullptr
   }
   if (ev) cudaEventRecord(ev[4], s);
   nvtxRangePushA("ybwd");
-  e[3] = chf::launch_ypass(1, G->prec, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0,
-                           G->py[G->prec], s, &ym);
+  e[3] = ch_launch_xy(G, 3, s);
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[5], s);
   nvtxRangePushA("xline");
-  e[4] = chf::launch_xline(G->prec, g, G->ya, G->yb, G->fsy, 1.0, G->px[G->prec], s);
+  e[4] = ch_launch_xy(G, 4, s);
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[6], s);
   nvtxRangePushA("yfwd");
-  e[5] = chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs,
-                           1.0 / ((double)g.Px * (double)g.Py), G->py[G->prec], s);
+  e[5] = ch_launch_xy(G, 5, s);
   nvtxRangePop();
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[7], s);
@@ -294,12 +289,113 @@ int bail(ch_grid* G, int code) {
   return code;
 }
 
+// gives back the newest n allocations
+void release_last(ch_grid* G, size_t n) {
+  for (; n > 0 && !G->allocs.empty(); --n) {
+    void* p = G->allocs.back();
+    if (G->ff) G->ff(p, G->actx);
+    else if (!G->af) cudaFree(p);
+    G->allocs.pop_back();
+  }
+}
+
+// one plan with its digits on the device; mode as in txy_plan
+int make_txy_plan(ch_grid* G, int mode, double scale, chf::TxyPlan* p) {
+  const GridDev& g = G->g;
+  std::vector<uint16_t> dig;
+  chf::txy_plan(mode, mode < 2 ? g.ny : g.Mx, mode < 2 ? g.Py : g.Px, scale, dig, p);
+  void* d = galloc(G, dig.size() * sizeof(uint16_t));
+  if (!d) return CH_ERR_ALLOC;
+  CK(cudaMemcpy(d, dig.data(), dig.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+  p->dig = (const uint16_t*)d;
+  return CH_OK;
+}
+
+// Plans and buffers of the tensor-core x/y transforms of a float64 grid.
+// Rule: from 2^15 modes on (below, a transform has fewer tiles than a third of the SMs and its
+// latency counts: 32 x 32 x 33, 16896 modes, y backward 25 against 21 us, x line 45 against 53,
+// y forward 30 against 33 by FFT; 48 x 48 x 49, 56448 modes, 39, 96 and 60 against 47, 137 and 75),
+// up to padded lengths of 1024 (the dense matrices grow with the length squared).
+constexpr int kTxyMaxP = 1024;
+constexpr long long kTxyMinModes = 1ll << 15;
+int setup_tx(ch_grid* G) {
+  const GridDev& g = G->g;
+  if (g.Px > kTxyMaxP || g.Py > kTxyMaxP || G->fs < kTxyMinModes) return CH_OK;
+  int dev = 0, nsm = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  chf::Txy t;
+  t.ctas = nsm < 1 ? 1 : nsm;
+  const double sc = 1.0 / ((double)g.Px * (double)g.Py);
+  chf::TxyPlan* plan[4] = {&t.yb, &t.yf, &t.xb, &t.xf};
+  const size_t before = G->allocs.size();
+  bool ok = true;
+  for (int i = 0; i < 4 && ok; ++i) {
+    const int r = make_txy_plan(G, i, i == 1 ? sc : 1.0, plan[i]);
+    if (r == CH_ERR_CUDA) return r;
+    ok = r == CH_OK;
+    t.keep_bytes = std::max(t.keep_bytes, chf::txy_keep_bytes(*plan[i]));
+  }
+  if (ok) ok = (t.keep = (char*)galloc(G, (size_t)t.ctas * t.keep_bytes)) != nullptr;
+  if (ok)
+    ok = (t.phys = (double*)galloc(G, (size_t)kNl * g.Px * g.Py * g.nz * sizeof(double))) != nullptr;
+  int* err = ok ? (int*)galloc(G, sizeof(int)) : nullptr;
+  if (!ok || !err) {   // no room: the float64 FFT kernels
+    cudaGetLastError();
+    release_last(G, G->allocs.size() - before);
+    return CH_OK;
+  }
+  CK(cudaMemset(err, 0, sizeof(int)));
+  t.err = G->tc_err = err;
+  G->tx = t;
+  G->use_tx = 1;
+  return CH_OK;
+}
+
 void drop_graph(ch_grid* G) {
   if (G->graph_ok) cudaGraphExecDestroy(G->gexec);
   G->graph_ok = 0;
 }
 
 }  // namespace
+
+cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s) {
+  const GridDev& g = G->g;
+  const FftPlan& py = G->py[G->prec];
+  if (stage == 3) {
+    chf::YMap ym = step_ymap();
+    ym.kys = 6.283185307179586476925 / g.ly;
+    return G->use_tx ? chf::launch_txy_y(1, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, ym, G->tx,
+                                         G->tx.yb, s)
+                     : chf::launch_ypass(1, G->prec, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0,
+                                         py, s, &ym);
+  }
+  if (stage == 4)
+    return G->use_tx ? chf::launch_txy_x(g, G->ya, G->yb, G->fsy, G->tx, s)
+                     : chf::launch_xline(G->prec, g, G->ya, G->yb, G->fsy, 1.0, G->px[G->prec], s);
+  return G->use_tx ? chf::launch_txy_ycomb(g, G->yb, G->nl, G->fsy, G->fs, G->tx, s)
+                   : chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs,
+                                       1.0 / ((double)g.Px * (double)g.Py), py, s);
+}
+
+cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out, int nf,
+                            cudaStream_t s) {
+  const GridDev& g = G->g;
+  const long long fi = dir == 1 ? G->fs : G->fsy, fo = dir == 1 ? G->fsy : G->fs;
+  if (!G->use_tx) return chf::launch_ypass(dir, 0, g, g.Py, in, out, nf, fi, fo, 1.0, G->py[0], s);
+  chf::YMap id;
+  for (int f = 0; f < chf::YMap::kMax; ++f) id.src[f] = f;
+  id.dy_mask = 0;
+  id.kys = 0.0;
+  return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, id, G->tx,
+                           dir == 1 ? G->tx.yb : G->tx_yf1, s);
+}
+
+// the reverse sweep's own plan (forward y transform without the step's 1 / (Px Py)), made once
+int ch_adjoint_plan(ch_grid* G) {
+  if (!G->use_tx || G->tx_yf1.dig) return CH_OK;
+  return make_txy_plan(G, 1, 1.0, &G->tx_yf1);
+}
 
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev) {
   return launch_step(G, first, s, ev);
@@ -492,6 +588,10 @@ int ch_init_grid(const ch_params* p, ch_alloc_fn alloc, ch_free_fn free_fn, void
   if (chf::zline_smem(g) > (size_t)kMaxSmem || chf::xline_smem(g.Px, sizeof(double2)) > (size_t)kMaxSmem) {
     return bail(G, CH_ERR_SIZE);
   }
+  if (G->prec == CH_PREC_FP64) {
+    st = setup_tx(G);
+    if (st != CH_OK) return bail(G, st);
+  }
   G->first = 1;
   G->fields_set = 0;
   G->nstep = 0;
@@ -586,7 +686,9 @@ int ch_step(ch_grid* G, int nsteps) {
 }
 
 int ch_launches_per_step(const ch_grid* G) {
-  return G ? (G->cheb == CH_CHEB_TC ? 8 : 6) : 0;
+  if (!G) return 0;
+  // the tensor-core x line is three launches (backward, products, forward), the forward y pass two
+  return (G->cheb == CH_CHEB_TC ? 8 : 6) + (G->use_tx ? 3 : 0);
 }
 
 int ch_step_timed(ch_grid* G, int nsteps, double* kernel_ms, double* total_ms) {
@@ -781,11 +883,19 @@ int ch_nonlinear(ch_grid* G, double* out9) {
   const double scale = 1.0 / ((double)g.Px * (double)g.Py);
   const int r = eval_products(G);
   if (r != CH_OK) return r;
-  CK(chf::launch_ypass(0, G->prec, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, scale,
-                       G->py[G->prec], G->stream));
+  if (G->use_tx) {
+    chf::YMap id;
+    for (int f = 0; f < chf::YMap::kMax; ++f) id.src[f] = f;
+    id.dy_mask = 0;
+    id.kys = 0.0;
+    CK(chf::launch_txy_y(0, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, id, G->tx, G->tx.yf,
+                         G->stream));
+  } else {
+    CK(chf::launch_ypass(0, G->prec, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, scale,
+                         G->py[G->prec], G->stream));
+  }
   CK(chf::launch_dct_lines(0, G->prec, g, G->nl, (double2*)out9, kNl, G->fs, G->pz, G->stream));
-  CK(chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs, scale, G->py[G->prec],
-                       G->stream));
+  CK(ch_launch_xy(G, 5, G->stream));
   return CH_OK;
 }
 
@@ -828,10 +938,10 @@ int ch_set_chebyshev(ch_grid* G, int method) {
         t[dir].keep = (char*)keep;
         t[dir].ctas = nsm;
       }
-      int* err = (int*)galloc(G, sizeof(int));
+      int* err = G->tc_err ? G->tc_err : (int*)galloc(G, sizeof(int));
       double2* cf = (double2*)galloc(G, (size_t)chf::kNc * G->fs * sizeof(double2));
       if (!err || !cf) return CH_ERR_ALLOC;
-      CK(cudaMemset(err, 0, sizeof(int)));
+      if (!G->tc_err) CK(cudaMemset(err, 0, sizeof(int)));
       G->tcf = t[0];
       G->tcb = t[1];
       G->tc_err = err;

@@ -126,6 +126,8 @@ struct ch_ensemble {
   int zsolve_tile;
   int ywq;                      // warp-FFT level of the grouped y passes (ensemble_ywq)
   int xwq;                      // the same for the grouped x line (padded x lengths)
+  int tx;                       // 1: a member's x/y stages run on the tensor cores; then every
+                                // member runs its own launches of those stages
   Tuning tune;
   std::string signature;
   cudaGraphExec_t gexec;
@@ -282,7 +284,10 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
   for (int st = 0; st < kStages; ++st) {
     cudaError_t e = cudaSuccess;
     if (tc && st == 0) e = member_transforms(E, 0, s);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && st >= 3 && E->tx) {
+      for (ch_grid* G : E->members)
+        if (e == cudaSuccess) e = ch_launch_xy(G, st, s);
+    } else if (e == cudaSuccess)
       e = chf::launch_grouped(st, E->prec, E->dmem, E->dbegin + (size_t)st * (n + 1), n,
                               grid_of(E, st), E->smem[st], E->zsolve_tile, tc,
                               st == 4 ? E->xwq : E->ywq, s);
@@ -410,6 +415,8 @@ int ch_ensemble_init(const ch_params* members, int n, ch_alloc_fn alloc, ch_free
     if (st == CH_OK) E->members.push_back(G);
   }
   if (st == CH_OK) E->signature = signature_of(E);
+  E->tx = 0;
+  for (ch_grid* G : E->members) E->tx |= G->use_tx;
   if (st == CH_OK) {
     E->dmem = (Member*)ealloc(E, n * sizeof(Member));
     E->dbegin = (int*)ealloc(E, (size_t)kStages * (n + 1) * sizeof(int));

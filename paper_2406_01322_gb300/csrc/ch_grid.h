@@ -96,11 +96,24 @@ struct ch_grid {
   chf::ChebTc tcf, tcb;
   double2* cf = nullptr;
   int* tc_err = nullptr;
+
+  // float64 y and x transforms of the step on the tensor cores (use_tx); tx_yf1: the forward y
+  // transform without the 1 / (Px Py), for the reverse sweep
+  int use_tx = 0;
+  chf::Txy tx;
+  chf::TxyPlan tx_yf1;
 };
 
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev);
 int ch_eval_nonlinear(ch_grid* G);
+// the x/y stages of the step on stream s: 3 y backward (bw -> ya), 4 x line (ya -> yb), 5 y
+// forward with the combinations (yb -> nl)
+cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s);
+// float64 y pass of the reverse sweep (identity field map, scale 1) on the padded grid
+cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out, int nf,
+                            cudaStream_t s);
+int ch_adjoint_plan(ch_grid* G);
 // u v w phi phi_x phi_y phi_z of the state on the unpadded grid into phys7 ((nz, ny, nx) each)
 int ch_state_phys7(ch_grid* G);
 // frees the reverse-sweep workspace if allocated

@@ -303,6 +303,34 @@ cudaError_t cheb_tc_prepare();
 cudaError_t launch_cheb_tc(int tin, int tout, const void* in, long long fsi, void* out,
                            long long fso, int nf, int nlines, int Nz, const ChebTc& t, int* err,
                            cudaStream_t s);
+// Float64 y and x transforms as exact-split products on the tensor cores (ch_txy.cu).  Plan of one
+// transform: nout columns in nsl slices of NT, nk inputs in nst stages of 16 cut into kc groups of
+// gst, `stages` stage buffers in smem bytes of shared memory.
+struct TxyPlan {
+  const uint16_t* dig = nullptr;   // device: matrix digits (txy_plan)
+  int nk = 0, nout = 0, NT = 0, nsl = 0, nst = 0, kc = 0, gst = 0, stages = 0, nmag = 0, q = 0;
+  long long ymid = 0;              // weight of the middle sample of a forward transform, times 2^q
+  size_t smem = 0;
+};
+struct Txy {
+  TxyPlan yb, yf, xb, xf;          // y backward / forward (padded), x backward / forward
+  char* keep = nullptr;            // per persistent CTA: keep_bytes of fixed-point values
+  size_t keep_bytes = 0;
+  double* phys = nullptr;          // nine real fields (Px, Py, Nz)
+  int ctas = 0;
+  int* err = nullptr;              // |= 1 if a bounded wait gave up
+};
+// mode 0 y backward, 1 y forward (times scale), 2 x backward, 3 x forward; n1 = Ny (y) or Mx (x), P
+// the transform length
+int txy_plan(int mode, int n1, int P, double scale, std::vector<uint16_t>& dig, TxyPlan* t);
+size_t txy_keep_bytes(const TxyPlan& t);
+cudaError_t launch_txy_y(int dir, const GridDev& g, int P, const void* in, void* out, int nf,
+                         long long fs_in, long long fs_out, const YMap& map, const Txy& x,
+                         const TxyPlan& plan, cudaStream_t s);
+cudaError_t launch_txy_ycomb(const GridDev& g, const void* in, void* out9, long long fs_in,
+                             long long fs_out, const Txy& x, cudaStream_t s);
+cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long long fs, const Txy& x,
+                         cudaStream_t s);
 // one bounded mbarrier wait that runs out on purpose (sets *err |= 1 after the wait bound)
 cudaError_t launch_wait_selftest(int* err, int nwaits, cudaStream_t s);
 // float64 FMA-rate probe: `blocks` CTAs of 256 threads, `iters` iterations of eight independent

@@ -94,7 +94,7 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
                                               TO* dst, uint32_t barAccFree, int lane) {
   for (int c0 = 0; c0 < CW; c0 += 4) {
     uint32_t v[7][4];
-    tmem_ld7x4(tb + (uint32_t)c0, NT, v);
+    tmem_ldx4<7>(tb + (uint32_t)c0, NT, v);
     if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -103,7 +103,7 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
     }
     long long T[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG>(v, e);
+    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG, 7>(v, e);
     if (kc > 1) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 goto drain;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               const uint32_t sA = sBase + slot * (uint32_t)kStageBytes;
-              issue_stage(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
+              issue_stage<7>(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
               any = true;
               mma_commit(barEmpty + 8 * slot);
               if (++slot == kStages) {
@@ -564,13 +564,6 @@ uint16_t bf16_bits(float f) {
   return (uint16_t)(u >> 16);   // exact: a digit has at most eight significant bits
 }
 
-// weight of input k in output n < N, times 2^q; cs[a] = cos(pi a / N)
-long long weight(const std::vector<long double>& cs, int N, int dir, int q, int n, int k) {
-  long double v = cs[((long long)n * k) % (2 * N)];
-  if (dir == 0) v *= (k == 0 ? 1.0L : 2.0L) / ((n == 0 ? 2.0L : 1.0L) * (long double)N);
-  return (long long)llroundl(ldexpl(v, q));
-}
-
 }  // namespace
 
 int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
@@ -586,14 +579,20 @@ int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
   t->q = 54;
   if (dir == 0)
     for (int h = H; h > 1; h >>= 1) ++t->q;
+  // the weights times 2^q: W_nk = w cos(pi n k / N), w = 2 / N (forward, half of it at n = 0 and at
+  // k = 0, where the cosine is 1) or 1; tabulated by angle
   const long double pi = 3.141592653589793238462643383279502884L;
-  std::vector<long double> cs(2 * N);   // cos(pi a / N)
+  const long double w = dir == 0 ? 2.0L / (long double)N : 1.0L;
+  std::vector<long long> Y(2 * N);
   for (int a = 0; a <= N; ++a) {
-    if (2 * a == N) cs[a] = 0.0L;
-    else if (2 * a < N) cs[a] = cosl(pi * (long double)a / (long double)N);
-    else cs[a] = -cosl(pi * (long double)(N - a) / (long double)N);
+    long double c = 0.0L;
+    if (2 * a < N) c = cosl(pi * (long double)a / (long double)N);
+    else if (2 * a > N) c = -cosl(pi * (long double)(N - a) / (long double)N);
+    Y[a] = (long long)llroundl(ldexpl(w * c, t->q));
   }
-  for (int a = N + 1; a < 2 * N; ++a) cs[a] = cs[2 * N - a];
+  for (int a = N + 1; a < 2 * N; ++a) Y[a] = Y[2 * N - a];
+  const long long Yh = (long long)llroundl(ldexpl(0.5L * w, t->q));
+  const long long Yq = (long long)llroundl(ldexpl(0.25L * w, t->q));
   t->ymid = dir == 0 ? (long long)llroundl(ldexpl(2.0L / (long double)N, t->q)) : 1ll << 54;
   const int NT = t->NT;
   double bound = 0.0, bound3 = 0.0;   // of all accumulators and of the first three
@@ -605,8 +604,11 @@ int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
       for (int k = 0; k < H; ++k) {
         const int st = k / kKS, kk = k % kKS;
         const int pos = 4 * (kk & 3) + (kk >> 2);   // k = 16 st + g + 4 e sits at position 4 g + e
-        const unsigned long long y =
-            (unsigned long long)weight(cs, N, dir, t->q, 2 * m + par, k) + kBias;
+        const int n = 2 * m + par;
+        const long long yk = dir == 1 || (n > 0 && k > 0) ? Y[((long long)n * k) % (2 * N)]
+                             : n == 0 && k == 0          ? Yq
+                                                         : Yh;
+        const unsigned long long y = (unsigned long long)yk + kBias;
         uint16_t* b = dig.data() + ((size_t)(2 * (m / NT) + par) * t->nst + st) * block;
         for (int j = 0; j < kPlanes; ++j) {
           const int row = j * NT + m % NT, d = (int)((y >> (8 * (6 - j))) & 255ull) - 128;

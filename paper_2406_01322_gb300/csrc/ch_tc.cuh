@@ -7,8 +7,9 @@
 //   X_k = sum_{i=0..6} a_ik 256^(6-i),  a_ik in [-128, 127],
 // which bf16 holds exactly.  A digit product sum_k a_ik b_jnk is an integer, and the products with
 // the same i + j = d share one fp32 accumulator G_d: |G_d| <= 7 2^14 K < 2^24 for K <= 144, so
-// every accumulation is exact.  d <= 6 is kept (28 products; the dropped ones are random-signed
-// and of order 2^-53 of max|x| max|B|), and
+// every accumulation is exact.  d <= 6 is kept (28 products; the dropped ones are random-signed,
+// about 2^-54 sqrt(K) of max|x| max|B| together), or d <= 7 (34 products, ND = 8 accumulators: the
+// dropped ones fall 2^8 below the quantisation of the operands), and
 //   sum_k X_k Y_nk = 256^6 U,  U = sum_{d<=6} 256^(6-d) G_d
 // is recombined in 64-bit integers.  Eight-bit digits need 28 products where seven-bit ones
 // (eight planes, K < 512) need 36; transforms with longer sums are cut into K groups of at most
@@ -130,11 +131,12 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       "l"(src), "r"(bytes), "r"(bar), "l"(pol)
       : "memory");
 }
-// seven 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32
-// lanes, then one wait that the values depend on
-__device__ __forceinline__ void tmem_ld7x4(uint32_t addr, int stride, uint32_t (&v)[7][4]) {
+// ND 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32 lanes,
+// then one wait that the values depend on
+template <int ND>
+__device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&v)[ND][4]) {
 #pragma unroll
-  for (int d = 0; d < 7; ++d)
+  for (int d = 0; d < ND; ++d)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3])
                  : "r"(addr + (uint32_t)(d * stride)));
@@ -144,7 +146,8 @@ __device__ __forceinline__ void tmem_ld7x4(uint32_t addr, int stride, uint32_t (
                  "+r"(v[2][2]), "+r"(v[2][3]), "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]),
                  "+r"(v[3][3]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[4][2]), "+r"(v[4][3]),
                  "+r"(v[5][0]), "+r"(v[5][1]), "+r"(v[5][2]), "+r"(v[5][3]), "+r"(v[6][0]),
-                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3])
+                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3]), "+r"(v[ND - 1][0]),
+                 "+r"(v[ND - 1][1]), "+r"(v[ND - 1][2]), "+r"(v[ND - 1][3])
                :
                : "memory");
 }
@@ -252,22 +255,23 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byt
   return *reinterpret_cast<uint32_t*>(&r);
 }
 
-// round(U / 64) of column e of the seven diagonal accumulators (exact integers below 2^24 held as
+// round(U / 64) of column e of the ND diagonal accumulators (exact integers below 2^24 held as
 // fp32), U = sum_d 256^(6-d) G_d.  Sums are formed modulo 2^64; |U| / 64 < 2^63 for sums of at most
 // 496 terms per row (|sum_k x_k B_nk| < 496 max|x| max|B|).  The first NMAG accumulators are known
 // to stay within 2^22 and convert by one float addition (the low bits of 1.5 2^23 + G are G), the
 // others by the conversion instruction (a quarter of the rate).
-template <int NMAG>
-__device__ __forceinline__ long long recombine(const uint32_t (&v)[7][4], int e) {
-  int g[7];
+template <int NMAG, int ND>
+__device__ __forceinline__ long long recombine(const uint32_t (&v)[ND][4], int e) {
+  int g[ND];
 #pragma unroll
-  for (int d = 0; d < 7; ++d)
+  for (int d = 0; d < ND; ++d)
     g[d] = d < NMAG ? __float_as_int(__uint_as_float(v[d][e]) + 12582912.0f) - 0x4B400000
                     : __float2int_rz(__uint_as_float(v[d][e]));
   const int h = g[0] * 256 + g[1], m = g[2] * 256 + g[3];
-  const long long l = (long long)g[4] * 65536 + ((long long)g[5] * 256 + (long long)g[6]);
-  return (long long)((unsigned long long)(unsigned)h << 34) + (long long)m * 262144 +
-         ((l + 32) >> 6);
+  long long l = (long long)g[4] * 65536 + ((long long)g[5] * 256 + (long long)g[6]);
+  if (ND == 8) l = (l * 256 + (long long)g[ND - 1] + 8192) >> 14;
+  else l = (l + 32) >> 6;
+  return (long long)((unsigned long long)(unsigned)h << 34) + (long long)m * 262144 + l;
 }
 
 // T 2^e rounded once to the output type: the integer converts in one instruction and the power of
@@ -318,7 +322,7 @@ template <> __device__ __forceinline__ df qnan<df>() {
 // (plane 0 covers all their columns).  NT is a template argument because the single issuing thread
 // is what limits the rate otherwise (NT = 64: 912 cycles of MMAs per stage; with the pieces worked
 // out at run time the issue took 2040).
-template <int NT>
+template <int NT, int ND>
 __device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint32_t sB, bool init) {
   // bf16 x bf16 -> fp32, both K-major, M = 128 (N added per MMA)
   constexpr uint32_t idesc0 =
@@ -326,7 +330,10 @@ __device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint3
   const uint64_t a0 = sdesc(sA, kALbo, 128), b0 = sdesc(sB, (uint32_t)(kPlanes * NT * 16), 128);
 #pragma unroll
   for (int i = 0; i < kPlanes; ++i) {
-    const int ntot = (kPlanes - i) * NT, np = (ntot + 255) / 256;
+    // diagonals i .. 6, and with ND = 8 diagonal 7 of planes 1 .. 6; plane 1 touches diagonal 7
+    // first, in an MMA of its own that may start it from zero
+    const int nb = (ND == 8 && i > 1) ? ND - i : kPlanes - i;
+    const int ntot = nb * NT, np = (ntot + 255) / 256;
     const int len = (ntot / np + 15) / 16 * 16;
 #pragma unroll
     for (int n0 = 0; n0 < ntot; n0 += len) {
@@ -335,15 +342,19 @@ __device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint3
                b0 + (uint64_t)n0, idesc0 | ((uint32_t)(nlen >> 3) << 17),
                (uint32_t)!(init && i == 0));
     }
+    if (ND == 8 && i == 1)
+      mma_bf16(tmem + (uint32_t)(7 * NT), a0 + (uint64_t)(kPlaneBytes / 16),
+               b0 + (uint64_t)(6 * NT), idesc0 | ((uint32_t)(NT >> 3) << 17), (uint32_t)!init);
   }
 }
+template <int ND>
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t sA, uint32_t sB, int NT,
                                             bool init) {
   switch (NT) {
-    case 16: issue_stage_nt<16>(tmem, sA, sB, init); break;
-    case 32: issue_stage_nt<32>(tmem, sA, sB, init); break;
-    case 48: issue_stage_nt<48>(tmem, sA, sB, init); break;
-    default: issue_stage_nt<64>(tmem, sA, sB, init); break;
+    case 16: issue_stage_nt<16, ND>(tmem, sA, sB, init); break;
+    case 32: issue_stage_nt<32, ND>(tmem, sA, sB, init); break;
+    case 48: issue_stage_nt<48, ND>(tmem, sA, sB, init); break;
+    default: issue_stage_nt<64, ND>(tmem, sA, sB, init); break;
   }
 }
 

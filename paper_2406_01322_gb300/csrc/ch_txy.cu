@@ -1,0 +1,803 @@
+// Float64 Fourier transforms along y and x (Sec. 3.2.1, with the 3/2-rule padding and truncation)
+// as exact-split products on the tensor cores (ch_tc.cuh): dense real cosine and sine matrices of
+// the padded lengths, float64-accurate, in place of shared-memory FFTs on the float64 pipe.
+//
+// GB300 issues about 1.6 float64 operations per clock per SM; a padded line of 192 points costs
+// about 12 of them per real sample by FFT, which is what bounded these passes.  As digit products
+// the same transforms need no float64 arithmetic: about 45 integer instructions per sample
+// converted, 30 per sample produced, and tensor work that stays below both for the lengths used.
+//
+// Four transforms, n = 0 .. nout - 1 and P the padded length:
+//   YB (modes -> samples in y):  f(n), f(P-n) = C +- i S,  C = sum_k s_k cos, S = sum_k d_k sin,
+//      s_k = c_k + c_{-k}, d_k = c_k - c_{-k} (s_0 = c_0), k < Ny / 2;
+//   YF (samples -> modes in y):  c_n, c_{-n} = C -+ i S,  s_k = f(k) + f(P-k), d_k = f(k) - f(P-k);
+//   XB (half spectrum -> real samples in x):  f(n), f(P-n) = E +- O,
+//      E = Re c_0 + 2 sum Re c_k cos, O = -2 sum Im c_k sin;
+//   XF (real samples -> half spectrum):  Re c_n = sum s_k cos, Im c_n = -sum d_k sin;
+// angles 2 pi k n / P.  The sums and differences s, d are exact in fixed point, both products of an
+// output are recombined as integers of one scale and added exactly, so every result is rounded
+// once.  For even P the sample k = P / 2 of a forward transform enters as (-1)^n times its weight
+// (added to the recombined integer), and the output n = P / 2 of a backward transform, an
+// alternating sum, is formed exactly by the producers.  Eight diagonals of digit products are kept
+// (34 products): with the 28 of seven diagonals a 128^3 step's error against 64 bits rose from
+// 1.8e-14 to 3.1e-14.
+//
+// Tiles, warps and stages as in the Chebyshev transform (ch_tc.cu): a tile is 64 complex lines
+// (re and im rows; YB, YF) or 128 lines (XB, XF), lines neighbouring in memory so that every load
+// and store of a warp covers whole sectors; passes are (output slice, cosine or sine product, K
+// group).  The recombined cosine products wait in shared memory for the sine ones.
+#include <math.h>
+#include <stdint.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "ch_internal.h"
+#include "ch_tc.cuh"
+
+namespace chf {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kPW = 8, kEW = 8, kSW = 3;               // producer, epilogue and scan warps
+constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
+constexpr int kMaxStages = 6;
+constexpr int kRB = 3;                                 // tiles whose row scales are held
+constexpr int kBars = 3 * kMaxStages + 3 + 2 * kRB;
+constexpr size_t kTail = kRB * kRows * (sizeof(long long) + sizeof(int)) + (size_t)(kBars + 1) * 8;
+// fixed-point values of one pass's stage block kept in global memory, eight per producer thread
+constexpr size_t kKeepStage = (size_t)kPW * 32 * 8 * sizeof(long long);
+
+__host__ __device__ constexpr int stage_bytes(int NT) { return kABytes + b_stage_bytes(NT); }
+
+enum { YB = 0, YF = 1, XB = 2, XF = 3 };
+
+struct Args {
+  const double* in;
+  double* out;
+  long long fsi, fso;         // field strides (complex elements; real samples for XB out, XF in)
+  int src[16];                // input field of each output field
+  unsigned dmask;             // output fields of i k times the input
+  double kscale;              // k of mode 1
+  int nlines, tpf, ntiles;    // lines per field, tiles per field, tiles
+  int ld;                     // line l: base (l / ld) * ihs + l % ld (inputs), * ohs (outputs)
+  long long ihs, ohs, estr, ostr;   // element strides along the transform, in and out
+  int n1, P;                  // modes of the full spectrum (Ny; unused for x), transform length
+  TxyPlan t;
+  char* keep;
+  long long keep_bytes;
+  int* err;
+};
+
+// row of complex line l (YB, YF): lines in blocks of eight, real parts then imaginary parts
+__device__ __forceinline__ int tile_row(int l, int part) { return (l >> 3) * 16 + part * 8 + (l & 7); }
+
+__device__ __forceinline__ unsigned dkey(double v) {
+  return FBits<double>::key(FBits<double>::bits(v));
+}
+template <bool TINY> __device__ __forceinline__ long long fix(double v, int maxe) {
+  return Fixed<double, TINY>::of(FBits<double>::bits(v), maxe);
+}
+
+// outputs of one thread in one pass: columns m0 .. m0 + CW - 1 of its row
+template <int MODE, int NMAG>
+__device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW, int m0, int grp,
+                                              int c, bool rowok, bool nan, bool safe, int ex,
+                                              long long mid, int part_c, long long* part,
+                                              long long* hold, double* dst, uint32_t barAccFree,
+                                              int lane) {
+  const int nout = A.t.nout;
+  for (int c0 = 0; c0 < CW; c0 += 4) {
+    uint32_t v[8][4];
+    tmem_ldx4<8>(tb + (uint32_t)c0, A.t.NT, v);
+    if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barAccFree) : "memory");
+    }
+    long long T[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG, 8>(v, e);
+    if (A.t.kc > 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (c > 0) T[e] += part[(c0 + e) * kEW * 32];
+        if (c + 1 < A.t.kc) part[(c0 + e) * kEW * 32] = T[e];
+      }
+      if (c + 1 < A.t.kc) continue;
+    }
+    if (grp == 0) {
+      if (MODE == YF || MODE == XF) {   // (-1)^n times the middle sample (m0 + c0 is even)
+        T[0] += mid;
+        T[1] -= mid;
+        T[2] += mid;
+        T[3] -= mid;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) hold[(c0 + e) * kEW * 32] = T[e];
+      continue;
+    }
+    double ra[4], rb[4];
+    long long a[4], b[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const long long h = hold[(c0 + e) * kEW * 32];
+      if (MODE == YB || MODE == YF) {
+        // the other part's sine product: re rows take -S_im (YB) or +S_im (YF), im rows the other
+        long long o = __shfl_xor_sync(0xffffffffu, T[e], 8);
+        if ((part_c == 0) == (MODE == YB)) o = -o;
+        a[e] = h + o;
+        b[e] = h - o;
+      } else if (MODE == XB) {
+        a[e] = h + T[e];
+        b[e] = h - T[e];
+      } else {
+        a[e] = h;
+        b[e] = T[e];
+      }
+    }
+    if (safe) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        ra[e] = scaled<double>(a[e], ex);
+        rb[e] = scaled<double>(b[e], ex);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        ra[e] = nan ? qnan<double>() : scaled_any<double>(a[e], ex);
+        rb[e] = nan ? qnan<double>() : scaled_any<double>(b[e], ex);
+      }
+    }
+    if (!rowok) continue;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int n = m0 + c0 + e;
+      if (n >= nout) continue;
+      if (MODE == XF) {
+        *reinterpret_cast<double2*>(dst + 2 * (size_t)n * A.ostr) = make_double2(ra[e], rb[e]);
+      } else if (MODE == XB) {
+        dst[(size_t)n * A.ostr] = ra[e];
+        if (n > 0) dst[(size_t)(A.P - n) * A.ostr] = rb[e];
+      } else if (MODE == YB) {
+        dst[2 * (size_t)n * A.ostr] = ra[e];
+        if (n > 0) dst[2 * (size_t)(A.P - n) * A.ostr] = rb[e];
+      } else {
+        // the y Nyquist row (n1 / 2) is zero
+        dst[2 * (size_t)n * A.ostr] = ra[e];
+        dst[2 * (size_t)(n > 0 ? A.n1 - n : A.n1 / 2) * A.ostr] = n > 0 ? rb[e] : 0.0;
+      }
+    }
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant__ Args A) {
+  constexpr bool CPX = MODE == YB || MODE == YF;   // rows: re and im of 64 lines; else 128 lines
+  constexpr int LPT = CPX ? kRows / 2 : kRows;     // lines per tile
+  constexpr int ISC = MODE == XF ? 1 : 2;          // doubles per input element
+  constexpr int OSC = MODE == XB ? 1 : 2;
+  extern __shared__ __align__(1024) unsigned char tsm[];
+  const int NT = A.t.NT, ns = A.t.stages, nst = A.t.nst;
+  const int sbytes = stage_bytes(NT);
+  unsigned char* stages = tsm;
+  long long* hold0 = reinterpret_cast<long long*>(tsm + (size_t)ns * sbytes);
+  long long* sC = hold0 + (NT / 2) * kEW * 32;
+  int* sE = reinterpret_cast<int*>(sC + kRB * kRows);
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + kRB * kRows);
+  uint32_t* sT = reinterpret_cast<uint32_t*>(bars + kBars);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t barFull = su32(bars), barB = barFull + 8 * kMaxStages;
+  const uint32_t barEmpty = barFull + 16 * kMaxStages, barAccFull = barFull + 24 * kMaxStages;
+  const uint32_t barAccFree = barAccFull + 8, barRow = barAccFull + 16;
+  const uint32_t barRowFree = barRow + 8 * kRB, barFin = barRowFree + 8 * kRB;
+  if (tid == 0) {
+    for (int b = 0; b < kMaxStages; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barFull + 8 * b), "r"(kPW));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barB + 8 * b));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barEmpty + 8 * b));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barAccFull));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barAccFree), "r"(kEW));
+    for (int b = 0; b < kRB; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRow + 8 * b), "r"(kSW));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barRowFree + 8 * b),
+                   "r"(kEW + kPW));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barFin));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  const bool issuer_warp = warp == kPW + kEW;
+  if (issuer_warp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     su32(sT)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();   // barriers and tensor-memory address visible to every warp
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *sT;
+  const uint32_t sBase = su32(stages);
+  char* kcta = A.keep + (long long)blockIdx.x * A.keep_bytes;
+  Waiter W;
+
+  if (issuer_warp) {
+    if (lane == 0) {
+      uint32_t slot = 0, use = 0, pass = 0;
+      bool any = false;
+      for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x)
+        for (int pp = 0; pp < 2 * A.t.nsl; ++pp)
+          for (int c = 0; c < A.t.kc; ++c, ++pass) {
+            if (pass > 0 && !W.wait(barAccFree, (pass - 1) & 1)) goto drain;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int s0 = c * A.t.gst, s1 = min(nst, s0 + A.t.gst);
+            for (int st = s0; st < s1; ++st) {
+              if (!W.wait(barFull + 8 * slot, use & 1) || !W.wait(barB + 8 * slot, use & 1))
+                goto drain;
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              const uint32_t sA = sBase + slot * (uint32_t)sbytes;
+              issue_stage<8>(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
+              any = true;
+              mma_commit(barEmpty + 8 * slot);
+              if ((int)++slot == ns) {
+                slot = 0;
+                ++use;
+              }
+            }
+            mma_commit(barAccFull);
+          }
+    drain:
+      if (!W.ok && any) {
+        // a wait ran out: nothing more is issued; wait (bounded) for the MMAs in flight before
+        // the tensor memory is released
+        mma_commit(barFin);
+        mbar_wait_until(barFin, 0, gtime() + kWaitNs);
+      }
+    }
+    __syncwarp();
+  } else if (warp > kPW + kEW) {
+    // ---- scan: lanes along the lines, 32 lines per group, one scale per line (a complex line's
+    // parts share it); the next tile's elements are prefetched into L2 on the way
+    const int sw = warp - (kPW + kEW + 1);
+    const int nel = MODE == YB ? A.n1 : MODE == XB ? A.t.nk : A.P;
+    int ti = 0;
+    for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
+      const int b = ti % kRB;
+      if (ti >= kRB && !W.wait_warp(barRowFree + 8 * b, (ti / kRB - 1) & 1)) break;
+      const int fld = tile / A.tpf;
+      const int tn = tile + gridDim.x, fn = tn / A.tpf;
+      const bool d = (A.dmask >> fld) & 1;
+      for (int gi = sw; gi < LPT / 32; gi += kSW) {
+        const int l = gi * 32 + lane;
+        const int line = (tile - fld * A.tpf) * LPT + l, linen = (tn - fn * A.tpf) * LPT + l;
+        const bool ok = line < A.nlines, okn = tn < A.ntiles && linen < A.nlines;
+        const double* src =
+            A.in + ((long long)A.src[fld] * A.fsi + (ok ? (line / A.ld) * A.ihs + line % A.ld : 0)) * ISC;
+        const double* nxt =
+            okn ? A.in + ((long long)A.src[fn] * A.fsi + (linen / A.ld) * A.ihs + linen % A.ld) * ISC
+                : src;
+        unsigned key = 0;
+        if (ok) {
+#pragma unroll 8
+          for (int j = 0; j < nel; ++j) {
+            if (okn)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt + (size_t)j * A.estr * ISC));
+            if (MODE == XF) {
+              key = max(key, dkey(src[(size_t)j * A.estr]));
+            } else if (!(MODE == YB && j == A.n1 / 2)) {
+              double2 x = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
+              if (d) {
+                const double k = A.kscale * (double)((MODE == YB && j > A.n1 / 2) ? j - A.n1 : j);
+                x = make_double2(k * x.x, k * x.y);
+              }
+              key = max(key, max(dkey(x.x), dkey(x.y)));
+            }
+          }
+        }
+        const int sc = row_scale<double>(key);
+        if (CPX) {
+          long long xr = 0, xi = 0;
+          if (MODE == YF && ok && !(A.P & 1)) {
+            const double2 x = *reinterpret_cast<const double2*>(src + 2 * (size_t)(A.P / 2) * A.estr);
+            xr = fix<true>(x.x, sc);
+            xi = fix<true>(x.y, sc);
+          }
+          const int ro = b * kRows + tile_row(l, 0);
+          sE[ro] = sc;
+          sE[ro + 8] = sc;
+          sC[ro] = __mul64hi(xr * 256, A.t.ymid * 4);   // x Y / 2^54
+          sC[ro + 8] = __mul64hi(xi * 256, A.t.ymid * 4);
+        } else {
+          long long x = 0;
+          if (MODE == XF && ok && !(A.P & 1)) x = fix<true>(src[(size_t)(A.P / 2) * A.estr], sc);
+          sE[b * kRows + l] = sc;
+          sC[b * kRows + l] = __mul64hi(x * 256, A.t.ymid * 4);
+        }
+      }
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRow + 8 * b) : "memory");
+    }
+  } else if (warp >= kEW) {
+    // ---- producers.  YB, YF: thread = (line l, g), K positions 4 g + e of a stage holding
+    // k = 16 st + g + 4 e, both parts.  XB, XF: thread = (line l, hf), positions 8 hf + e holding
+    // k = 16 st + hf + 2 e.
+    const int p = tid - 32 * kEW, pw = warp - kEW;
+    const int l = CPX ? pw * 8 + ((lane >> 1) & 7) : pw * 16 + (lane & 15);
+    const int g = CPX ? (lane >> 4) * 2 + (lane & 1) : lane >> 4;
+    constexpr int KS = CPX ? 4 : 2, NE = CPX ? 4 : 8;   // k step and values per stage
+    const int row = CPX ? tile_row(l, 0) : l;
+    const uint32_t oa = CPX ? (uint32_t)((g >> 1) * (int)kALbo + row * 16 + (g & 1) * 8)
+                            : (uint32_t)(g * (int)kALbo + row * 16);
+    const uint32_t bbytes = (uint32_t)b_stage_bytes(NT);
+    const size_t bstride = (size_t)bbytes / 2;   // elements of a stage block
+    const uint64_t pol = policy_evict_last();
+    longlong2* kp = reinterpret_cast<longlong2*>(kcta) + p;
+    uint32_t slot = 0, use = 0;
+    int ti = 0;
+    // the stage's digit planes of v (biased) and, by one thread, the copy of its matrix digits;
+    // false after a wait ran out
+    auto put = [&](const unsigned long long (&v)[8], const uint16_t* bsrc) {
+      if (use > 0 && !W.wait_warp(barEmpty + 8 * slot, (use & 1) ^ 1)) return false;
+      unsigned char* sA = stages + (size_t)slot * sbytes;
+      if (p == 0) bulk_load(su32(sA) + (uint32_t)kABytes, bsrc, bbytes, barB + 8 * slot, pol);
+#pragma unroll
+      for (int i = 0; i < kPlanes; ++i) {
+        const int b = 6 - i, sh = b < 4 ? 0 : 32;
+        uint32_t w[8], r[4];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = (uint32_t)(v[e] >> sh);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) r[e] = digit_pair(w[2 * e], w[2 * e + 1], b & 3);
+        if (CPX) {
+          *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + oa) = make_uint2(r[0], r[1]);
+          *reinterpret_cast<uint2*>(sA + i * kPlaneBytes + oa + 128) = make_uint2(r[2], r[3]);
+        } else {
+          *reinterpret_cast<uint4*>(sA + i * kPlaneBytes + oa) = make_uint4(r[0], r[1], r[2], r[3]);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barFull + 8 * slot)
+                     : "memory");
+      if ((int)++slot == ns) {
+        slot = 0;
+        ++use;
+      }
+      return true;
+    };
+    auto keep_at = [&](int grp, int st) { return kp + (size_t)(grp * nst + st) * (4 * kPW * 32); };
+    auto store_keep = [&](longlong2* d, const unsigned long long (&v)[8]) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        __stcg(d + i * kPW * 32, make_longlong2((long long)v[2 * i], (long long)v[2 * i + 1]));
+    };
+    for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
+      const int fld = tile / A.tpf;
+      const int line = (tile - fld * A.tpf) * LPT + l;
+      const bool rowok = line < A.nlines, d = (A.dmask >> fld) & 1;
+      const int lh = line / A.ld, ll = line - lh * A.ld;
+      const double* src =
+          A.in + ((long long)A.src[fld] * A.fsi + (rowok ? lh * A.ihs + ll : 0)) * ISC;
+      // complex inputs: x (k) and, folded, y (L - k); real ones: two samples per element
+      double2 x[8];
+      auto load = [&](int st) {
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+          const int k = 16 * st + g + KS * e;
+          const bool ok = rowok && k < A.t.nk, okm = ok && k > 0;
+          if (CPX) {
+            const int L = MODE == YB ? A.n1 : A.P;
+            x[e] = make_double2(0.0, 0.0);
+            x[4 + e] = make_double2(0.0, 0.0);
+            if (ok) x[e] = *reinterpret_cast<const double2*>(src + 2 * (size_t)k * A.estr);
+            if (okm) x[4 + e] = *reinterpret_cast<const double2*>(src + 2 * (size_t)(L - k) * A.estr);
+          } else if (MODE == XB) {
+            x[e] = make_double2(0.0, 0.0);
+            if (ok) x[e] = *reinterpret_cast<const double2*>(src + 2 * (size_t)k * A.estr);
+          } else {
+            x[e] = make_double2(0.0, 0.0);
+            if (ok) x[e].x = src[(size_t)k * A.estr];
+            if (okm) x[e].y = src[(size_t)(A.P - k) * A.estr];
+          }
+        }
+      };
+      load(0);
+      const int rbuf = ti % kRB;
+      if (!W.wait_warp(barRow + 8 * rbuf, (ti / kRB) & 1)) break;
+      const int sc = sE[rbuf * kRows + row];
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
+                     : "memory");
+      const bool tiny = __any_sync(0xffffffffu, sc < kTinyScale) != 0;
+      unsigned long long sumr = 0, sumi = 0, s0 = 0;
+      bool ok = true;
+      for (int st = 0; st < nst && ok; ++st) {
+        if ((MODE == YB || MODE == XB) && d) {   // i k times the mode
+#pragma unroll
+          for (int e = 0; e < NE; ++e) {
+            const double k = A.kscale * (double)(16 * st + g + KS * e);
+            x[e] = make_double2(-k * x[e].y, k * x[e].x);
+            if (CPX) x[4 + e] = make_double2(k * x[4 + e].y, -k * x[4 + e].x);
+          }
+        }
+        unsigned long long s[8], dd[8];
+        auto convert = [&](auto tag) {
+          constexpr bool TINY = decltype(tag)::value;
+#pragma unroll
+          for (int e = 0; e < NE; ++e) {
+            if (CPX) {
+              const long long a = fix<TINY>(x[e].x, sc), b = fix<TINY>(x[4 + e].x, sc);
+              const long long u = fix<TINY>(x[e].y, sc), v = fix<TINY>(x[4 + e].y, sc);
+              s[e] = a + b + kBias;
+              dd[e] = a - b + kBias;
+              s[4 + e] = u + v + kBias;
+              dd[4 + e] = u - v + kBias;
+            } else {
+              const long long a = fix<TINY>(x[e].x, sc), b = fix<TINY>(x[e].y, sc);
+              s[e] = MODE == XB ? a + kBias : a + b + kBias;
+              dd[e] = MODE == XB ? b + kBias : a - b + kBias;
+            }
+          }
+        };
+        if (tiny) convert(std::true_type());
+        else convert(std::false_type());
+        if (st + 1 < nst) load(st + 1);
+        store_keep(keep_at(1, st), dd);
+        if (A.t.nsl > 1) store_keep(keep_at(0, st), s);
+        if (MODE == YB || MODE == XB) {
+#pragma unroll
+          for (int e = 0; e < NE; ++e) {
+            sumr += s[e];
+            if (CPX) sumi += s[4 + e];
+          }
+          if (st == 0) s0 = s[0];
+        }
+        ok = put(s, A.t.dig + (size_t)st * bstride);
+      }
+      if (!ok) break;
+      if ((MODE == YB || MODE == XB) && !(A.P & 1)) {
+        // output n = P / 2: sum_k (-1)^k s_k (YB), 2 sum_k (-1)^k Re c_k - Re c_0 (XB);
+        // (-1)^k = (-1)^g.  High and low parts (27 bits) are added apart.
+        const unsigned long long nb = (unsigned long long)(NE * nst) * kBias;
+        const int f = MODE == XB ? 2 : 1;
+        long long tr = (long long)(sumr - nb), tm = (long long)(sumi - nb);
+        if (g & 1) {
+          tr = -tr;
+          tm = -tm;
+        }
+        long long hr = f * (tr >> 27), lr = f * (tr & 0x7FFFFFF);
+        long long hm = tm >> 27, lm = tm & 0x7FFFFFF;
+        if (MODE == XB && g == 0) {
+          const long long z = (long long)(s0 - kBias);
+          hr -= z >> 27;
+          lr -= z & 0x7FFFFFF;
+        }
+#pragma unroll
+        for (int off = CPX ? 1 : 16; off <= 16; off <<= 4) {   // the threads of the line
+          hr += __shfl_xor_sync(0xffffffffu, hr, off);
+          lr += __shfl_xor_sync(0xffffffffu, lr, off);
+          if (CPX) {
+            hm += __shfl_xor_sync(0xffffffffu, hm, off);
+            lm += __shfl_xor_sync(0xffffffffu, lm, off);
+          }
+        }
+        if (g == 0 && rowok) {
+          const int e2 = sc - FBits<double>::EOFF - 51;   // sum 2^(E - 54), T = sum / 8
+          const double vr = sc == kNanRow ? qnan<double>()
+                                          : scaled_any<double>(hr * 16777216ll + ((lr + 4) >> 3), e2);
+          double* o = A.out + ((long long)fld * A.fso + lh * A.ohs + ll + (long long)(A.P / 2) * A.ostr) * OSC;
+          if (CPX) {
+            const double vi = sc == kNanRow ? qnan<double>()
+                                            : scaled_any<double>(hm * 16777216ll + ((lm + 4) >> 3), e2);
+            *reinterpret_cast<double2*>(o) = make_double2(vr, vi);
+          } else {
+            *o = vr;
+          }
+        }
+      }
+      for (int pp = 1; pp < 2 * A.t.nsl && ok; ++pp) {
+        longlong2 nx[4];
+        auto fetch = [&](int st) {
+          const longlong2* s = keep_at(pp & 1, st);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) nx[i] = __ldcg(s + i * kPW * 32);
+        };
+        fetch(0);
+        for (int st = 0; st < nst && ok; ++st) {
+          unsigned long long v[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            v[2 * i] = (unsigned long long)nx[i].x;
+            v[2 * i + 1] = (unsigned long long)nx[i].y;
+          }
+          if (st + 1 < nst) fetch(st + 1);
+          ok = put(v, A.t.dig + ((size_t)pp * nst + st) * bstride);
+        }
+      }
+      if (!ok) break;
+    }
+    // after a failed wait the copies still in flight finish (bounded) before the CTA ends
+    if (!W.ok && p == 0) {
+      const uint64_t dl = gtime() + kWaitNs;
+      for (int b = 0; b < ns; ++b) {
+        const uint32_t n = use + (b < (int)slot ? 1u : 0u);   // copies issued to slot b
+        if (n > 0) mbar_wait_until(barB + 8 * b, (n - 1) & 1, dl);
+      }
+    }
+  } else {
+    // ---- epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
+    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators
+    const int qd = warp & 3, cg = warp >> 2, CW = NT / 2;
+    const int row = qd * 32 + lane;
+    const int l = CPX ? (row >> 4) * 8 + (row & 7) : row, part_c = CPX ? (row >> 3) & 1 : 0;
+    const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cg * CW);
+    long long* part = reinterpret_cast<long long*>(kcta + (size_t)2 * nst * kKeepStage) + tid;
+    uint32_t pass = 0;
+    int ti = 0;
+    for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
+      const int fld = tile / A.tpf, rbuf = ti % kRB;
+      const int line = (tile - fld * A.tpf) * LPT + l;
+      if (!W.wait_warp(barRow + 8 * rbuf, (ti / kRB) & 1)) break;
+      const int me = sE[rbuf * kRows + row];
+      const long long mid = sC[rbuf * kRows + row];
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
+                     : "memory");
+      const bool rowok = line < A.nlines, nan = me == kNanRow;
+      const int ex = me - FBits<double>::EOFF - A.t.q;   // result = T 2^(E - q)
+      const bool safe =
+          __all_sync(0xffffffffu, !rowok || (!nan && safe_exp<double>(ex))) != 0;
+      const int lh = line / A.ld, ll = line - lh * A.ld;
+      double* dst =
+          A.out + ((long long)fld * A.fso + (rowok ? lh * A.ohs + ll : 0)) * OSC + part_c;
+      bool ok = true;
+      for (int pp = 0; pp < 2 * A.t.nsl && ok; ++pp) {
+        const int m0 = (pp >> 1) * NT + cg * CW;
+        for (int c = 0; c < A.t.kc; ++c, ++pass) {
+          if (!(ok = W.wait_warp(barAccFull, pass & 1))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (A.t.nmag == 8)
+            epilogue_pass<MODE, 8>(A, tb, CW, m0, pp & 1, c, rowok, nan, safe, ex, mid, part_c, part,
+                                   hold0 + tid, dst, barAccFree, lane);
+          else
+            epilogue_pass<MODE, 0>(A, tb, CW, m0, pp & 1, c, rowok, nan, safe, ex, mid, part_c, part,
+                                   hold0 + tid, dst, barAccFree, lane);
+        }
+      }
+      if (!ok) break;
+    }
+  }
+  if (!W.ok) atomicOr(A.err, 1);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (issuer_warp)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// The nine products (in place: seven physical fields u v w phi phi_x phi_y phi_z in, Sxx - Szz,
+// Syy - Szz, Sxy, Sxz, Syz, phi^3, u phi, v phi, w phi out) of n samples per field.  About 20
+// float64 operations per sample: bound by the float64 pipe and by HBM about equally.
+__global__ void __launch_bounds__(256) products_kernel(double* __restrict__ f, long long n,
+                                                       double kappa) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const double u = f[i], v = f[n + i], w = f[2 * n + i], ph = f[3 * n + i];
+    const double fx = f[4 * n + i], fy = f[5 * n + i], fz = f[6 * n + i];
+    const double kx = kappa * fx, ky = kappa * fy, kz = kappa * fz;
+    const double wz = fma(w, w, kz * fz);
+    f[i] = fma(-u, u, fma(-kx, fx, wz));
+    f[n + i] = fma(-v, v, fma(-ky, fy, wz));
+    f[2 * n + i] = -fma(u, v, kx * fy);
+    f[3 * n + i] = -fma(u, w, kx * fz);
+    f[4 * n + i] = -fma(v, w, ky * fz);
+    f[5 * n + i] = ph * ph * ph;
+    f[6 * n + i] = u * ph;
+    f[7 * n + i] = v * ph;
+    f[8 * n + i] = w * ph;
+  }
+}
+
+// The assembly's z-independent combinations (launch_ycomb), in place on the nine products' modes:
+//   P = kx ky (Sxx' - Syy') + (ky^2 - kx^2) Sxy, Q = i (kx Syz - ky Sxz), C = i (kx Sxz + ky Syz),
+//   R = -(kx^2 Sxx' + 2 kx ky Sxy + ky^2 Syy'), F = -i (kx u phi + ky v phi), w phi, phi^3
+// (on the kx = ky = 0 line P and Q hold Sxz and Syz).  One thread per mode and z.
+__global__ void __launch_bounds__(256) combine_kernel(double2* __restrict__ f, long long fs, int Ny,
+                                                      int Nz, double kxs, double kys) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= fs) return;
+  const long long line = i / Nz;
+  const int mx = (int)(line / Ny), j = (int)(line - (long long)mx * Ny);
+  const double kx = kxs * mx, ky = kys * (j < Ny / 2 ? j : j - Ny);
+  const double2 xx = f[i], yy = f[fs + i], xy = f[2 * fs + i], xz = f[3 * fs + i];
+  const double2 yz = f[4 * fs + i], p3 = f[5 * fs + i], uf = f[6 * fs + i], vf = f[7 * fs + i];
+  const double2 wf = f[8 * fs + i];
+  const double a = kx * ky, b = fma(ky, ky, -kx * kx), c = kx * kx, d = ky * ky, a2 = 2.0 * a;
+  if (line == 0) {
+    f[i] = xz;
+    f[fs + i] = yz;
+  } else {
+    f[i] = make_double2(fma(b, xy.x, a * (xx.x - yy.x)), fma(b, xy.y, a * (xx.y - yy.y)));
+    f[fs + i] = mul_i(make_double2(fma(kx, yz.x, -ky * xz.x), fma(kx, yz.y, -ky * xz.y)));
+  }
+  f[2 * fs + i] = mul_i(make_double2(fma(kx, xz.x, ky * yz.x), fma(kx, xz.y, ky * yz.y)));
+  f[3 * fs + i] = make_double2(-fma(c, xx.x, fma(a2, xy.x, d * yy.x)),
+                               -fma(c, xx.y, fma(a2, xy.y, d * yy.y)));
+  f[4 * fs + i] = mul_mi(make_double2(fma(kx, uf.x, ky * vf.x), fma(kx, uf.y, ky * vf.y)));
+  f[5 * fs + i] = wf;
+  f[6 * fs + i] = p3;
+}
+
+uint16_t bf16_bits(float f) {
+  uint32_t u;
+  memcpy(&u, &f, sizeof u);
+  return (uint16_t)(u >> 16);   // exact: a digit has at most eight significant bits
+}
+
+size_t plan_smem(int NT, int ns) {
+  return (size_t)ns * stage_bytes(NT) + (size_t)(NT / 2) * kEW * 32 * sizeof(long long) + kTail;
+}
+
+template <int MODE> cudaError_t launch_mode(Args& a, int nf, const Txy& x, cudaStream_t s) {
+  constexpr int LPT = MODE == YB || MODE == YF ? kRows / 2 : kRows;
+  static SmemLimit cur;
+  cudaError_t e = ensure_smem(txy_kernel<MODE>, a.t.smem, &cur);
+  if (e != cudaSuccess) return e;
+  a.tpf = (a.nlines + LPT - 1) / LPT;
+  a.ntiles = a.tpf * nf;
+  a.keep = x.keep;
+  a.keep_bytes = (long long)x.keep_bytes;
+  a.err = x.err;
+  if (a.ntiles <= 0) return cudaSuccess;
+  txy_kernel<MODE><<<std::min(a.ntiles, x.ctas), kThreads, a.t.smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t txy_keep_bytes(const TxyPlan& t) {
+  return 2 * (size_t)t.nst * kKeepStage + (size_t)(kNTMax / 2) * kEW * 32 * sizeof(long long);
+}
+
+int txy_plan(int mode, int n1, int P, double scale, std::vector<uint16_t>& dig, TxyPlan* t) {
+  const int half = (P + 1) / 2;   // samples n and P - n share a column: n < half (and P / 2)
+  t->nk = mode == YB ? n1 / 2 : mode == XB ? n1 : half;
+  t->nout = mode == YF ? n1 / 2 : mode == XF ? n1 : half;
+  t->nsl = (t->nout + kNTMax - 1) / kNTMax;
+  t->NT = ((t->nout + t->nsl - 1) / t->nsl + 15) / 16 * 16;
+  t->nst = (t->nk + kKS - 1) / kKS;
+  t->kc = (t->nst * kKS + kMaxK - 1) / kMaxK;
+  t->gst = (t->nst + t->kc - 1) / t->kc;
+  t->stages = kMaxStages;
+  while (t->stages > 2 && plan_smem(t->NT, t->stages) > 226 * 1024) --t->stages;
+  t->smem = plan_smem(t->NT, t->stages);
+  // matrix scale 2^q: the largest weight at most 2^54, and the recombined sums (2^-54 of the sum of
+  // at most nterm products) below 2^62
+  const double wmax = mode == XB ? 2.0 : mode == YF ? fabs(scale) : 1.0;
+  const double nterm = mode == YB ? 2.0 * n1 : mode == XB ? 2.0 * n1 : mode == YF ? 2.0 * P : P;
+  t->q = (int)floor(std::min(54.0 - log2(wmax), 62.0 - log2(nterm * wmax)));
+  t->ymid = mode == YF ? (long long)llround(ldexp(scale, t->q)) : mode == XF ? 1ll << t->q : 0;
+  const long double pi2 = 6.283185307179586476925286766559005768L;
+  // the weights times 2^q by angle 2 pi a / P, of cosine and sine, and at k = 0 (cosine 1, sine 0)
+  std::vector<long long> Y[2] = {std::vector<long long>(P), std::vector<long long>(P)};
+  const long double w = mode == YF ? (long double)scale : mode == XB ? 2.0L : 1.0L;
+  const long double ws = mode == XB || mode == XF ? -w : w;
+  for (int a = 0; a < P; ++a) {
+    const long double c = cosl(pi2 * (long double)a / (long double)P);
+    const long double sn = sinl(pi2 * (long double)a / (long double)P);
+    Y[0][a] = (long long)llroundl(ldexpl(w * c, t->q));
+    Y[1][a] = (long long)llroundl(ldexpl(ws * sn, t->q));
+  }
+  const long long Y0 = mode == XB ? 1ll << t->q : Y[0][0];
+  const int NT = t->NT;
+  const size_t block = (size_t)kPlanes * NT * kKS;
+  dig.assign((size_t)2 * t->nsl * t->nst * block, 0);
+  double bound = 0.0;
+  for (int n = 0; n < t->nout; ++n)
+    for (int grp = 0; grp < 2; ++grp) {
+      double acc = 0.0;
+      for (int k = 0; k < t->nk; ++k) {
+        const long long yk = k == 0 ? (grp == 0 ? Y0 : 0) : Y[grp][((long long)n * k) % P];
+        const unsigned long long y = (unsigned long long)yk + kBias;
+        const int st = k / kKS, kk = k % kKS;
+        // stage position of k: 4 g + e holds g + 4 e (complex lines), 8 hf + e holds hf + 2 e
+        const int pos = mode == YB || mode == YF ? 4 * (kk & 3) + (kk >> 2) : 8 * (kk & 1) + (kk >> 1);
+        uint16_t* b = dig.data() + ((size_t)(2 * (n / NT) + grp) * t->nst + st) * block;
+        for (int j = 0; j < kPlanes; ++j) {
+          const int row = j * NT + n % NT, dgt = (int)((y >> (8 * (6 - j))) & 255ull) - 128;
+          b[((size_t)(pos >> 3) * kPlanes * NT + row) * 8 + (pos & 7)] = bf16_bits((float)dgt);
+          acc += 128.0 * abs(dgt);   // |G_d| <= 128 sum_j sum_k |b_jk|
+        }
+      }
+      bound = std::max(bound, acc);
+    }
+  t->nmag = bound <= 4194304.0 ? 8 : 0;
+  return 0;
+}
+
+// y pass of nf fields: dir 1 modes (Mx, Ny, Nz) -> samples (Mx, P, Nz), dir 0 the inverse
+// (truncated, times the plan's scale); arguments as in launch_ypass
+cudaError_t launch_txy_y(int dir, const GridDev& g, int P, const void* in, void* out, int nf,
+                         long long fs_in, long long fs_out, const YMap& map, const Txy& x,
+                         const TxyPlan& plan, cudaStream_t s) {
+  Args a;
+  memset(&a, 0, sizeof a);
+  a.in = (const double*)in;
+  a.out = (double*)out;
+  a.fsi = fs_in;
+  a.fso = fs_out;
+  for (int f = 0; f < nf; ++f) a.src[f] = map.src[f];
+  a.dmask = dir == 1 ? map.dy_mask : 0;
+  a.kscale = map.kys;
+  a.nlines = g.Mx * g.nz;
+  a.ld = g.nz;
+  a.ihs = (long long)(dir == 1 ? g.ny : P) * g.nz;
+  a.ohs = (long long)(dir == 1 ? P : g.ny) * g.nz;
+  a.estr = a.ostr = g.nz;
+  a.n1 = g.ny;
+  a.P = P;
+  a.t = plan;
+  return dir == 1 ? launch_mode<YB>(a, nf, x, s) : launch_mode<YF>(a, nf, x, s);
+}
+
+cudaError_t launch_txy_ycomb(const GridDev& g, const void* in, void* out9, long long fs_in,
+                             long long fs_out, const Txy& x, cudaStream_t s) {
+  YMap map;
+  for (int f = 0; f < YMap::kMax; ++f) map.src[f] = f;
+  map.dy_mask = 0;
+  map.kys = 0.0;
+  cudaError_t e = launch_txy_y(0, g, g.Py, in, out9, 9, fs_in, fs_out, map, x, x.yf, s);
+  if (e != cudaSuccess) return e;
+  combine_kernel<<<(unsigned)((fs_out + 255) / 256), 256, 0, s>>>(
+      (double2*)out9, fs_out, g.ny, g.nz, 6.283185307179586476925 / g.lx,
+      6.283185307179586476925 / g.ly);
+  return cudaGetLastError();
+}
+
+// x line: six fields (Mx, Py, Nz) -> seven physical fields -> nine products -> nine fields
+cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long long fs, const Txy& x,
+                         cudaStream_t s) {
+  const int Q = g.Py * g.nz;
+  const long long np = (long long)g.Px * Q;
+  Args a;
+  memset(&a, 0, sizeof a);
+  a.in = (const double*)in6;
+  a.out = x.phys;
+  a.fsi = fs;
+  a.fso = np;
+  const int src[7] = {0, 1, 2, 3, 3, 4, 5};   // u v w phi (phi -> i kx phi) phi_y phi_z
+  for (int f = 0; f < 7; ++f) a.src[f] = src[f];
+  a.dmask = 1u << 4;
+  a.kscale = 6.283185307179586476925 / g.lx;
+  a.nlines = Q;
+  a.ld = Q;
+  a.estr = a.ostr = Q;
+  a.P = g.Px;
+  a.t = x.xb;
+  cudaError_t e = launch_mode<XB>(a, 7, x, s);
+  if (e != cudaSuccess) return e;
+  products_kernel<<<(unsigned)std::min<long long>((np + 255) / 256, (long long)x.ctas * 32), 256, 0, s>>>(
+      x.phys, np, g.kappa);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  a.in = x.phys;
+  a.out = (double*)out9;
+  a.fsi = np;
+  a.fso = fs;
+  for (int f = 0; f < 9; ++f) a.src[f] = f;
+  a.dmask = 0;
+  a.t = x.xf;
+  return launch_mode<XF>(a, 9, x, s);
+}
+
+}  // namespace chf
