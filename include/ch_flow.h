@@ -116,7 +116,11 @@ int ch_set_fields_host(ch_grid* g, const double* u, const double* v, const doubl
                        const double* phi);
 
 /* Advance nsteps full time steps (Sec. 2.2 steps i)-v)), asynchronously on the stream.  After
- * the first step the per-step launch sequence is replayed from a captured CUDA graph. */
+ * the first step the per-step launch sequence is replayed from a captured CUDA graph.
+ * Float64 grids of at least 2^15 modes (nx/2 ny nz) and padded lengths up to
+ * 1024 do their x and y transforms as exact-split products on the tensor cores (float64-accurate;
+ * nine real padded fields of extra memory; the FFT kernels if that memory is not to be had); the
+ * radix schedules of ch_set_fft_pruning do not apply to them. */
 int ch_step(ch_grid* g, int nsteps);
 
 /* The kernels of one time step in the order ch_step_timed reports them in: zrhs (DCT,
@@ -193,7 +197,8 @@ int ch_fp64_fma_rate(double* tflops);
  * the last.  kernel_ms may be NULL.  Used by the benchmark to attribute step time. */
 int ch_step_timed(ch_grid* g, int nsteps, double* kernel_ms, double* total_ms);
 
-/* Number of kernel launches one ch_step makes per time step. */
+/* Number of kernel launches one ch_step makes per time step (six; two more with CH_CHEB_TC, three
+ * more with the x/y transforms on the tensor cores). */
 int ch_launches_per_step(const ch_grid* g);
 
 /* Spectral state -> physical u, v, w, phi (device, (nz,ny,nx) float64) on the unpadded grid. */

@@ -265,11 +265,8 @@ int ch_adjoint_gradient(ch_grid* G, double* gu, double* gv, double* gw, double* 
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
   CK(chf::launch_adj_project(g, G->a_L, G->fs, G->auxA, G->pz, s));
-  CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, 4, G->fs, G->fs, 1.0, G->pyu, s));
   double* out[4] = {gu, gv, gw, gphi};
-  for (int f = 0; f < 4; ++f)
-    CK(chf::launch_x_c2r(g, G->auxB + f * G->fs, out[f], 1, G->fs, G->fsp, G->pxu, s));
-  return CH_OK;
+  return ch_z_to_rows(G, G->auxA, G->auxB, 4, out);
 }
 
 int ch_adjoint_end(ch_grid* G) {

@@ -188,7 +188,13 @@ thread_local cudaError_t t_last_cuda = cudaSuccess;
 int eval_products(ch_grid* G) {
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  CK(chf::launch_zbwd(0, G->prec, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s));
+  if (G->cheb == CH_CHEB_TC) {   // as the step itself forms the fields
+    CK(chf::launch_fields_coef(g, G->om, G->w, G->phi, G->cf, G->fs, G->pz, s));
+    CK(chf::launch_cheb_tc(0, G->prec, G->cf, G->fs, G->bw, G->fs, kBw, g.Mx * g.ny, g.nz, G->tcb,
+                           G->tc_err, s));
+  } else {
+    CK(chf::launch_zbwd(0, G->prec, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s));
+  }
   CK(ch_launch_xy(G, 3, s));
   CK(ch_launch_xy(G, 4, s));
   return CH_OK;
@@ -271,10 +277,22 @@ int launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev = nullptr
 // cheb_fwd cheb_bwd)
 const int kStepPos[CH_STEP_KERNELS] = {1, 2, 3, 5, 6, 7, 0, 4};
 
+int coef_to_rows(ch_grid* G, const double2* coef, int nf, const chf::YMap& ym, int ny_out,
+                 const int* xsrc, unsigned xmask, int nx_out, double* const* out);
+
 // the 7 backward fields of the state, evaluated on the unpadded grid, into phys7
 int state_to_phys7(ch_grid* G, int nf) {
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
+  if (G->use_ax) {
+    CK(chf::launch_fields_coef(g, G->om, G->w, G->phi, G->auxB, G->fs, G->pz, s));
+    chf::YMap ym = step_ymap();   // u v w phi i ky phi D phi
+    ym.kys = 6.283185307179586476925 / g.ly;
+    const int xsrc[7] = {0, 1, 2, 3, 3, 4, 5};
+    double* out[7];
+    for (int f = 0; f < 7; ++f) out[f] = G->phys7 + f * G->fsp;
+    return coef_to_rows(G, G->auxB, kBw, ym, kYa, xsrc, 1u << 4, 7, out);
+  }
   CK(chf::launch_zbwd(0, 0, 7, g, G->R, G->om, G->w, G->phi, G->auxA, G->fs, G->pz, s));
   CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, nf, G->fs, G->fs, 1.0, G->pyu, s));
   CK(chf::launch_x_c2r(g, G->auxB, G->phys7, nf, G->fs, G->fsp, G->pxu, s));
@@ -299,11 +317,47 @@ void release_last(ch_grid* G, size_t n) {
   }
 }
 
-// one plan with its digits on the device; mode as in txy_plan
-int make_txy_plan(ch_grid* G, int mode, double scale, chf::TxyPlan* p) {
+// Plans, digits and scratch of the tensor-core Chebyshev transforms, made once per handle;
+// CH_ERR_SIZE: length not supported, CH_ERR_ALLOC with nothing kept
+int ensure_cheb(ch_grid* G) {
+  if (G->tcf.dig) return CH_OK;
+  chf::ChebTc t[2];
+  const size_t before = G->allocs.size();
+  int dev = 0, nsm = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  if (nsm < 1) nsm = 1;
+  // one persistent CTA per SM, each with room for one tile's fixed-point rows
+  void* keep = nullptr;
+  int* err = G->tc_err;
+  for (int dir = 0; dir < 2; ++dir) {
+    std::vector<uint16_t> dig;
+    if (chf::cheb_tc_tables(G->g.N, dir, dig, &t[dir]) != 0) return CH_ERR_SIZE;
+    void* d = galloc(G, dig.size() * sizeof(uint16_t));
+    if (dir == 0) keep = galloc(G, (size_t)nsm * chf::cheb_tc_keep_bytes(G->g.N));
+    if (dir == 0 && !err) err = (int*)galloc(G, sizeof(int));
+    if (!d || !keep || !err) {
+      release_last(G, G->allocs.size() - before);
+      return CH_ERR_ALLOC;
+    }
+    CK(cudaMemcpy(d, dig.data(), dig.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+    t[dir].dig = (const uint16_t*)d;
+    t[dir].keep = (char*)keep;
+    t[dir].ctas = nsm;
+  }
+  CK(chf::cheb_tc_prepare());
+  if (!G->tc_err) CK(cudaMemset(err, 0, sizeof(int)));
+  G->tc_err = err;
+  G->tcf = t[0];
+  G->tcb = t[1];
+  return CH_OK;
+}
+
+// one plan with its digits on the device; mode as in txy_plan, P the transform length
+int make_txy_plan(ch_grid* G, int mode, int P, double scale, chf::TxyPlan* p) {
   const GridDev& g = G->g;
   std::vector<uint16_t> dig;
-  chf::txy_plan(mode, mode < 2 ? g.ny : g.Mx, mode < 2 ? g.Py : g.Px, scale, dig, p);
+  chf::txy_plan(mode, mode < 2 ? g.ny : g.Mx, P, scale, dig, p);
   void* d = galloc(G, dig.size() * sizeof(uint16_t));
   if (!d) return CH_ERR_ALLOC;
   CK(cudaMemcpy(d, dig.data(), dig.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
@@ -311,44 +365,84 @@ int make_txy_plan(ch_grid* G, int mode, double scale, chf::TxyPlan* p) {
   return CH_OK;
 }
 
-// Plans and buffers of the tensor-core x/y transforms of a float64 grid.
+// Plans and buffers of the tensor-core x/y transforms: of the unpadded grid for the entry points
+// that read and write physical fields (use_ax, with the Chebyshev transforms), and of the padded one
+// for the steps of a float64 grid (use_tx).
 // Rule: from 2^15 modes on (below, a transform has fewer tiles than a third of the SMs and its
 // latency counts: 32 x 32 x 33, 16896 modes, y backward 25 against 21 us, x line 45 against 53,
 // y forward 30 against 33 by FFT; 48 x 48 x 49, 56448 modes, 39, 96 and 60 against 47, 137 and 75),
-// up to padded lengths of 1024 (the dense matrices grow with the length squared).
+// up to transform lengths of 1024 (the dense matrices grow with the length squared).
 constexpr int kTxyMaxP = 1024;
 constexpr long long kTxyMinModes = 1ll << 15;
 int setup_tx(ch_grid* G) {
   const GridDev& g = G->g;
-  if (g.Px > kTxyMaxP || g.Py > kTxyMaxP || G->fs < kTxyMinModes) return CH_OK;
-  int dev = 0, nsm = 0;
-  CK(cudaGetDevice(&dev));
-  CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  if (g.nx > kTxyMaxP || g.ny > kTxyMaxP || G->fs < kTxyMinModes) return CH_OK;
+  const int c = ensure_cheb(G);
+  if (c == CH_ERR_CUDA) return c;
+  if (c != CH_OK) {   // a length the Chebyshev transform does not take, or no room
+    cudaGetLastError();
+    return CH_OK;
+  }
   chf::Txy t;
-  t.ctas = nsm < 1 ? 1 : nsm;
-  const double sc = 1.0 / ((double)g.Px * (double)g.Py);
-  chf::TxyPlan* plan[4] = {&t.yb, &t.yf, &t.xb, &t.xf};
+  t.ctas = G->tcf.ctas;
+  t.err = G->tc_err;
   const size_t before = G->allocs.size();
+  const bool padded = G->prec == CH_PREC_FP64 && g.Px <= kTxyMaxP && g.Py <= kTxyMaxP;
+  const double su = 1.0 / ((double)g.nx * (double)g.ny), sp = 1.0 / ((double)g.Px * (double)g.Py);
+  chf::TxyPlan* plan[8] = {&t.ybu, &t.yfu, &t.xbu, &t.xfu, &t.yb, &t.yf, &t.xb, &t.xf};
+  const int len[8] = {g.ny, g.ny, g.nx, g.nx, g.Py, g.Py, g.Px, g.Px};
   bool ok = true;
-  for (int i = 0; i < 4 && ok; ++i) {
-    const int r = make_txy_plan(G, i, i == 1 ? sc : 1.0, plan[i]);
+  for (int i = 0; i < (padded ? 8 : 4) && ok; ++i) {
+    const int r = make_txy_plan(G, i & 3, len[i], i == 1 ? su : i == 5 ? sp : 1.0, plan[i]);
     if (r == CH_ERR_CUDA) return r;
     ok = r == CH_OK;
     t.keep_bytes = std::max(t.keep_bytes, chf::txy_keep_bytes(*plan[i]));
   }
   if (ok) ok = (t.keep = (char*)galloc(G, (size_t)t.ctas * t.keep_bytes)) != nullptr;
-  if (ok)
-    ok = (t.phys = (double*)galloc(G, (size_t)kNl * g.Px * g.Py * g.nz * sizeof(double))) != nullptr;
-  int* err = ok ? (int*)galloc(G, sizeof(int)) : nullptr;
-  if (!ok || !err) {   // no room: the float64 FFT kernels
+  if (!ok) {   // no room: the float64 FFT kernels
     cudaGetLastError();
     release_last(G, G->allocs.size() - before);
     return CH_OK;
   }
-  CK(cudaMemset(err, 0, sizeof(int)));
-  t.err = G->tc_err = err;
+  if (padded)
+    t.phys = (double*)galloc(G, (size_t)kNl * g.Px * g.Py * g.nz * sizeof(double));
+  if (!t.phys) cudaGetLastError();
   G->tx = t;
-  G->use_tx = 1;
+  G->use_ax = 1;
+  G->use_tx = t.phys != nullptr;
+  return CH_OK;
+}
+
+// ---- physical fields on the unpadded grid by the tensor-core transforms (use_ax)
+chf::YMap identity_ymap() {
+  chf::YMap m;
+  for (int f = 0; f < chf::YMap::kMax; ++f) m.src[f] = f;
+  m.dy_mask = 0;
+  m.kys = 0.0;
+  return m;
+}
+
+// nf coefficient fields in `coef` -> physical rows out[f]; uses auxA (samples in z) and auxB; map,
+// dmask: y-pass fields and x fields as in launch_txy_y and launch_txy_rows (nullptr: identity)
+int coef_to_rows(ch_grid* G, const double2* coef, int nf, const chf::YMap& ym, int ny_out,
+                 const int* xsrc, unsigned xmask, int nx_out, double* const* out) {
+  const GridDev& g = G->g;
+  cudaStream_t s = G->stream;
+  CK(chf::launch_cheb_tc(0, 0, coef, G->fs, G->auxA, G->fs, nf, g.Mx * g.ny, g.nz, G->tcb,
+                         G->tc_err, s));
+  CK(chf::launch_txy_y(1, g, g.ny, G->auxA, G->auxB, ny_out, G->fs, G->fs, ym, G->tx, G->tx.ybu, s));
+  CK(chf::launch_txy_rows(1, g, out, G->auxB, G->fs, nx_out, xsrc, xmask, G->tx, s));
+  return CH_OK;
+}
+// nf physical rows -> coefficient fields `coef` (not auxA or auxB's first nf fields)
+int rows_to_coef(ch_grid* G, double* const* phys, int nf, double2* coef) {
+  const GridDev& g = G->g;
+  cudaStream_t s = G->stream;
+  CK(chf::launch_txy_rows(0, g, phys, G->auxA, G->fs, nf, nullptr, 0, G->tx, s));
+  CK(chf::launch_txy_y(0, g, g.ny, G->auxA, G->auxB, nf, G->fs, G->fs, identity_ymap(), G->tx,
+                       G->tx.yfu, s));
+  CK(chf::launch_cheb_tc(0, 0, G->auxB, G->fs, coef, G->fs, nf, g.Mx * g.ny, g.nz, G->tcf,
+                         G->tc_err, s));
   return CH_OK;
 }
 
@@ -383,24 +477,34 @@ cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out
   const GridDev& g = G->g;
   const long long fi = dir == 1 ? G->fs : G->fsy, fo = dir == 1 ? G->fsy : G->fs;
   if (!G->use_tx) return chf::launch_ypass(dir, 0, g, g.Py, in, out, nf, fi, fo, 1.0, G->py[0], s);
-  chf::YMap id;
-  for (int f = 0; f < chf::YMap::kMax; ++f) id.src[f] = f;
-  id.dy_mask = 0;
-  id.kys = 0.0;
-  return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, id, G->tx,
+  return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, identity_ymap(), G->tx,
                            dir == 1 ? G->tx.yb : G->tx_yf1, s);
 }
 
 // the reverse sweep's own plan (forward y transform without the step's 1 / (Px Py)), made once
 int ch_adjoint_plan(ch_grid* G) {
   if (!G->use_tx || G->tx_yf1.dig) return CH_OK;
-  return make_txy_plan(G, 1, 1.0, &G->tx_yf1);
+  return make_txy_plan(G, 1, G->g.Py, 1.0, &G->tx_yf1);
 }
 
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev) {
   return launch_step(G, first, s, ev);
 }
 int ch_state_phys7(ch_grid* G) { return state_to_phys7(G, 7); }
+int ch_z_to_rows(ch_grid* G, const double2* in, double2* tmp, int nf, double* const* out) {
+  const GridDev& g = G->g;
+  cudaStream_t s = G->stream;
+  if (G->use_ax) {
+    CK(chf::launch_txy_y(1, g, g.ny, in, tmp, nf, G->fs, G->fs, identity_ymap(), G->tx, G->tx.ybu,
+                         s));
+    CK(chf::launch_txy_rows(1, g, out, tmp, G->fs, nf, nullptr, 0, G->tx, s));
+    return CH_OK;
+  }
+  CK(chf::launch_ypass(1, 0, g, g.ny, in, tmp, nf, G->fs, G->fs, 1.0, G->pyu, s));
+  for (int f = 0; f < nf; ++f)
+    CK(chf::launch_x_c2r(g, tmp + f * G->fs, out[f], 1, G->fs, G->fsp, G->pxu, s));
+  return CH_OK;
+}
 int ch_eval_nonlinear(ch_grid* G) { return eval_nonlinear_impl(G); }
 
 extern "C" {
@@ -588,10 +692,8 @@ int ch_init_grid(const ch_params* p, ch_alloc_fn alloc, ch_free_fn free_fn, void
   if (chf::zline_smem(g) > (size_t)kMaxSmem || chf::xline_smem(g.Px, sizeof(double2)) > (size_t)kMaxSmem) {
     return bail(G, CH_ERR_SIZE);
   }
-  if (G->prec == CH_PREC_FP64) {
-    st = setup_tx(G);
-    if (st != CH_OK) return bail(G, st);
-  }
+  st = setup_tx(G);
+  if (st != CH_OK) return bail(G, st);
   G->first = 1;
   G->fields_set = 0;
   G->nstep = 0;
@@ -619,11 +721,18 @@ static int set_from_phys(ch_grid* G, const double* u, const double* v, const dou
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
   const double* f4[4] = {u, v, w, phi};
-  for (int f = 0; f < 4; ++f)
-    CK(chf::launch_x_r2c(g, f4[f], G->auxA + f * G->fs, 1, G->fsp, G->fs, G->pxu, s));
-  CK(chf::launch_ypass(0, 0, g, g.ny, G->auxA, G->auxB, 4, G->fs, G->fs,
-                       1.0 / ((double)g.nx * (double)g.ny), G->pyu, s));
-  CK(chf::launch_project(g, G->auxB, G->fs, G->om, G->w, G->phi, G->hom, G->hw, G->hphi, G->pz, s));
+  if (G->use_ax) {
+    const int r = rows_to_coef(G, const_cast<double* const*>(f4), 4, G->auxA);
+    if (r != CH_OK) return r;
+    CK(chf::launch_project(g, G->auxA, G->fs, G->om, G->w, G->phi, G->hom, G->hw, G->hphi, G->pz, s,
+                           1));
+  } else {
+    for (int f = 0; f < 4; ++f)
+      CK(chf::launch_x_r2c(g, f4[f], G->auxA + f * G->fs, 1, G->fsp, G->fs, G->pxu, s));
+    CK(chf::launch_ypass(0, 0, g, g.ny, G->auxA, G->auxB, 4, G->fs, G->fs,
+                         1.0 / ((double)g.nx * (double)g.ny), G->pyu, s));
+    CK(chf::launch_project(g, G->auxB, G->fs, G->om, G->w, G->phi, G->hom, G->hw, G->hphi, G->pz, s));
+  }
   G->first = 1;
   G->nstep = 0;
   G->t = 0.0;
@@ -728,9 +837,13 @@ int ch_get_fields(ch_grid* G, double* u, double* v, double* w, double* phi) {
   if (!G || !u || !v || !w || !phi) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
+  double* f4[4] = {u, v, w, phi};
+  if (G->use_ax) {
+    CK(chf::launch_fields_coef(g, G->om, G->w, G->phi, G->auxB, G->fs, G->pz, s));
+    return coef_to_rows(G, G->auxB, 4, identity_ymap(), 4, nullptr, 0, 4, f4);
+  }
   CK(chf::launch_zbwd(0, 0, 7, g, G->R, G->om, G->w, G->phi, G->auxA, G->fs, G->pz, s));
   CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, 4, G->fs, G->fs, 1.0, G->pyu, s));
-  double* f4[4] = {u, v, w, phi};
   for (int f = 0; f < 4; ++f)
     CK(chf::launch_x_c2r(g, G->auxB + f * G->fs, f4[f], 1, G->fs, G->fsp, G->pxu, s));
   return CH_OK;
@@ -857,6 +970,10 @@ int ch_transform_forward(ch_grid* G, const double* phys, double* spec) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
+  if (G->use_ax) {
+    double* p[1] = {const_cast<double*>(phys)};
+    return rows_to_coef(G, p, 1, (double2*)spec);
+  }
   CK(chf::launch_x_r2c(g, phys, G->auxA, 1, G->fsp, G->fs, G->pxu, s));
   CK(chf::launch_ypass(0, 0, g, g.ny, G->auxA, G->auxB, 1, G->fs, G->fs,
                        1.0 / ((double)g.nx * (double)g.ny), G->pyu, s));
@@ -868,6 +985,8 @@ int ch_transform_backward(ch_grid* G, const double* spec, double* phys) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
+  if (G->use_ax)
+    return coef_to_rows(G, (const double2*)spec, 1, identity_ymap(), 1, nullptr, 0, 1, &phys);
   CK(chf::launch_dct_lines(1, 0, g, spec, G->auxA, 1, G->fs, G->pz, s));
   CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, 1, G->fs, G->fs, 1.0, G->pyu, s));
   CK(chf::launch_x_c2r(g, G->auxB, phys, 1, G->fs, G->fsp, G->pxu, s));
@@ -884,12 +1003,8 @@ int ch_nonlinear(ch_grid* G, double* out9) {
   const int r = eval_products(G);
   if (r != CH_OK) return r;
   if (G->use_tx) {
-    chf::YMap id;
-    for (int f = 0; f < chf::YMap::kMax; ++f) id.src[f] = f;
-    id.dy_mask = 0;
-    id.kys = 0.0;
-    CK(chf::launch_txy_y(0, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, id, G->tx, G->tx.yf,
-                         G->stream));
+    CK(chf::launch_txy_y(0, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, identity_ymap(), G->tx,
+                         G->tx.yf, G->stream));
   } else {
     CK(chf::launch_ypass(0, G->prec, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, scale,
                          G->py[G->prec], G->stream));
@@ -914,37 +1029,11 @@ int ch_set_chebyshev(ch_grid* G, int method) {
   if (G->adj_block) return CH_ERR_STATE;   // not while a reverse sweep is open
   if (method == CH_CHEB_TC) {
     if (!G->cf) {
-      const GridDev& g = G->g;
-      std::vector<uint16_t> dig[2];
-      chf::ChebTc t[2];
-      for (int dir = 0; dir < 2; ++dir) {
-        if (chf::cheb_tc_tables(g.N, dir, dig[dir], &t[dir]) != 0) return CH_ERR_SIZE;
-        void* dd = galloc(G, dig[dir].size() * sizeof(uint16_t));
-        if (!dd) return CH_ERR_ALLOC;
-        CK(cudaMemcpy(dd, dig[dir].data(), dig[dir].size() * sizeof(uint16_t),
-                      cudaMemcpyHostToDevice));
-        t[dir].dig = (const uint16_t*)dd;
-      }
-      CK(chf::cheb_tc_prepare());
-      CK(chf::zline_coef_prepare(g));
-      // one persistent CTA per SM, each with room for one tile's fixed-point rows
-      int dev = 0, nsm = 0;
-      CK(cudaGetDevice(&dev));
-      CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-      if (nsm < 1) nsm = 1;
-      void* keep = galloc(G, (size_t)nsm * chf::cheb_tc_keep_bytes(g.N));
-      if (!keep) return CH_ERR_ALLOC;
-      for (int dir = 0; dir < 2; ++dir) {
-        t[dir].keep = (char*)keep;
-        t[dir].ctas = nsm;
-      }
-      int* err = G->tc_err ? G->tc_err : (int*)galloc(G, sizeof(int));
+      const int r = ensure_cheb(G);
+      if (r != CH_OK) return r;
+      CK(chf::zline_coef_prepare(G->g));
       double2* cf = (double2*)galloc(G, (size_t)chf::kNc * G->fs * sizeof(double2));
-      if (!err || !cf) return CH_ERR_ALLOC;
-      if (!G->tc_err) CK(cudaMemset(err, 0, sizeof(int)));
-      G->tcf = t[0];
-      G->tcb = t[1];
-      G->tc_err = err;
+      if (!cf) return CH_ERR_ALLOC;
       G->cf = cf;
     }
   }

@@ -327,6 +327,7 @@ std::string signature_of(const ch_ensemble* E) {
   return sig + b;
 }
 
+
 void drop_graph(ch_ensemble* E) {
   if (E->graph_ok) cudaGraphExecDestroy(E->gexec);
   E->graph_ok = 0;

@@ -97,9 +97,10 @@ struct ch_grid {
   double2* cf = nullptr;
   int* tc_err = nullptr;
 
-  // float64 y and x transforms of the step on the tensor cores (use_tx); tx_yf1: the forward y
+  // tensor-core transforms of the unpadded grid for the entry points that take or give physical
+  // fields (use_ax) and of the step's float64 y and x stages (use_tx); tx_yf1: the forward y
   // transform without the 1 / (Px Py), for the reverse sweep
-  int use_tx = 0;
+  int use_ax = 0, use_tx = 0;
   chf::Txy tx;
   chf::TxyPlan tx_yf1;
 };
@@ -114,6 +115,8 @@ cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s);
 cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out, int nf,
                             cudaStream_t s);
 int ch_adjoint_plan(ch_grid* G);
+// nf fields of z samples (Mx, Ny, Nz) -> physical rows out[f]; tmp: nf fields
+int ch_z_to_rows(ch_grid* G, const double2* in, double2* tmp, int nf, double* const* out);
 // u v w phi phi_x phi_y phi_z of the state on the unpadded grid into phys7 ((nz, ny, nx) each)
 int ch_state_phys7(ch_grid* G);
 // frees the reverse-sweep workspace if allocated

@@ -97,9 +97,13 @@ cudaError_t build_factor_table(const GridDev& g, double* fac, cudaStream_t s);
 
 // Projection of four physical-z fields (u, v, w, phi as (Mx, Ny, Nz) complex, already
 // Fourier-transformed in x, y) onto the state (omega_z / mean flow, w, phi); zeroes history.
+// coef = 1: uvwp holds Chebyshev coefficients already.
 cudaError_t launch_project(const GridDev& g, const double2* uvwp, long long fs, double2* st_om,
                            double2* st_w, double2* st_phi, double2* h_om, double2* h_w,
-                           double2* h_phi, const FftPlan& pz, cudaStream_t s);
+                           double2* h_phi, const FftPlan& pz, cudaStream_t s, int coef = 0);
+// coefficients of the fields u v w phi D phi of the state as is (no update) into cf
+cudaError_t launch_fields_coef(const GridDev& g, double2* st_om, double2* st_w, double2* st_phi,
+                               double2* cf, long long fs, const FftPlan& pz, cudaStream_t s);
 
 // DCT-I of nf fields of (Mx, Ny, Nz) lines: dir 0 = samples -> coefficients (input precision
 // prec), dir 1 = coefficients -> samples (fp64 in and out).
@@ -314,6 +318,7 @@ struct TxyPlan {
 };
 struct Txy {
   TxyPlan yb, yf, xb, xf;          // y backward / forward (padded), x backward / forward
+  TxyPlan ybu, yfu, xbu, xfu;      // the same on the unpadded grid (yfu: times 1 / (Nx Ny))
   char* keep = nullptr;            // per persistent CTA: keep_bytes of fixed-point values
   size_t keep_bytes = 0;
   double* phys = nullptr;          // nine real fields (Px, Py, Nz)
@@ -329,6 +334,12 @@ cudaError_t launch_txy_y(int dir, const GridDev& g, int P, const void* in, void*
                          const TxyPlan& plan, cudaStream_t s);
 cudaError_t launch_txy_ycomb(const GridDev& g, const void* in, void* out9, long long fs_in,
                              long long fs_out, const Txy& x, cudaStream_t s);
+// x transforms between rows of physical samples (Nz, Ny, Nx), one pointer per field, and modes
+// (Mx, Ny, Nz): dir 0 forward (unnormalised), 1 backward (output f from field src[f], i kx times it
+// where dmask has bit f)
+cudaError_t launch_txy_rows(int dir, const GridDev& g, double* const* phys, double2* spec,
+                            long long fs, int nf, const int* src, unsigned dmask, const Txy& x,
+                            cudaStream_t s);
 cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long long fs, const Txy& x,
                          cudaStream_t s);
 // one bounded mbarrier wait that runs out on purpose (sets *err |= 1 after the wait bound)

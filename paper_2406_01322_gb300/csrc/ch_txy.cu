@@ -47,6 +47,7 @@ using namespace tc;
 constexpr int kPW = 8, kEW = 8, kSW = 3;               // producer, epilogue and scan warps
 constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
 constexpr int kMaxStages = 6;
+constexpr int kMaxFields = 9;
 constexpr int kRB = 3;                                 // tiles whose row scales are held
 constexpr int kBars = 3 * kMaxStages + 3 + 2 * kRB;
 constexpr size_t kTail = kRB * kRows * (sizeof(long long) + sizeof(int)) + (size_t)(kBars + 1) * 8;
@@ -58,15 +59,16 @@ __host__ __device__ constexpr int stage_bytes(int NT) { return kABytes + b_stage
 enum { YB = 0, YF = 1, XB = 2, XF = 3 };
 
 struct Args {
-  const double* in;
-  double* out;
-  long long fsi, fso;         // field strides (complex elements; real samples for XB out, XF in)
-  int src[16];                // input field of each output field
+  const double* in[kMaxFields];   // input and output of each output field
+  double* out[kMaxFields];
   unsigned dmask;             // output fields of i k times the input
   double kscale;              // k of mode 1
   int nlines, tpf, ntiles;    // lines per field, tiles per field, tiles
-  int ld;                     // line l: base (l / ld) * ihs + l % ld (inputs), * ohs (outputs)
-  long long ihs, ohs, estr, ostr;   // element strides along the transform, in and out
+  // line l starts at element (l / ld) ihs + (l % ld) ils of the input (complex elements; real
+  // samples for XF) and (l / ld) ohs + (l % ld) ols of the output (real samples for XB)
+  int ld;
+  long long ihs, ils, ohs, ols;
+  long long estr, ostr;       // element strides along the transform, in and out
   int n1, P;                  // modes of the full spectrum (Ny; unused for x), transform length
   TxyPlan t;
   char* keep;
@@ -163,7 +165,12 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
       if (MODE == XF) {
         *reinterpret_cast<double2*>(dst + 2 * (size_t)n * A.ostr) = make_double2(ra[e], rb[e]);
       } else if (MODE == XB) {
-        dst[(size_t)n * A.ostr] = ra[e];
+        // in rows of samples (ostr = 1) on 16-byte boundaries, samples n, n + 1 (n even) in one store
+        const bool rows = A.ostr == 1 && ((uintptr_t)dst & 15) == 0;
+        if (rows && !(e & 1) && n + 1 < nout)
+          *reinterpret_cast<double2*>(dst + n) = make_double2(ra[e], ra[e | 1]);
+        else if (!rows || !(e & 1))
+          dst[(size_t)n * A.ostr] = ra[e];
         if (n > 0) dst[(size_t)(A.P - n) * A.ostr] = rb[e];
       } else if (MODE == YB) {
         dst[2 * (size_t)n * A.ostr] = ra[e];
@@ -279,10 +286,9 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
         const int line = (tile - fld * A.tpf) * LPT + l, linen = (tn - fn * A.tpf) * LPT + l;
         const bool ok = line < A.nlines, okn = tn < A.ntiles && linen < A.nlines;
         const double* src =
-            A.in + ((long long)A.src[fld] * A.fsi + (ok ? (line / A.ld) * A.ihs + line % A.ld : 0)) * ISC;
+            A.in[fld] + (ok ? (line / A.ld) * A.ihs + (line % A.ld) * A.ils : 0) * ISC;
         const double* nxt =
-            okn ? A.in + ((long long)A.src[fn] * A.fsi + (linen / A.ld) * A.ihs + linen % A.ld) * ISC
-                : src;
+            okn ? A.in[fn] + ((linen / A.ld) * A.ihs + (linen % A.ld) * A.ils) * ISC : src;
         unsigned key = 0;
         if (ok) {
 #pragma unroll 8
@@ -385,8 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       const int line = (tile - fld * A.tpf) * LPT + l;
       const bool rowok = line < A.nlines, d = (A.dmask >> fld) & 1;
       const int lh = line / A.ld, ll = line - lh * A.ld;
-      const double* src =
-          A.in + ((long long)A.src[fld] * A.fsi + (rowok ? lh * A.ihs + ll : 0)) * ISC;
+      const double* src = A.in[fld] + (rowok ? lh * A.ihs + ll * A.ils : 0) * ISC;
       // complex inputs: x (k) and, folded, y (L - k); real ones: two samples per element
       double2 x[8];
       auto load = [&](int st) {
@@ -495,7 +500,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           const int e2 = sc - FBits<double>::EOFF - 51;   // sum 2^(E - 54), T = sum / 8
           const double vr = sc == kNanRow ? qnan<double>()
                                           : scaled_any<double>(hr * 16777216ll + ((lr + 4) >> 3), e2);
-          double* o = A.out + ((long long)fld * A.fso + lh * A.ohs + ll + (long long)(A.P / 2) * A.ostr) * OSC;
+          double* o = A.out[fld] + (lh * A.ohs + ll * A.ols + (long long)(A.P / 2) * A.ostr) * OSC;
           if (CPX) {
             const double vi = sc == kNanRow ? qnan<double>()
                                             : scaled_any<double>(hm * 16777216ll + ((lm + 4) >> 3), e2);
@@ -559,8 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       const bool safe =
           __all_sync(0xffffffffu, !rowok || (!nan && safe_exp<double>(ex))) != 0;
       const int lh = line / A.ld, ll = line - lh * A.ld;
-      double* dst =
-          A.out + ((long long)fld * A.fso + (rowok ? lh * A.ohs + ll : 0)) * OSC + part_c;
+      double* dst = A.out[fld] + (rowok ? lh * A.ohs + ll * A.ols : 0) * OSC + part_c;
       bool ok = true;
       for (int pp = 0; pp < 2 * A.t.nsl && ok; ++pp) {
         const int m0 = (pp >> 1) * NT + cg * CW;
@@ -699,25 +703,40 @@ int txy_plan(int mode, int n1, int P, double scale, std::vector<uint16_t>& dig, 
     Y[1][a] = (long long)llroundl(ldexpl(ws * sn, t->q));
   }
   const long long Y0 = mode == XB ? 1ll << t->q : Y[0][0];
+  // their digits as bf16, and the sum of the digits' magnitudes; entry P: k = 0
+  struct Dig {
+    uint16_t d[kPlanes];
+    int sum;
+  };
+  std::vector<Dig> D[2] = {std::vector<Dig>(P + 1), std::vector<Dig>(P + 1)};
+  for (int grp = 0; grp < 2; ++grp)
+    for (int a = 0; a <= P; ++a) {
+      const long long v = a < P ? Y[grp][a] : (grp == 0 ? Y0 : 0);
+      const unsigned long long y = (unsigned long long)v + kBias;
+      D[grp][a].sum = 0;
+      for (int j = 0; j < kPlanes; ++j) {
+        const int dgt = (int)((y >> (8 * (6 - j))) & 255ull) - 128;
+        D[grp][a].d[j] = bf16_bits((float)dgt);
+        D[grp][a].sum += abs(dgt);
+      }
+    }
   const int NT = t->NT;
   const size_t block = (size_t)kPlanes * NT * kKS;
   dig.assign((size_t)2 * t->nsl * t->nst * block, 0);
   double bound = 0.0;
   for (int n = 0; n < t->nout; ++n)
     for (int grp = 0; grp < 2; ++grp) {
-      double acc = 0.0;
-      for (int k = 0; k < t->nk; ++k) {
-        const long long yk = k == 0 ? (grp == 0 ? Y0 : 0) : Y[grp][((long long)n * k) % P];
-        const unsigned long long y = (unsigned long long)yk + kBias;
+      double acc = 0.0;   // |G_d| <= 128 sum_j sum_k |b_jk|
+      uint16_t* b0 = dig.data() + (size_t)(2 * (n / NT) + grp) * t->nst * block + (size_t)(n % NT) * 8;
+      int a = 0;          // n k mod P
+      for (int k = 0; k < t->nk; ++k, a = a + n >= P ? a + n - P : a + n) {
+        const Dig& e = D[grp][k == 0 ? P : a];
         const int st = k / kKS, kk = k % kKS;
         // stage position of k: 4 g + e holds g + 4 e (complex lines), 8 hf + e holds hf + 2 e
         const int pos = mode == YB || mode == YF ? 4 * (kk & 3) + (kk >> 2) : 8 * (kk & 1) + (kk >> 1);
-        uint16_t* b = dig.data() + ((size_t)(2 * (n / NT) + grp) * t->nst + st) * block;
-        for (int j = 0; j < kPlanes; ++j) {
-          const int row = j * NT + n % NT, dgt = (int)((y >> (8 * (6 - j))) & 255ull) - 128;
-          b[((size_t)(pos >> 3) * kPlanes * NT + row) * 8 + (pos & 7)] = bf16_bits((float)dgt);
-          acc += 128.0 * abs(dgt);   // |G_d| <= 128 sum_j sum_k |b_jk|
-        }
+        uint16_t* b = b0 + st * block + (size_t)(pos >> 3) * kPlanes * NT * 8 + (pos & 7);
+        for (int j = 0; j < kPlanes; ++j) b[(size_t)j * NT * 8] = e.d[j];
+        acc += 128.0 * e.sum;
       }
       bound = std::max(bound, acc);
     }
@@ -732,17 +751,18 @@ cudaError_t launch_txy_y(int dir, const GridDev& g, int P, const void* in, void*
                          const TxyPlan& plan, cudaStream_t s) {
   Args a;
   memset(&a, 0, sizeof a);
-  a.in = (const double*)in;
-  a.out = (double*)out;
-  a.fsi = fs_in;
-  a.fso = fs_out;
-  for (int f = 0; f < nf; ++f) a.src[f] = map.src[f];
+  if (nf > kMaxFields) return cudaErrorInvalidValue;
+  for (int f = 0; f < nf; ++f) {
+    a.in[f] = (const double*)in + 2 * map.src[f] * fs_in;
+    a.out[f] = (double*)out + 2 * f * fs_out;
+  }
   a.dmask = dir == 1 ? map.dy_mask : 0;
   a.kscale = map.kys;
   a.nlines = g.Mx * g.nz;
   a.ld = g.nz;
   a.ihs = (long long)(dir == 1 ? g.ny : P) * g.nz;
   a.ohs = (long long)(dir == 1 ? P : g.ny) * g.nz;
+  a.ils = a.ols = 1;
   a.estr = a.ostr = g.nz;
   a.n1 = g.ny;
   a.P = P;
@@ -771,16 +791,15 @@ cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long lon
   const long long np = (long long)g.Px * Q;
   Args a;
   memset(&a, 0, sizeof a);
-  a.in = (const double*)in6;
-  a.out = x.phys;
-  a.fsi = fs;
-  a.fso = np;
   const int src[7] = {0, 1, 2, 3, 3, 4, 5};   // u v w phi (phi -> i kx phi) phi_y phi_z
-  for (int f = 0; f < 7; ++f) a.src[f] = src[f];
+  for (int f = 0; f < 7; ++f) {
+    a.in[f] = (const double*)in6 + 2 * src[f] * fs;
+    a.out[f] = x.phys + f * np;
+  }
   a.dmask = 1u << 4;
   a.kscale = 6.283185307179586476925 / g.lx;
-  a.nlines = Q;
-  a.ld = Q;
+  a.nlines = a.ld = Q;
+  a.ils = a.ols = 1;
   a.estr = a.ostr = Q;
   a.P = g.Px;
   a.t = x.xb;
@@ -790,14 +809,44 @@ cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long lon
       x.phys, np, g.kappa);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  a.in = x.phys;
-  a.out = (double*)out9;
-  a.fsi = np;
-  a.fso = fs;
-  for (int f = 0; f < 9; ++f) a.src[f] = f;
+  for (int f = 0; f < 9; ++f) {
+    a.in[f] = x.phys + f * np;
+    a.out[f] = (double*)out9 + 2 * f * fs;
+  }
   a.dmask = 0;
   a.t = x.xf;
   return launch_mode<XF>(a, 9, x, s);
+}
+
+// x transforms between rows of physical samples (Nz, Ny, Nx) and modes (Mx, Ny, Nz) on the unpadded
+// grid: dir 0 phys[f] -> spec field f, dir 1 the inverse (field map src, i kx times the input for
+// the fields of dmask)
+cudaError_t launch_txy_rows(int dir, const GridDev& g, double* const* phys, double2* spec,
+                            long long fs, int nf, const int* src, unsigned dmask, const Txy& x,
+                            cudaStream_t s) {
+  Args a;
+  memset(&a, 0, sizeof a);
+  if (nf > kMaxFields) return cudaErrorInvalidValue;
+  for (int f = 0; f < nf; ++f) {
+    double* m = (double*)spec + 2 * (src ? src[f] : f) * fs;
+    a.in[f] = dir == 0 ? phys[f] : m;
+    a.out[f] = dir == 0 ? m : phys[f];
+  }
+  a.dmask = dir == 1 ? dmask : 0;
+  a.kscale = 6.283185307179586476925 / g.lx;
+  a.nlines = g.ny * g.nz;
+  a.ld = g.nz;                                        // line = y Nz + z
+  const long long rh = g.nx, rl = (long long)g.ny * g.nx, mh = g.nz, ml = 1;
+  a.ihs = dir == 0 ? rh : mh;
+  a.ils = dir == 0 ? rl : ml;
+  a.ohs = dir == 0 ? mh : rh;
+  a.ols = dir == 0 ? ml : rl;
+  const long long ms = (long long)g.ny * g.nz;
+  a.estr = dir == 0 ? 1 : ms;
+  a.ostr = dir == 0 ? ms : 1;
+  a.P = g.nx;
+  a.t = dir == 0 ? x.xfu : x.xbu;
+  return dir == 0 ? launch_mode<XF>(a, nf, x, s) : launch_mode<XB>(a, nf, x, s);
 }
 
 }  // namespace chf

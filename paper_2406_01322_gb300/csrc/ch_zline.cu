@@ -1129,6 +1129,8 @@ __global__ void __launch_bounds__(COEF ? ZTC : ZT) zbwd_kernel(GridDev g, const 
 }
 
 // set_fields projection: u, v, w, phi samples (after the x/y transforms) -> state
+// (COEF: their Chebyshev coefficients)
+template <int COEF>
 __global__ void __launch_bounds__(ZT) project_kernel(GridDev g, const double2* __restrict__ in,
                                                      long long fs, double2* st_om, double2* st_w,
                                                      double2* st_phi, double2* h_om,
@@ -1143,21 +1145,26 @@ __global__ void __launch_bounds__(ZT) project_kernel(GridDev g, const double2* _
   const bool nyq = (j == g.ny / 2);
   const bool is00 = (mx == 0 && j == 0);
   const ZSmem z = carve(zsm, Nz, N);
-  for (int idx = threadIdx.x; idx < 4 * Nz; idx += blockDim.x) {
-    const int f = idx / Nz, n = idx - f * Nz;
-    LN(z, f, Nz)[n] = in[(long long)f * fs + off + n];
+  if (!COEF) {
+    for (int idx = threadIdx.x; idx < 4 * Nz; idx += blockDim.x) {
+      const int f = idx / Nz, n = idx - f * Nz;
+      LN(z, f, Nz)[n] = in[(long long)f * fs + off + n];
+    }
+    __syncthreads();
+    dct_forward_lines(z, 0, 4, Nz, N, pz, g.zcs, is00);
   }
-  __syncthreads();
-  dct_forward_lines(z, 0, 4, Nz, N, pz, g.zcs, is00);
   const double2 zero = make_double2(0.0, 0.0);
+  auto fld = [&](int f, int n) {
+    return COEF ? in[(long long)f * fs + off + n] : LN(z, f, Nz)[n];
+  };
   for (int n = threadIdx.x; n < Nz; n += blockDim.x) {
-    const double2 u = LN(z, 0, Nz)[n], v = LN(z, 1, Nz)[n];
+    const double2 u = fld(0, n), v = fld(1, n);
     double2 om;
     if (is00) om = make_double2(u.x, v.x);           // ubar + i vbar
     else om = mul_i(kx * v - ky * u);                // i kx v - i ky u
     st_om[off + n] = nyq ? zero : om;
-    st_w[off + n] = (nyq || is00) ? zero : LN(z, 2, Nz)[n];
-    st_phi[off + n] = nyq ? zero : LN(z, 3, Nz)[n];
+    st_w[off + n] = (nyq || is00) ? zero : fld(2, n);
+    st_phi[off + n] = nyq ? zero : fld(3, n);
     h_om[off + n] = zero;
     h_w[off + n] = zero;
     h_phi[off + n] = zero;
@@ -1203,7 +1210,7 @@ __global__ void __launch_bounds__(DT) diag_partial_kernel(GridDev g, const doubl
                                                           const double* __restrict__ dzl,
                                                           double* __restrict__ part) {
   const long long npt = (long long)g.nz * g.ny * g.nx;
-  const double dx = g.lx / g.nx, dy = g.ly / g.ny;
+  const double dx = g.lx / g.nx, dy = g.ly / g.ny, rdx = 1.0 / dx, rdy = 1.0 / dy;
   double ke = 0, g2s = 0, fe = 0, cfl = 0, mphi = 0, nan = 0;
   for (long long i = blockIdx.x * (long long)DT + threadIdx.x; i < npt; i += (long long)gridDim.x * DT) {
     const int k = (int)(i / ((long long)g.ny * g.nx));
@@ -1215,7 +1222,7 @@ __global__ void __launch_bounds__(DT) diag_partial_kernel(GridDev g, const doubl
     g2s += wk * gg;
     const double q = ph * ph - 1.0;
     fe += wk * (0.25 * q * q + 0.5 * g.ch * g.ch * gg);
-    const double c = g.dt * (fabs(u) / dx + fabs(v) / dy + fabs(w) / dzl[k]);
+    const double c = g.dt * (fabs(u) * rdx + fabs(v) * rdy + fabs(w) / dzl[k]);
     cfl = fmax(cfl, c);
     mphi = fmax(mphi, fabs(ph));
     if (!isfinite(u) || !isfinite(v) || !isfinite(w) || !isfinite(ph)) nan = 1.0;
@@ -1238,24 +1245,34 @@ __global__ void __launch_bounds__(DT) diag_partial_kernel(GridDev g, const doubl
   if (threadIdx.x < 6) part[blockIdx.x * 6 + threadIdx.x] = red[threadIdx.x][0];
 }
 
-__global__ void diag_final_kernel(GridDev g, int nblk, const double* __restrict__ part,
-                                  const double2* __restrict__ st_phi, const double* __restrict__ qint,
-                                  double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[3] = {0, 0, 0}, m[3] = {0, 0, 0};
-  for (int b = 0; b < nblk; ++b) {
-    for (int q = 0; q < 3; ++q) s[q] += part[b * 6 + q];
-    for (int q = 0; q < 3; ++q) m[q] = fmax(m[q], part[b * 6 + 3 + q]);
+// one block: a thread per partial (nblk <= 304), tree over the block.  (One thread that added them
+// all in a loop took 114 us, a third of the partial sums' kernel.)
+constexpr int DFT = 512;
+__global__ void __launch_bounds__(DFT) diag_final_kernel(GridDev g, int nblk,
+                                                         const double* __restrict__ part,
+                                                         const double2* __restrict__ st_phi,
+                                                         const double* __restrict__ qint,
+                                                         double* __restrict__ out) {
+  __shared__ double red[7][DFT];
+  const int t = threadIdx.x;
+  double v[7] = {0, 0, 0, 0, 0, 0, 0};
+  for (int b = t; b < nblk; b += DFT) {
+    for (int q = 0; q < 3; ++q) v[q] += part[b * 6 + q];
+    for (int q = 3; q < 6; ++q) v[q] = fmax(v[q], part[b * 6 + q]);
   }
-  double mass = 0.0;  // line (0,0) is the first line of the state
-  for (int n = 0; n < g.nz; ++n) mass = fma(qint[n], st_phi[n].x, mass);
-  out[0] = mass * g.lx * g.ly;
-  out[1] = s[0];
-  out[2] = s[1];
-  out[3] = s[2];
-  out[4] = m[0];
-  out[5] = m[1];
-  out[6] = m[2];
+  // mass: line (0,0) is the first line of the state
+  for (int n = t; n < g.nz; n += DFT) v[6] = fma(qint[n], st_phi[n].x, v[6]);
+  for (int q = 0; q < 7; ++q) red[q][t] = v[q];
+  __syncthreads();
+  for (int s = DFT / 2; s > 0; s >>= 1) {
+    if (t < s)
+      for (int q = 0; q < 7; ++q)
+        red[q][t] = (q >= 3 && q < 6) ? fmax(red[q][t], red[q][t + s]) : red[q][t] + red[q][t + s];
+    __syncthreads();
+  }
+  if (t != 0) return;
+  out[0] = red[6][0] * g.lx * g.ly;
+  for (int q = 0; q < 6; ++q) out[1 + q] = red[q][0];
 }
 
 // ---- discrete adjoint of the step (float64) ----------------------------------------------
@@ -2279,12 +2296,29 @@ cudaError_t launch_zbwd(int update, int prec, int nout, const GridDev& g, const 
 
 cudaError_t launch_project(const GridDev& g, const double2* uvwp, long long fs, double2* st_om,
                            double2* st_w, double2* st_phi, double2* h_om, double2* h_w,
-                           double2* h_phi, const FftPlan& pz, cudaStream_t s) {
+                           double2* h_phi, const FftPlan& pz, cudaStream_t s, int coef) {
+  if (coef) {
+    project_kernel<1><<<g.Mx * g.ny, ZT, 0, s>>>(g, uvwp, fs, st_om, st_w, st_phi, h_om, h_w, h_phi,
+                                                 pz);
+    return cudaGetLastError();
+  }
   const size_t smem = zline_smem(g);
   static SmemLimit cur;
-  cudaError_t e = ensure_smem(project_kernel, smem, &cur);
+  cudaError_t e = ensure_smem(project_kernel<0>, smem, &cur);
   if (e != cudaSuccess) return e;
-  project_kernel<<<g.Mx * g.ny, ZT, smem, s>>>(g, uvwp, fs, st_om, st_w, st_phi, h_om, h_w, h_phi, pz);
+  project_kernel<0><<<g.Mx * g.ny, ZT, smem, s>>>(g, uvwp, fs, st_om, st_w, st_phi, h_om, h_w,
+                                                  h_phi, pz);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fields_coef(const GridDev& g, double2* st_om, double2* st_w, double2* st_phi,
+                               double2* cf, long long fs, const FftPlan& pz, cudaStream_t s) {
+  const size_t smem = zbwd_coef_smem(g);
+  static SmemLimit cur;
+  cudaError_t e = ensure_smem(zbwd_kernel<double, 0, 5, 1>, smem, &cur);
+  if (e != cudaSuccess) return e;
+  zbwd_kernel<double, 0, 5, 1><<<g.Mx * g.ny, ZTC, smem, s>>>(g, nullptr, st_om, st_w, st_phi, cf,
+                                                             fs, pz);
   return cudaGetLastError();
 }
 
@@ -2313,7 +2347,7 @@ cudaError_t launch_diag(const GridDev& g, const double* phys7, long long fs,
   diag_partial_kernel<<<nblk, DT, 0, s>>>(g, phys7, fs, ccw, dzl, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, 32, 0, s>>>(g, nblk, part, st_phi, qint, out);
+  diag_final_kernel<<<1, DFT, 0, s>>>(g, nblk, part, st_phi, qint, out);
   return cudaGetLastError();
 }
 
