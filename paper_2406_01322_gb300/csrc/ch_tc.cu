@@ -123,7 +123,8 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
     TO r[4];
     if (safe) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) r[e] = scaled<TO>(T[e], ex);
+      for (int e = 0; e < 4; ++e)
+        r[e] = (e & 1) ? scaled_alu<TO>(T[e], ex) : scaled<TO>(T[e], ex);
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e) r[e] = nan ? qnan<TO>() : scaled_any<TO>(T[e], ex);

@@ -267,11 +267,20 @@ __device__ __forceinline__ long long recombine(const uint32_t (&v)[ND][4], int e
   for (int d = 0; d < ND; ++d)
     g[d] = d < NMAG ? __float_as_int(__uint_as_float(v[d][e]) + 12582912.0f) - 0x4B400000
                     : __float2int_rz(__uint_as_float(v[d][e]));
+  // h, m (and q, when every |G| <= 2^22) fit 32 bits; G_4 256^2 + G_5 256 = 2^8 q and
+  // G_6 256 + G_7 (or G_6) = r contribute 4 q + round(r / 2^14) (round(r / 64)) to U / 64
   const int h = g[0] * 256 + g[1], m = g[2] * 256 + g[3];
-  long long l = (long long)g[4] * 65536 + ((long long)g[5] * 256 + (long long)g[6]);
-  if (ND == 8) l = (l * 256 + (long long)g[ND - 1] + 8192) >> 14;
-  else l = (l + 32) >> 6;
-  return (long long)((unsigned long long)(unsigned)h << 34) + (long long)m * 262144 + l;
+  long long l;
+  if (NMAG == ND) {
+    const int q = g[4] * 256 + g[5];
+    const int r = ND == 8 ? (g[6] * 256 + g[ND - 1] + 8192) >> 14 : (g[6] + 32) >> 6;
+    l = (long long)q * 4 + (long long)r;
+  } else {
+    l = (long long)g[4] * 1024 + ((long long)g[5] * 4 +
+        (ND == 8 ? ((long long)g[6] * 256 + (long long)g[ND - 1] + 8192) >> 14
+                 : (long long)((g[6] + 32) >> 6)));
+  }
+  return (long long)((unsigned long long)(unsigned)h << 34) + ((long long)m * 262144 + l);
 }
 
 // T 2^e rounded once to the output type: the integer converts in one instruction and the power of
@@ -284,6 +293,21 @@ template <typename TO> __device__ TO scaled(long long T, int e);
 template <> __device__ __forceinline__ double scaled<double>(long long T, int e) {
   const double v = __ll2double_rn(T);
   return __hiloint2double(__double2hiint(v) + (T != 0 ? e << 20 : 0), __double2loint(v));
+}
+// the same to nearest even by integer operations alone: the conversion instruction runs on the
+// float64 pipe (1.9 a clock per SM), so the epilogues send every second value this way
+template <typename TO> __device__ __forceinline__ TO scaled_alu(long long T, int e) {
+  return scaled<TO>(T, e);
+}
+template <> __device__ __forceinline__ double scaled_alu<double>(long long T, int e) {
+  const int sg = (int)(T >> 63);
+  const unsigned long long a = ((unsigned long long)T ^ (unsigned long long)(long long)sg) -
+                               (unsigned long long)(long long)sg;   // |T| < 2^63
+  const int lz = __clzll((long long)a);
+  const unsigned long long n = a << (lz - 1);                // leading one at bit 62
+  const unsigned long long m = (n + 0x1FFull + ((n >> 10) & 1ull)) >> 10;   // 53 bits, or 2^53
+  const int hi = (int)(m >> 32) + ((1085 - lz + e) << 20);   // m carries the implicit bit
+  return __hiloint2double((T != 0 ? hi : 0) | (sg & (int)0x80000000), T != 0 ? (int)m : 0);
 }
 template <> __device__ __forceinline__ float scaled<float>(long long T, int e) {
   return __int_as_float(__float_as_int(__ll2float_rn(T)) + (T != 0 ? e << 23 : 0));

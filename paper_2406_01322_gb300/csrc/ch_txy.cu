@@ -148,7 +148,7 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         ra[e] = scaled<double>(a[e], ex);
-        rb[e] = scaled<double>(b[e], ex);
+        rb[e] = scaled_alu<double>(b[e], ex);
       }
     } else {
 #pragma unroll
@@ -290,21 +290,34 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
         const double* nxt =
             okn ? A.in[fn] + ((linen / A.ld) * A.ihs + (linen % A.ld) * A.ils) * ISC : src;
         unsigned key = 0;
-        if (ok) {
-#pragma unroll 8
-          for (int j = 0; j < nel; ++j) {
-            if (okn)
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt + (size_t)j * A.estr * ISC));
-            if (MODE == XF) {
-              key = max(key, dkey(src[(size_t)j * A.estr]));
-            } else if (!(MODE == YB && j == A.n1 / 2)) {
-              double2 x = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
-              if (d) {
-                const double k = A.kscale * (double)((MODE == YB && j > A.n1 / 2) ? j - A.n1 : j);
-                x = make_double2(k * x.x, k * x.y);
-              }
-              key = max(key, max(dkey(x.x), dkey(x.y)));
+        constexpr int U = MODE == XF ? 16 : 8;   // loads in flight per lane
+        for (int j0 = 0; j0 < nel; j0 += U) {
+          double2 v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int j = j0 + u;
+            v[u] = make_double2(0.0, 0.0);
+            if (ok && j < nel && !(MODE == YB && j == A.n1 / 2)) {
+              if (MODE == XF) v[u].x = src[(size_t)j * A.estr];
+              else v[u] = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
             }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (okn && j0 + u < nel)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt + (size_t)(j0 + u) * A.estr * ISC));
+          if (MODE != XF && d) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int j = j0 + u;
+              const double k = A.kscale * (double)((MODE == YB && j > A.n1 / 2) ? j - A.n1 : j);
+              v[u] = make_double2(k * v[u].x, k * v[u].y);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            key = max(key, dkey(v[u].x));
+            if (MODE != XF) key = max(key, dkey(v[u].y));
           }
         }
         const int sc = row_scale<double>(key);
