@@ -48,9 +48,12 @@ constexpr int kPW = 8, kEW = 8, kSW = 3;               // producer, epilogue and
 constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
 constexpr int kMaxStages = 6;
 constexpr int kMaxFields = 9;
-constexpr int kRB = 3;                                 // tiles whose row scales are held
-constexpr int kBars = 3 * kMaxStages + 3 + 2 * kRB;
-constexpr size_t kTail = kRB * kRows * (sizeof(long long) + sizeof(int)) + (size_t)(kBars + 1) * 8;
+// tiles whose row scales are held: the scan runs at most this far ahead (with three, and an L2
+// prefetch of a fourth, tiles left L2 before they were converted: 256x256x129 y forward 1.75 ms
+// against 1.49)
+constexpr int kRB = 2;
+constexpr int kBars = 3 * kMaxStages + 4 + 2 * kRB;
+constexpr size_t kTail = kRB * kRows * (sizeof(long long) + 2 * sizeof(int)) + (size_t)(kBars + 1) * 8;
 // fixed-point values of one pass's stage block kept in global memory, eight per producer thread
 constexpr size_t kKeepStage = (size_t)kPW * 32 * 8 * sizeof(long long);
 
@@ -194,16 +197,20 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
   const int NT = A.t.NT, ns = A.t.stages, nst = A.t.nst;
   const int sbytes = stage_bytes(NT);
   unsigned char* stages = tsm;
+  // the recombined cosine products of a pass, per epilogue thread (in L2 instead, with room for five
+  // stages, the epilogue was slower: y backward 0.20 -> 0.23, x backward 0.28 -> 0.31 ms at 128^3)
   long long* hold0 = reinterpret_cast<long long*>(tsm + (size_t)ns * sbytes);
   long long* sC = hold0 + (NT / 2) * kEW * 32;
   int* sE = reinterpret_cast<int*>(sC + kRB * kRows);
-  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sE + kRB * kRows);
+  unsigned* sK = reinterpret_cast<unsigned*>(sE + kRB * kRows);   // largest key of each line
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(sK + kRB * kRows);
   uint32_t* sT = reinterpret_cast<uint32_t*>(bars + kBars);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t barFull = su32(bars), barB = barFull + 8 * kMaxStages;
   const uint32_t barEmpty = barFull + 16 * kMaxStages, barAccFull = barFull + 24 * kMaxStages;
   const uint32_t barAccFree = barAccFull + 8, barRow = barAccFull + 16;
-  const uint32_t barRowFree = barRow + 8 * kRB, barFin = barRowFree + 8 * kRB;
+  const uint32_t barRowFree = barRow + 8 * kRB, barFin = barRowFree + 8 * kRB, barKey = barFin + 8;
+  for (int i = tid; i < kRB * kRows; i += kThreads) sK[i] = 0;
   if (tid == 0) {
     for (int b = 0; b < kMaxStages; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barFull + 8 * b), "r"(kPW));
@@ -218,6 +225,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
                    "r"(kEW + kPW));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(barFin));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(barKey), "r"(kSW));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   const bool issuer_warp = warp == kPW + kEW;
@@ -270,42 +278,38 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
     }
     __syncwarp();
   } else if (warp > kPW + kEW) {
-    // ---- scan: lanes along the lines, 32 lines per group, one scale per line (a complex line's
-    // parts share it); the next tile's elements are prefetched into L2 on the way
-    const int sw = warp - (kPW + kEW + 1);
+    // ---- scan: one scale per line (a complex line's parts share it).  Each warp takes a third of the
+    // elements of every line, lanes along the lines, U loads in flight per lane.
+    const int sw = warp - (kPW + kEW + 1), st = sw * 32 + lane;
     const int nel = MODE == YB ? A.n1 : MODE == XB ? A.t.nk : A.P;
+    const int ja = nel * sw / kSW, jz = nel * (sw + 1) / kSW;
+    constexpr int U = MODE == XF ? 24 : 12;
     int ti = 0;
     for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
       const int b = ti % kRB;
       if (ti >= kRB && !W.wait_warp(barRowFree + 8 * b, (ti / kRB - 1) & 1)) break;
       const int fld = tile / A.tpf;
-      const int tn = tile + gridDim.x, fn = tn / A.tpf;
       const bool d = (A.dmask >> fld) & 1;
-      for (int gi = sw; gi < LPT / 32; gi += kSW) {
+#pragma unroll 1
+      for (int gi = 0; gi < LPT / 32; ++gi) {
         const int l = gi * 32 + lane;
-        const int line = (tile - fld * A.tpf) * LPT + l, linen = (tn - fn * A.tpf) * LPT + l;
-        const bool ok = line < A.nlines, okn = tn < A.ntiles && linen < A.nlines;
+        const int line = (tile - fld * A.tpf) * LPT + l;
+        const bool ok = line < A.nlines;
         const double* src =
             A.in[fld] + (ok ? (line / A.ld) * A.ihs + (line % A.ld) * A.ils : 0) * ISC;
-        const double* nxt =
-            okn ? A.in[fn] + ((linen / A.ld) * A.ihs + (linen % A.ld) * A.ils) * ISC : src;
         unsigned key = 0;
-        constexpr int U = MODE == XF ? 16 : 8;   // loads in flight per lane
-        for (int j0 = 0; j0 < nel; j0 += U) {
+#pragma unroll 1
+        for (int j0 = ja; j0 < jz; j0 += U) {
           double2 v[U];
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const int j = j0 + u;
             v[u] = make_double2(0.0, 0.0);
-            if (ok && j < nel && !(MODE == YB && j == A.n1 / 2)) {
+            if (ok && j < jz && !(MODE == YB && j == A.n1 / 2)) {
               if (MODE == XF) v[u].x = src[(size_t)j * A.estr];
               else v[u] = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
             }
           }
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (okn && j0 + u < nel)
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt + (size_t)(j0 + u) * A.estr * ISC));
           if (MODE != XF && d) {
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -320,11 +324,24 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
             if (MODE != XF) key = max(key, dkey(v[u].y));
           }
         }
-        const int sc = row_scale<double>(key);
+        if (key) atomicMax(&sK[b * kRows + l], key);
+      }
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barKey) : "memory");
+      if (!W.wait_warp(barKey, ti & 1)) break;
+      for (int l = st; l < LPT; l += 32 * kSW) {
+        const int line = (tile - fld * A.tpf) * LPT + l;
+        const bool ok = line < A.nlines && !(A.P & 1);
+        const double* mp = A.in[fld] + (ok ? (line / A.ld) * A.ihs + (line % A.ld) * A.ils +
+                                                 (long long)(A.P / 2) * A.estr
+                                           : 0) * ISC;
+        const int sc = row_scale<double>(sK[b * kRows + l]);
+        sK[b * kRows + l] = 0;   // for tile ti + kRB, whose scan waits for this one's readers
         if (CPX) {
           long long xr = 0, xi = 0;
-          if (MODE == YF && ok && !(A.P & 1)) {
-            const double2 x = *reinterpret_cast<const double2*>(src + 2 * (size_t)(A.P / 2) * A.estr);
+          if (MODE == YF && ok) {
+            const double2 x = *reinterpret_cast<const double2*>(mp);
             xr = fix<true>(x.x, sc);
             xi = fix<true>(x.y, sc);
           }
@@ -334,8 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           sC[ro] = __mul64hi(xr * 256, A.t.ymid * 4);   // x Y / 2^54
           sC[ro + 8] = __mul64hi(xi * 256, A.t.ymid * 4);
         } else {
-          long long x = 0;
-          if (MODE == XF && ok && !(A.P & 1)) x = fix<true>(src[(size_t)(A.P / 2) * A.estr], sc);
+          const long long x = MODE == XF && ok ? fix<true>(*mp, sc) : 0;
           sE[b * kRows + l] = sc;
           sC[b * kRows + l] = __mul64hi(x * 256, A.t.ymid * 4);
         }
@@ -559,6 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
     const int row = qd * 32 + lane;
     const int l = CPX ? (row >> 4) * 8 + (row & 7) : row, part_c = CPX ? (row >> 3) & 1 : 0;
     const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cg * CW);
+    // sums over several K groups are kept here between the groups
     long long* part = reinterpret_cast<long long*>(kcta + (size_t)2 * nst * kKeepStage) + tid;
     uint32_t pass = 0;
     int ti = 0;

@@ -678,7 +678,7 @@ __device__ void w_correct_mixed(const GridDev& g, double2* __restrict__ row, int
 // new phi on exit.
 constexpr int ST = 128;   // threads per zsolve CTA
 __device__ __forceinline__ void zsolve_body(const GridDev& g, double2* __restrict__ R, long long fs,
-                                            int nlines, int t) {
+                                            int nlines, int t, int prob) {
   const int N = g.N, Nz = g.nz;
   const int line = t >> 1, p = t & 1;
   if (line >= nlines) return;
@@ -698,13 +698,25 @@ __device__ __forceinline__ void zsolve_body(const GridDev& g, double2* __restric
   const unsigned pm = 0x3u << (threadIdx.x & 30);  // the two lanes (parities) of this line
   const int oo = fsl ? 3 : 0;
   double2* row = R + (size_t)line * Nz;
-  if (mixed)
-    tau_sweep_mixed(row, p, N, k2 + g.beta, g.bc, t1, t2, t3, fac_ptr(g, 0, 0, K),
-                    fac_ptr(g, 0, 1, K), fac_ptr(g, 0, 2, K), g.NK,
-                    g.fac + fac_mixed_off(g, 0) + K, pm);
-  else
-    tau_sweep_c<true>(row, p, N, k2 + g.beta, fsl, t1, t2, t3, fac_ptr(g, oo, 0, K),
-                fac_ptr(g, oo, 1, K), fac_ptr(g, oo, 2, K), g.NK, fac_rsq(g, oo, p, K));
+  if (prob == 0) {
+    if (mixed)
+      tau_sweep_mixed(row, p, N, k2 + g.beta, g.bc, t1, t2, t3, fac_ptr(g, 0, 0, K),
+                      fac_ptr(g, 0, 1, K), fac_ptr(g, 0, 2, K), g.NK,
+                      g.fac + fac_mixed_off(g, 0) + K, pm);
+    else
+      tau_sweep_c<true>(row, p, N, k2 + g.beta, fsl, t1, t2, t3, fac_ptr(g, oo, 0, K),
+                  fac_ptr(g, oo, 1, K), fac_ptr(g, oo, 2, K), g.NK, fac_rsq(g, oo, p, K));
+    return;
+  }
+  if (prob == 2) {
+    // phi: two Neumann problems with the same operator (D^2 - k^2 - lam)
+    row = R + 2 * fs + (size_t)line * Nz;
+    const double a = k2 + g.lam;
+    for (int rep = 0; rep < 2; ++rep)
+      tau_sweep_c<true>(row, p, N, a, true, t1, t2, t3, fac_ptr(g, 2, 0, K), fac_ptr(g, 2, 1, K),
+                  fac_ptr(g, 2, 2, K), g.NK, fac_rsq(g, 2, p, K));
+    return;
+  }
   // w: influence problem (theta, w) with w = w' = 0 at both walls, or (free-slip) theta and w
   // each with Dirichlet rows
   row = R + fs + (size_t)line * Nz;
@@ -739,17 +751,11 @@ __device__ __forceinline__ void zsolve_body(const GridDev& g, double2* __restric
       row[n] = v;
     }
   }
-  // phi: two Neumann problems with the same operator (D^2 - k^2 - lam)
-  row = R + 2 * fs + (size_t)line * Nz;
-  const double a = k2 + g.lam;
-  for (int rep = 0; rep < 2; ++rep)
-    tau_sweep_c<true>(row, p, N, a, true, t1, t2, t3, fac_ptr(g, 2, 0, K), fac_ptr(g, 2, 1, K),
-                fac_ptr(g, 2, 2, K), g.NK, fac_rsq(g, 2, p, K));
 }
 
 __global__ void __launch_bounds__(ST) zsolve_kernel(GridDev g, double2* __restrict__ R,
                                                     long long fs, int nlines) {
-  zsolve_body(g, R, fs, nlines, blockIdx.x * blockDim.x + threadIdx.x);
+  zsolve_body(g, R, fs, nlines, blockIdx.x * blockDim.x + threadIdx.x, 2 - blockIdx.y);
 }
 
 constexpr int TL = 32;    // lines per tile-variant CTA (2 TL chains: one per (line, parity))
@@ -832,7 +838,7 @@ __device__ __forceinline__ void solve_tile_problem(const GridDev& g, double2* __
 // parity), the three problems in turn.  R holds [omega | theta-w | phi] right-hand sides on
 // entry and the solved sums / new phi on exit (line-major, like the state).
 __device__ __forceinline__ void zsolve_tile_body(const GridDev& g, double2* __restrict__ R,
-                                                 long long fs, int nlines, int bid) {
+                                                 long long fs, int nlines, int bid, int prob) {
   extern __shared__ double2 ssm[];
   const int Nz = g.nz;
   double2* tile = ssm;
@@ -859,20 +865,17 @@ __device__ __forceinline__ void zsolve_tile_body(const GridDev& g, double2* __re
   const bool is00 = (mx == 0 && j == 0);
   const int ntile = min(TL, nlines - line0);
   const unsigned pm = 0x3u << (threadIdx.x & 30);  // the two lanes of this line
-  for (int prob = 0; prob < 3; ++prob) {
-    double2* Rp = R + prob * fs + (size_t)line0 * Nz;
-    tile_copy(tile, Rp, ntile * Nz);
-    __syncthreads();
-    if (valid) solve_tile_problem(g, tile + l * Nz, prob, p, K, k2, is00, t1, t2, t3, pm);
-    __syncthreads();
-    tile_copy(Rp, tile, ntile * Nz);
-    __syncthreads();
-  }
+  double2* Rp = R + prob * fs + (size_t)line0 * Nz;
+  tile_copy(tile, Rp, ntile * Nz);
+  __syncthreads();
+  if (valid) solve_tile_problem(g, tile + l * Nz, prob, p, K, k2, is00, t1, t2, t3, pm);
+  __syncthreads();
+  tile_copy(Rp, tile, ntile * Nz);
 }
 
 __global__ void __launch_bounds__(TLT) zsolve_tile_kernel(GridDev g, double2* __restrict__ R,
                                                         long long fs, int nlines) {
-  zsolve_tile_body(g, R, fs, nlines, blockIdx.x);
+  zsolve_tile_body(g, R, fs, nlines, blockIdx.x, 2 - blockIdx.y);
 }
 
 // ---- operator table (init time) -------------------------------------------------------------
@@ -1987,8 +1990,10 @@ __global__ void __launch_bounds__(TLT) grouped_zsolve_tile_kernel(const Member* 
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int m = member_of(begin, nmem, item);
     const Member& M = mem[m];
-    zsolve_tile_body(M.g, M.R, M.fs, M.g.Mx * M.g.ny, item - begin[m]);
-    __syncthreads();
+    for (int prob = 0; prob < 3; ++prob) {
+      zsolve_tile_body(M.g, M.R, M.fs, M.g.Mx * M.g.ny, item - begin[m], prob);
+      __syncthreads();
+    }
   }
 }
 
@@ -1998,7 +2003,8 @@ __global__ void __launch_bounds__(ST) grouped_zsolve_kernel(const Member* __rest
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int m = member_of(begin, nmem, item);
     const Member& M = mem[m];
-    zsolve_body(M.g, M.R, M.fs, M.g.Mx * M.g.ny, (item - begin[m]) * ST + threadIdx.x);
+    for (int prob = 0; prob < 3; ++prob)
+      zsolve_body(M.g, M.R, M.fs, M.g.Mx * M.g.ny, (item - begin[m]) * ST + threadIdx.x, prob);
   }
 }
 
@@ -2256,11 +2262,11 @@ cudaError_t launch_zsolve(const GridDev& g, double2* R, long long fs, cudaStream
     static SmemLimit cur;
     cudaError_t e = ensure_smem(zsolve_tile_kernel, tile, &cur);
     if (e != cudaSuccess) return e;
-    zsolve_tile_kernel<<<(nlines + TL - 1) / TL, TLT, tile, s>>>(g, R, fs, nlines);
+    zsolve_tile_kernel<<<dim3((nlines + TL - 1) / TL, 3), TLT, tile, s>>>(g, R, fs, nlines);
   } else {
     // long lines: sweep in global memory (L1/L2), occupancy set by registers
     const int nthreads = 2 * nlines;
-    zsolve_kernel<<<(nthreads + ST - 1) / ST, ST, 0, s>>>(g, R, fs, nlines);
+    zsolve_kernel<<<dim3((nthreads + ST - 1) / ST, 3), ST, 0, s>>>(g, R, fs, nlines);
   }
   return cudaGetLastError();
 }
