@@ -135,7 +135,7 @@ int reverse_core(ch_grid* G, const double2* ya, int first, cudaEvent_t* ev) {
   if (ev) cudaEventRecord(ev[2], s);
   e[2] = ch_launch_y_adj(G, 1, G->a_nlb, (double2*)G->yb, kNl, s);
   if (ev) cudaEventRecord(ev[3], s);
-  e[3] = chf::launch_adj_xline(g, ya, (const double2*)G->yb, G->a_x6, G->fsy, G->px[0], s);
+  e[3] = ch_launch_x_adj(G, ya, G->a_x6, s);
   if (ev) cudaEventRecord(ev[4], s);
   e[4] = ch_launch_y_adj(G, 0, G->a_x6, G->auxA, kYa, s);
   if (ev) cudaEventRecord(ev[5], s);

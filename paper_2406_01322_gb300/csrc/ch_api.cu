@@ -393,7 +393,7 @@ int setup_tx(ch_grid* G) {
   const int len[8] = {g.ny, g.ny, g.nx, g.nx, g.Py, g.Py, g.Px, g.Px};
   bool ok = true;
   for (int i = 0; i < (padded ? 8 : 4) && ok; ++i) {
-    const int r = make_txy_plan(G, i & 3, len[i], i == 1 ? su : i == 5 ? sp : 1.0, plan[i]);
+    const int r = make_txy_plan(G, i & 3, len[i], i == 1 ? su : i == 5 ? sp : 2.0, plan[i]);
     if (r == CH_ERR_CUDA) return r;
     ok = r == CH_OK;
     t.keep_bytes = std::max(t.keep_bytes, chf::txy_keep_bytes(*plan[i]));
@@ -476,15 +476,36 @@ cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out
                             cudaStream_t s) {
   const GridDev& g = G->g;
   const long long fi = dir == 1 ? G->fs : G->fsy, fo = dir == 1 ? G->fsy : G->fs;
-  if (!G->use_tx) return chf::launch_ypass(dir, 0, g, g.Py, in, out, nf, fi, fo, 1.0, G->py[0], s);
+  if (!G->use_tx || !(dir == 1 ? G->tx.yb : G->tx_yf1).dig)
+    return chf::launch_ypass(dir, 0, g, g.Py, in, out, nf, fi, fo, 1.0, G->py[0], s);
   return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, identity_ymap(), G->tx,
                            dir == 1 ? G->tx.yb : G->tx_yf1, s);
 }
 
-// the reverse sweep's own plan (forward y transform without the step's 1 / (Px Py)), made once
+cudaError_t ch_launch_x_adj(ch_grid* G, const double2* ya, double2* out6, cudaStream_t s) {
+  const GridDev& g = G->g;
+  if (!G->use_tx || !G->tx_xb1.dig)
+    return chf::launch_adj_xline(g, ya, (const double2*)G->yb, out6, G->fsy, G->px[0], s);
+  // the padded physical fields (9/4 of an unpadded one) use the buffers of seven unpadded fields that
+  // the reverse step does not need here
+  const long long np = (long long)g.Px * g.Py * g.nz;
+  double *a = (double*)G->auxA, *b = (double*)G->auxB;
+  double* const phys7[7] = {a, a + np, a + 2 * np, b, b + np, b + 2 * np, G->phys7};
+  return chf::launch_txy_adj_x(g, ya, G->yb, out6, G->fsy, phys7, G->tx, G->tx_xb1, s);
+}
+
+// the reverse sweep's own plans, made once; without room for them the FFT kernels run
 int ch_adjoint_plan(ch_grid* G) {
-  if (!G->use_tx || G->tx_yf1.dig) return CH_OK;
-  return make_txy_plan(G, 1, G->g.Py, 1.0, &G->tx_yf1);
+  if (!G->use_tx) return CH_OK;
+  for (int i = 0; i < 2; ++i) {
+    chf::TxyPlan t, *p = i == 0 ? &G->tx_yf1 : &G->tx_xb1;
+    if (p->dig) continue;
+    const int r = make_txy_plan(G, i == 0 ? 1 : 2, i == 0 ? G->g.Py : G->g.Px, 1.0, &t);
+    if (r == CH_ERR_CUDA) return r;
+    if (r == CH_OK) *p = t;
+    else cudaGetLastError();
+  }
+  return CH_OK;
 }
 
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev) {

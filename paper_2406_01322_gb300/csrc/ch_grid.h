@@ -98,11 +98,12 @@ struct ch_grid {
   int* tc_err = nullptr;
 
   // tensor-core transforms of the unpadded grid for the entry points that take or give physical
-  // fields (use_ax) and of the step's float64 y and x stages (use_tx); tx_yf1: the forward y
-  // transform without the 1 / (Px Py), for the reverse sweep
+  // fields (use_ax) and of the step's float64 y and x stages (use_tx); for the reverse sweep,
+  // made when it first begins, tx_yf1: the forward y transform without the 1 / (Px Py), tx_xb1: the
+  // transposed forward x transform
   int use_ax = 0, use_tx = 0;
   chf::Txy tx;
-  chf::TxyPlan tx_yf1;
+  chf::TxyPlan tx_yf1, tx_xb1;
 };
 
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
@@ -114,6 +115,9 @@ cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s);
 // float64 y pass of the reverse sweep (identity field map, scale 1) on the padded grid
 cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out, int nf,
                             cudaStream_t s);
+// transposed x line of the reverse sweep: ya (y-padded fields of the state), yb (product adjoints,
+// overwritten) -> out6
+cudaError_t ch_launch_x_adj(ch_grid* G, const double2* ya, double2* out6, cudaStream_t s);
 int ch_adjoint_plan(ch_grid* G);
 // nf fields of z samples (Mx, Ny, Nz) -> physical rows out[f]; tmp: nf fields
 int ch_z_to_rows(ch_grid* G, const double2* in, double2* tmp, int nf, double* const* out);

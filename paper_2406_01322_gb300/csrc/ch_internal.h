@@ -313,6 +313,7 @@ cudaError_t launch_cheb_tc(int tin, int tout, const void* in, long long fsi, voi
 struct TxyPlan {
   const uint16_t* dig = nullptr;   // device: matrix digits (txy_plan)
   int nk = 0, nout = 0, NT = 0, nsl = 0, nst = 0, kc = 0, gst = 0, stages = 0, nmag = 0, q = 0;
+  int unit = 0;                    // x backward with weight 1 at every mode
   long long ymid = 0;              // weight of the middle sample of a forward transform, times 2^q
   size_t smem = 0;
 };
@@ -325,7 +326,8 @@ struct Txy {
   int ctas = 0;
   int* err = nullptr;              // |= 1 if a bounded wait gave up
 };
-// mode 0 y backward, 1 y forward (times scale), 2 x backward, 3 x forward; n1 = Ny (y) or Mx (x), P
+// mode 0 y backward, 1 y forward (times scale), 2 x backward (scale: the weight of the modes k >= 1,
+// 2 for a half spectrum, 1 for the transpose of the forward transform), 3 x forward; n1 = Ny (y) or Mx (x), P
 // the transform length
 int txy_plan(int mode, int n1, int P, double scale, std::vector<uint16_t>& dig, TxyPlan* t);
 size_t txy_keep_bytes(const TxyPlan& t);
@@ -342,6 +344,10 @@ cudaError_t launch_txy_rows(int dir, const GridDev& g, double* const* phys, doub
                             cudaStream_t s);
 cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long long fs, const Txy& x,
                          cudaStream_t s);
+// transposed x line; phys7: scratch, seven real fields (Px, Py, Nz); xb1: x backward plan of scale 1;
+// overwrites pb9
+cudaError_t launch_txy_adj_x(const GridDev& g, const void* in6, void* pb9, void* out6, long long fs,
+                             double* const* phys7, const Txy& x, const TxyPlan& xb1, cudaStream_t s);
 // one bounded mbarrier wait that runs out on purpose (sets *err |= 1 after the wait bound)
 cudaError_t launch_wait_selftest(int* err, int nwaits, cudaStream_t s);
 // float64 FMA-rate probe: `blocks` CTAs of 256 threads, `iters` iterations of eight independent
