@@ -139,11 +139,12 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
 // elements, line stride Nz = N + 1; dig: the matrix digits, stage blocks of 7 NT rows x 16 K in
 // the order slice, parity, stage; keep: keep_bytes per CTA; nst stages per parity in kc groups of
 // gst; nmag: accumulators known to stay within 2^22 (7, 3 or 0); q: log2 of the matrix scale;
-// ymid: middle weight times 2^q; lastf: factor of output N (forward).
+// ymid: middle weight times 2^q; lastf: factor of output N (forward).  The 2 nsl passes of a tile are
+// cut into items of np passes; several items a tile only where all items have a CTA each (launch_t).
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kThreads, 1)
     cheb_tc_kernel(const TI* __restrict__ in, long long fsi, TO* __restrict__ out, long long fso,
-                   int nlines, int Nz, int tpf, int ntiles, int NT, int nsl, int nst, int kc,
+                   int nlines, int Nz, int tpf, int ntiles, int np, int NT, int nsl, int nst, int kc,
                    int gst, int nmag, const uint16_t* __restrict__ dig, char* __restrict__ keep,
                    long long keep_bytes, int fwd, int q, long long ymid, double lastf,
                    int* __restrict__ err) {
@@ -183,6 +184,53 @@ __global__ void __launch_bounds__(kThreads, 1)
                  "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  const int nparts = 2 * nsl / np, nitems = ntiles * nparts;
+  // row scales and middle terms of lines l0 .. l0 + 3 of a tile, a warp's lanes along the lines
+  auto scan4 = [&](int tile, int b, int l0) {
+    const int fld = tile / tpf;
+    const int line0 = (tile - fld * tpf) * (kRows / 2);
+    const int nl = min(kRows / 2, nlines - line0);
+    const TI* src = in + ((size_t)fld * fsi + (size_t)line0 * Nz) * 2;
+    unsigned kr[4] = {0, 0, 0, 0}, ki[4] = {0, 0, 0, 0};
+#pragma unroll 2
+    for (int k = lane; k < Nz; k += 32) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (l0 + i < nl) {
+          const CBits<TI> x = ld_cplx(src + ((size_t)(l0 + i) * Nz + k) * 2);
+          kr[i] = max(kr[i], F::key(x.re));
+          ki[i] = max(ki[i], F::key(x.im));
+        }
+    }
+    unsigned mr = 0, mi = 0;   // lane i < 4: the keys of line l0 + i
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned a = __reduce_max_sync(0xffffffffu, kr[i]);
+      const unsigned c = __reduce_max_sync(0xffffffffu, ki[i]);
+      if (lane == i) {
+        mr = a;
+        mi = c;
+      }
+    }
+    if (lane < 4 && l0 + lane < kRows / 2) {
+      const int l = l0 + lane, er = row_scale<TI>(mr), ei = row_scale<TI>(mi);
+      long long xr = 0, xi = 0;
+      if (l < nl) {
+        const CBits<TI> x = ld_cplx(src + ((size_t)l * Nz + H) * 2);
+        xr = Fixed<TI, true>::of(x.re, er);
+        xi = Fixed<TI, true>::of(x.im, ei);
+      }
+      const int ro = b * kRows + tile_row(l, 0);
+      sE[ro] = er;
+      sE[ro + 8] = ei;
+      // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
+      sC[ro] = __mul64hi(xr * 256, ymid * 4);
+      sC[ro + 8] = __mul64hi(xi * 256, ymid * 4);
+    }
+  };
+  // the first tile by every warp (scanned by three, it kept the others waiting: a launch of one tile per
+  // CTA 13 -> 10 us at N = 16, 19 -> 13 at N = 64)
+  if (4 * warp < kRows / 2) scan4(blockIdx.x / nparts, 0, 4 * warp);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();   // barriers and tensor-memory address visible to every warp
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -197,8 +245,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t slot = 0, use = 0;   // stage slot and how often it was used
       uint32_t pass = 0;
       bool any = false;
-      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-        for (int pp = 0; pp < 2 * nsl; ++pp)
+      for (int item = blockIdx.x; item < nitems; item += gridDim.x)
+        for (int pp = 0; pp < np; ++pp)
           for (int c = 0; c < kc; ++c, ++pass) {
             if (pass > 0 && !W.wait(barAccFree, (pass - 1) & 1)) goto drain;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -228,16 +276,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp > kPW + kEW) {
-    // ---- scan: four lines at a time, a warp's lanes along the line
+    // ---- scan: four lines at a time
     const int sw = warp - (kPW + kEW + 1);
     int ti = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
-      const int fld = tile / tpf;
-      const int line0 = (tile - fld * tpf) * (kRows / 2);
-      const int nl = min(kRows / 2, nlines - line0);
-      const TI* src = in + ((size_t)fld * fsi + (size_t)line0 * Nz) * 2;
-      if (sw == 0 && lane == 0 && tile + (int)gridDim.x < ntiles) {
-        const int tn = tile + gridDim.x, fn = tn / tpf, ln = (tn - fn * tpf) * (kRows / 2);
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++ti) {
+      const int tile = item / nparts;
+      if (sw == 0 && lane == 0 && item + (int)gridDim.x < nitems) {
+        const int tn = (item + gridDim.x) / nparts, fn = tn / tpf, ln = (tn - fn * tpf) * (kRows / 2);
         const char* a = reinterpret_cast<const char*>(in + ((size_t)fn * fsi + (size_t)ln * Nz) * 2);
         const char* z = a + (size_t)min(kRows / 2, nlines - ln) * Nz * 2 * sizeof(TI);
         const uintptr_t a16 = ((uintptr_t)a + 15) & ~(uintptr_t)15;
@@ -249,44 +294,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const int b = ti % kRB;
       if (ti >= kRB && !W.wait_warp(barRowFree + 8 * b, (ti / kRB - 1) & 1)) break;
-      for (int l0 = 4 * sw; l0 < kRows / 2; l0 += 4 * kSW) {
-        unsigned kr[4] = {0, 0, 0, 0}, ki[4] = {0, 0, 0, 0};
-#pragma unroll 2
-        for (int k = lane; k < Nz; k += 32) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (l0 + i < nl) {
-              const CBits<TI> x = ld_cplx(src + ((size_t)(l0 + i) * Nz + k) * 2);
-              kr[i] = max(kr[i], F::key(x.re));
-              ki[i] = max(ki[i], F::key(x.im));
-            }
-        }
-        unsigned mr = 0, mi = 0;   // lane i < 4: the keys of line l0 + i
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const unsigned a = __reduce_max_sync(0xffffffffu, kr[i]);
-          const unsigned c = __reduce_max_sync(0xffffffffu, ki[i]);
-          if (lane == i) {
-            mr = a;
-            mi = c;
-          }
-        }
-        if (lane < 4 && l0 + lane < kRows / 2) {
-          const int l = l0 + lane, er = row_scale<TI>(mr), ei = row_scale<TI>(mi);
-          long long xr = 0, xi = 0;
-          if (l < nl) {
-            const CBits<TI> x = ld_cplx(src + ((size_t)l * Nz + H) * 2);
-            xr = Fixed<TI, true>::of(x.re, er);
-            xi = Fixed<TI, true>::of(x.im, ei);
-          }
-          const int ro = b * kRows + tile_row(l, 0);
-          sE[ro] = er;
-          sE[ro + 8] = ei;
-          // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
-          sC[ro] = __mul64hi(xr * 256, ymid * 4);
-          sC[ro + 8] = __mul64hi(xi * 256, ymid * 4);
-        }
-      }
+      if (ti > 0)
+        for (int l0 = 4 * sw; l0 < kRows / 2; l0 += 4 * kSW) scan4(tile, b, l0);
       __syncwarp();
       if (lane == 0)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRow + 8 * b) : "memory");
@@ -337,7 +346,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         __stcg(d + i * kPW * 32, make_longlong2((long long)v[2 * i], (long long)v[2 * i + 1]));
     };
     const size_t bstride = (size_t)bbytes / 2;   // elements of a stage block
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++ti) {
+      const int tile = item / nparts, pp0 = (item - tile * nparts) * np;
       const int fld = tile / tpf;
       const int line = (tile - fld * tpf) * (kRows / 2) + l;
       const bool rowok = line < nlines;
@@ -365,7 +375,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
                      : "memory");
       const bool tiny = __any_sync(0xffffffffu, min(ere, eim) < kTinyScale) != 0;
-      // first pass: convert, fold, write the sums' planes, keep the differences (all biased)
+      // first pass: convert, fold, write the sums' (odd passes: the differences') planes, keep what the
+      // item's other passes need (all biased)
       unsigned long long sumr = 0, sumi = 0, s0r = 0, s0i = 0;
       bool ok = true;
       for (int st = 0; st < nst && ok; ++st) {
@@ -392,8 +403,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (st + 1 < nst) load(st + 1);
-        store_keep(keep_at(1, st), d);
-        if (nsl > 1) store_keep(keep_at(0, st), s);
+        if (np > 1) store_keep(keep_at(1, st), d);   // for np = 2 pp0 is even
+        if (np > 2) store_keep(keep_at(0, st), s);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {   // at most 64 values below 2^56
           sumr += s[e];
@@ -403,12 +414,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           s0r = s[0];
           s0i = s[4];
         }
-        ok = put(s, dig + (size_t)st * bstride);
+        const uint16_t* bsrc = dig + ((size_t)pp0 * nst + st) * bstride;
+        ok = pp0 & 1 ? put(d, bsrc) : put(s, bsrc);
       }
       if (!ok) break;
       // the last output n = N: sum_k w_k (-1)^k x_k, (-1)^k = (-1)^g for this thread's k; weights
       // e_k = 2 except k = 0, N (forward) or 1.  High and low parts (27 bits) are added apart.
-      {
+      if (pp0 == 0) {
         const unsigned long long nb = (unsigned long long)(4 * nst) * kBias;
         long long tr = (long long)(sumr - nb), tm = (long long)(sumi - nb);
         if (g & 1) {
@@ -460,8 +472,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           o[1] = vi;
         }
       }
-      // the later passes: slice 0 odd, then even and odd of each further slice, from the kept values
-      for (int pp = 1; pp < 2 * nsl && ok; ++pp) {
+      // the later passes: odd, then even and odd of each further slice, from the kept values
+      for (int pp = pp0 + 1; pp < pp0 + np && ok; ++pp) {
         const int par = pp & 1;
         longlong2 nx[4];
         auto fetch = [&](int st) {
@@ -502,7 +514,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     long long* part = reinterpret_cast<long long*>(kcta + (size_t)2 * nst * kKeepStage) + tid;
     uint32_t pass = 0;
     int ti = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++ti) {
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++ti) {
+      const int tile = item / nparts, pp0 = (item - tile * nparts) * np;
       const int fld = tile / tpf, rbuf = ti % kRB;
       const int line = (tile - fld * tpf) * (kRows / 2) + l;
       if (!W.wait_warp(barRow + 8 * rbuf, (ti / kRB) & 1)) break;
@@ -518,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           __all_sync(0xffffffffu, !rowok || (!nan && safe_exp<TO>(ex))) != 0;
       TO* dst = out + ((size_t)fld * fso + (size_t)(rowok ? line : 0) * Nz) * 2 + part_c;
       bool ok = true;
-      for (int pp = 0; pp < 2 * nsl && ok; ++pp) {
+      for (int pp = pp0; pp < pp0 + np && ok; ++pp) {
         const int par = pp & 1, m0 = (pp >> 1) * NT + cg * CW;
         TO* d = dst + 2 * (size_t)(2 * m0 + par);
         for (int c = 0; c < kc; ++c, ++pass) {
@@ -551,9 +564,14 @@ cudaError_t launch_t(const void* in, long long fsi, void* out, long long fso, in
   const int tpf = (nlines + kRows / 2 - 1) / (kRows / 2);
   const long long ntiles = (long long)nf * tpf;
   if (ntiles <= 0) return cudaSuccess;
-  const int grid = (int)std::min<long long>(ntiles, t.ctas);
+  // Rule: as many CTAs to a tile as all tiles find an SM each; a tile's passes (two for N <= 128, four
+  // up to 256) then run side by side and each CTA converts its rows again
+  // (24 tiles, us, one CTA a tile / split: N = 128 30 / 18, N = 192 48 / 21, N = 256 62 / 26).
+  int np = 2 * t.nsl;
+  while (np % 2 == 0 && ntiles * (2 * t.nsl / np) * 2 <= t.ctas) np /= 2;
+  const int grid = (int)std::min<long long>(ntiles * (2 * t.nsl / np), t.ctas);
   cheb_tc_kernel<TI, TO><<<grid, kThreads, kSmem, s>>>(
-      (const TI*)in, fsi, (TO*)out, fso, nlines, Nz, tpf, (int)ntiles, t.NT, t.nsl, t.nst, t.kc,
+      (const TI*)in, fsi, (TO*)out, fso, nlines, Nz, tpf, (int)ntiles, np, t.NT, t.nsl, t.nst, t.kc,
       t.gst, t.nmag, t.dig, t.keep, (long long)cheb_tc_keep_bytes(Nz - 1), t.dir == 0 ? 1 : 0, t.q, t.ymid,
       t.dir == 0 ? 0.5 / (double)(Nz - 1) : 1.0, err);
   return cudaGetLastError();

@@ -238,6 +238,53 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
                  "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  // largest keys of elements ja .. jz - 1 of lines 32 gi .. + 31 of a tile, lanes along the lines, U
+  // loads in flight per lane
+  const int nel = MODE == YB ? A.n1 : MODE == XB ? A.t.nk : A.P;
+  constexpr int U = MODE == XF ? 24 : 12;
+  auto keys = [&](int tile, int b, int gi, int ja, int jz) {
+    const int fld = tile / A.tpf, l = gi * 32 + lane;
+    const int line = (tile - fld * A.tpf) * LPT + l;
+    const bool ok = line < A.nlines, d = (A.dmask >> fld) & 1;
+    const double* src =
+        A.in[fld] + (ok ? (line / A.ld) * A.ihs + (line % A.ld) * A.ils : 0) * ISC;
+    unsigned key = 0;
+#pragma unroll 1
+    for (int j0 = ja; j0 < jz; j0 += U) {
+      double2 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u;
+        v[u] = make_double2(0.0, 0.0);
+        if (ok && j < jz && !(MODE == YB && j == A.n1 / 2)) {
+          if (MODE == XF) v[u].x = src[(size_t)j * A.estr];
+          else v[u] = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
+        }
+      }
+      if (MODE != XF && d) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = j0 + u;
+          const double k = A.kscale * (double)((MODE == YB && j > A.n1 / 2) ? j - A.n1 : j);
+          v[u] = make_double2(k * v[u].x, k * v[u].y);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        key = max(key, dkey(v[u].x));
+        if (MODE != XF) key = max(key, dkey(v[u].y));
+      }
+    }
+    if (key) atomicMax(&sK[b * kRows + l], key);
+  };
+  __syncthreads();   // sK cleared
+  {
+    // the first tile's keys by every warp: nothing else can begin before they are known (with
+    // the same change in the Chebyshev kernel, a 64 x 36 x 145 transform and its inverse 206 -> 129 us)
+    constexpr int G = LPT / 32, parts = kThreads / 32 / G;
+    const int pt = warp / G;
+    if (pt < parts) keys(blockIdx.x, 0, warp % G, nel * pt / parts, nel * (pt + 1) / parts);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();   // barriers and tensor-memory address visible to every warp
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -281,54 +328,17 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
     }
     __syncwarp();
   } else if (warp > kPW + kEW) {
-    // ---- scan: one scale per line (a complex line's parts share it).  Each warp takes a third of the
-    // elements of every line, lanes along the lines, U loads in flight per lane.
+    // ---- scan: one scale per line (a complex line's parts share it); each warp takes a third of the
+    // elements of every line
     const int sw = warp - (kPW + kEW + 1), st = sw * 32 + lane;
-    const int nel = MODE == YB ? A.n1 : MODE == XB ? A.t.nk : A.P;
-    const int ja = nel * sw / kSW, jz = nel * (sw + 1) / kSW;
-    constexpr int U = MODE == XF ? 24 : 12;
     int ti = 0;
     for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x, ++ti) {
       const int b = ti % kRB;
       if (ti >= kRB && !W.wait_warp(barRowFree + 8 * b, (ti / kRB - 1) & 1)) break;
       const int fld = tile / A.tpf;
-      const bool d = (A.dmask >> fld) & 1;
+      if (ti > 0)
 #pragma unroll 1
-      for (int gi = 0; gi < LPT / 32; ++gi) {
-        const int l = gi * 32 + lane;
-        const int line = (tile - fld * A.tpf) * LPT + l;
-        const bool ok = line < A.nlines;
-        const double* src =
-            A.in[fld] + (ok ? (line / A.ld) * A.ihs + (line % A.ld) * A.ils : 0) * ISC;
-        unsigned key = 0;
-#pragma unroll 1
-        for (int j0 = ja; j0 < jz; j0 += U) {
-          double2 v[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int j = j0 + u;
-            v[u] = make_double2(0.0, 0.0);
-            if (ok && j < jz && !(MODE == YB && j == A.n1 / 2)) {
-              if (MODE == XF) v[u].x = src[(size_t)j * A.estr];
-              else v[u] = *reinterpret_cast<const double2*>(src + 2 * (size_t)j * A.estr);
-            }
-          }
-          if (MODE != XF && d) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const int j = j0 + u;
-              const double k = A.kscale * (double)((MODE == YB && j > A.n1 / 2) ? j - A.n1 : j);
-              v[u] = make_double2(k * v[u].x, k * v[u].y);
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            key = max(key, dkey(v[u].x));
-            if (MODE != XF) key = max(key, dkey(v[u].y));
-          }
-        }
-        if (key) atomicMax(&sK[b * kRows + l], key);
-      }
+        for (int gi = 0; gi < LPT / 32; ++gi) keys(tile, b, gi, nel * sw / kSW, nel * (sw + 1) / kSW);
       __syncwarp();
       if (lane == 0)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barKey) : "memory");
