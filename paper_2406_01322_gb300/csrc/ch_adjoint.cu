@@ -181,7 +181,7 @@ int adjoint_step_impl(ch_grid* G, const void* state, cudaEvent_t* ev) {
   G->nl_stale = 1;
   if (ev) cudaEventRecord(ev[0], s);
   // forward fields of s_n on the y-padded grid (the x line's linearisation point)
-  cudaError_t e0 = chf::launch_zbwd(0, 0, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s);
+  cudaError_t e0 = ch_launch_fields(G, s);
   if (ev) cudaEventRecord(ev[1], s);
   cudaError_t e1 = ch_launch_xy(G, 3, s);
   if (ev) cudaEventRecord(ev[2], s);

@@ -186,15 +186,8 @@ thread_local cudaError_t t_last_cuda = cudaSuccess;
 // the nine products of the current state on the y-padded grid: bw <- 5 fields; ya <- y
 // backward; yb <- x line
 int eval_products(ch_grid* G) {
-  const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  if (G->cheb == CH_CHEB_TC) {   // as the step itself forms the fields
-    CK(chf::launch_fields_coef(g, G->om, G->w, G->phi, G->cf, G->fs, G->pz, s));
-    CK(chf::launch_cheb_tc(0, G->prec, G->cf, G->fs, G->bw, G->fs, kBw, g.Mx * g.ny, g.nz, G->tcb,
-                           G->tc_err, s));
-  } else {
-    CK(chf::launch_zbwd(0, G->prec, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s));
-  }
+  CK(ch_launch_fields(G, s));
   CK(ch_launch_xy(G, 3, s));
   CK(ch_launch_xy(G, 4, s));
   return CH_OK;
@@ -210,12 +203,12 @@ int eval_nonlinear_impl(ch_grid* G) {
 }
 
 // The step's launch schedule (the only copy).  Launch positions: 0 Chebyshev forward transform
-// on the tensor cores (CH_CHEB_TC only), 1 zrhs, 2 zsolve, 3 zbwd, 4 Chebyshev backward
-// transform (CH_CHEB_TC only), 5 y backward, 6 x line, 7 y forward.  ev, when given, holds
+// on the tensor cores (ch_z_coef only), 1 zrhs, 2 zsolve, 3 zbwd, 4 Chebyshev backward
+// transform (ch_z_coef only), 5 y backward, 6 x line, 7 y forward.  ev, when given, holds
 // CH_STEP_KERNELS events: ev[p] is recorded after position p (right away for an empty position).
 int launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev = nullptr) {
   const GridDev& g = G->g;
-  const bool tc = G->cheb == CH_CHEB_TC;
+  const bool tc = ch_z_coef(G);
   const int nlines = g.Mx * g.ny;
   cudaError_t e[CH_STEP_KERNELS];
   for (int k = 0; k < CH_STEP_KERNELS; ++k) e[k] = cudaSuccess;
@@ -374,6 +367,7 @@ int make_txy_plan(ch_grid* G, int mode, int P, double scale, chf::TxyPlan* p) {
 // up to transform lengths of 1024 (the dense matrices grow with the length squared).
 constexpr int kTxyMaxP = 1024;
 constexpr long long kTxyMinModes = 1ll << 15;
+constexpr long long kCoefMinModes = 1ll << 18;
 int setup_tx(ch_grid* G) {
   const GridDev& g = G->g;
   if (g.nx > kTxyMaxP || g.ny > kTxyMaxP || G->fs < kTxyMinModes) return CH_OK;
@@ -452,6 +446,16 @@ void drop_graph(ch_grid* G) {
 }
 
 }  // namespace
+
+cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s) {
+  const GridDev& g = G->g;
+  if (!ch_z_coef(G))
+    return chf::launch_zbwd(0, G->prec, kBw, g, G->R, G->om, G->w, G->phi, G->bw, G->fs, G->pz, s);
+  const cudaError_t e = chf::launch_fields_coef(g, G->om, G->w, G->phi, G->cf, G->fs, G->pz, s);
+  if (e != cudaSuccess) return e;
+  return chf::launch_cheb_tc(0, G->prec, G->cf, G->fs, G->bw, G->fs, kBw, g.Mx * g.ny, g.nz, G->tcb,
+                             G->tc_err, s);
+}
 
 cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s) {
   const GridDev& g = G->g;
@@ -619,7 +623,7 @@ int ch_init_grid(const ch_params* p, ch_alloc_fn alloc, ch_free_fn free_fn, void
   G->bw = A((size_t)kBw * G->fs * esz);
   G->ya = A((size_t)kYa * G->fsy * esz);
   G->yb = A((size_t)kNl * G->fsy * esz);
-  G->auxA = (double2*)A((size_t)7 * sb);
+  G->auxA = G->cf = (double2*)A((size_t)7 * sb);   // kNc = 7 fields
   G->auxB = (double2*)A((size_t)7 * sb);
   G->phys7 = (double*)A((size_t)7 * G->fsp * sizeof(double));
   G->tab = (double*)A((size_t)6 * nz * sizeof(double));
@@ -714,6 +718,15 @@ int ch_init_grid(const ch_params* p, ch_alloc_fn alloc, ch_free_fn free_fn, void
     return bail(G, CH_ERR_SIZE);
   }
   st = setup_tx(G);
+  // Rule for the step's z transforms while no method is selected: on the tensor cores from 2^18
+  // modes on.  The whole step by FFT / on the tensor cores, us: 48 x 48 x 193 (2^17.8 modes)
+  // 1043 / 895 float64, 920 / 734 mixed; 96 x 96 x 65 (2^18.2) 1112 / 859, 931 / 651; 192 x 128 x
+  // 163 6884 / 4751, 5248 / 2870.  Below, with a tenth to a quarter to gain, a step keeps its six
+  // or nine launches.
+  if (st == CH_OK && G->use_ax && G->fs >= kCoefMinModes) {
+    if (chf::zline_coef_prepare(G->g) == cudaSuccess) G->z_auto = 1;
+    else cudaGetLastError();
+  }
   if (st != CH_OK) return bail(G, st);
   G->first = 1;
   G->fields_set = 0;
@@ -818,7 +831,7 @@ int ch_step(ch_grid* G, int nsteps) {
 int ch_launches_per_step(const ch_grid* G) {
   if (!G) return 0;
   // the tensor-core x line is three launches (backward, products, forward), the forward y pass two
-  return (G->cheb == CH_CHEB_TC ? 8 : 6) + (G->use_tx ? 3 : 0);
+  return (ch_z_coef(G) ? 8 : 6) + (G->use_tx ? 3 : 0);
 }
 
 int ch_step_timed(ch_grid* G, int nsteps, double* kernel_ms, double* total_ms) {
@@ -1049,17 +1062,13 @@ int ch_set_chebyshev(ch_grid* G, int method) {
   if (!G || (method != CH_CHEB_FFT && method != CH_CHEB_TC)) return CH_ERR_ARG;
   if (G->adj_block) return CH_ERR_STATE;   // not while a reverse sweep is open
   if (method == CH_CHEB_TC) {
-    if (!G->cf) {
-      const int r = ensure_cheb(G);
-      if (r != CH_OK) return r;
-      CK(chf::zline_coef_prepare(G->g));
-      double2* cf = (double2*)galloc(G, (size_t)chf::kNc * G->fs * sizeof(double2));
-      if (!cf) return CH_ERR_ALLOC;
-      G->cf = cf;
-    }
+    const int r = ensure_cheb(G);
+    if (r != CH_OK) return r;
+    CK(chf::zline_coef_prepare(G->g));
   }
   drop_graph(G);
   G->cheb = method;
+  G->z_auto = 0;
   return CH_OK;
 }
 
@@ -1090,7 +1099,7 @@ int ch_get_fft_pruning(const ch_grid* G) { return G ? G->px[0].prune : CH_ERR_AR
 int ch_chebyshev_lines(ch_grid* G, int dir, const double* in, double* out, int nf) {
   if (!G || !in || !out || nf < 1 || (dir != 0 && dir != 1)) return CH_ERR_ARG;
   const GridDev& g = G->g;
-  if (G->cheb == CH_CHEB_TC) {
+  if (ch_z_coef(G)) {
     CK(chf::launch_cheb_tc(0, 0, in, G->fs, out, G->fs, nf, g.Mx * g.ny, g.nz,
                            dir == 0 ? G->tcf : G->tcb, G->tc_err, G->stream));
   } else {

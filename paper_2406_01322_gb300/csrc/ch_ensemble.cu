@@ -94,6 +94,10 @@ using chf::Member;
 namespace {
 
 constexpr int kStages = CH_ENSEMBLE_STAGES;
+// work lists: the six stages, then zrhs and zbwd of the members whose z transforms run on the tensor
+// cores (ch_z_coef; the others are in lists 0 and 2, so that every member steps as it would alone)
+constexpr int kLists = kStages + 2;
+int stage_of(int list) { return list < kStages ? list : list == kStages ? 0 : 2; }
 
 struct Tuning {
   int style[3] = {0, 0, 0};        // radix style of x, y, z transforms
@@ -110,6 +114,8 @@ struct ch_ensemble {
   std::vector<ch_grid*> members;
   int prec;
   int cheb;                     // Chebyshev method of the grouped step (CH_CHEB_FFT / CH_CHEB_TC)
+  int z_auto;                   // no method selected yet: each member's own
+  std::vector<char> zc;         // members in the coefficient lists
   int nsm;
   cudaStream_t stream;
   cudaStream_t cap;
@@ -118,11 +124,11 @@ struct ch_ensemble {
   void* actx;
   std::vector<void*> allocs;
   Member* dmem;                 // device descriptors
-  int* dbegin;                  // device work lists, kStages x (n + 1)
+  int* dbegin;                  // device work lists, kLists x (n + 1)
   std::vector<Member> hmem;
   std::vector<int> hbegin;
-  size_t smem[kStages];
-  int occ[kStages];
+  size_t smem[kLists];
+  int occ[kLists];
   int zsolve_tile;
   int ywq;                      // warp-FFT level of the grouped y passes (ensemble_ywq)
   int xwq;                      // the same for the grouped x line (padded x lengths)
@@ -221,16 +227,19 @@ int build_descriptors(ch_ensemble* E) {
     M.yscale = 1.0 / ((double)G->g.Px * (double)G->g.Py);
     M.kxs = 6.283185307179586476925 / G->g.lx;
   }
-  E->hbegin.assign((size_t)kStages * (n + 1), 0);
-  for (int s = 0; s < kStages; ++s) {
+  E->hbegin.assign((size_t)kLists * (n + 1), 0);
+  for (int l = 0; l < kLists; ++l) {
+    const int s = stage_of(l), coef = l >= kStages;
     size_t mx = 0;
-    int* b = &E->hbegin[(size_t)s * (n + 1)];
+    int* b = &E->hbegin[(size_t)l * (n + 1)];
     for (int i = 0; i < n; ++i) {
-      b[i + 1] = b[i] + chf::stage_items(s, E->hmem[i], E->prec);
-      const size_t sm = chf::stage_smem(s, E->hmem[i], E->prec, E->cheb == CH_CHEB_TC);
+      b[i + 1] = b[i];
+      if ((s == 0 || s == 2) && (int)E->zc[i] != coef) continue;
+      b[i + 1] += chf::stage_items(s, E->hmem[i], E->prec);
+      const size_t sm = chf::stage_smem(s, E->hmem[i], E->prec, coef);
       if (sm > mx) mx = sm;
     }
-    E->smem[s] = mx;
+    E->smem[l] = mx;
     if (mx > (size_t)chf::kMaxSmem) return CH_ERR_SIZE;
   }
   return CH_OK;
@@ -248,23 +257,29 @@ int upload(ch_ensemble* E) {
   return CH_OK;
 }
 
-int grid_of(ch_ensemble* E, int s) {
-  const int n = (int)E->members.size();
-  const int total = E->hbegin[(size_t)s * (n + 1) + n];
-  int per = E->tune.ctas_per_sm[s];
-  if (per <= 0 || per > E->occ[s]) per = E->occ[s];
+int list_items(const ch_ensemble* E, int l) {
+  const size_t n = E->members.size();
+  return E->hbegin[(size_t)l * (n + 1) + n];
+}
+
+int grid_of(ch_ensemble* E, int l) {
+  const int total = list_items(E, l);
+  int per = E->tune.ctas_per_sm[stage_of(l)];
+  if (per <= 0 || per > E->occ[l]) per = E->occ[l];
   if (per <= 0) per = 1;
   long long g = (long long)per * E->nsm;
   if (g > total) g = total;
   return g < 1 ? 1 : (int)g;
 }
 
-// tensor-core Chebyshev method: one transform launch per member around the grouped z stages,
+// one Chebyshev transform launch per member of the coefficient lists around the grouped z stages,
 // dir 0 (before zrhs) the nine products' samples -> coefficients, dir 1 (after zbwd) the five
 // backward fields' coefficients -> samples.  Each launch is a persistent grid over that member's
 // tiles of rows.
 cudaError_t member_transforms(ch_ensemble* E, int dir, cudaStream_t s) {
-  for (ch_grid* G : E->members) {
+  for (size_t i = 0; i < E->members.size(); ++i) {
+    ch_grid* G = E->members[i];
+    if (!E->zc[i]) continue;
     const int nlines = G->g.Mx * G->g.ny;
     const cudaError_t e =
         dir == 0 ? chf::launch_cheb_tc(E->prec, 0, G->nl, G->fs, G->cf, G->fs, chf::kNc, nlines,
@@ -276,22 +291,24 @@ cudaError_t member_transforms(ch_ensemble* E, int dir, cudaStream_t s) {
   return cudaSuccess;
 }
 
-// one ensemble step: the six grouped stages; with the tensor-core method the member transforms
-// run before stage 0 and after stage 2 and are timed with those stages
+// one ensemble step: the six grouped stages, zrhs and zbwd in one launch per kind of member; the
+// members' transforms run before stage 0 and after stage 2 and are timed with those stages
 int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
   const int n = (int)E->members.size();
-  const int tc = E->cheb == CH_CHEB_TC;
   for (int st = 0; st < kStages; ++st) {
     cudaError_t e = cudaSuccess;
-    if (tc && st == 0) e = member_transforms(E, 0, s);
+    if (st == 0) e = member_transforms(E, 0, s);
     if (e == cudaSuccess && st >= 3 && E->tx) {
       for (ch_grid* G : E->members)
         if (e == cudaSuccess) e = ch_launch_xy(G, st, s);
-    } else if (e == cudaSuccess)
-      e = chf::launch_grouped(st, E->prec, E->dmem, E->dbegin + (size_t)st * (n + 1), n,
-                              grid_of(E, st), E->smem[st], E->zsolve_tile, tc,
-                              st == 4 ? E->xwq : E->ywq, s);
-    if (e == cudaSuccess && tc && st == 2) e = member_transforms(E, 1, s);
+    } else {
+      for (int l = 0; l < kLists && e == cudaSuccess; ++l)
+        if (stage_of(l) == st && list_items(E, l) > 0)
+          e = chf::launch_grouped(st, E->prec, E->dmem, E->dbegin + (size_t)l * (n + 1), n,
+                                  grid_of(E, l), E->smem[l], E->zsolve_tile, l >= kStages,
+                                  st == 4 ? E->xwq : E->ywq, s);
+    }
+    if (e == cudaSuccess && st == 2) e = member_transforms(E, 1, s);
     if (ev) cudaEventRecord(ev[st], s);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -309,9 +326,9 @@ void compute_occupancy(ch_ensemble* E) {
   }
   E->ywq = chf::ensemble_ywq(py, E->prec);
   E->xwq = chf::ensemble_ywq(px, E->prec);
-  for (int s = 0; s < kStages; ++s)
-    E->occ[s] = chf::stage_occupancy(s, E->prec, E->smem[s], E->zsolve_tile,
-                                     E->cheb == CH_CHEB_TC, s == 4 ? E->xwq : E->ywq);
+  for (int l = 0; l < kLists; ++l)
+    E->occ[l] = chf::stage_occupancy(stage_of(l), E->prec, E->smem[l], E->zsolve_tile, l >= kStages,
+                                     stage_of(l) == 4 ? E->xwq : E->ywq);
 }
 
 // tuning cache key: member sizes, precision and Chebyshev method
@@ -323,7 +340,7 @@ std::string signature_of(const ch_ensemble* E) {
     snprintf(b, sizeof(b), "%dx%dx%d:%d/", G->g.nx, G->g.ny, G->g.nz, G->g.bc);
     sig += b;
   }
-  snprintf(b, sizeof(b), "p%d/c%d", E->prec, E->cheb);
+  snprintf(b, sizeof(b), "p%d/c%d", E->prec, E->z_auto ? 2 : E->cheb);
   return sig + b;
 }
 
@@ -396,6 +413,7 @@ int ch_ensemble_init(const ch_params* members, int n, ch_alloc_fn alloc, ch_free
   if (!E) return CH_ERR_ALLOC;
   E->prec = members[0].precision;
   E->cheb = CH_CHEB_FFT;
+  E->z_auto = 1;
   E->stream = (cudaStream_t)stream;
   E->af = alloc;
   E->ff = free_fn;
@@ -417,10 +435,13 @@ int ch_ensemble_init(const ch_params* members, int n, ch_alloc_fn alloc, ch_free
   }
   if (st == CH_OK) E->signature = signature_of(E);
   E->tx = 0;
-  for (ch_grid* G : E->members) E->tx |= G->use_tx;
+  for (ch_grid* G : E->members) {
+    E->tx |= G->use_tx;
+    E->zc.push_back((char)ch_z_coef(G));
+  }
   if (st == CH_OK) {
     E->dmem = (Member*)ealloc(E, n * sizeof(Member));
-    E->dbegin = (int*)ealloc(E, (size_t)kStages * (n + 1) * sizeof(int));
+    E->dbegin = (int*)ealloc(E, (size_t)kLists * (n + 1) * sizeof(int));
     if (!E->dmem || !E->dbegin) st = CH_ERR_ALLOC;
   }
   if (st == CH_OK) {
@@ -455,14 +476,17 @@ int ch_ensemble_member(ch_ensemble* E, int i, ch_grid** out) {
 
 int ch_ensemble_set_chebyshev(ch_ensemble* E, int method) {
   if (!E || (method != CH_CHEB_FFT && method != CH_CHEB_TC)) return CH_ERR_ARG;
-  if (method == E->cheb) return CH_OK;
+  if (method == E->cheb && !E->z_auto) return CH_OK;
   // every member takes the method (its tables and coefficient buffer stay allocated for the
   // member's lifetime once made, so a later change of a member's own method leaves the
   // ensemble's step intact)
   for (size_t i = 0; i < E->members.size(); ++i) {
     const int st = ch_set_chebyshev(E->members[i], method);
     if (st != CH_OK) {
-      for (size_t j = 0; j < i; ++j) ch_set_chebyshev(E->members[j], E->cheb);
+      for (size_t j = 0; j < i; ++j) {
+        ch_set_chebyshev(E->members[j], E->cheb);
+        E->members[j]->z_auto = E->z_auto && E->zc[j];
+      }
       return st;
     }
   }
@@ -471,6 +495,8 @@ int ch_ensemble_set_chebyshev(ch_ensemble* E, int method) {
     return CH_ERR_CUDA;
   }
   E->cheb = method;
+  E->z_auto = 0;
+  E->zc.assign(E->members.size(), (char)(method == CH_CHEB_TC));
   E->signature = signature_of(E);
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
@@ -618,8 +644,9 @@ int ch_ensemble_tuning(const ch_ensemble* E, char* buf, size_t n) {
            "\"zsolve_tile\": %d, \"chebyshev\": %d}",
            E->tune.tuned, E->tune.style[0], E->tune.style[1], E->tune.style[2],
            E->tune.ctas_per_sm[0], E->tune.ctas_per_sm[1], E->tune.ctas_per_sm[2],
-           E->tune.ctas_per_sm[3], E->tune.ctas_per_sm[4], E->tune.ctas_per_sm[5], E->occ[0],
-           E->occ[1], E->occ[2], E->occ[3], E->occ[4], E->occ[5], E->zsolve_tile, E->cheb);
+           E->tune.ctas_per_sm[3], E->tune.ctas_per_sm[4], E->tune.ctas_per_sm[5],
+           E->occ[list_items(E, 0) ? 0 : kStages], E->occ[1],
+           E->occ[list_items(E, 2) ? 2 : kStages + 1], E->occ[3], E->occ[4], E->occ[5], E->zsolve_tile, E->cheb);
   return CH_OK;
 }
 

@@ -90,9 +90,9 @@ struct ch_grid {
   int nl_stale = 0;  // 1: the state was replaced by a reverse step; products not recomputed
 
   // Chebyshev transform of the step: CH_CHEB_FFT (inside zrhs / zbwd) or CH_CHEB_TC (tensor
-  // cores, two extra launches); the tables, the coefficient buffer (9 fields) and the error flag
-  // of the bounded device waits exist once CH_CHEB_TC was selected
-  int cheb = 0;
+  // cores, two extra launches); z_auto: the tensor cores although no method was selected.  cf: the
+  // coefficients between the transforms and zrhs / zbwd (auxA)
+  int cheb = 0, z_auto = 0;
   chf::ChebTc tcf, tcb;
   double2* cf = nullptr;
   int* tc_err = nullptr;
@@ -106,9 +106,13 @@ struct ch_grid {
   chf::TxyPlan tx_yf1, tx_xb1;
 };
 
+// the step's z kernels work on Chebyshev coefficients, transformed on the tensor cores
+inline bool ch_z_coef(const ch_grid* G) { return G->cheb == CH_CHEB_TC || G->z_auto; }
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev);
 int ch_eval_nonlinear(ch_grid* G);
+// bw <- the five backward fields u v w phi D phi of the state, as the step itself forms them
+cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s);
 // the x/y stages of the step on stream s: 3 y backward (bw -> ya), 4 x line (ya -> yb), 5 y
 // forward with the combinations (yb -> nl)
 cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s);
