@@ -84,6 +84,39 @@ bool make_radices_style(int n, int style, FftPlan* pl) {
   return true;
 }
 
+// cos and sin of 2 pi t / n, t < n.  Angles that are images of one another (t, n - t, n / 2 - t, n / 4 -
+// t, ...) share one evaluation: extended precision is software on some hosts, about a microsecond a
+// call, and a grid's plans need thousands of values.
+void circle(int n, std::vector<long double>& c, std::vector<long double>& s) {
+  c.assign(n, 0.0L);
+  s.assign(n, 0.0L);
+  std::vector<char> done(n, 0);
+  const long double pi2 = 6.283185307179586476925286766559005768L;
+  auto set = [&](int t, long double x, long double y) {
+    t = (t % n + n) % n;
+    if (done[t]) return;
+    done[t] = 1;
+    c[t] = x;
+    s[t] = y;
+  };
+  for (int t = 0; t < n; ++t) {
+    if (done[t]) continue;
+    const long double a = pi2 * (long double)t / (long double)n, x = cosl(a), y = sinl(a);
+    set(t, x, y);
+    set(-t, x, -y);
+    if (n % 2 == 0) {
+      set(n / 2 - t, -x, y);
+      set(n / 2 + t, -x, -y);
+    }
+    if (n % 4 == 0) {
+      set(n / 4 - t, y, x);
+      set(n / 4 + t, -y, x);
+      set(3 * (n / 4) - t, -y, -x);
+      set(3 * (n / 4) + t, y, -x);
+    }
+  }
+}
+
 // size rules of ch_params (see include/ch_flow.h): CH_OK or CH_ERR_SIZE
 int check_sizes(int nx, int ny, int nz) {
   if (nx < 4 || ny < 4 || nz < 5 || nx % 2 || ny % 2) return CH_ERR_SIZE;
@@ -128,10 +161,10 @@ int make_plan(ch_grid* G, int n, int prec, FftPlan* pl, int style = 0) {
   std::vector<double2> h64(n);
   std::vector<float2> h32(n);
   std::vector<float> hdf(4 * (size_t)n);  // double-float pairs (h, l) of re and im
-  const long double pi2 = 6.283185307179586476925286766559L;
+  std::vector<long double> cs, sn;
+  chf::circle(n, cs, sn);
   for (int t = 0; t < n; ++t) {
-    const long double a = pi2 * (long double)t / (long double)n;
-    const long double c = cosl(a), s = -sinl(a);
+    const long double c = cs[t], s = -sn[t];
     h64[t] = make_double2((double)c, (double)s);
     h32[t] = make_float2((float)c, (float)s);
     const float ch = (float)c, sh = (float)s;

@@ -326,6 +326,8 @@ struct Txy {
   int ctas = 0;
   int* err = nullptr;              // |= 1 if a bounded wait gave up
 };
+// cos and sin of 2 pi t / n, t < n
+void circle(int n, std::vector<long double>& c, std::vector<long double>& s);
 // mode 0 y backward, 1 y forward (times scale), 2 x backward (scale: the weight of the modes k >= 1,
 // 2 for a half spectrum, 1 for the transpose of the forward transform), 3 x forward; n1 = Ny (y) or Mx (x), P
 // the transform length

@@ -773,16 +773,15 @@ int txy_plan(int mode, int n1, int P, double scale, std::vector<uint16_t>& dig, 
   const double nterm = mode == YB ? 2.0 * n1 : mode == XB ? 2.0 * n1 : mode == YF ? 2.0 * P : P;
   t->q = (int)floor(std::min(54.0 - log2(wmax), 62.0 - log2(nterm * wmax)));
   t->ymid = mode == YF ? (long long)llround(ldexp(scale, t->q)) : mode == XF ? 1ll << t->q : 0;
-  const long double pi2 = 6.283185307179586476925286766559005768L;
   // the weights times 2^q by angle 2 pi a / P, of cosine and sine, and at k = 0 (cosine 1, sine 0)
+  std::vector<long double> cs, sn;
+  circle(P, cs, sn);
   std::vector<long long> Y[2] = {std::vector<long long>(P), std::vector<long long>(P)};
   const long double w = mode == YF || mode == XB ? (long double)scale : 1.0L;
   const long double ws = mode == XB || mode == XF ? -w : w;
   for (int a = 0; a < P; ++a) {
-    const long double c = cosl(pi2 * (long double)a / (long double)P);
-    const long double sn = sinl(pi2 * (long double)a / (long double)P);
-    Y[0][a] = (long long)llroundl(ldexpl(w * c, t->q));
-    Y[1][a] = (long long)llroundl(ldexpl(ws * sn, t->q));
+    Y[0][a] = (long long)llroundl(ldexpl(w * cs[a], t->q));
+    Y[1][a] = (long long)llroundl(ldexpl(ws * sn[a], t->q));
   }
   const long long Y0 = mode == XB ? 1ll << t->q : Y[0][0];
   // their digits as bf16, and the sum of the digits' magnitudes; entry P: k = 0
