@@ -24,7 +24,7 @@
 //   scan (3 warps): the rows' scales of the next tile (the rows' first, cold read, after an L2
 //     prefetch of the tile one further ahead) and the middle elements' terms;
 //   producers (8 warps): per K stage of 16 (one MMA k-step) a thread converts four pairs
-//     (x_k, x_{N-k}) of the real and imaginary rows of one line to fixed point, writes the seven
+//     (x_k, x_{N-k}) of the real and imaginary rows of one line to fixed point, writes the eight
 //     digit planes of the sums to the stage's shared buffer and keeps the differences (and, with
 //     several slices, the sums) in a per-CTA buffer in global memory (L2), read back by the same
 //     thread for the later passes; thread 0 also issues the bulk copy of the stage's matrix digits;
@@ -50,7 +50,7 @@ using namespace tc;
 
 constexpr int kPW = 8, kEW = 8, kSW = 3;          // producer, epilogue and scan warps
 constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
-constexpr int kStages = 5;                        // K stages in flight
+constexpr int kStages = 4;                        // K stages in flight
 constexpr int kRB = 3;                            // tiles whose row scales are held
 constexpr int kStageBytes = kABytes + b_stage_bytes(kNTMax);
 // per stage full, bfull, empty; accfull, accfree, rowfull[kRB], rowfree[kRB], fin
@@ -85,7 +85,7 @@ __device__ __forceinline__ CBits<df> ld_cplx(const df* p) {
 }
 
 // One pass's outputs of one thread: columns m0 .. m0 + CW - 1 of its row, four at a time, from the
-// seven accumulators at tensor-memory address tb; dst: output column m0 (columns 4 scalars apart).
+// eight accumulators at tensor-memory address tb; dst: output column m0 (columns 4 scalars apart).
 // Arguments as in the kernel.
 template <typename TO, int NMAG>
 __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m0, int H, int c,
@@ -93,8 +93,8 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
                                               int ex, long long mid, bool halve0, long long* part,
                                               TO* dst, uint32_t barAccFree, int lane) {
   for (int c0 = 0; c0 < CW; c0 += 4) {
-    uint32_t v[7][4];
-    tmem_ldx4<7>(tb + (uint32_t)c0, NT, v);
+    uint32_t v[kDiags][4];
+    tmem_ldx4(tb + (uint32_t)c0, NT, v);
     if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -103,7 +103,7 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
     }
     long long T[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG, 7>(v, e);
+    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG>(v, e);
     if (kc > 1) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -138,7 +138,7 @@ __device__ __forceinline__ void epilogue_pass(uint32_t tb, int NT, int CW, int m
 // in / out: nf fields of complex lines (re, im interleaved), field stride fsi / fso complex
 // elements, line stride Nz = N + 1; dig: the matrix digits, stage blocks of 7 NT rows x 16 K in
 // the order slice, parity, stage; keep: keep_bytes per CTA; nst stages per parity in kc groups of
-// gst; nmag: accumulators known to stay within 2^22 (7, 3 or 0); q: log2 of the matrix scale;
+// gst; nmag: accumulators known to stay within 2^22 (8, 3 or 0); q: log2 of the matrix scale;
 // ymid: middle weight times 2^q; lastf: factor of output N (forward).  The 2 nsl passes of a tile are
 // cut into items of np passes; several items a tile only where all items have a CTA each (launch_t).
 template <typename TI, typename TO>
@@ -223,9 +223,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int ro = b * kRows + tile_row(l, 0);
       sE[ro] = er;
       sE[ro + 8] = ei;
-      // x_H Y_H / 2^54 (|x_H| < 2^54, Y_H <= 2^54)
-      sC[ro] = __mul64hi(xr * 256, ymid * 4);
-      sC[ro + 8] = __mul64hi(xi * 256, ymid * 4);
+      // X_H Y_H / 2^62 (|X_H| < 2^62, Y_H <= 2^54)
+      sC[ro] = __mul64hi(xr, ymid * 4);
+      sC[ro + 8] = __mul64hi(xi, ymid * 4);
     }
   };
   // the first tile by every warp (scanned by three, it kept the others waiting: a launch of one tile per
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 goto drain;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               const uint32_t sA = sBase + slot * (uint32_t)kStageBytes;
-              issue_stage<7>(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
+              issue_stage(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
               any = true;
               mma_commit(barEmpty + 8 * slot);
               if (++slot == kStages) {
@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       unsigned char* sA = stages + (size_t)slot * kStageBytes;
       if (p == 0) bulk_load(su32(sA) + (uint32_t)kABytes, bsrc, bbytes, barB + 8 * slot, pol);
 #pragma unroll
-      for (int i = 0; i < kPlanes; ++i) {
-        const int b = 6 - i, sh = b < 4 ? 0 : 32;
+      for (int i = 0; i < kAPlanes; ++i) {
+        const int b = 7 - i, sh = b < 4 ? 0 : 32;
         uint32_t w[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) w[e] = (uint32_t)(v[e] >> sh);
@@ -377,7 +377,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool tiny = __any_sync(0xffffffffu, min(ere, eim) < kTinyScale) != 0;
       // first pass: convert, fold, write the sums' (odd passes: the differences') planes, keep what the
       // item's other passes need (all biased)
-      unsigned long long sumr = 0, sumi = 0, s0r = 0, s0i = 0;
+      WordSums sumr, sumi;
+      unsigned long long s0r = 0, s0i = 0;
       bool ok = true;
       for (int st = 0; st < nst && ok; ++st) {
         unsigned long long s[8], d[8];
@@ -386,29 +387,29 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int e = 0; e < 4; ++e) {
             const long long x = Fixed<TI, false>::of(xa[e].re, ere), y = Fixed<TI, false>::of(xb[e].re, ere);
             const long long z = Fixed<TI, false>::of(xa[e].im, eim), w = Fixed<TI, false>::of(xb[e].im, eim);
-            s[e] = x + y + kBias;
-            d[e] = x - y + kBias;
-            s[4 + e] = z + w + kBias;
-            d[4 + e] = z - w + kBias;
+            s[e] = x + y + kABias;
+            d[e] = x - y + kABias;
+            s[4 + e] = z + w + kABias;
+            d[4 + e] = z - w + kABias;
           }
         } else {
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const long long x = Fixed<TI, true>::of(xa[e].re, ere), y = Fixed<TI, true>::of(xb[e].re, ere);
             const long long z = Fixed<TI, true>::of(xa[e].im, eim), w = Fixed<TI, true>::of(xb[e].im, eim);
-            s[e] = x + y + kBias;
-            d[e] = x - y + kBias;
-            s[4 + e] = z + w + kBias;
-            d[4 + e] = z - w + kBias;
+            s[e] = x + y + kABias;
+            d[e] = x - y + kABias;
+            s[4 + e] = z + w + kABias;
+            d[4 + e] = z - w + kABias;
           }
         }
         if (st + 1 < nst) load(st + 1);
         if (np > 1) store_keep(keep_at(1, st), d);   // for np = 2 pp0 is even
         if (np > 2) store_keep(keep_at(0, st), s);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {   // at most 64 values below 2^56
-          sumr += s[e];
-          sumi += s[4 + e];
+        for (int e = 0; e < 4; ++e) {
+          sumr.add(s[e]);
+          sumi.add(s[4 + e]);
         }
         if (st == 0) {
           s0r = s[0];
@@ -419,17 +420,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       // the last output n = N: sum_k w_k (-1)^k x_k, (-1)^k = (-1)^g for this thread's k; weights
-      // e_k = 2 except k = 0, N (forward) or 1.  High and low parts (27 bits) are added apart.
+      // e_k = 2 except k = 0, N (forward) or 1.  High and low words are added apart.
       if (pp0 == 0) {
-        const unsigned long long nb = (unsigned long long)(4 * nst) * kBias;
-        long long tr = (long long)(sumr - nb), tm = (long long)(sumi - nb);
-        if (g & 1) {
-          tr = -tr;
-          tm = -tm;
-        }
-        const int f2 = fwd ? 2 : 1;
-        long long hr = f2 * (tr >> 27), lr = f2 * (tr & 0x7FFFFFF);
-        long long hm = f2 * (tm >> 27), lm = f2 * (tm & 0x7FFFFFF);
+        const int f2 = fwd ? 2 : 1, sf = g & 1 ? -f2 : f2;
+        long long hr = sf * sumr.high(4 * nst), lr = sf * sumr.low(4 * nst);
+        long long hm = sf * sumi.high(4 * nst), lm = sf * sumi.low(4 * nst);
         if (g == 0) {
           const int wm = (H & 1) ? -f2 : f2;
           long long xr = 0, xi = 0;
@@ -438,16 +433,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             xr = Fixed<TI, true>::of(x.re, ere);
             xi = Fixed<TI, true>::of(x.im, eim);
           }
-          hr += wm * (xr >> 27);
-          lr += wm * (xr & 0x7FFFFFF);
-          hm += wm * (xi >> 27);
-          lm += wm * (xi & 0x7FFFFFF);
+          hr += wm * (xr >> 32);
+          lr += wm * (long long)(unsigned)xr;
+          hm += wm * (xi >> 32);
+          lm += wm * (long long)(unsigned)xi;
           if (fwd) {   // s_0 was counted twice
-            const long long a = (long long)(s0r - kBias), c = (long long)(s0i - kBias);
-            hr -= a >> 27;
-            lr -= a & 0x7FFFFFF;
-            hm -= c >> 27;
-            lm -= c & 0x7FFFFFF;
+            const long long a = (long long)(s0r - kABias), c = (long long)(s0i - kABias);
+            hr -= a >> 32;
+            lr -= (long long)(unsigned)a;
+            hm -= c >> 32;
+            lm -= (long long)(unsigned)c;
           }
         }
 #pragma unroll
@@ -458,11 +453,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           lm += __shfl_xor_sync(0xffffffffu, lm, off);
         }
         if (g == 0 && rowok) {
-          // sum = 2^(E - 54) (h 2^27 + l) = T 2^(E - 51), T = h 2^24 + l / 8
           TO vr = ere == kNanRow ? qnan<TO>()
-                                 : scaled_any<TO>(hr * 16777216ll + ((lr + 4) >> 3), ere - F::EOFF - 51);
+                                 : scaled_any<TO>(words_to_t(hr, lr), ere - F::EOFF - 51);
           TO vi = eim == kNanRow ? qnan<TO>()
-                                 : scaled_any<TO>(hm * 16777216ll + ((lm + 4) >> 3), eim - F::EOFF - 51);
+                                 : scaled_any<TO>(words_to_t(hm, lm), eim - F::EOFF - 51);
           if (fwd) {
             vr = times<TO>(vr, lastf);
             vi = times<TO>(vi, lastf);
@@ -505,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ---- epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
-    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators
+    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the eight accumulators
     const int qd = warp & 3, cg = warp >> 2, CW = NT / 2;
     const int row = qd * 32 + lane;
     const int l = (row >> 4) * 8 + (row & 7), part_c = (row >> 3) & 1;
@@ -537,8 +531,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int c = 0; c < kc; ++c, ++pass) {
           if (!(ok = W.wait_warp(barAccFull, pass & 1))) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (nmag == 7)
-            epilogue_pass<TO, 7>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
+          if (nmag == 8)
+            epilogue_pass<TO, 8>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
                                  d, barAccFree, lane);
           else if (nmag == 3)
             epilogue_pass<TO, 3>(tb, NT, CW, m0, H, c, kc, par, rowok, nan, safe, ex, mid, fwd, part,
@@ -643,7 +637,7 @@ int cheb_tc_tables(int N, int dir, std::vector<uint16_t>& dig, ChebTc* t) {
       }
       bound = std::max(bound, acc);
     }
-  t->nmag = bound <= 4194304.0 ? 7 : (bound3 <= 4194304.0 ? 3 : 0);
+  t->nmag = bound <= 4194304.0 ? 8 : (bound3 <= 4194304.0 ? 3 : 0);
   return 0;
 }
 

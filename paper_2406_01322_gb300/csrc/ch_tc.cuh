@@ -2,22 +2,26 @@
 // bounded waits, float <-> fixed point, the digit planes, and the issue of one K stage's MMAs.
 //
 // A product of a float64 row x with a fixed matrix B is made exact up to the rounding of the two
-// operands: x becomes the integers X_k = round(x_k 2^(54-E)) (|x_k| < 0.98 2^E over the row), B
-// the integers Y_nk = round(B_nk 2^q), both written with seven signed base-256 digits,
-//   X_k = sum_{i=0..6} a_ik 256^(6-i),  a_ik in [-128, 127],
+// operands: x becomes the integers X_k = round(x_k 2^(62-E)) (|x_k| < 0.98 2^E over the row), B
+// the integers Y_nk = round(B_nk 2^q), |Y| <= 2^54, written with eight and seven signed base-256
+// digits,
+//   X_k = sum_{i=0..7} a_ik 256^(7-i),  a_ik in [-128, 127],
 // which bf16 holds exactly.  A digit product sum_k a_ik b_jnk is an integer, and the products with
 // the same i + j = d share one fp32 accumulator G_d: |G_d| <= 7 2^14 K < 2^24 for K <= 144, so
-// every accumulation is exact.  d <= 6 is kept (28 products; the dropped ones are random-signed,
-// about 2^-54 sqrt(K) of max|x| max|B| together), or d <= 7 (34 products, ND = 8 accumulators: the
-// dropped ones fall 2^8 below the quantisation of the operands), and
-//   sum_k X_k Y_nk = 256^6 U,  U = sum_{d<=6} 256^(6-d) G_d
-// is recombined in 64-bit integers.  Eight-bit digits need 28 products where seven-bit ones
-// (eight planes, K < 512) need 36; transforms with longer sums are cut into K groups of at most
-// 144 whose recombined integers are added.
+// every accumulation is exact.  d <= 7 is kept (35 products), and
+//   sum_k X_k Y_nk = 256^7 U,  U = sum_{d<=6} 256^(6-d) G_d + G_7 / 256
+// is recombined in 64-bit integers; transforms with longer sums are cut into K groups of at most 144
+// whose recombined integers are added.
+//
+// The error against exact sums (rows of decaying coefficients, transforms of 96 x 96 x 65 fields): the
+// eighth digit of X takes the rounding of the small elements of a row, 2^-55 of its largest in seven
+// digits, out of the result, and the eighth diagonal the dropped products, which with seven (28
+// products) are 2^-51 of max|x| max|B|.  With seven digits and 28 (z) and 34 (x, y) products a backward
+// transform was four times less accurate than by FFT (7.8e-16 against 1.9e-16 of the field).
 //
 // The seven B digit planes of an output slice are stacked into one 7 NT-row operand, so A plane i
-// needs one MMA chain over rows 0 .. (7-i) NT with its accumulator at column i NT: product (i, j)
-// lands on diagonal i + j.
+// needs one MMA chain over rows 0 .. (8-i) NT (at most 7 NT) with its accumulator at column i NT:
+// product (i, j) lands on diagonal i + j.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -30,15 +34,18 @@ namespace chf {
 namespace tc {
 
 constexpr int kRows = 128;        // rows per tile = tensor-memory lanes
-constexpr int kPlanes = 7;        // base-256 digits of an operand
+constexpr int kPlanes = 7;        // base-256 digits of a matrix element
+constexpr int kAPlanes = 8;       // and of a row's element
+constexpr int kDiags = 8;         // accumulators (diagonals of digit products)
 constexpr int kKS = 16;           // K per pipeline stage (one MMA k-step)
 constexpr int kMaxK = 144;        // K up to which the fp32 accumulators stay exact
-constexpr int kNTMax = 64;        // columns of an output slice (7 x 64 tensor-memory columns)
+constexpr int kNTMax = 64;        // columns of an output slice (8 x 64 tensor-memory columns)
 constexpr int kPlaneBytes = kRows * kKS * 2;             // one A digit plane of a stage
-constexpr int kABytes = kPlanes * kPlaneBytes;           // the A planes of a stage
+constexpr int kABytes = kAPlanes * kPlaneBytes;           // the A planes of a stage
 constexpr uint32_t kALbo = kRows * 16;                   // A: bytes between 8-element K groups
 __host__ __device__ constexpr int b_stage_bytes(int NT) { return kPlanes * NT * kKS * 2; }
 constexpr unsigned long long kBias = 0x0080808080808080ull;   // 128 sum_{t<7} 256^t
+constexpr unsigned long long kABias = 0x8080808080808080ull;  // 128 sum_{t<8} 256^t
 constexpr uint64_t kWaitNs = 1000000000ull;                   // bound of every device wait
 
 // ---- PTX wrappers -----------------------------------------------------------------------------
@@ -131,12 +138,11 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       "l"(src), "r"(bytes), "r"(bar), "l"(pol)
       : "memory");
 }
-// ND 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32 lanes,
+// 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32 lanes,
 // then one wait that the values depend on
-template <int ND>
-__device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&v)[ND][4]) {
+__device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&v)[kDiags][4]) {
 #pragma unroll
-  for (int d = 0; d < ND; ++d)
+  for (int d = 0; d < kDiags; ++d)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v[d][0]), "=r"(v[d][1]), "=r"(v[d][2]), "=r"(v[d][3])
                  : "r"(addr + (uint32_t)(d * stride)));
@@ -146,8 +152,8 @@ __device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&
                  "+r"(v[2][2]), "+r"(v[2][3]), "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]),
                  "+r"(v[3][3]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[4][2]), "+r"(v[4][3]),
                  "+r"(v[5][0]), "+r"(v[5][1]), "+r"(v[5][2]), "+r"(v[5][3]), "+r"(v[6][0]),
-                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3]), "+r"(v[ND - 1][0]),
-                 "+r"(v[ND - 1][1]), "+r"(v[ND - 1][2]), "+r"(v[ND - 1][3])
+                 "+r"(v[6][1]), "+r"(v[6][2]), "+r"(v[6][3]), "+r"(v[7][0]),
+                 "+r"(v[7][1]), "+r"(v[7][2]), "+r"(v[7][3])
                :
                : "memory");
 }
@@ -157,7 +163,7 @@ __device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&
 // orders |x|; infinities and NaNs are the largest) and the exponent field of the row scale.
 // maxe = row_scale(largest key) is the exponent field of the row's largest element, plus one when
 // that element is above 0.975 of the next power of two: |x| < 0.976 2^E with E = maxe - EOFF, so
-// the sum or difference of two elements stays inside the seven signed base-256 digits (0.996 2^55).
+// the sum or difference of two elements stays inside the eight signed base-256 digits (0.996 2^63).
 template <typename T> struct FBits;
 template <> struct FBits<double> {
   static constexpr int EMAX = 0x7FF, EOFF = 1022, KEY_MB = 20;
@@ -196,7 +202,7 @@ template <typename T> __device__ __forceinline__ int row_scale(unsigned key) {
   return max(e, 1) + (frac > (unsigned)(0.95 * (1 << F::KEY_MB)) ? 1 : 0);
 }
 
-// round(x 2^(54-E)) of the element with bit pattern b in a row of scale maxe (E = maxe - EOFF);
+// round(x 2^(62-E)) of the element with bit pattern b in a row of scale maxe (E = maxe - EOFF);
 // zero in a row that holds an infinity or NaN (kNanRow), whose results are NaN.  TINY = false: the
 // implicit mantissa bit is set whatever the exponent field, which is right for normal numbers and
 // harmless for zeros and subnormals once the row scale is at least kTinyScale (they shift out).
@@ -208,7 +214,7 @@ template <bool TINY> __device__ __forceinline__ long long fixed_f32(unsigned b, 
     ef = 1;
   }
   const int sh = min(maxe - ef, 63);
-  const unsigned long long r = (((unsigned long long)m << 31 >> sh) + 1ull) >> 1;
+  const unsigned long long r = (((unsigned long long)m << 39 >> sh) + 1ull) >> 1;
   const long long s = (long long)((int)b >> 31);
   return ((long long)r ^ s) - s;
 }
@@ -223,7 +229,7 @@ template <bool TINY> struct Fixed<double, TINY> {
       ef = 1;
     }
     const int sh = min(maxe - ef, 63);
-    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)b) << 2;
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)b) << 10;
     const unsigned long long r = ((m >> sh) + 1ull) >> 1;
     const long long s = (long long)((int)hi >> 31);
     return ((long long)r ^ s) - s;
@@ -242,7 +248,7 @@ template <bool TINY> struct Fixed<df, TINY> {
 };
 
 // Digit plane i (0 = most significant) of two values, as two bf16 in one word (first in the low
-// half): byte 6 - i of the biased integers, u, stands for the digit u - 128.  With l = u mod 128,
+// half): byte 7 - i of the biased integers, u, stands for the digit u - 128.  With l = u mod 128,
 // the bf16 128 + l is 0x4300 | l, and the digit is (128 + l) - 256 or (128 + l) - 128 (bit 7 of u
 // clear or set; the bf16 -256 and -128 differ in exactly that bit of 0xC380), one exact bf16 add.
 __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byte) {
@@ -255,30 +261,49 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byt
   return *reinterpret_cast<uint32_t*>(&r);
 }
 
-// round(U / 64) of column e of the ND diagonal accumulators (exact integers below 2^24 held as
+// the high and low words of biased fixed-point values, added apart
+struct WordSums {
+  unsigned long long h = 0, l = 0;
+  __device__ __forceinline__ void add(unsigned long long v) {
+    h += (unsigned)(v >> 32);
+    l += (unsigned)v;
+  }
+  // the sums of the values without their bias, of n values: h 2^32 + l
+  __device__ __forceinline__ long long high(int n) const {
+    return (long long)(h - (unsigned long long)n * (unsigned)(kABias >> 32));
+  }
+  __device__ __forceinline__ long long low(int n) const {
+    return (long long)(l - (unsigned long long)n * (unsigned)kABias);
+  }
+};
+// such a sum, in units of 2^(E-62), as the T of T 2^(E-51)
+__device__ __forceinline__ long long words_to_t(long long h, long long l) {
+  return h * 2097152ll + ((l + 1024) >> 11);
+}
+
+// round(U / 64) of column e of the diagonal accumulators (exact integers below 2^24 held as
 // fp32), U = sum_d 256^(6-d) G_d.  Sums are formed modulo 2^64; |U| / 64 < 2^63 for sums of at most
 // 496 terms per row (|sum_k x_k B_nk| < 496 max|x| max|B|).  The first NMAG accumulators are known
 // to stay within 2^22 and convert by one float addition (the low bits of 1.5 2^23 + G are G), the
 // others by the conversion instruction (a quarter of the rate).
-template <int NMAG, int ND>
-__device__ __forceinline__ long long recombine(const uint32_t (&v)[ND][4], int e) {
-  int g[ND];
+template <int NMAG>
+__device__ __forceinline__ long long recombine(const uint32_t (&v)[kDiags][4], int e) {
+  int g[kDiags];
 #pragma unroll
-  for (int d = 0; d < ND; ++d)
+  for (int d = 0; d < kDiags; ++d)
     g[d] = d < NMAG ? __float_as_int(__uint_as_float(v[d][e]) + 12582912.0f) - 0x4B400000
                     : __float2int_rz(__uint_as_float(v[d][e]));
   // h, m (and q, when every |G| <= 2^22) fit 32 bits; G_4 256^2 + G_5 256 = 2^8 q and
-  // G_6 256 + G_7 (or G_6) = r contribute 4 q + round(r / 2^14) (round(r / 64)) to U / 64
+  // G_6 256 + G_7 = r contribute 4 q + round(r / 2^14) to U / 64
   const int h = g[0] * 256 + g[1], m = g[2] * 256 + g[3];
   long long l;
-  if (NMAG == ND) {
+  if (NMAG == kDiags) {
     const int q = g[4] * 256 + g[5];
-    const int r = ND == 8 ? (g[6] * 256 + g[ND - 1] + 8192) >> 14 : (g[6] + 32) >> 6;
+    const int r = (g[6] * 256 + g[7] + 8192) >> 14;
     l = (long long)q * 4 + (long long)r;
   } else {
     l = (long long)g[4] * 1024 + ((long long)g[5] * 4 +
-        (ND == 8 ? ((long long)g[6] * 256 + (long long)g[ND - 1] + 8192) >> 14
-                 : (long long)((g[6] + 32) >> 6)));
+        (((long long)g[6] * 256 + (long long)g[7] + 8192) >> 14));
   }
   return (long long)((unsigned long long)(unsigned)h << 34) + ((long long)m * 262144 + l);
 }
@@ -341,22 +366,22 @@ template <> __device__ __forceinline__ df qnan<df>() {
 // ---- one K stage's MMAs -----------------------------------------------------------------------
 // A planes at shared address sA, the stacked B planes (7 NT rows) at sB, both 16 K wide in the
 // canonical no-swizzle K-major core-matrix layout; accumulators from tensor-memory column tmem.
-// A plane i times B rows 0 .. (7-i) NT, in pieces of at most 256 columns of equal width (an MMA of
+// A plane i times B rows 0 .. min(7, 8-i) NT, in pieces of at most 256 columns of equal width (an MMA of
 // M = 128 takes N / 2 cycles, but not less than about 50).  init: the accumulators start from zero
 // (plane 0 covers all their columns).  NT is a template argument because the single issuing thread
-// is what limits the rate otherwise (NT = 64: 912 cycles of MMAs per stage; with the pieces worked
-// out at run time the issue took 2040).
-template <int NT, int ND>
+// is what limits the rate otherwise (NT = 64: 28 products took 912 cycles of MMAs per stage;
+// with the pieces worked out at run time the issue took 2040).
+template <int NT>
 __device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint32_t sB, bool init) {
   // bf16 x bf16 -> fp32, both K-major, M = 128 (N added per MMA)
   constexpr uint32_t idesc0 =
       (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 4) << 24);
   const uint64_t a0 = sdesc(sA, kALbo, 128), b0 = sdesc(sB, (uint32_t)(kPlanes * NT * 16), 128);
 #pragma unroll
-  for (int i = 0; i < kPlanes; ++i) {
-    // diagonals i .. 6, and with ND = 8 diagonal 7 of planes 1 .. 6; plane 1 touches diagonal 7
-    // first, in an MMA of its own that may start it from zero
-    const int nb = (ND == 8 && i > 1) ? ND - i : kPlanes - i;
+  for (int i = 0; i < kAPlanes; ++i) {
+    // diagonals i .. 6, and diagonal 7 of planes 1 .. 7; plane 1 touches diagonal 7 first, in an MMA
+    // of its own that may start it from zero
+    const int nb = i > 1 ? kDiags - i : kPlanes - i;
     const int ntot = nb * NT, np = (ntot + 255) / 256;
     const int len = (ntot / np + 15) / 16 * 16;
 #pragma unroll
@@ -366,19 +391,18 @@ __device__ __forceinline__ void issue_stage_nt(uint32_t tmem, uint32_t sA, uint3
                b0 + (uint64_t)n0, idesc0 | ((uint32_t)(nlen >> 3) << 17),
                (uint32_t)!(init && i == 0));
     }
-    if (ND == 8 && i == 1)
+    if (i == 1)
       mma_bf16(tmem + (uint32_t)(7 * NT), a0 + (uint64_t)(kPlaneBytes / 16),
                b0 + (uint64_t)(6 * NT), idesc0 | ((uint32_t)(NT >> 3) << 17), (uint32_t)!init);
   }
 }
-template <int ND>
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t sA, uint32_t sB, int NT,
                                             bool init) {
   switch (NT) {
-    case 16: issue_stage_nt<16, ND>(tmem, sA, sB, init); break;
-    case 32: issue_stage_nt<32, ND>(tmem, sA, sB, init); break;
-    case 48: issue_stage_nt<48, ND>(tmem, sA, sB, init); break;
-    default: issue_stage_nt<64, ND>(tmem, sA, sB, init); break;
+    case 16: issue_stage_nt<16>(tmem, sA, sB, init); break;
+    case 32: issue_stage_nt<32>(tmem, sA, sB, init); break;
+    case 48: issue_stage_nt<48>(tmem, sA, sB, init); break;
+    default: issue_stage_nt<64>(tmem, sA, sB, init); break;
   }
 }
 

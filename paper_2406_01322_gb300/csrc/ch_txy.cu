@@ -4,7 +4,7 @@
 //
 // GB300 issues about 1.6 float64 operations per clock per SM; a padded line of 192 points costs
 // about 12 of them per real sample by FFT, which is what bounded these passes.  As digit products
-// the same transforms need no float64 arithmetic: about 45 integer instructions per sample
+// the same transforms need no float64 arithmetic: about 50 integer instructions per sample
 // converted, 30 per sample produced, and tensor work that stays below both for the lengths used.
 //
 // Four transforms, n = 0 .. nout - 1 and P the padded length:
@@ -18,9 +18,7 @@
 // output are recombined as integers of one scale and added exactly, so every result is rounded
 // once.  For even P the sample k = P / 2 of a forward transform enters as (-1)^n times its weight
 // (added to the recombined integer), and the output n = P / 2 of a backward transform, an
-// alternating sum, is formed exactly by the producers.  Eight diagonals of digit products are kept
-// (34 products): with the 28 of seven diagonals a 128^3 step's error against 64 bits rose from
-// 1.8e-14 to 3.1e-14.
+// alternating sum, is formed exactly by the producers.
 //
 // Tiles, warps and stages as in the Chebyshev transform (ch_tc.cu): a tile is 64 complex lines
 // (re and im rows; YB, YF) or 128 lines (XB, XF), lines neighbouring in memory so that every load
@@ -99,8 +97,8 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
                                               int lane) {
   const int nout = A.t.nout;
   for (int c0 = 0; c0 < CW; c0 += 4) {
-    uint32_t v[8][4];
-    tmem_ldx4<8>(tb + (uint32_t)c0, A.t.NT, v);
+    uint32_t v[kDiags][4];
+    tmem_ldx4(tb + (uint32_t)c0, A.t.NT, v);
     if (c0 + 4 >= CW) {   // all read: the accumulators are free for the next pass
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -109,7 +107,7 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
     }
     long long T[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG, 8>(v, e);
+    for (int e = 0; e < 4; ++e) T[e] = recombine<NMAG>(v, e);
     if (A.t.kc > 1) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -308,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
                 goto drain;
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               const uint32_t sA = sBase + slot * (uint32_t)sbytes;
-              issue_stage<8>(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
+              issue_stage(tmem, sA, sA + (uint32_t)kABytes, NT, st == s0);
               any = true;
               mma_commit(barEmpty + 8 * slot);
               if ((int)++slot == ns) {
@@ -361,12 +359,12 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           const int ro = b * kRows + tile_row(l, 0);
           sE[ro] = sc;
           sE[ro + 8] = sc;
-          sC[ro] = __mul64hi(xr * 256, A.t.ymid * 4);   // x Y / 2^54
-          sC[ro + 8] = __mul64hi(xi * 256, A.t.ymid * 4);
+          sC[ro] = __mul64hi(xr, A.t.ymid * 4);   // X Y / 2^62
+          sC[ro + 8] = __mul64hi(xi, A.t.ymid * 4);
         } else {
           const long long x = MODE == XF && ok ? fix<true>(*mp, sc) : 0;
           sE[b * kRows + l] = sc;
-          sC[b * kRows + l] = __mul64hi(x * 256, A.t.ymid * 4);
+          sC[b * kRows + l] = __mul64hi(x, A.t.ymid * 4);
         }
       }
       __syncwarp();
@@ -397,8 +395,8 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       unsigned char* sA = stages + (size_t)slot * sbytes;
       if (p == 0) bulk_load(su32(sA) + (uint32_t)kABytes, bsrc, bbytes, barB + 8 * slot, pol);
 #pragma unroll
-      for (int i = 0; i < kPlanes; ++i) {
-        const int b = 6 - i, sh = b < 4 ? 0 : 32;
+      for (int i = 0; i < kAPlanes; ++i) {
+        const int b = 7 - i, sh = b < 4 ? 0 : 32;
         uint32_t w[8], r[4];
 #pragma unroll
         for (int e = 0; e < 8; ++e) w[e] = (uint32_t)(v[e] >> sh);
@@ -466,7 +464,8 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(barRowFree + 8 * rbuf)
                      : "memory");
       const bool tiny = __any_sync(0xffffffffu, sc < kTinyScale) != 0;
-      unsigned long long sumr = 0, sumi = 0, s0 = 0;
+      WordSums sumr, sumi;
+      unsigned long long s0 = 0;
       bool ok = true;
       for (int st = 0; st < nst && ok; ++st) {
         if ((MODE == YB || MODE == XB) && d) {   // i k times the mode
@@ -485,14 +484,14 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
             if (CPX) {
               const long long a = fix<TINY>(x[e].x, sc), b = fix<TINY>(x[4 + e].x, sc);
               const long long u = fix<TINY>(x[e].y, sc), v = fix<TINY>(x[4 + e].y, sc);
-              s[e] = a + b + kBias;
-              dd[e] = a - b + kBias;
-              s[4 + e] = u + v + kBias;
-              dd[4 + e] = u - v + kBias;
+              s[e] = a + b + kABias;
+              dd[e] = a - b + kABias;
+              s[4 + e] = u + v + kABias;
+              dd[4 + e] = u - v + kABias;
             } else {
               const long long a = fix<TINY>(x[e].x, sc), b = fix<TINY>(x[e].y, sc);
-              s[e] = MODE == XB ? a + kBias : a + b + kBias;
-              dd[e] = MODE == XB ? b + kBias : a - b + kBias;
+              s[e] = MODE == XB ? a + kABias : a + b + kABias;
+              dd[e] = MODE == XB ? b + kABias : a - b + kABias;
             }
           }
         };
@@ -504,8 +503,8 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
         if (MODE == YB || MODE == XB) {
 #pragma unroll
           for (int e = 0; e < NE; ++e) {
-            sumr += s[e];
-            if (CPX) sumi += s[4 + e];
+            sumr.add(s[e]);
+            if (CPX) sumi.add(s[4 + e]);
           }
           if (st == 0) s0 = s[0];
         }
@@ -515,20 +514,15 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       if ((MODE == YB || MODE == XB) && !(A.P & 1)) {
         // output n = P / 2: sum_k (-1)^k s_k (YB, and XB of unit weights), 2 sum_k (-1)^k Re c_k -
         // Re c_0 (XB);
-        // (-1)^k = (-1)^g.  High and low parts (27 bits) are added apart.
-        const unsigned long long nb = (unsigned long long)(NE * nst) * kBias;
+        // (-1)^k = (-1)^g.  High and low words are added apart.
         const int f = MODE == XB && !A.t.unit ? 2 : 1;
-        long long tr = (long long)(sumr - nb), tm = (long long)(sumi - nb);
-        if (g & 1) {
-          tr = -tr;
-          tm = -tm;
-        }
-        long long hr = f * (tr >> 27), lr = f * (tr & 0x7FFFFFF);
-        long long hm = tm >> 27, lm = tm & 0x7FFFFFF;
+        const int sf = g & 1 ? -f : f, cnt = NE * nst;
+        long long hr = sf * sumr.high(cnt), lr = sf * sumr.low(cnt);
+        long long hm = CPX ? sf * sumi.high(cnt) : 0, lm = CPX ? sf * sumi.low(cnt) : 0;
         if (f == 2 && g == 0) {
-          const long long z = (long long)(s0 - kBias);
-          hr -= z >> 27;
-          lr -= z & 0x7FFFFFF;
+          const long long z = (long long)(s0 - kABias);
+          hr -= z >> 32;
+          lr -= (long long)(unsigned)z;
         }
 #pragma unroll
         for (int off = CPX ? 1 : 16; off <= 16; off <<= 4) {   // the threads of the line
@@ -540,13 +534,13 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           }
         }
         if (g == 0 && rowok) {
-          const int e2 = sc - FBits<double>::EOFF - 51;   // sum 2^(E - 54), T = sum / 8
+          const int e2 = sc - FBits<double>::EOFF - 51;
           const double vr = sc == kNanRow ? qnan<double>()
-                                          : scaled_any<double>(hr * 16777216ll + ((lr + 4) >> 3), e2);
+                                          : scaled_any<double>(words_to_t(hr, lr), e2);
           double* o = A.out[fld] + (lh * A.ohs + ll * A.ols + (long long)(A.P / 2) * A.ostr) * OSC;
           if (CPX) {
             const double vi = sc == kNanRow ? qnan<double>()
-                                            : scaled_any<double>(hm * 16777216ll + ((lm + 4) >> 3), e2);
+                                            : scaled_any<double>(words_to_t(hm, lm), e2);
             *reinterpret_cast<double2*>(o) = make_double2(vr, vi);
           } else {
             *o = vr;
@@ -584,7 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
     }
   } else {
     // ---- epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its rows), columns
-    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the seven accumulators
+    // (w / 4) NT / 2 .. + NT / 2 - 1 of each of the eight accumulators
     const int qd = warp & 3, cg = warp >> 2, CW = NT / 2;
     const int row = qd * 32 + lane;
     const int l = CPX ? (row >> 4) * 8 + (row & 7) : row, part_c = CPX ? (row >> 3) & 1 : 0;
