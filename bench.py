@@ -53,8 +53,6 @@ DF_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 9.67 / 1e12
 # current build from one ncu capture each (128 x 128 x 129 workloads, steady-state launches);
 # absent entries report null.  Re-capture when a kernel changes.
 TRAFFIC_MB = {
-    ("channel_128x128x129", 0, "xline"): 152.8 + 185.4,
-    ("channel_128x128x129", 0, "ybwd"): 84.6 + 135.3,
     ("channel_128x128x129", 2, "xline"): 153.2 + 193.1,
     ("channel_128x128x129", 2, "ybwd"): 84.7 + 134.8,
     # coefficient-space z kernels of the tensor-core method (the same kernels at any precision)
@@ -67,12 +65,8 @@ TRAFFIC_MB = {
     ("channel_512x256x257_mixed", 1, "zbwd"): 1343.6 + 1427.6,
     ("channel_512x256x257_mixed", 0, "zsolve"): 4753.3 + 3623.4,
     ("channel_512x256x257_mixed", 0, "zbwd"): 1343.7 + 2096.8,
-    ("channel_512x256x257_mixed", 0, "xline"): 2434.1 + 3591.5,
-    ("channel_512x256x257_mixed", 0, "ybwd"): 1610.9 + 2393.1,
     # current step kernels (full-size captures of the default bench command's kernels with
     # --cheb tc, and of the 128^3 mixed tensor-core and float64 FFT-method steps)
-    ("channel_512x256x257_mixed", 1, "cheb_fwd"): 964.4 + 2390.7,
-    ("channel_512x256x257_mixed", 1, "cheb_bwd"): 1368.9 + 1220.4,
     ("channel_512x256x257_mixed", 1, "zrhs_coef"): 3331.3 + 2004.2,
     ("channel_512x256x257_mixed", 1, "zbwd_coef"): 1342.3 + 2287.4,
     ("channel_512x256x257_mixed", 1, "xline"): 1783.4 + 2107.7,
@@ -87,9 +81,7 @@ TRAFFIC_MB = {
     ("channel_128x128x129", 1, "yfwd"): 114.2 + 32.6,
     ("channel_128x128x129", 1, "ybwd"): 42.0 + 27.9,
     ("channel_128x128x129", 0, "zrhs"): 218.3 + 73.3,
-    ("channel_128x128x129", 0, "yfwd"): 228.3 + 85.9,
     ("channel_128x128x129", 0, "zbwd"): 84.0 + 82.6,
-    ("channel_128x128x129_adjoint", 0, "adj_xline"): 380.7 + 130.9,
     ("channel_128x128x129_adjoint", 0, "adj_zsolve"): 102.4 + 28.2,
     ("channel_128x128x129_adjoint", 0, "adj_zrhs"): 135.1 + 223.7,
 }
@@ -166,9 +158,10 @@ def kernel_work(w, prec, cheb="fft"):
     # for the i kx, i ky combinations)
     yf_fl = 9 * Mx * nz * fft_flops(Py) + 42 * S
     yf_by = (9 * Y + 7 * S) * b
-    # Chebyshev transforms on the tensor cores (CH_CHEB_TC): tensor-pipe flops issued (36 digit
-    # products of 2 M Nout K each, M = real rows, Nout and K padded as the kernel pads them) and
-    # the bytes of the fields read and written once
+    # Chebyshev transforms on the tensor cores: the flops of the plain matrix product in an exact
+    # split of eight 7-bit digits (36 digit products of 2 M Nout K each, M = real rows, Nout and K
+    # padded to its tiles), a yardstick that does not change with the kernel (what the kernel
+    # issues: cheb_issued_flops), and the bytes of the fields read and written once
     Kp, NT, nNt = tc_tiles(nz)
     rows = 2 * lines
     tcf_fl = 36 * 2.0 * (7 * rows) * (NT * nNt) * Kp
@@ -186,14 +179,24 @@ def kernel_work(w, prec, cheb="fft"):
 
 
 def tc_tiles(nz):
-    """K padding, output slice width and slice count of the tensor-core Chebyshev kernel (the
-    library's rule: the slices cover the outputs n < N = nz - 1, 48 wide unless 64-wide ones pad
-    20 % less; the last output is summed exactly outside the MMAs)."""
+    """K padding, output slice width and slice count of the unfolded tensor-core product (the
+    slices cover the outputs n < N = nz - 1, 48 wide unless 64-wide ones pad 20 % less)."""
     N = nz - 1
     Kp = (nz + 15) // 16 * 16
     c48, c64 = (N + 47) // 48 * 48, (N + 63) // 64 * 64
     NT = 48 if 5 * c48 <= 4 * c64 else 64
     return Kp, NT, (N + NT - 1) // NT
+
+
+def cheb_issued_flops(w, nf):
+    """Tensor-pipe flops that one Chebyshev launch of nf fields issues: two folded products (even
+    and odd outputs) of K = N / 2 and N / 2 outputs, in slices of at most 64 columns and stages of
+    16 K, 35 digit products each, for the real and imaginary rows of every line."""
+    H = (w["nz"] - 1) // 2
+    nsl = (H + 63) // 64
+    NT = ((H + nsl - 1) // nsl + 15) // 16 * 16
+    K = (H + 15) // 16 * 16
+    return 35 * 2.0 * (2 * nf * (w["nx"] // 2) * w["ny"]) * (2 * NT * nsl) * K
 
 
 def cufft_transforms_ms(w, prec, reps=5, warmup=2, dev="cuda"):
@@ -737,6 +740,7 @@ def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
                              "9.67 float32 instructions per float64-equivalent flop (nominal)"}
     elif name.startswith("cheb"):
         tpk, tpk_kind = tensor_peak()
+        fl = cheb_issued_flops(w, 7 if name == "cheb_fwd" else 5)
         ach = fl / (per_launch_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": tpk, "unit": "TFLOP/s",
                 "frac": ach / tpk, "traffic": traffic, "kernel": name, "peak_kind": tpk_kind}

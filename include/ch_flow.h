@@ -126,24 +126,27 @@ int ch_step(ch_grid* g, int nsteps);
 /* The kernels of one time step in the order ch_step_timed reports them in: zrhs (DCT,
  * assembly, AB2, right-hand sides), zsolve (tau solves), zbwd (update, velocity, backward DCT),
  * y backward, x line, y forward, then the two Chebyshev transforms on the tensor cores
- * (forward of the nine products before zrhs, backward of the five fields after zbwd), which run
- * only under CH_CHEB_TC (zero time otherwise; zrhs and zbwd then skip their DCTs). */
+ * (forward of the seven combined lines before zrhs, backward of the five fields after zbwd), which
+ * run under CH_CHEB_TC and on large grids without a selected method (ch_set_chebyshev; zero time
+ * otherwise; zrhs and zbwd then skip their DCTs). */
 #define CH_STEP_KERNELS 8
 
 /* Method of the Chebyshev transforms (Sec. 3.2.1) inside the step:
- * CH_CHEB_FFT: DCT-I through one N-point complex FFT per line, in float64, fused into zrhs/zbwd
- *   (the default);
- * CH_CHEB_TC: the transform as a product with the fixed Nz x Nz Chebyshev matrix on the tensor
- *   cores, float64-accurate by an exact split of both operands into eight signed 7-bit digits
- *   (bf16, Ozaki scheme; fp32 accumulation is exact for these integers) and a recombination in
- *   64-bit integers; error a few units of 2^-53 of max|row| x max_n sum_k |B_nk| per line, the
- *   accuracy of a float64 transform.  Two extra launches per step and a 9-field float64 coefficient buffer.
- *   Single grids (any precision) with nz <= 496; not with the adjoint. */
+ * CH_CHEB_FFT: DCT-I through one N-point complex FFT per line, in float64, fused into zrhs/zbwd;
+ * CH_CHEB_TC: the transform as a product with the fixed Chebyshev matrix, folded into its even and
+ *   odd halves, on the tensor cores; float64-accurate by an exact split of both operands into signed
+ *   base-256 digits (bf16, Ozaki scheme; fp32 accumulation is exact for these integers) and a
+ *   recombination in 64-bit integers; error a few units of 2^-53 of max|row| x max_n sum_k |B_nk|
+ *   per line, the accuracy of a float64 transform.  Two extra launches per step.  Single grids (any
+ *   precision) with nz <= 496; not with the adjoint.
+ * While no method was selected, ch_get_chebyshev says CH_CHEB_FFT and grids of fewer than 2^18
+ * modes (nx/2 ny nz) work that way; larger ones (nz <= 496, nx, ny <= 1024) use the tensor cores as
+ * under CH_CHEB_TC, reverse sweeps included. */
 #define CH_CHEB_FFT 0
 #define CH_CHEB_TC 1
 
-/* Select the step's Chebyshev method; allocates the tensor-core tables and buffer on the first
- * CH_CHEB_TC (synchronous).  CH_ERR_ARG: bad method; CH_ERR_STATE: a reverse sweep is open;
+/* Select the step's Chebyshev method; allocates the tensor-core tables, where the grid does not have
+ * them yet, on the first CH_CHEB_TC (synchronous).  CH_ERR_ARG: bad method; CH_ERR_STATE: a reverse sweep is open;
  * CH_ERR_SIZE: nz > 496.
  * The captured step graph is rebuilt at the next ch_step. */
 int ch_set_chebyshev(ch_grid* g, int method);
@@ -161,7 +164,7 @@ int ch_get_fft_pruning(const ch_grid* g);
 
 /* Chebyshev transform along z of nf fields of complex lines (device, float64 (re, im) pairs,
  * layout [field][mx * ny + j][n], field stride (nx/2) ny nz, the layout of ch_get_spectral) with
- * the selected method: dir 0 samples at z_k = cos(pi k / N) -> coefficients a_n, dir 1 the
+ * the method in use: dir 0 samples at z_k = cos(pi k / N) -> coefficients a_n, dir 1 the
  * inverse.  in and out must not overlap.  Asynchronous on the handle's stream. */
 int ch_chebyshev_lines(ch_grid* g, int dir, const double* in, double* out, int nf);
 
@@ -197,8 +200,8 @@ int ch_fp64_fma_rate(double* tflops);
  * the last.  kernel_ms may be NULL.  Used by the benchmark to attribute step time. */
 int ch_step_timed(ch_grid* g, int nsteps, double* kernel_ms, double* total_ms);
 
-/* Number of kernel launches one ch_step makes per time step (six; two more with CH_CHEB_TC, three
- * more with the x/y transforms on the tensor cores). */
+/* Number of kernel launches one ch_step makes per time step (six; two more with the Chebyshev
+ * transforms on the tensor cores, three more with the x/y transforms there). */
 int ch_launches_per_step(const ch_grid* g);
 
 /* Spectral state -> physical u, v, w, phi (device, (nz,ny,nx) float64) on the unpadded grid. */
@@ -300,7 +303,8 @@ int ch_render_interface(ch_grid* g, unsigned char* rgb, double* depth, int width
  * (created here with the given allocator and stream; all members share one `precision`, any of
  * the three; CH_ERR_ARG if they differ).  One ensemble step advances every member by one time
  * step with six grouped persistent launches (one per stage; their CTAs walk a work list spanning
- * all members; with CH_CHEB_TC two more per member), captured once into a CUDA graph and
+ * all members; two more per member whose Chebyshev transforms run on the tensor cores; members with
+ * and without get a zrhs and a zbwd launch of their own), captured once into a CUDA graph and
  * replayed.  Members are set, read and diagnosed through their ch_grid handles
  * (ch_ensemble_member); ch_ensemble_step needs every member set.  ch_ensemble_autotune times the
  * transforms' radix schedules and the persistent CTAs per SM of each stage on the live members
@@ -318,7 +322,9 @@ int ch_ensemble_step(ch_ensemble* e, int nsteps);
 #define CH_ENSEMBLE_STAGES 6
 int ch_ensemble_step_timed(ch_ensemble* e, int nsteps, double* stage_ms, double* total_ms);
 int ch_ensemble_autotune(ch_ensemble* e, int reps);
-/* Chebyshev method of the ensemble step (CH_CHEB_FFT default, CH_CHEB_TC): with CH_CHEB_TC the
+/* Chebyshev method of the ensemble step (CH_CHEB_FFT, CH_CHEB_TC; while none was selected
+ * ch_ensemble_get_chebyshev says CH_CHEB_FFT and each member works as it would alone): with
+ * CH_CHEB_TC the
  * grouped zrhs and zbwd stages read and write float64 Chebyshev coefficients and each member's
  * z transforms (Sec. 3.2.1) run on the tensor cores as in ch_set_chebyshev, one launch per
  * member before zrhs and one after zbwd, inside the step's graph and timed with stages 0 and 2

@@ -287,7 +287,8 @@ class Grid:
     KERNELS = ("zrhs", "zsolve", "zbwd", "ybwd", "xline", "yfwd", "cheb_fwd", "cheb_bwd")
 
     def set_chebyshev(self, method):
-        """CHEB_FFT (default) or CHEB_TC: how the step does its Chebyshev transforms."""
+        """CHEB_FFT or CHEB_TC: how the step does its Chebyshev transforms (until one is selected,
+        CHEB_FFT on small grids and the tensor cores on large ones; see ch_flow.h)."""
         _ck("ch_set_chebyshev", lib().ch_set_chebyshev(self.h, int(method)))
 
     def chebyshev(self):

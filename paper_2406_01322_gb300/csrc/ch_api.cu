@@ -1,10 +1,12 @@
 // C-ABI of the channel solver (declared in include/ch_flow.h): validation, plans, twiddle
 // tables, internal buffers, the per-step launch schedule and its CUDA-graph replay.
 //
-// One time step (paper Sec. 2.2, steps i)-v)) is six launches on the handle's stream (eight with
-// the tensor-core Chebyshev method: the forward transform of the nine products before zrhs and
-// the backward transform of the five fields after zbwd, zrhs and zbwd then skipping their DCTs):
-//   zrhs    : Chebyshev DCT-I of the nine non-linear fields (as seven combinations), assembly,
+// One time step (paper Sec. 2.2, steps i)-v)) is six launches on the handle's stream; two more with
+// the Chebyshev transforms on the tensor cores (the forward transform of the seven combined lines
+// before zrhs and the backward one of the five fields after zbwd, zrhs and zbwd then skipping their
+// DCTs), three more with the float64 x/y transforms there (x backward, products, x forward; y
+// forward, combinations):
+//   zrhs    : Chebyshev DCT-I of the seven combinations of the nine non-linear fields, assembly,
 //             AB2 / CN / IE right-hand sides;
 //   zsolve  : the Chebyshev-tau solves of every wavenumber line;
 //   zbwd    : state update, velocity from continuity, backward DCT-I of the five fields the next

@@ -835,8 +835,10 @@ __device__ __forceinline__ void solve_tile_problem(const GridDev& g, double2* __
 }
 
 // zsolve, tile variant (short lines): TL lines per CTA staged in shared memory, thread = (line,
-// parity), the three problems in turn.  R holds [omega | theta-w | phi] right-hand sides on
-// entry and the solved sums / new phi on exit (line-major, like the state).
+// parity) of one problem; single grids give each problem its own blocks (the chains are latency-bound:
+// one thread for all three took 78 against 39 us at 32 x 32 x 33, 0.55 against 0.35 ms at 162 x 108 x
+// 163), the grouped kernels, with items enough, loop over them.  R holds [omega | theta-w | phi]
+// right-hand sides on entry and the solved sums / new phi on exit (line-major, like the state).
 __device__ __forceinline__ void zsolve_tile_body(const GridDev& g, double2* __restrict__ R,
                                                  long long fs, int nlines, int bid, int prob) {
   extern __shared__ double2 ssm[];
