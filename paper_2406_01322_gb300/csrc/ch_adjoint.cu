@@ -130,8 +130,15 @@ int reverse_core(ch_grid* G, const double2* ya, int first, cudaEvent_t* ev) {
   cudaError_t e[7];
   e[0] = chf::launch_adj_zsolve(g, G->a_L, G->a_Rb, G->fs, G->a_bb, s);
   if (ev) cudaEventRecord(ev[1], s);
-  e[1] = chf::launch_adj_zrhs(g, G->a_Rb, G->a_L, G->a_mu, G->a_lam, G->a_mu2, G->a_nlb, G->fs,
-                              first, G->a_bb, G->pz, s);
+  // Chebyshev transforms on the tensor cores where the step has them there: the transposed forward
+  // one is the forward one (its matrix is symmetric), the transposed backward one the backward one
+  const bool tc = ch_z_coef(G);
+  const int nlines = g.Mx * g.ny;
+  e[1] = chf::launch_adj_zrhs(g, G->a_Rb, G->a_L, G->a_mu, G->a_lam, G->a_mu2,
+                              tc ? (double2*)G->yb : G->a_nlb, G->fs, first, G->a_bb, G->pz, tc, s);
+  if (tc && e[1] == cudaSuccess)
+    e[1] = chf::launch_cheb_tc(0, 0, G->yb, G->fs, G->a_nlb, G->fs, kNl, nlines, g.nz, G->tcf,
+                               G->tc_err, s);
   if (ev) cudaEventRecord(ev[2], s);
   e[2] = ch_launch_y_adj(G, 1, G->a_nlb, (double2*)G->yb, kNl, s);
   if (ev) cudaEventRecord(ev[3], s);
@@ -141,7 +148,12 @@ int reverse_core(ch_grid* G, const double2* ya, int first, cudaEvent_t* ev) {
   if (ev) cudaEventRecord(ev[5], s);
   e[5] = chf::launch_fold_dy(g, G->auxA, G->fs, s);
   if (ev) cudaEventRecord(ev[6], s);
-  e[6] = chf::launch_adj_zbwd(g, G->auxA, G->fs, G->a_lam, G->fs, G->pz, s);
+  e[6] = cudaSuccess;
+  if (tc)
+    e[6] = chf::launch_cheb_tc(0, 0, G->auxA, G->fs, G->auxB, G->fs, kBw, nlines, g.nz, G->tcb,
+                               G->tc_err, s);
+  if (e[6] == cudaSuccess)
+    e[6] = chf::launch_adj_zbwd(g, tc ? G->auxB : G->auxA, G->fs, G->a_lam, G->fs, G->pz, tc, s);
   if (ev) cudaEventRecord(ev[7], s);
   for (int k = 0; k < 7; ++k)
     if (e[k] != cudaSuccess) {

@@ -249,6 +249,7 @@ cudaError_t launch_x_c2r(const GridDev& g, const double2* in, double* phys, int 
 // adj_zrhs: from Rb, L, bb and mu (adjoint of this step's AB2 history h_n): lam = adjoint of the
 //   state s_n except its non-linear dependence, mu_prev = adjoint of h_{n-1}, nlb = adjoint of
 //   the 9 spectral non-linear fields times 1/(Px Py).
+//   (adj_zrhs, adj_zbwd with coef = 1: without their Chebyshev transforms.)
 // adj_xline: transposed x-line (in6 = the forward y-padded fields of s_n, pb9 = adjoints of the
 //   9 products after the transposed forward y pass) -> out6 adjoints of u v w phi phi_y phi_z.
 // fold_dy: f6[3] += -i ky f6[4]; f6[4] = f6[5].
@@ -260,9 +261,9 @@ cudaError_t launch_adj_zsolve(const GridDev& g, const double2* L, double2* Rb, l
 cudaError_t launch_adj_zrhs(const GridDev& g, const double2* Rb, const double2* L,
                             const double2* mu, double2* lam, double2* mu_prev, double2* nlb,
                             long long fs, int first, const double2* bb, const FftPlan& pz,
-                            cudaStream_t s);
+                            int coef, cudaStream_t s);
 cudaError_t launch_adj_zbwd(const GridDev& g, const double2* in5, long long fs_in, double2* lam,
-                            long long fs, const FftPlan& pz, cudaStream_t s);
+                            long long fs, const FftPlan& pz, int coef, cudaStream_t s);
 cudaError_t launch_objective(const GridDev& g, const double2* om, const double2* w,
                              const double2* phi, double2* lam, long long fs, double* part,
                              cudaStream_t s);

@@ -1446,8 +1446,9 @@ __device__ double2 tau_sweep_ct(double2* x, int p, int N, double alpha, bool neu
   return make_double2(rsq * a0.x, rsq * a0.y);
 }
 
-// adjoint of zsolve + state update: one thread per (line, parity); L = adjoint of the new
-// state (3 fields), Rb = adjoint of the right-hand sides (3 fields, written).
+// adjoint of zsolve + state update: one thread per (line, parity, problem), blockIdx.y = 2 - problem
+// (128 x 128 x 129: 0.47 ms with the three problems in turn, 0.29 apart); L = adjoint of the new state (3 fields), Rb = adjoint
+// of the right-hand sides (3 fields, written).
 // The adjoint differentiates the literal Crank-Nicolson map, whose solves impose the wall
 // conditions on q^{n+1}.  The forward sweeps solve for S = q^{n+1} + q^n with homogeneous wall
 // rows; on states that meet the wall conditions that is the same as imposing S's wall values =
@@ -1470,24 +1471,31 @@ __global__ void __launch_bounds__(ST) adj_zsolve_kernel(GridDev g, const double2
   const double *t1 = g.go1, *t2 = g.go2, *t3 = g.go3;
   const double2 zero = make_double2(0.0, 0.0);
   double2* bl = bb + (size_t)t * 3;
-  for (int f = 0; f < 3; ++f) {
-    const double2* in = L + f * fs + (size_t)line * Nz;
-    double2* row = Rb + f * fs + (size_t)line * Nz;
-    for (int n = p; n <= N; n += 2) row[n] = nyq ? zero : in[n];
-  }
+  const int prob = 2 - blockIdx.y;
+  const double2* in = L + prob * fs + (size_t)line * Nz;
+  double2* row = Rb + prob * fs + (size_t)line * Nz;
+  for (int n = p; n <= N; n += 2) row[n] = nyq ? zero : in[n];
   if (nyq) {
-    bl[0] = zero;
-    bl[1] = zero;
-    bl[2] = zero;
+    if (prob == 0) bl[0] = zero;
+    if (prob == 1) {
+      bl[1] = zero;
+      bl[2] = zero;
+    }
     return;
   }
-  // omega (and the mean flow): S = Sol_beta(r; wall value of omega^n)
-  double2* row = Rb + (size_t)line * Nz;
-  bl[0] = tau_sweep_ct(row, p, N, k2 + g.beta, false, t1, t2, t3, fac_ptr(g, 0, 0, K),
-                       fac_ptr(g, 0, 1, K), fac_ptr(g, 0, 2, K), g.NK, fac_rsq(g, 0, p, K));
+  if (prob == 0) {   // omega (and the mean flow): S = Sol_beta(r; wall value of omega^n)
+    bl[0] = tau_sweep_ct(row, p, N, k2 + g.beta, false, t1, t2, t3, fac_ptr(g, 0, 0, K),
+                         fac_ptr(g, 0, 1, K), fac_ptr(g, 0, 2, K), g.NK, fac_rsq(g, 0, p, K));
+    return;
+  }
+  if (prob == 2) {   // phi: two Neumann solves with the same operator (implicit Euler: no wall term)
+    for (int rep = 0; rep < 2; ++rep)
+      tau_sweep_ct(row, p, N, k2 + g.lam, true, t1, t2, t3, fac_ptr(g, 2, 0, K),
+                   fac_ptr(g, 2, 1, K), fac_ptr(g, 2, 2, K), g.NK, fac_rsq(g, 2, p, K));
+    return;
+  }
   // w: S_w = Omega_p + c Omega_h, Omega_p = Sol_0(Sol_beta r; wall value of w^n),
   //    c = (D w^n wall value - sum n^2 Omega_p) rsh
-  row = Rb + fs + (size_t)line * Nz;
   if (is00) {
     for (int n = p; n <= N; n += 2) row[n] = zero;
     bl[1] = zero;
@@ -1515,11 +1523,6 @@ __global__ void __launch_bounds__(ST) adj_zsolve_kernel(GridDev g, const double2
     tau_sweep_ct(row, p, N, k2 + g.beta, false, t1, t2, t3, fac_ptr(g, 0, 0, K),
                  fac_ptr(g, 0, 1, K), fac_ptr(g, 0, 2, K), g.NK, fac_rsq(g, 0, p, K));
   }
-  // phi: two Neumann solves with the same operator (implicit Euler: no wall-value term)
-  row = Rb + 2 * fs + (size_t)line * Nz;
-  for (int rep = 0; rep < 2; ++rep)
-    tau_sweep_ct(row, p, N, k2 + g.lam, true, t1, t2, t3, fac_ptr(g, 2, 0, K), fac_ptr(g, 2, 1, K),
-                 fac_ptr(g, 2, 2, K), g.NK, fac_rsq(g, 2, p, K));
 }
 
 // transpose of the forward DCT on lines [first, first+cnt): a = F x with F[n][j] =
@@ -1543,7 +1546,11 @@ __device__ void dct_forward_transpose_lines(const ZSmem& z, int first, int cnt, 
 // adjoint of zrhs (right-hand sides, AB2, assembly, forward DCT and combinations):
 // inputs Rb (rhs adjoints), L (new-state adjoint), mu (adjoint of h_n), state s_n;
 // outputs lam (adjoint of s_n, partial: update + rhs + phi in G), mu_prev (adjoint of h_{n-1}),
-// nlb (9 non-linear sample adjoints, fp64)
+// nlb (9 non-linear sample adjoints, fp64).  COEF: nlb takes what the transposed transform is to be
+// applied to; the forward DCT's matrix 2 cos(pi n j / N) / (cbar_n cbar_j N) is symmetric, so the
+// forward transform on the tensor cores does it (128 x 128 x 129: 1.31 ms with the DCTs, 0.66 as
+// coefficients and the transform).
+template <int COEF>
 __global__ void __launch_bounds__(ZT) adj_zrhs_kernel(GridDev g, const double2* __restrict__ Rb,
                                                       const double2* __restrict__ L,
                                                       const double2* __restrict__ mu,
@@ -1650,7 +1657,7 @@ __global__ void __launch_bounds__(ZT) adj_zrhs_kernel(GridDev g, const double2* 
     LN(z, 6, Nz)[n] = Gb;                               // phi^3 line
   }
   __syncthreads();
-  for (int f0 = 0; f0 < 7; f0 += NBF)
+  for (int f0 = 0; f0 < 7 && !COEF; f0 += NBF)
     dct_forward_transpose_lines(z, f0, (7 - f0 < NBF) ? 7 - f0 : NBF, Nz, N, pz, g.zcs);
   // combinations transposed: samples of the nine non-linear fields
   for (int n = tid; n < Nz; n += blockDim.x) {
@@ -1682,7 +1689,9 @@ __global__ void __launch_bounds__(ZT) adj_zrhs_kernel(GridDev g, const double2* 
 }
 
 // adjoint of the backward fields of s_n (u, v, w, phi, D phi -> backward DCT): in = 5 sample
-// adjoint fields; adds the state adjoint into lam
+// adjoint fields (COEF: their backward transforms, done on the tensor cores: 128 x 128 x 129 0.69 ->
+// 0.29 ms); adds the state adjoint into lam
+template <int COEF>
 __global__ void __launch_bounds__(ZT) adj_zbwd_kernel(GridDev g, const double2* __restrict__ in5,
                                                       long long fs_in, double2* __restrict__ lam,
                                                       long long fs, FftPlan pz) {
@@ -1702,8 +1711,10 @@ __global__ void __launch_bounds__(ZT) adj_zbwd_kernel(GridDev g, const double2* 
   }
   __syncthreads();
   // the backward DCT matrix C[j][n] = cos(pi n j / N) is symmetric: its transpose is itself
-  dct1_lines(z, 0, 4, Nz, N, pz, g.zcs, 1);
-  dct1_lines(z, 4, 1, Nz, N, pz, g.zcs, 1);
+  if (!COEF) {
+    dct1_lines(z, 0, 4, Nz, N, pz, g.zcs, 1);
+    dct1_lines(z, 4, 1, Nz, N, pz, g.zcs, 1);
+  }
   const double k2 = ksq(kx, ky);
   const double rk2 = is00 ? 0.0 : 1.0 / k2;
   for (int n = threadIdx.x; n < Nz; n += blockDim.x) {
@@ -2197,30 +2208,36 @@ int occupancy_z(int stage, int prec, size_t smem, int zsolve_tile, int coef) {
 cudaError_t launch_adj_zsolve(const GridDev& g, const double2* L, double2* Rb, long long fs,
                               double2* bb, cudaStream_t s) {
   const int nlines = g.Mx * g.ny;
-  adj_zsolve_kernel<<<(2 * nlines + ST - 1) / ST, ST, 0, s>>>(g, L, Rb, fs, nlines, bb);
+  adj_zsolve_kernel<<<dim3((2 * nlines + ST - 1) / ST, 3), ST, 0, s>>>(g, L, Rb, fs, nlines, bb);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_zrhs(const GridDev& g, const double2* Rb, const double2* L,
                             const double2* mu, double2* lam, double2* mu_prev, double2* nlb,
                             long long fs, int first, const double2* bb, const FftPlan& pz,
-                            cudaStream_t s) {
-  const size_t smem = zline_smem(g);
-  static SmemLimit cur;
-  cudaError_t e = ensure_smem(adj_zrhs_kernel, smem, &cur);
+                            int coef, cudaStream_t s) {
+  const size_t smem = coef ? (size_t)15 * g.nz * sizeof(double2) : zline_smem(g);   // lines 0..14
+  static SmemLimit cur[2];
+  cudaError_t e = ensure_smem(coef ? adj_zrhs_kernel<1> : adj_zrhs_kernel<0>, smem, &cur[coef]);
   if (e != cudaSuccess) return e;
-  adj_zrhs_kernel<<<g.Mx * g.ny, ZT, smem, s>>>(g, Rb, L, mu, lam, mu_prev, nlb, fs, first,
-                                                 1.0 / ((double)g.Px * (double)g.Py), bb, pz);
+  const double nls = 1.0 / ((double)g.Px * (double)g.Py);
+  if (coef)
+    adj_zrhs_kernel<1><<<g.Mx * g.ny, ZT, smem, s>>>(g, Rb, L, mu, lam, mu_prev, nlb, fs, first, nls,
+                                                     bb, pz);
+  else
+    adj_zrhs_kernel<0><<<g.Mx * g.ny, ZT, smem, s>>>(g, Rb, L, mu, lam, mu_prev, nlb, fs, first, nls,
+                                                     bb, pz);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_zbwd(const GridDev& g, const double2* in5, long long fs_in, double2* lam,
-                            long long fs, const FftPlan& pz, cudaStream_t s) {
-  const size_t smem = zline_smem(g);
-  static SmemLimit cur;
-  cudaError_t e = ensure_smem(adj_zbwd_kernel, smem, &cur);
+                            long long fs, const FftPlan& pz, int coef, cudaStream_t s) {
+  const size_t smem = coef ? (size_t)14 * g.nz * sizeof(double2) : zline_smem(g);   // lines 0..13
+  static SmemLimit cur[2];
+  cudaError_t e = ensure_smem(coef ? adj_zbwd_kernel<1> : adj_zbwd_kernel<0>, smem, &cur[coef]);
   if (e != cudaSuccess) return e;
-  adj_zbwd_kernel<<<g.Mx * g.ny, ZT, smem, s>>>(g, in5, fs_in, lam, fs, pz);
+  if (coef) adj_zbwd_kernel<1><<<g.Mx * g.ny, ZT, smem, s>>>(g, in5, fs_in, lam, fs, pz);
+  else adj_zbwd_kernel<0><<<g.Mx * g.ny, ZT, smem, s>>>(g, in5, fs_in, lam, fs, pz);
   return cudaGetLastError();
 }
 
