@@ -754,6 +754,9 @@ def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
         roof = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
                 "traffic": traffic, "kernel": name, "peak_kind": f"{hbm_kind} copy bandwidth"}
     roof["algorithmic_per_launch"] = {"flops": fl, "bytes": by}
+    if prec == 0 and name in ("ybwd", "xline", "yfwd"):
+        roof["note"] = ("float64 FFT flops as the yardstick; from 2^15 modes on the transforms run "
+                        "on the tensor cores")
     if roof["bound"] == "alu" and roof["peak"] == FP64_PEAK_TFLOPS and MEASURED_FMA.get("tflops"):
         roof["fp64_fma_measured_tflops"] = MEASURED_FMA["tflops"]
         roof["frac_of_measured_fma_rate"] = roof["achieved"] / MEASURED_FMA["tflops"]

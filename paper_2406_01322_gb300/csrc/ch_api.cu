@@ -397,8 +397,8 @@ int make_txy_plan(ch_grid* G, int mode, int P, double scale, chf::TxyPlan* p) {
 // that read and write physical fields (use_ax, with the Chebyshev transforms), and of the padded one
 // for the steps of a float64 grid (use_tx).
 // Rule: from 2^15 modes on (below, a transform has fewer tiles than a third of the SMs and its
-// latency counts: 32 x 32 x 33, 16896 modes, y backward 25 against 21 us, x line 45 against 53,
-// y forward 30 against 33 by FFT; 48 x 48 x 49, 56448 modes, 39, 96 and 60 against 47, 137 and 75),
+// latency counts: 32 x 32 x 33, 16896 modes, y backward, x line and y forward 28, 56 and 27 against
+// 22, 53 and 33 us by FFT; 48 x 48 x 49, 56448 modes, 34, 88 and 46 against 47, 137 and 75),
 // up to transform lengths of 1024 (the dense matrices grow with the length squared).
 constexpr int kTxyMaxP = 1024;
 constexpr long long kTxyMinModes = 1ll << 15;
