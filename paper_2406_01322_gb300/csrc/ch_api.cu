@@ -475,6 +475,15 @@ int rows_to_coef(ch_grid* G, double* const* phys, int nf, double2* coef) {
   return CH_OK;
 }
 
+// Rule for a transform of one field (its tiles are few; several fields together always gain): on the
+// tensor cores from 3 2^15 modes on with at least 8 x lines per x point.  A pair of transforms by FFT /
+// on the tensor cores, us: 128 x 48 x 33 165 / 141, 288 x 72 x 33 416 / 303, 64 x 36 x 145 162 / 129;
+// below 96 x 24 x 65 111 / 121, 256 x 24 x 25 152 / 228, 216 x 24 x 17 130 / 203.
+bool ax_one_field(const ch_grid* G) {
+  const GridDev& g = G->g;
+  return G->use_ax && G->fs >= 3 * kTxyMinModes && (long long)g.ny * g.nz >= 8ll * g.nx;
+}
+
 void drop_graph(ch_grid* G) {
   if (G->graph_ok) cudaGraphExecDestroy(G->gexec);
   G->graph_ok = 0;
@@ -1039,7 +1048,7 @@ int ch_transform_forward(ch_grid* G, const double* phys, double* spec) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  if (G->use_ax) {
+  if (ax_one_field(G)) {
     double* p[1] = {const_cast<double*>(phys)};
     return rows_to_coef(G, p, 1, (double2*)spec);
   }
@@ -1054,7 +1063,7 @@ int ch_transform_backward(ch_grid* G, const double* spec, double* phys) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  if (G->use_ax)
+  if (ax_one_field(G))
     return coef_to_rows(G, (const double2*)spec, 1, identity_ymap(), 1, nullptr, 0, 1, &phys);
   CK(chf::launch_dct_lines(1, 0, g, spec, G->auxA, 1, G->fs, G->pz, s));
   CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, 1, G->fs, G->fs, 1.0, G->pyu, s));
