@@ -139,8 +139,11 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 // 4-column loads (one per diagonal accumulator, `stride` columns apart) of this warp's 32 lanes,
-// then one wait that the values depend on
+// then one wait that the values depend on.  The loads are .aligned: every lane of the warp executes
+// them together, so the warp is brought together here, after whatever its lanes did apart (the
+// stores of a ragged last tile, whose rows only some lanes have).
 __device__ __forceinline__ void tmem_ldx4(uint32_t addr, int stride, uint32_t (&v)[kDiags][4]) {
+  __syncwarp();
 #pragma unroll
   for (int d = 0; d < kDiags; ++d)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"

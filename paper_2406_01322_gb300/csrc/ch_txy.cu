@@ -161,11 +161,10 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
     }
     if (MODE == XF && A.lift && m0 + c0 == 0)
       ra[0] = nan ? qnan<double>() : scaled_any<double>(a[0], ex - A.lift);
-    if (!rowok) continue;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int n = m0 + c0 + e;
-      if (n >= nout) continue;
+      if (!rowok || n >= nout) continue;
       if (MODE == XF) {
         *reinterpret_cast<double2*>(dst + 2 * (size_t)n * A.ostr) = make_double2(ra[e], rb[e]);
       } else if (MODE == XB) {
