@@ -267,11 +267,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             mma_commit(barAccFull);
           }
     drain:
-      if (!W.ok && any) {
-        // a wait ran out: nothing more is issued; wait (bounded) for the MMAs in flight before
-        // the tensor memory is released
+      // however the loop ended, here or in another warp (an epilogue that gave up waits for no MMA):
+      // the MMAs in flight finish (bounded) before the tensor memory is released
+      if (any) {
         mma_commit(barFin);
-        mbar_wait_until(barFin, 0, gtime() + kWaitNs);
+        W.ok = mbar_wait(barFin, 0) && W.ok;
       }
     }
     __syncwarp();
@@ -489,12 +489,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
     }
-    // after a failed wait the copies still in flight finish (bounded) before the CTA ends
-    if (!W.ok && p == 0) {
+    // the copies still in flight finish (bounded) before the CTA ends: all were consumed unless a
+    // wait ran out, in this warp or in the issuer
+    if (p == 0) {
       const uint64_t dl = gtime() + kWaitNs;
       for (int b = 0; b < kStages; ++b) {
         const uint32_t n = use + (b < (int)slot ? 1u : 0u);   // copies issued to slot b
-        if (n > 0) mbar_wait_until(barB + 8 * b, (n - 1) & 1, dl);
+        if (n > 0 && !mbar_wait_until(barB + 8 * b, (n - 1) & 1, dl)) W.ok = false;
       }
     }
   } else {
