@@ -170,7 +170,12 @@ int ch_chebyshev_lines(ch_grid* g, int dir, const double* in, double* out, int n
 
 /* Synchronise the handle's stream; CH_ERR_TIMEOUT (and the flag cleared) if a bounded device
  * wait of the tensor-core kernels gave up since the last check (its outputs are then invalid),
- * else CH_OK.  ch_diagnostics reports the same condition. */
+ * else CH_OK.  These kernels serve CH_CHEB_TC and, on larger grids, ch_step, the calls that take or
+ * give physical fields and the reverse sweep.  Calls that only enqueue work answer CH_OK whatever
+ * becomes of it; every call that waits for the stream to give a result (ch_get_fields_host,
+ * ch_diagnostics, ch_get_state, ch_objective, ch_adjoint_begin / _step / _segment / _end, the timed
+ * calls, ch_ensemble_step_timed / _autotune for any member) reports the condition too, with its
+ * outputs invalid, until ch_device_status clears it. */
 int ch_device_status(ch_grid* g);
 
 /* Test of the failure path of the bounded device waits (not in the paper; library

@@ -51,7 +51,7 @@ int objective_impl(ch_grid* G, double2* lam, double* J) {
   CK(chf::launch_sum(G->obj_part, nlines, G->obj_part + nlines, s));
   if (J) {
     CK(cudaMemcpyAsync(J, G->obj_part + nlines, sizeof(double), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    return ch_sync_status(G);
   }
   return CH_OK;
 }
@@ -112,7 +112,10 @@ int ch_adjoint_begin(ch_grid* G, double* J) {
   }
   // lambda_K = dJ/ds_K, mu_{K-1} = 0 (the last history is not used by J)
   int r = objective_impl(G, G->a_L, J);
-  if (r != CH_OK) return r;
+  if (r != CH_OK) {
+    ch_adjoint_release(G);
+    return r;
+  }
   CK(cudaMemsetAsync(G->a_mu, 0, (size_t)3 * G->fs * sizeof(double2), G->stream));
   return CH_OK;
 }
@@ -179,7 +182,8 @@ int adjoint_step_impl(ch_grid* G, const void* state, cudaEvent_t* ev) {
   chf::StateHeader h;
   const char* b = (const char*)state;
   CK(cudaMemcpyAsync(&h, b, sizeof(h), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  const int r = ch_sync_status(G);   // of the reverse steps before this one
+  if (r != CH_OK) return r;
   if (h.magic != chf::kStateMagic || h.nx != g.nx || h.ny != g.ny || h.nz != g.nz ||
       !h.fields_set)
     return CH_ERR_ARG;
@@ -228,7 +232,7 @@ int ch_adjoint_step_timed(ch_grid* G, const void* state, double* kernel_ms) {
   }
   for (int i = 0; i <= CH_ADJ_KERNELS; ++i) cudaEventDestroy(ev[i]);
   if (st == CH_ERR_CUDA) cudaGetLastError();
-  return st;
+  return st != CH_OK ? st : ch_sync_status(G);
 }
 
 int ch_adjoint_segment(ch_grid* G, const void* checkpoint, int nsteps) {
@@ -252,8 +256,10 @@ int ch_adjoint_segment(ch_grid* G, const void* checkpoint, int nsteps) {
     G->seg_cap = nsteps;
   }
   char* seg = (char*)G->seg_block;
+  int r = ch_sync_status(G);                 // of the segments before this one
+  if (r != CH_OK) return r;
   // recompute the segment from its checkpoint, keeping each state's y-padded fields
-  int r = ch_set_state(G, checkpoint);       // also evaluates the fields of the first state
+  r = ch_set_state(G, checkpoint);           // also evaluates the fields of the first state
   if (r != CH_OK) return r;
   std::vector<int> first((size_t)nsteps);
   for (int k = 0; k < nsteps; ++k) {
@@ -283,8 +289,10 @@ int ch_adjoint_gradient(ch_grid* G, double* gu, double* gv, double* gw, double* 
 
 int ch_adjoint_end(ch_grid* G) {
   if (!G) return CH_ERR_ARG;
+  if (!G->adj_block) return CH_OK;
+  const int r = ch_sync_status(G);   // of the gradient and the reverse steps
   ch_adjoint_release(G);
-  return CH_OK;
+  return r;
 }
 
 }  // extern "C"

@@ -575,6 +575,13 @@ int ch_z_to_rows(ch_grid* G, const double2* in, double2* tmp, int nf, double* co
   return CH_OK;
 }
 int ch_eval_nonlinear(ch_grid* G) { return eval_nonlinear_impl(G); }
+int ch_sync_status(ch_grid* G) {
+  int te = 0;
+  if (G->tc_err)
+    CK(cudaMemcpyAsync(&te, G->tc_err, sizeof(int), cudaMemcpyDeviceToHost, G->stream));
+  CK(cudaStreamSynchronize(G->stream));
+  return te ? CH_ERR_TIMEOUT : CH_OK;
+}
 
 extern "C" {
 
@@ -908,7 +915,7 @@ int ch_step_timed(ch_grid* G, int nsteps, double* kernel_ms, double* total_ms) {
   if (kernel_ms)
     for (int k = 0; k < NKER; ++k) kernel_ms[k] = ks[k];
   *total_ms = tot;
-  return st;
+  return st != CH_OK ? st : ch_sync_status(G);
 }
 
 int ch_get_fields(ch_grid* G, double* u, double* v, double* w, double* phi) {
@@ -936,8 +943,7 @@ int ch_get_fields_host(ch_grid* G, double* u, double* v, double* w, double* phi)
   double* f4[4] = {u, v, w, phi};
   for (int f = 0; f < 4; ++f)
     CK(cudaMemcpyAsync(f4[f], G->phys7 + f * G->fsp, b, cudaMemcpyDeviceToHost, G->stream));
-  CK(cudaStreamSynchronize(G->stream));
-  return CH_OK;
+  return ch_sync_status(G);
 }
 
 int ch_diagnostics(ch_grid* G, ch_diag* out) {
@@ -950,12 +956,8 @@ int ch_diagnostics(ch_grid* G, ch_diag* out) {
                       G->tab + 5 * nz, G->diag_part, G->diag_out, G->stream));
   double h[8];
   CK(cudaMemcpyAsync(h, G->diag_out, 7 * sizeof(double), cudaMemcpyDeviceToHost, G->stream));
-  CK(cudaStreamSynchronize(G->stream));
-  if (G->tc_err) {
-    int te = 0;
-    CK(cudaMemcpy(&te, G->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (te) return CH_ERR_TIMEOUT;
-  }
+  r = ch_sync_status(G);
+  if (r != CH_OK) return r;
   out->t = G->t;
   out->step = G->nstep;
   out->mass = h[0];
@@ -995,8 +997,7 @@ int ch_get_state(ch_grid* G, void* buf) {
   const double2* src[6] = {G->om, G->w, G->phi, G->hom, G->hw, G->hphi};
   for (int i = 0; i < 6; ++i)
     CK(cudaMemcpyAsync(b + sizeof(h) + i * sb, src[i], sb, cudaMemcpyDeviceToDevice, G->stream));
-  CK(cudaStreamSynchronize(G->stream));
-  return CH_OK;
+  return ch_sync_status(G);
 }
 
 int ch_set_state(ch_grid* G, const void* buf) {
@@ -1209,16 +1210,9 @@ int ch_fp64_fma_rate(double* tflops) {
 
 int ch_device_status(ch_grid* G) {
   if (!G) return CH_ERR_ARG;
-  CK(cudaStreamSynchronize(G->stream));
-  if (G->tc_err) {
-    int te = 0;
-    CK(cudaMemcpy(&te, G->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (te) {
-      CK(cudaMemset(G->tc_err, 0, sizeof(int)));
-      return CH_ERR_TIMEOUT;
-    }
-  }
-  return CH_OK;
+  const int r = ch_sync_status(G);
+  if (r == CH_ERR_TIMEOUT) CK(cudaMemsetAsync(G->tc_err, 0, sizeof(int), G->stream));
+  return r;
 }
 
 }  // extern "C"

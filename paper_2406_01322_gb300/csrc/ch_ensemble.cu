@@ -399,6 +399,16 @@ int timed_steps(ch_ensemble* E, int nsteps, double* stage_ms, double* total_ms) 
   return st;
 }
 
+// synchronises: CH_ERR_TIMEOUT while a member's device-wait flag is set
+int members_status(ch_ensemble* E) {
+  int st = CH_OK;
+  for (ch_grid* G : E->members) {
+    const int r = ch_sync_status(G);
+    if (st == CH_OK) st = r;
+  }
+  return st;
+}
+
 }  // namespace
 
 extern "C" {
@@ -558,7 +568,8 @@ int ch_ensemble_step_timed(ch_ensemble* E, int nsteps, double* stage_ms, double*
   if (!E || nsteps < 0 || !total_ms) return CH_ERR_ARG;
   for (ch_grid* G : E->members)
     if (!G->fields_set) return CH_ERR_STATE;
-  return timed_steps(E, nsteps, stage_ms, total_ms);
+  const int st = timed_steps(E, nsteps, stage_ms, total_ms);
+  return st != CH_OK ? st : members_status(E);
 }
 
 int ch_ensemble_autotune(ch_ensemble* E, int reps) {
@@ -626,6 +637,7 @@ int ch_ensemble_autotune(ch_ensemble* E, int reps) {
     cudaGetLastError();
     if (st == CH_OK) st = CH_ERR_CUDA;
   }
+  if (st == CH_OK) st = members_status(E);   // (the states are restored by now)
   for (int i = 0; i < n; ++i)
     if (saved[i]) efree(E, saved[i]);
   drop_graph(E);

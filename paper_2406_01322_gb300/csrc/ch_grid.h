@@ -111,6 +111,9 @@ inline bool ch_z_coef(const ch_grid* G) { return G->cheb == CH_CHEB_TC || G->z_a
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev);
 int ch_eval_nonlinear(ch_grid* G);
+// synchronises the stream: CH_ERR_TIMEOUT while the flag of the bounded device waits is set (it stays
+// set until ch_device_status), else CH_OK
+int ch_sync_status(ch_grid* G);
 // bw <- the five backward fields u v w phi D phi of the state, as the step itself forms them
 cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s);
 // the x/y stages of the step on stream s: 3 y backward (bw -> ya), 4 x line (ya -> yb), 5 y
