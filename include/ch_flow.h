@@ -118,9 +118,9 @@ int ch_set_fields_host(ch_grid* g, const double* u, const double* v, const doubl
 /* Advance nsteps full time steps (Sec. 2.2 steps i)-v)), asynchronously on the stream.  After
  * the first step the per-step launch sequence is replayed from a captured CUDA graph.
  * Float64 grids of at least 2^15 modes (nx/2 ny nz) and padded lengths up to
- * 1024 do their x and y transforms as exact-split products on the tensor cores (float64-accurate;
- * nine real padded fields of extra memory; the FFT kernels if that memory is not to be had); the
- * radix schedules of ch_set_fft_pruning do not apply to them. */
+ * 1024 (and nz <= 496) do their x and y transforms as exact-split products on the tensor cores
+ * (float64-accurate; the FFT kernels if the memory for the matrices is not to be had); the radix
+ * schedules of ch_set_fft_pruning do not apply to them. */
 int ch_step(ch_grid* g, int nsteps);
 
 /* The kernels of one time step in the order ch_step_timed reports them in: zrhs (DCT,
@@ -252,7 +252,8 @@ int ch_nonlinear(ch_grid* g, double* out9);
  * with respect to the physical initial fields u, v, w, phi given to ch_set_fields.
  * ch_objective: J of the current state (host double; synchronises the stream).
  * ch_adjoint_begin: allocates the reverse-sweep workspace (24 spectral fields plus six y-padded
- *   fields, with the grid's allocator) and seeds the sweep with dJ/ds of the CURRENT state (the
+ *   fields, with the grid's allocator; nine real padded fields more where the x transforms run on the
+ *   tensor cores, by FFT if that memory is not to be had) and seeds the sweep with dJ/ds of the CURRENT state (the
  *   final state of the forward run); *J receives J (may be NULL).
  * ch_adjoint_step: reverses ONE forward step.  `state` is a device buffer written by
  *   ch_get_state just before that forward step; steps are reversed last to first.  The handle's

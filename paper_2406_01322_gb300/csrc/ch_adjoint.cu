@@ -64,6 +64,11 @@ void ch_adjoint_release(ch_grid* G) {
   if (G->ff) G->ff(G->adj_block, G->actx);
   else if (!G->af) cudaFree(G->adj_block);
   G->adj_block = nullptr;
+  if (G->a_phys) {
+    if (G->ff) G->ff(G->a_phys, G->actx);
+    else if (!G->af) cudaFree(G->a_phys);
+    G->a_phys = nullptr;
+  }
   G->a_lam = G->a_L = G->a_Rb = G->a_mu = G->a_mu2 = G->a_nlb = G->a_x6 = G->a_bb = nullptr;
   if (G->seg_block) {
     if (G->ff) G->ff(G->seg_block, G->actx);
@@ -109,6 +114,13 @@ int ch_adjoint_begin(ch_grid* G, double* J) {
     G->a_nlb = b + 15 * fs;
     G->a_x6 = b + 24 * fs;
     G->a_bb = G->a_x6 + 6 * G->fsy;
+  }
+  if (G->use_tx && !G->a_phys) {   // without room for it the x line runs by FFT
+    const size_t bytes = (size_t)kNl * G->g.Px * G->g.Py * G->g.nz * sizeof(double);
+    void* p = nullptr;
+    if (G->af) p = G->af(bytes, G->actx);
+    else if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
+    G->a_phys = (double*)p;
   }
   // lambda_K = dJ/ds_K, mu_{K-1} = 0 (the last history is not used by J)
   int r = objective_impl(G, G->a_L, J);

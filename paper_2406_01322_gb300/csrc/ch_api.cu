@@ -433,12 +433,14 @@ int setup_tx(ch_grid* G) {
     release_last(G, G->allocs.size() - before);
     return CH_OK;
   }
-  if (padded)
-    t.phys = (double*)galloc(G, (size_t)kNl * g.Px * g.Py * g.nz * sizeof(double));
-  if (!t.phys) cudaGetLastError();
+  // the x line's nine padded physical fields (9/4 of an unpadded one): three each in the buffers of seven
+  // unpadded fields that serve the calls between steps and the Chebyshev coefficients
+  for (int f = 0; f < 9; ++f)
+    t.phys[f] = (f < 3 ? (double*)G->auxA : f < 6 ? (double*)G->auxB : G->phys7) +
+                (long long)(f % 3) * g.Px * g.Py * g.nz;
   G->tx = t;
   G->use_ax = 1;
-  G->use_tx = t.phys != nullptr;
+  G->use_tx = padded;
   return CH_OK;
 }
 
@@ -532,14 +534,9 @@ cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out
 
 cudaError_t ch_launch_x_adj(ch_grid* G, const double2* ya, double2* out6, cudaStream_t s) {
   const GridDev& g = G->g;
-  if (!G->use_tx || !G->tx_xb1.dig)
+  if (!G->use_tx || !G->tx_xb1.dig || !G->a_phys)
     return chf::launch_adj_xline(g, ya, (const double2*)G->yb, out6, G->fsy, G->px[0], s);
-  // the padded physical fields (9/4 of an unpadded one) use the buffers of seven unpadded fields that
-  // the reverse step does not need here
-  const long long np = (long long)g.Px * g.Py * g.nz;
-  double *a = (double*)G->auxA, *b = (double*)G->auxB;
-  double* const phys7[7] = {a, a + np, a + 2 * np, b, b + np, b + 2 * np, G->phys7};
-  return chf::launch_txy_adj_x(g, ya, G->yb, out6, G->fsy, phys7, G->tx, G->tx_xb1, s);
+  return chf::launch_txy_adj_x(g, ya, G->yb, out6, G->fsy, G->a_phys, G->tx, G->tx_xb1, s);
 }
 
 // the reverse sweep's own plans, made once; without room for them the FFT kernels run

@@ -323,7 +323,7 @@ struct Txy {
   TxyPlan ybu, yfu, xbu, xfu;      // the same on the unpadded grid (yfu: times 1 / (Nx Ny))
   char* keep = nullptr;            // per persistent CTA: keep_bytes of fixed-point values
   size_t keep_bytes = 0;
-  double* phys = nullptr;          // nine real fields (Px, Py, Nz)
+  double* phys[9] = {};            // nine real fields (Px, Py, Nz), scratch of the x line
   int ctas = 0;
   int* err = nullptr;              // |= 1 if a bounded wait gave up
 };
@@ -347,10 +347,10 @@ cudaError_t launch_txy_rows(int dir, const GridDev& g, double* const* phys, doub
                             cudaStream_t s);
 cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long long fs, const Txy& x,
                          cudaStream_t s);
-// transposed x line; phys7: scratch, seven real fields (Px, Py, Nz); xb1: x backward plan of scale 1;
-// overwrites pb9
+// transposed x line; adj9: scratch, nine real fields (Px, Py, Nz) besides x.phys; xb1: x backward plan
+// of scale 1; overwrites pb9
 cudaError_t launch_txy_adj_x(const GridDev& g, const void* in6, void* pb9, void* out6, long long fs,
-                             double* const* phys7, const Txy& x, const TxyPlan& xb1, cudaStream_t s);
+                             double* adj9, const Txy& x, const TxyPlan& xb1, cudaStream_t s);
 // one bounded mbarrier wait that runs out on purpose (sets *err |= 1 after the wait bound)
 cudaError_t launch_wait_selftest(int* err, int nwaits, cudaStream_t s);
 // float64 FMA-rate probe: `blocks` CTAs of 256 threads, `iters` iterations of eight independent

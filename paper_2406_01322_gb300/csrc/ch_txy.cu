@@ -630,23 +630,25 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
 // The nine products (in place: seven physical fields u v w phi phi_x phi_y phi_z in, Sxx - Szz,
 // Syy - Szz, Sxy, Sxz, Syz, phi^3, u phi, v phi, w phi out) of n samples per field.  About 20
 // float64 operations per sample: bound by the float64 pipe and by HBM about equally.
-__global__ void __launch_bounds__(256) products_kernel(double* __restrict__ f, long long n,
-                                                       double kappa) {
+struct Phys9 {
+  double* f[9];
+};
+__global__ void __launch_bounds__(256) products_kernel(const Phys9 p, long long n, double kappa) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const double u = f[i], v = f[n + i], w = f[2 * n + i], ph = f[3 * n + i];
-    const double fx = f[4 * n + i], fy = f[5 * n + i], fz = f[6 * n + i];
+    const double u = p.f[0][i], v = p.f[1][i], w = p.f[2][i], ph = p.f[3][i];
+    const double fx = p.f[4][i], fy = p.f[5][i], fz = p.f[6][i];
     const double kx = kappa * fx, ky = kappa * fy, kz = kappa * fz;
     const double wz = fma(w, w, kz * fz);
-    f[i] = fma(-u, u, fma(-kx, fx, wz));
-    f[n + i] = fma(-v, v, fma(-ky, fy, wz));
-    f[2 * n + i] = -fma(u, v, kx * fy);
-    f[3 * n + i] = -fma(u, w, kx * fz);
-    f[4 * n + i] = -fma(v, w, ky * fz);
-    f[5 * n + i] = ph * ph * ph;
-    f[6 * n + i] = u * ph;
-    f[7 * n + i] = v * ph;
-    f[8 * n + i] = w * ph;
+    p.f[0][i] = fma(-u, u, fma(-kx, fx, wz));
+    p.f[1][i] = fma(-v, v, fma(-ky, fy, wz));
+    p.f[2][i] = -fma(u, v, kx * fy);
+    p.f[3][i] = -fma(u, w, kx * fz);
+    p.f[4][i] = -fma(v, w, ky * fz);
+    p.f[5][i] = ph * ph * ph;
+    p.f[6][i] = u * ph;
+    p.f[7][i] = v * ph;
+    p.f[8][i] = w * ph;
   }
 }
 
@@ -683,10 +685,7 @@ __global__ void __launch_bounds__(256) combine_kernel(double2* __restrict__ f, l
 // Transposed Jacobian of the nine products, point by point: the fields u v w phi phi_x phi_y phi_z
 // (p, in) and the product adjoints b (nine fields of n samples) give the fields' adjoints (p, out).
 // 33 float64 operations per sample (0.34 ms at 192 x 192 x 129 samples) bound it.
-struct Phys7 {
-  double* f[7];
-};
-__global__ void __launch_bounds__(256) adj_products_kernel(const Phys7 p,
+__global__ void __launch_bounds__(256) adj_products_kernel(const Phys9 p,
                                                            const double* __restrict__ b, long long n,
                                                            double kappa) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -869,7 +868,7 @@ cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long lon
   const int src[7] = {0, 1, 2, 3, 3, 4, 5};   // u v w phi (phi -> i kx phi) phi_y phi_z
   for (int f = 0; f < 7; ++f) {
     a.in[f] = (const double*)in6 + 2 * src[f] * fs;
-    a.out[f] = x.phys + f * np;
+    a.out[f] = x.phys[f];
   }
   a.dmask = 1u << 4;
   a.kscale = 6.283185307179586476925 / g.lx;
@@ -880,12 +879,14 @@ cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long lon
   a.t = x.xb;
   cudaError_t e = launch_mode<XB>(a, 7, x, s);
   if (e != cudaSuccess) return e;
+  Phys9 p;
+  memcpy(p.f, x.phys, sizeof p.f);
   products_kernel<<<(unsigned)std::min<long long>((np + 255) / 256, (long long)x.ctas * 32), 256, 0, s>>>(
-      x.phys, np, g.kappa);
+      p, np, g.kappa);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   for (int f = 0; f < 9; ++f) {
-    a.in[f] = x.phys + f * np;
+    a.in[f] = x.phys[f];
     a.out[f] = (double*)out9 + 2 * f * fs;
   }
   a.dmask = 0;
@@ -899,7 +900,7 @@ cudaError_t launch_txy_x(const GridDev& g, const void* in6, void* out9, long lon
 // the padded backward transform (a forward transform with the modes k >= 1 doubled); phi_x's adjoint
 // folds into phi's.  At 128^3 the five launches take 1.3 ms in place of the 3.3 of the FFT kernel.
 cudaError_t launch_txy_adj_x(const GridDev& g, const void* in6, void* pb9, void* out6, long long fs,
-                             double* const* phys7, const Txy& x, const TxyPlan& xb1, cudaStream_t s) {
+                             double* adj9, const Txy& x, const TxyPlan& xb1, cudaStream_t s) {
   const int Q = g.Py * g.nz;
   const long long np = (long long)g.Px * Q;
   const double kxs = 6.283185307179586476925 / g.lx;
@@ -908,7 +909,7 @@ cudaError_t launch_txy_adj_x(const GridDev& g, const void* in6, void* pb9, void*
   const int src[7] = {0, 1, 2, 3, 3, 4, 5};
   for (int f = 0; f < 7; ++f) {
     a.in[f] = (const double*)in6 + 2 * src[f] * fs;
-    a.out[f] = phys7[f];
+    a.out[f] = x.phys[f];
   }
   a.dmask = 1u << 4;
   a.kscale = kxs;
@@ -921,18 +922,18 @@ cudaError_t launch_txy_adj_x(const GridDev& g, const void* in6, void* pb9, void*
   if (e != cudaSuccess) return e;
   for (int f = 0; f < 9; ++f) {
     a.in[f] = (const double*)pb9 + 2 * f * fs;
-    a.out[f] = x.phys + f * np;
+    a.out[f] = adj9 + f * np;
   }
   a.dmask = 0;
   a.t = xb1;
   if ((e = launch_mode<XB>(a, 9, x, s)) != cudaSuccess) return e;
-  Phys7 p;
-  for (int f = 0; f < 7; ++f) p.f[f] = phys7[f];
+  Phys9 p;
+  memcpy(p.f, x.phys, sizeof p.f);
   adj_products_kernel<<<(unsigned)std::min<long long>((np + 255) / 256, (long long)x.ctas * 32), 256, 0,
-                        s>>>(p, x.phys, np, g.kappa);
+                        s>>>(p, adj9, np, g.kappa);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (int f = 0; f < 7; ++f) {
-    a.in[f] = phys7[f];
+    a.in[f] = x.phys[f];
     a.out[f] = f == 4 ? (double*)pb9 : (double*)out6 + 2 * src[f] * fs;
   }
   a.lift = 1;
