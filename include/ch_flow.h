@@ -309,20 +309,21 @@ int ch_render_interface(ch_grid* g, unsigned char* rgb, double* depth, int width
  * (created here with the given allocator and stream; all members share one `precision`, any of
  * the three; CH_ERR_ARG if they differ).  One ensemble step advances every member by one time
  * step with six grouped persistent launches (one per stage; their CTAs walk a work list spanning
- * all members; two more per member whose Chebyshev transforms run on the tensor cores; members with
- * and without get a zrhs and a zbwd launch of their own), captured once into a CUDA graph and
- * replayed.  Members are set, read and diagnosed through their ch_grid handles
+ * all members; two more per member whose Chebyshev transforms run on the tensor cores, and members
+ * with and without get a zrhs and a zbwd launch of their own; members whose x and y transforms run
+ * there, see ch_step, make the six launches of those stages themselves and leave the grouped ones to
+ * the others), captured once into a CUDA graph and replayed.  Members are set, read and diagnosed through their ch_grid handles
  * (ch_ensemble_member); ch_ensemble_step needs every member set.  ch_ensemble_autotune times the
  * transforms' radix schedules and the persistent CTAs per SM of each stage on the live members
- * (their states are saved and restored bit for bit) and keeps the fastest; the choice is cached
- * per size signature for the process.  ch_ensemble_tuning writes the choice as a JSON object. */
+ * (their states are saved and restored bit for bit) and keeps the fastest (a stage without grouped
+ * members keeps its defaults); the choice is cached per size signature for the process.  ch_ensemble_tuning writes the choice as a JSON object. */
 typedef struct ch_ensemble ch_ensemble;
 int ch_ensemble_init(const ch_params* members, int n, ch_alloc_fn alloc, ch_free_fn free_fn,
                      void* alloc_ctx, void* stream, ch_ensemble** out);
 int ch_ensemble_size(const ch_ensemble* e);
 int ch_ensemble_member(ch_ensemble* e, int i, ch_grid** out);
 int ch_ensemble_step(ch_ensemble* e, int nsteps);
-/* as ch_ensemble_step with events between the six grouped launches (stream synchronised):
+/* as ch_ensemble_step with events between the six stages (stream synchronised):
  * stage_ms[0..CH_ENSEMBLE_STAGES-1] summed per stage (zrhs zsolve zbwd y backward x line
  * y forward), *total_ms over all steps */
 #define CH_ENSEMBLE_STAGES 6

@@ -95,7 +95,9 @@ namespace {
 
 constexpr int kStages = CH_ENSEMBLE_STAGES;
 // work lists: the six stages, then zrhs and zbwd of the members whose z transforms run on the tensor
-// cores (ch_z_coef; the others are in lists 0 and 2, so that every member steps as it would alone)
+// cores (ch_z_coef; the others are in lists 0 and 2, so that every member steps as it would alone).
+// Members whose x and y transforms run there (use_tx) are in none of the lists 3 to 5: each launches
+// those stages itself, the others stay grouped.
 constexpr int kLists = kStages + 2;
 int stage_of(int list) { return list < kStages ? list : list == kStages ? 0 : 2; }
 
@@ -132,8 +134,6 @@ struct ch_ensemble {
   int zsolve_tile;
   int ywq;                      // warp-FFT level of the grouped y passes (ensemble_ywq)
   int xwq;                      // the same for the grouped x line (padded x lengths)
-  int tx;                       // 1: a member's x/y stages run on the tensor cores; then every
-                                // member runs its own launches of those stages
   Tuning tune;
   std::string signature;
   cudaGraphExec_t gexec;
@@ -235,6 +235,7 @@ int build_descriptors(ch_ensemble* E) {
     for (int i = 0; i < n; ++i) {
       b[i + 1] = b[i];
       if ((s == 0 || s == 2) && (int)E->zc[i] != coef) continue;
+      if (s >= 3 && E->members[i]->use_tx) continue;
       b[i + 1] += chf::stage_items(s, E->hmem[i], E->prec);
       const size_t sm = chf::stage_smem(s, E->hmem[i], E->prec, coef);
       if (sm > mx) mx = sm;
@@ -292,22 +293,21 @@ cudaError_t member_transforms(ch_ensemble* E, int dir, cudaStream_t s) {
 }
 
 // one ensemble step: the six grouped stages, zrhs and zbwd in one launch per kind of member; the
-// members' transforms run before stage 0 and after stage 2 and are timed with those stages
+// members' own transforms run before stage 0, after stage 2 and after the grouped part of stages 3 to 5,
+// and are timed with those stages (float64, thirty members of 32 x 32 x 33 beside one of 64 x 64 x 17 or
+// 128 x 128 x 129: 4.78 and 6.94 ms a step with every member launching them itself, 4.08 and 6.25 so)
 int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
   const int n = (int)E->members.size();
   for (int st = 0; st < kStages; ++st) {
     cudaError_t e = cudaSuccess;
     if (st == 0) e = member_transforms(E, 0, s);
-    if (e == cudaSuccess && st >= 3 && E->tx) {
-      for (ch_grid* G : E->members)
-        if (e == cudaSuccess) e = ch_launch_xy(G, st, s);
-    } else {
-      for (int l = 0; l < kLists && e == cudaSuccess; ++l)
-        if (stage_of(l) == st && list_items(E, l) > 0)
-          e = chf::launch_grouped(st, E->prec, E->dmem, E->dbegin + (size_t)l * (n + 1), n,
-                                  grid_of(E, l), E->smem[l], E->zsolve_tile, l >= kStages,
-                                  st == 4 ? E->xwq : E->ywq, s);
-    }
+    for (int l = 0; l < kLists && e == cudaSuccess; ++l)
+      if (stage_of(l) == st && list_items(E, l) > 0)
+        e = chf::launch_grouped(st, E->prec, E->dmem, E->dbegin + (size_t)l * (n + 1), n,
+                                grid_of(E, l), E->smem[l], E->zsolve_tile, l >= kStages,
+                                st == 4 ? E->xwq : E->ywq, s);
+    for (size_t i = 0; i < E->members.size() && st >= 3 && e == cudaSuccess; ++i)
+      if (E->members[i]->use_tx) e = ch_launch_xy(E->members[i], st, s);
     if (e == cudaSuccess && st == 2) e = member_transforms(E, 1, s);
     if (ev) cudaEventRecord(ev[st], s);
     if (e != cudaSuccess) {
@@ -320,10 +320,11 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
 
 void compute_occupancy(ch_ensemble* E) {
   std::vector<int> py, px;
-  for (ch_grid* G : E->members) {
-    py.push_back(G->g.Py);
-    px.push_back(G->g.Px);
-  }
+  for (ch_grid* G : E->members)
+    if (!G->use_tx) {
+      py.push_back(G->g.Py);
+      px.push_back(G->g.Px);
+    }
   E->ywq = chf::ensemble_ywq(py, E->prec);
   E->xwq = chf::ensemble_ywq(px, E->prec);
   for (int l = 0; l < kLists; ++l)
@@ -343,7 +344,6 @@ std::string signature_of(const ch_ensemble* E) {
   snprintf(b, sizeof(b), "p%d/c%d", E->prec, E->z_auto ? 2 : E->cheb);
   return sig + b;
 }
-
 
 void drop_graph(ch_ensemble* E) {
   if (E->graph_ok) cudaGraphExecDestroy(E->gexec);
@@ -444,11 +444,7 @@ int ch_ensemble_init(const ch_params* members, int n, ch_alloc_fn alloc, ch_free
     if (st == CH_OK) E->members.push_back(G);
   }
   if (st == CH_OK) E->signature = signature_of(E);
-  E->tx = 0;
-  for (ch_grid* G : E->members) {
-    E->tx |= G->use_tx;
-    E->zc.push_back((char)ch_z_coef(G));
-  }
+  for (ch_grid* G : E->members) E->zc.push_back((char)ch_z_coef(G));
   if (st == CH_OK) {
     E->dmem = (Member*)ealloc(E, n * sizeof(Member));
     E->dbegin = (int*)ealloc(E, (size_t)kLists * (n + 1) * sizeof(int));
@@ -602,7 +598,9 @@ int ch_ensemble_autotune(ch_ensemble* E, int reps) {
     cost[1][style] = stage_ms[3] + stage_ms[5];
     cost[2][style] = stage_ms[0] + stage_ms[2];
   }
+  // (a schedule that no member's grouped x or y stage uses stays as it is: only noise would choose it)
   for (int k = 0; k < 3 && st == CH_OK; ++k) {
+    if (k < 2 && list_items(E, 4 - k) == 0) continue;
     int b = 0;
     for (int style = 1; style < (k < 2 ? 4 : 3); ++style)
       if (cost[k][style] < cost[k][b]) b = style;
@@ -619,7 +617,7 @@ int ch_ensemble_autotune(ch_ensemble* E, int reps) {
     if (st == CH_OK) st = upload(E);
     if (st == CH_OK) st = timed_steps(E, reps, stage_ms, &tot);
     for (int s = 0; s < kStages && st == CH_OK; ++s)
-      if (stage_ms[s] < bestms[s]) {
+      if ((s < 3 || list_items(E, s) > 0) && stage_ms[s] < bestms[s]) {
         bestms[s] = stage_ms[s];
         best.ctas_per_sm[s] = cand[c];
       }
