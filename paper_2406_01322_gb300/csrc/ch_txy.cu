@@ -46,6 +46,7 @@ constexpr int kPW = 8, kEW = 8, kSW = 3;               // producer, epilogue and
 constexpr int kThreads = 32 * (kPW + kEW + 1 + kSW);   // epilogue 0..7, producers, issuer, scan
 constexpr int kMaxStages = 6;
 constexpr int kMaxFields = 9;
+constexpr int kMaxSlices = 8;   // transforms of up to 1024 points
 // tiles whose row scales are held: the scan runs at most this far ahead (with three, and an L2
 // prefetch of a fourth, tiles left L2 before they were converted: 256x256x129 y forward 1.75 ms
 // against 1.49)
@@ -65,6 +66,9 @@ struct Args {
   unsigned dmask;             // output fields of i k times the input
   double kscale;              // k of mode 1
   int nlines, tpf, ntiles;    // lines per field, tiles per field, tiles
+  // SPLIT: the output slices of a tile are shared by gridDim.y CTAs, cut[blockIdx.y] ..
+  // cut[blockIdx.y + 1] - 1
+  short cut[kMaxSlices + 1];
   // line l starts at element (l / ld) ihs + (l % ld) ils of the input (complex elements; real
   // samples for XF) and (l / ld) ohs + (l % ld) ols of the output (real samples for XB)
   int ld;
@@ -187,7 +191,9 @@ __device__ __forceinline__ void epilogue_pass(const Args& A, uint32_t tb, int CW
   }
 }
 
-template <int MODE>
+// SPLIT: several CTAs to a tile (its own instantiation: with the passes' bounds at run time in the only
+// one, the x line of 128 x 128 x 129 went from 0.81 to 0.84 ms)
+template <int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant__ Args A) {
   constexpr bool CPX = MODE == YB || MODE == YF;   // rows: re and im of 64 lines; else 128 lines
   constexpr int LPT = CPX ? kRows / 2 : kRows;     // lines per tile
@@ -195,6 +201,9 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
   constexpr int OSC = MODE == XB ? 1 : 2;
   extern __shared__ __align__(1024) unsigned char tsm[];
   const int NT = A.t.NT, ns = A.t.stages, nst = A.t.nst;
+  // this CTA's passes
+  const int pp0 = SPLIT ? 2 * A.cut[blockIdx.y] : 0;
+  const int pp1 = SPLIT ? 2 * A.cut[blockIdx.y + 1] : 2 * A.t.nsl;
   const int sbytes = stage_bytes(NT);
   unsigned char* stages = tsm;
   // the recombined cosine products of a pass, per epilogue thread (in L2 instead, with room for five
@@ -287,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *sT;
   const uint32_t sBase = su32(stages);
-  char* kcta = A.keep + (long long)blockIdx.x * A.keep_bytes;
+  char* kcta = A.keep + (long long)(SPLIT ? blockIdx.y * gridDim.x + blockIdx.x : blockIdx.x) * A.keep_bytes;
   Waiter W;
 
   if (issuer_warp) {
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       uint32_t slot = 0, use = 0, pass = 0;
       bool any = false;
       for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x)
-        for (int pp = 0; pp < 2 * A.t.nsl; ++pp)
+        for (int pp = pp0; pp < pp1; ++pp)
           for (int c = 0; c < A.t.kc; ++c, ++pass) {
             if (pass > 0 && !W.wait(barAccFree, (pass - 1) & 1)) goto drain;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -498,7 +507,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
         else convert(std::false_type());
         if (st + 1 < nst) load(st + 1);
         store_keep(keep_at(1, st), dd);
-        if (A.t.nsl > 1) store_keep(keep_at(0, st), s);
+        if (SPLIT ? (int)gridDim.y < A.t.nsl : A.t.nsl > 1) store_keep(keep_at(0, st), s);   // more than one slice
         if (MODE == YB || MODE == XB) {
 #pragma unroll
           for (int e = 0; e < NE; ++e) {
@@ -507,10 +516,10 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           }
           if (st == 0) s0 = s[0];
         }
-        ok = put(s, A.t.dig + (size_t)st * bstride);
+        ok = put(s, A.t.dig + ((size_t)pp0 * nst + st) * bstride);
       }
       if (!ok) break;
-      if ((MODE == YB || MODE == XB) && !(A.P & 1)) {
+      if ((MODE == YB || MODE == XB) && !(A.P & 1) && (!SPLIT || blockIdx.y == 0)) {
         // output n = P / 2: sum_k (-1)^k s_k (YB, and XB of unit weights), 2 sum_k (-1)^k Re c_k -
         // Re c_0 (XB);
         // (-1)^k = (-1)^g.  High and low words are added apart.
@@ -546,7 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           }
         }
       }
-      for (int pp = 1; pp < 2 * A.t.nsl && ok; ++pp) {
+      for (int pp = pp0 + 1; pp < pp1 && ok; ++pp) {
         longlong2 nx[4];
         auto fetch = [&](int st) {
           const longlong2* s = keep_at(pp & 1, st);
@@ -604,7 +613,7 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
       const int lh = line / A.ld, ll = line - lh * A.ld;
       double* dst = A.out[fld] + (rowok ? lh * A.ohs + ll * A.ols : 0) * OSC + part_c;
       bool ok = true;
-      for (int pp = 0; pp < 2 * A.t.nsl && ok; ++pp) {
+      for (int pp = pp0; pp < pp1 && ok; ++pp) {
         const int m0 = (pp >> 1) * NT + cg * CW;
         for (int c = 0; c < A.t.kc; ++c, ++pass) {
           if (!(ok = W.wait_warp(barAccFull, pass & 1))) break;
@@ -728,8 +737,9 @@ size_t plan_smem(int NT, int ns) {
 
 template <int MODE> cudaError_t launch_mode(Args& a, int nf, const Txy& x, cudaStream_t s) {
   constexpr int LPT = MODE == YB || MODE == YF ? kRows / 2 : kRows;
-  static SmemLimit cur;
-  cudaError_t e = ensure_smem(txy_kernel<MODE>, a.t.smem, &cur);
+  static SmemLimit cur[2];
+  cudaError_t e = ensure_smem(txy_kernel<MODE, false>, a.t.smem, &cur[0]);
+  if (e == cudaSuccess) e = ensure_smem(txy_kernel<MODE, true>, a.t.smem, &cur[1]);
   if (e != cudaSuccess) return e;
   a.tpf = (a.nlines + LPT - 1) / LPT;
   a.ntiles = a.tpf * nf;
@@ -737,7 +747,17 @@ template <int MODE> cudaError_t launch_mode(Args& a, int nf, const Txy& x, cudaS
   a.keep_bytes = (long long)x.keep_bytes;
   a.err = x.err;
   if (a.ntiles <= 0) return cudaSuccess;
-  txy_kernel<MODE><<<std::min(a.ntiles, x.ctas), kThreads, a.t.smem, s>>>(a);
+  // Rule: as many CTAs to a tile as all tiles find an SM each, up to one per output slice (its cosine and
+  // sine products meet in shared memory); each converts the tile's rows again.  One CTA a tile / this, us:
+  // y backward 16 x 648 x 65 (54 tiles, two CTAs each) 607 / 360, 8 x 648 x 17 (12 tiles, eight) 598 / 163;
+  // x backward, products and x forward of 512 x 24 x 9 (21 and 27 tiles) 690 / 263.
+  const int parts = std::max(1, std::min(std::min(a.t.nsl, kMaxSlices), x.ctas / a.ntiles));
+  if (parts == 1) {
+    txy_kernel<MODE, false><<<std::min(a.ntiles, x.ctas), kThreads, a.t.smem, s>>>(a);
+  } else {
+    for (int i = 0; i <= parts; ++i) a.cut[i] = (short)(i * a.t.nsl / parts);
+    txy_kernel<MODE, true><<<dim3(a.ntiles, parts), kThreads, a.t.smem, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
