@@ -119,8 +119,8 @@ int ch_set_fields_host(ch_grid* g, const double* u, const double* v, const doubl
  * the first step the per-step launch sequence is replayed from a captured CUDA graph.
  * Float64 grids of at least 2^15 modes (nx/2 ny nz) and padded lengths up to
  * 1024 (and nz <= 496) do their x and y transforms as exact-split products on the tensor cores
- * (float64-accurate; the FFT kernels if the memory for the matrices is not to be had); the radix
- * schedules of ch_set_fft_pruning do not apply to them. */
+ * (float64-accurate; y passes of few long lines, and all if the memory for the matrices is not to be
+ * had, by FFT); the radix schedules of ch_set_fft_pruning do not apply to them. */
 int ch_step(ch_grid* g, int nsteps);
 
 /* The kernels of one time step in the order ch_step_timed reports them in: zrhs (DCT,
@@ -206,7 +206,7 @@ int ch_fp64_fma_rate(double* tflops);
 int ch_step_timed(ch_grid* g, int nsteps, double* kernel_ms, double* total_ms);
 
 /* Number of kernel launches one ch_step makes per time step (six; two more with the Chebyshev
- * transforms on the tensor cores, three more with the x/y transforms there). */
+ * transforms on the tensor cores, two more with the x line and one with the forward y pass there). */
 int ch_launches_per_step(const ch_grid* g);
 
 /* Spectral state -> physical u, v, w, phi (device, (nz,ny,nx) float64) on the unpadded grid. */

@@ -393,13 +393,71 @@ int make_txy_plan(ch_grid* G, int mode, int P, double scale, chf::TxyPlan* p) {
   return CH_OK;
 }
 
+// Where a transform may run either way, both times are estimated (us on GB300).  On the tensor cores the
+// CTA with the most tiles does per K stage (16 inputs) one conversion and two products of each of its
+// output slices; by FFT the time grows with the points, over a latency that grows with the length.  The
+// coefficients are least-squares fits to 127 grids of 2^14 to 2^23 modes with lengths from 4 to 1024 in x and y
+// (the estimates are within 9 % and 17 % rms).
+struct TxCost {
+  double conv, mma;   // per stage
+};
+double tx_us(const TxCost& c, const chf::TxyPlan& t, long long lines, int rows, int nf, int ctas) {
+  const long long tiles = std::max(1ll, (lines + rows - 1) / rows * nf);
+  const long long parts = std::max(1ll, std::min<long long>(t.nsl, ctas / tiles));
+  const long long waves = (tiles * parts + ctas - 1) / ctas, slices = (t.nsl + parts - 1) / parts;
+  return (double)(waves * t.nst) * (c.conv + c.mma * 2.0 * (double)slices * t.NT / 64.0);
+}
+// Rule for a y pass of several padded fields: by FFT where that is a quarter faster by estimate, few long
+// lines.  FFT / tensor cores, us: backward 8 x 648 x 17 64 / 163, 8 x 512 x 17 41 / 131, 16 x 512 x 33 98 / 178,
+// forward 8 x 512 x 17 76 / 110; on the tensor cores backward 16 x 648 x 65 355 / 360, 128 x 648 x 17 777 / 620,
+// 512 x 6 x 33 108 / 43, forward 48 x 648 x 17 487 / 370.
+bool y_on_tc(const ch_grid* G, int dir, const chf::TxyPlan& t, int nf) {
+  const GridDev& g = G->g;
+  const long long lines = (long long)g.Mx * g.nz;
+  const double m = 1e-6 * (double)nf * (double)lines, P = g.Py;
+  const double tc = dir == 1 ? 20.0 + tx_us({3.23, 1.48}, t, lines, 64, nf, G->tx.ctas)
+                             : 18.5 + tx_us({2.72, 1.47}, t, lines, 64, nf, G->tx.ctas);
+  const double fft = dir == 1 ? 2.6 + 69.8 * m * (P + 16.6) + 0.041 * P
+                              : 71.5 * m * (P + 23.8) + 0.071 * P;
+  return tc <= 1.25 * fft;
+}
+// Rule for the transforms of nf physical fields to coefficients (set_fields: four) and of one field back
+// (get_fields and diagnostics, four fields and seven, always gain): on the tensor cores where that is faster by
+// estimate, with a margin for its error.  FFT / tensor cores, us: one field 128 x 48 x 33 81 / 108, 256 x 24 x 25
+// 77 / 134, 72 x 72 x 49 79 / 92, 64 x 36 x 145 81 / 76, 512 x 48 x 33 244 / 218, 256 x 256 x 17 477 / 193; four 512 x 6 x
+// 33 164 / 232, 256 x 16 x 17 118 / 135, 512 x 24 x 17 271 / 262, 64 x 64 x 17 102 / 79, 128 x 48 x 33 171 / 129;
+// one back 128 x 16 x 33 46 / 62, 8 x 648 x 17 108 / 125, 128 x 48 x 33 85 / 71, 384 x 48 x 17 153 / 109.
+bool ax_forward(const ch_grid* G, int nf) {
+  if (!G->use_ax) return false;
+  const GridDev& g = G->g;
+  const long long xl = (long long)g.ny * g.nz, yl = (long long)g.Mx * g.nz;
+  const double m = 1e-6 * (double)nf * (double)G->fsp;
+  return 49.9 + 16.9 * m + tx_us({4.30, 2.67}, G->tx.xfu, xl, 128, nf, G->tx.ctas) +
+             tx_us({0.74, 1.56}, G->tx.yfu, yl, 64, nf, G->tx.ctas) <=
+         0.95 * (16.8 + 5.0 * nf + 198.0 * m + 0.069 * g.nx + 0.141 * g.ny + 0.038 * g.nz);
+}
+bool ax_backward_one(const ch_grid* G) {
+  if (!G->use_ax) return false;
+  const GridDev& g = G->g;
+  const long long xl = (long long)g.ny * g.nz, yl = (long long)g.Mx * g.nz;
+  const double m = 1e-6 * (double)G->fsp;
+  return 43.1 + 16.9 * m + tx_us({1.46, 1.42}, G->tx.xbu, xl, 128, 1, G->tx.ctas) +
+             tx_us({0.73, 1.39}, G->tx.ybu, yl, 64, 1, G->tx.ctas) <=
+         0.9 * (22.4 + 200.0 * m + 0.069 * g.nx + 0.133 * g.ny + 0.031 * g.nz);
+}
+
 // Plans and buffers of the tensor-core x/y transforms: of the unpadded grid for the entry points
 // that read and write physical fields (use_ax, with the Chebyshev transforms), and of the padded one
 // for the steps of a float64 grid (use_tx).
 // Rule: from 2^15 modes on (below, a transform has fewer tiles than a third of the SMs and its
 // latency counts: 32 x 32 x 33, 16896 modes, y backward, x line and y forward 28, 56 and 27 against
-// 22, 53 and 33 us by FFT; 48 x 48 x 49, 56448 modes, 34, 88 and 46 against 47, 137 and 75),
-// up to transform lengths of 1024 (the dense matrices grow with the length squared).
+// 22, 53 and 33 us by FFT; 48 x 48 x 49, 56448 modes, 34, 88 and 46 against 47, 137 and 75; get_fields of a
+// mixed grid of 32 x 64 x 33 142 by FFT, 62 here), up to transform lengths of 1024 (the dense matrices grow
+// with the length squared; 192 x 648 x 33, padded 972, y backward and forward 2082 and 3323 by FFT, 1142 and
+// 2028 here; a field of 24 x 1024 x 33 330 by FFT, 192 here).  Below the limits y passes and transforms of few
+// long lines stay with the FFT by the rules above; the x line does not: few x lines cost it more only below
+// about 300 of 576 points and more (512 x 16 x 9, 216 lines, 142 by FFT and 260 here, 512 x 6 x 33, 297 lines,
+// 275 and 264, 384 x 24 x 17, 612 lines, 318 and 259), where the y passes gain about as much.
 constexpr int kTxyMaxP = 1024;
 constexpr long long kTxyMinModes = 1ll << 15;
 constexpr long long kCoefMinModes = 1ll << 18;
@@ -441,6 +499,8 @@ int setup_tx(ch_grid* G) {
   G->tx = t;
   G->use_ax = 1;
   G->use_tx = padded;
+  G->tx_y[0] = padded && y_on_tc(G, 0, t.yf, kNl);
+  G->tx_y[1] = padded && y_on_tc(G, 1, t.yb, kYa);
   return CH_OK;
 }
 
@@ -477,15 +537,6 @@ int rows_to_coef(ch_grid* G, double* const* phys, int nf, double2* coef) {
   return CH_OK;
 }
 
-// Rule for a transform of one field (its tiles are few; several fields together always gain): on the
-// tensor cores from 3 2^15 modes on with at least 8 x lines per x point.  A pair of transforms by FFT /
-// on the tensor cores, us: 128 x 48 x 33 165 / 141, 288 x 72 x 33 416 / 303, 64 x 36 x 145 162 / 129;
-// below 96 x 24 x 65 111 / 121, 256 x 24 x 25 152 / 228, 216 x 24 x 17 130 / 203.
-bool ax_one_field(const ch_grid* G) {
-  const GridDev& g = G->g;
-  return G->use_ax && G->fs >= 3 * kTxyMinModes && (long long)g.ny * g.nz >= 8ll * g.nx;
-}
-
 void drop_graph(ch_grid* G) {
   if (G->graph_ok) cudaGraphExecDestroy(G->gexec);
   G->graph_ok = 0;
@@ -506,30 +557,30 @@ cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s) {
 cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s) {
   const GridDev& g = G->g;
   const FftPlan& py = G->py[G->prec];
+  const bool tc = ch_tx_stage(G, stage);
   if (stage == 3) {
     chf::YMap ym = step_ymap();
     ym.kys = 6.283185307179586476925 / g.ly;
-    return G->use_tx ? chf::launch_txy_y(1, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, ym, G->tx,
-                                         G->tx.yb, s)
-                     : chf::launch_ypass(1, G->prec, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0,
-                                         py, s, &ym);
+    return tc ? chf::launch_txy_y(1, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, ym, G->tx, G->tx.yb, s)
+              : chf::launch_ypass(1, G->prec, g, g.Py, G->bw, G->ya, kYa, G->fs, G->fsy, 1.0, py, s,
+                                  &ym);
   }
   if (stage == 4)
-    return G->use_tx ? chf::launch_txy_x(g, G->ya, G->yb, G->fsy, G->tx, s)
-                     : chf::launch_xline(G->prec, g, G->ya, G->yb, G->fsy, 1.0, G->px[G->prec], s);
-  return G->use_tx ? chf::launch_txy_ycomb(g, G->yb, G->nl, G->fsy, G->fs, G->tx, s)
-                   : chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs,
-                                       1.0 / ((double)g.Px * (double)g.Py), py, s);
+    return tc ? chf::launch_txy_x(g, G->ya, G->yb, G->fsy, G->tx, s)
+              : chf::launch_xline(G->prec, g, G->ya, G->yb, G->fsy, 1.0, G->px[G->prec], s);
+  return tc ? chf::launch_txy_ycomb(g, G->yb, G->nl, G->fsy, G->fs, G->tx, s)
+            : chf::launch_ycomb(G->prec, g, G->yb, G->nl, G->fsy, G->fs,
+                                1.0 / ((double)g.Px * (double)g.Py), py, s);
 }
 
 cudaError_t ch_launch_y_adj(ch_grid* G, int dir, const double2* in, double2* out, int nf,
                             cudaStream_t s) {
   const GridDev& g = G->g;
   const long long fi = dir == 1 ? G->fs : G->fsy, fo = dir == 1 ? G->fsy : G->fs;
-  if (!G->use_tx || !(dir == 1 ? G->tx.yb : G->tx_yf1).dig)
+  const chf::TxyPlan& plan = dir == 1 ? G->tx.yb : G->tx_yf1;
+  if (!G->use_tx || !plan.dig || !y_on_tc(G, dir, plan, nf))
     return chf::launch_ypass(dir, 0, g, g.Py, in, out, nf, fi, fo, 1.0, G->py[0], s);
-  return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, identity_ymap(), G->tx,
-                           dir == 1 ? G->tx.yb : G->tx_yf1, s);
+  return chf::launch_txy_y(dir, g, g.Py, in, out, nf, fi, fo, identity_ymap(), G->tx, plan, s);
 }
 
 cudaError_t ch_launch_x_adj(ch_grid* G, const double2* ya, double2* out6, cudaStream_t s) {
@@ -803,7 +854,7 @@ static int set_from_phys(ch_grid* G, const double* u, const double* v, const dou
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
   const double* f4[4] = {u, v, w, phi};
-  if (G->use_ax) {
+  if (ax_forward(G, 4)) {
     const int r = rows_to_coef(G, const_cast<double* const*>(f4), 4, G->auxA);
     if (r != CH_OK) return r;
     CK(chf::launch_project(g, G->auxA, G->fs, G->om, G->w, G->phi, G->hom, G->hw, G->hphi, G->pz, s,
@@ -879,7 +930,7 @@ int ch_step(ch_grid* G, int nsteps) {
 int ch_launches_per_step(const ch_grid* G) {
   if (!G) return 0;
   // the tensor-core x line is three launches (backward, products, forward), the forward y pass two
-  return (ch_z_coef(G) ? 8 : 6) + (G->use_tx ? 3 : 0);
+  return (ch_z_coef(G) ? 8 : 6) + (ch_tx_stage(G, 4) ? 2 : 0) + (ch_tx_stage(G, 5) ? 1 : 0);
 }
 
 int ch_step_timed(ch_grid* G, int nsteps, double* kernel_ms, double* total_ms) {
@@ -1046,7 +1097,7 @@ int ch_transform_forward(ch_grid* G, const double* phys, double* spec) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  if (ax_one_field(G)) {
+  if (ax_forward(G, 1)) {
     double* p[1] = {const_cast<double*>(phys)};
     return rows_to_coef(G, p, 1, (double2*)spec);
   }
@@ -1061,7 +1112,7 @@ int ch_transform_backward(ch_grid* G, const double* spec, double* phys) {
   if (!G || !phys || !spec) return CH_ERR_ARG;
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;
-  if (ax_one_field(G))
+  if (ax_backward_one(G))
     return coef_to_rows(G, (const double2*)spec, 1, identity_ymap(), 1, nullptr, 0, 1, &phys);
   CK(chf::launch_dct_lines(1, 0, g, spec, G->auxA, 1, G->fs, G->pz, s));
   CK(chf::launch_ypass(1, 0, g, g.ny, G->auxA, G->auxB, 1, G->fs, G->fs, 1.0, G->pyu, s));
@@ -1078,7 +1129,7 @@ int ch_nonlinear(ch_grid* G, double* out9) {
   const double scale = 1.0 / ((double)g.Px * (double)g.Py);
   const int r = eval_products(G);
   if (r != CH_OK) return r;
-  if (G->use_tx) {
+  if (ch_tx_stage(G, 5)) {
     CK(chf::launch_txy_y(0, g, g.Py, G->yb, G->nl, kNl, G->fsy, G->fs, identity_ymap(), G->tx,
                          G->tx.yf, G->stream));
   } else {

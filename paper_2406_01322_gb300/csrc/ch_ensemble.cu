@@ -96,8 +96,8 @@ namespace {
 constexpr int kStages = CH_ENSEMBLE_STAGES;
 // work lists: the six stages, then zrhs and zbwd of the members whose z transforms run on the tensor
 // cores (ch_z_coef; the others are in lists 0 and 2, so that every member steps as it would alone).
-// Members whose x and y transforms run there (use_tx) are in none of the lists 3 to 5: each launches
-// those stages itself, the others stay grouped.
+// Members whose x or y transforms run there (ch_tx_stage) are not in that stage's list: each launches it
+// itself, the others stay grouped.
 constexpr int kLists = kStages + 2;
 int stage_of(int list) { return list < kStages ? list : list == kStages ? 0 : 2; }
 
@@ -235,7 +235,7 @@ int build_descriptors(ch_ensemble* E) {
     for (int i = 0; i < n; ++i) {
       b[i + 1] = b[i];
       if ((s == 0 || s == 2) && (int)E->zc[i] != coef) continue;
-      if (s >= 3 && E->members[i]->use_tx) continue;
+      if (s >= 3 && ch_tx_stage(E->members[i], s)) continue;
       b[i + 1] += chf::stage_items(s, E->hmem[i], E->prec);
       const size_t sm = chf::stage_smem(s, E->hmem[i], E->prec, coef);
       if (sm > mx) mx = sm;
@@ -307,7 +307,7 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
                                 grid_of(E, l), E->smem[l], E->zsolve_tile, l >= kStages,
                                 st == 4 ? E->xwq : E->ywq, s);
     for (size_t i = 0; i < E->members.size() && st >= 3 && e == cudaSuccess; ++i)
-      if (E->members[i]->use_tx) e = ch_launch_xy(E->members[i], st, s);
+      if (ch_tx_stage(E->members[i], st)) e = ch_launch_xy(E->members[i], st, s);
     if (e == cudaSuccess && st == 2) e = member_transforms(E, 1, s);
     if (ev) cudaEventRecord(ev[st], s);
     if (e != cudaSuccess) {
@@ -320,11 +320,10 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
 
 void compute_occupancy(ch_ensemble* E) {
   std::vector<int> py, px;
-  for (ch_grid* G : E->members)
-    if (!G->use_tx) {
-      py.push_back(G->g.Py);
-      px.push_back(G->g.Px);
-    }
+  for (ch_grid* G : E->members) {
+    if (!ch_tx_stage(G, 3) || !ch_tx_stage(G, 5)) py.push_back(G->g.Py);
+    if (!ch_tx_stage(G, 4)) px.push_back(G->g.Px);
+  }
   E->ywq = chf::ensemble_ywq(py, E->prec);
   E->xwq = chf::ensemble_ywq(px, E->prec);
   for (int l = 0; l < kLists; ++l)
@@ -600,7 +599,7 @@ int ch_ensemble_autotune(ch_ensemble* E, int reps) {
   }
   // (a schedule that no member's grouped x or y stage uses stays as it is: only noise would choose it)
   for (int k = 0; k < 3 && st == CH_OK; ++k) {
-    if (k < 2 && list_items(E, 4 - k) == 0) continue;
+    if (k == 0 ? list_items(E, 4) == 0 : k == 1 && list_items(E, 3) + list_items(E, 5) == 0) continue;
     int b = 0;
     for (int style = 1; style < (k < 2 ? 4 : 3); ++style)
       if (cost[k][style] < cost[k][b]) b = style;

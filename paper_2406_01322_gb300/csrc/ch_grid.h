@@ -99,16 +99,21 @@ struct ch_grid {
   int* tc_err = nullptr;
 
   // tensor-core transforms of the unpadded grid for the entry points that take or give physical
-  // fields (use_ax) and of the step's float64 y and x stages (use_tx); for the reverse sweep,
+  // fields (use_ax) and of the step's float64 x stage (use_tx) and y stages (tx_y: forward, backward); for
+  // the reverse sweep,
   // made when it first begins, tx_yf1: the forward y transform without the 1 / (Px Py), tx_xb1: the
   // transposed forward x transform
-  int use_ax = 0, use_tx = 0;
+  int use_ax = 0, use_tx = 0, tx_y[2] = {0, 0};
   chf::Txy tx;
   chf::TxyPlan tx_yf1, tx_xb1;
 };
 
 // the step's z kernels work on Chebyshev coefficients, transformed on the tensor cores
 inline bool ch_z_coef(const ch_grid* G) { return G->cheb == CH_CHEB_TC || G->z_auto; }
+// stage 3 y backward, 4 x line, 5 y forward of the step runs on the tensor cores
+inline bool ch_tx_stage(const ch_grid* G, int stage) {
+  return stage == 4 ? G->use_tx != 0 : G->tx_y[stage == 3] != 0;
+}
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev);
 int ch_eval_nonlinear(ch_grid* G);
