@@ -554,6 +554,19 @@ cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s) {
                              G->tc_err, s);
 }
 
+// Rule for the x line of an ensemble's member: by FFT, grouped, where that is a quarter faster by estimate.
+// A grouped launch has no latency of its own (the fits as in y_on_tc, without it): sixteen members of
+// 512 x 8 x 17 10.8 ms alone on the tensor cores with one CTA a tile, 4.1 with the slices shared out, 1.9
+// grouped; 384 x 16 x 17 3.4 and 2.8; 48 x 48 x 33 1.2 and 1.4.
+bool ch_tx_member(const ch_grid* G, int stage) {
+  if (!ch_tx_stage(G, stage) || stage != 4) return ch_tx_stage(G, stage);
+  const long long Q = (long long)G->g.Py * G->g.nz;
+  const double m = 1e-6 * (double)Q, P = G->g.Px;
+  return 32.1 + 26.7 * m * P + tx_us({6.47, 0.70}, G->tx.xb, Q, 128, 7, G->tx.ctas) +
+             tx_us({2.84, 1.48}, G->tx.xf, Q, 128, 9, G->tx.ctas) <=
+         1.25 * 487.0 * m * (P + 12.8);
+}
+
 cudaError_t ch_launch_xy(ch_grid* G, int stage, cudaStream_t s) {
   const GridDev& g = G->g;
   const FftPlan& py = G->py[G->prec];

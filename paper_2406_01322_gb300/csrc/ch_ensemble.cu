@@ -96,7 +96,7 @@ namespace {
 constexpr int kStages = CH_ENSEMBLE_STAGES;
 // work lists: the six stages, then zrhs and zbwd of the members whose z transforms run on the tensor
 // cores (ch_z_coef; the others are in lists 0 and 2, so that every member steps as it would alone).
-// Members whose x or y transforms run there (ch_tx_stage) are not in that stage's list: each launches it
+// Members whose x or y transforms run there (ch_tx_member) are not in that stage's list: each launches it
 // itself, the others stay grouped.
 constexpr int kLists = kStages + 2;
 int stage_of(int list) { return list < kStages ? list : list == kStages ? 0 : 2; }
@@ -235,7 +235,7 @@ int build_descriptors(ch_ensemble* E) {
     for (int i = 0; i < n; ++i) {
       b[i + 1] = b[i];
       if ((s == 0 || s == 2) && (int)E->zc[i] != coef) continue;
-      if (s >= 3 && ch_tx_stage(E->members[i], s)) continue;
+      if (s >= 3 && ch_tx_member(E->members[i], s)) continue;
       b[i + 1] += chf::stage_items(s, E->hmem[i], E->prec);
       const size_t sm = chf::stage_smem(s, E->hmem[i], E->prec, coef);
       if (sm > mx) mx = sm;
@@ -307,7 +307,7 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
                                 grid_of(E, l), E->smem[l], E->zsolve_tile, l >= kStages,
                                 st == 4 ? E->xwq : E->ywq, s);
     for (size_t i = 0; i < E->members.size() && st >= 3 && e == cudaSuccess; ++i)
-      if (ch_tx_stage(E->members[i], st)) e = ch_launch_xy(E->members[i], st, s);
+      if (ch_tx_member(E->members[i], st)) e = ch_launch_xy(E->members[i], st, s);
     if (e == cudaSuccess && st == 2) e = member_transforms(E, 1, s);
     if (ev) cudaEventRecord(ev[st], s);
     if (e != cudaSuccess) {
@@ -321,8 +321,8 @@ int launch_all(ch_ensemble* E, cudaStream_t s, cudaEvent_t* ev) {
 void compute_occupancy(ch_ensemble* E) {
   std::vector<int> py, px;
   for (ch_grid* G : E->members) {
-    if (!ch_tx_stage(G, 3) || !ch_tx_stage(G, 5)) py.push_back(G->g.Py);
-    if (!ch_tx_stage(G, 4)) px.push_back(G->g.Px);
+    if (!ch_tx_member(G, 3) || !ch_tx_member(G, 5)) py.push_back(G->g.Py);
+    if (!ch_tx_member(G, 4)) px.push_back(G->g.Px);
   }
   E->ywq = chf::ensemble_ywq(py, E->prec);
   E->xwq = chf::ensemble_ywq(px, E->prec);

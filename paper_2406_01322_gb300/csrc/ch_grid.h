@@ -114,6 +114,8 @@ inline bool ch_z_coef(const ch_grid* G) { return G->cheb == CH_CHEB_TC || G->z_a
 inline bool ch_tx_stage(const ch_grid* G, int stage) {
   return stage == 4 ? G->use_tx != 0 : G->tx_y[stage == 3] != 0;
 }
+// the same for a member of an ensemble, whose other choice is a grouped launch
+bool ch_tx_member(const ch_grid* G, int stage);
 // launch schedule of one step on stream s (events optional) and the non-linear evaluation
 int ch_launch_step(ch_grid* G, int first, cudaStream_t s, cudaEvent_t* ev);
 int ch_eval_nonlinear(ch_grid* G);

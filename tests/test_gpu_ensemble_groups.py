@@ -63,3 +63,27 @@ def test_stages_without_grouped_members_keep_their_defaults(binding):
     assert t["radix_style"]["x"] == 0 and t["radix_style"]["y"] == 0
     assert t["ctas_per_sm"][3:] == [0, 0, 0]
     e.close()
+
+
+def test_members_of_few_long_x_lines_are_grouped_there(binding):
+    """512 x 8 x 17: a grid of its own has its x line on the tensor cores, a member the grouped FFT (the last
+    bits tell them apart); both agree to the float64 bar of the step, 1e-10, and a member evolves the
+    same bit for bit whatever is beside it."""
+    m = dict(nx=512, ny=8, nz=17, **PHYS)
+    alone = evolve(ensemble(binding, [m]), (7,))[0]
+    among = evolve(ensemble(binding, [LARGE, m, SMALL]), (8, 7, 9))[1]
+    assert torch.equal(alone, among)
+    e = ensemble(binding, [m])
+    g = binding.Grid(**m)
+    assert g.launches_per_step() == 9
+    f = [torch.from_numpy(np.ascontiguousarray(a))
+         for a in inputs.initial_fields(512, 8, 17, 150.0, 0.05, 1, 0.4, 7)]
+    for x in (g, e.grids[0]):
+        x.set_fields(*f)
+    g.step(3)
+    e.step(3)
+    assert not torch.equal(g.get_state(), e.grids[0].get_state())
+    for a, b in zip(g.get_fields(), e.grids[0].get_fields()):
+        assert float((a - b).abs().max()) <= 1e-10 * float(b.abs().max())
+    e.close()
+    g.close()
