@@ -454,9 +454,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (g == 0 && rowok) {
           TO vr = ere == kNanRow ? qnan<TO>()
-                                 : scaled_any<TO>(words_to_t(hr, lr), ere - F::EOFF - 51);
+                                 : words_scaled<TO>(hr, lr, ere - F::EOFF - 62);
           TO vi = eim == kNanRow ? qnan<TO>()
-                                 : scaled_any<TO>(words_to_t(hm, lm), eim - F::EOFF - 51);
+                                 : words_scaled<TO>(hm, lm, eim - F::EOFF - 62);
           if (fwd) {
             vr = times<TO>(vr, lastf);
             vi = times<TO>(vi, lastf);

@@ -279,9 +279,18 @@ struct WordSums {
     return (long long)(l - (unsigned long long)n * (unsigned)kABias);
   }
 };
-// such a sum, in units of 2^(E-62), as the T of T 2^(E-51)
-__device__ __forceinline__ long long words_to_t(long long h, long long l) {
-  return h * 2097152ll + ((l + 1024) >> 11);
+// such a sum times 2^e, rounded once (both words are below 2^53, so their conversions are exact)
+template <typename TO> __device__ TO words_scaled(long long h, long long l, int e);
+template <> __device__ __forceinline__ double words_scaled<double>(long long h, long long l, int e) {
+  return ldexp(fma(__ll2double_rn(h), 4294967296.0, __ll2double_rn(l)), e);
+}
+template <> __device__ __forceinline__ float words_scaled<float>(long long h, long long l, int e) {
+  return (float)words_scaled<double>(h, l, e);
+}
+template <> __device__ __forceinline__ df words_scaled<df>(long long h, long long l, int e) {
+  const double v = words_scaled<double>(h, l, e);
+  const float hi = (float)v;
+  return df(hi, (float)(v - (double)hi));
 }
 
 // round(U / 64) of column e of the diagonal accumulators (exact integers below 2^24 held as

@@ -542,13 +542,13 @@ __global__ void __launch_bounds__(kThreads, 1) txy_kernel(const __grid_constant_
           }
         }
         if (g == 0 && rowok) {
-          const int e2 = sc - FBits<double>::EOFF - 51;
+          const int e2 = sc - FBits<double>::EOFF - 62;
           const double vr = sc == kNanRow ? qnan<double>()
-                                          : scaled_any<double>(words_to_t(hr, lr), e2);
+                                          : words_scaled<double>(hr, lr, e2);
           double* o = A.out[fld] + (lh * A.ohs + ll * A.ols + (long long)(A.P / 2) * A.ostr) * OSC;
           if (CPX) {
             const double vi = sc == kNanRow ? qnan<double>()
-                                            : scaled_any<double>(words_to_t(hm, lm), e2);
+                                            : words_scaled<double>(hm, lm, e2);
             *reinterpret_cast<double2*>(o) = make_double2(vr, vi);
           } else {
             *o = vr;

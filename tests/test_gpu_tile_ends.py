@@ -73,3 +73,29 @@ def test_back_to_back_launches_leave_nothing_in_flight(binding, nz):
     for a, b in zip(first, last):
         assert torch.equal(a, b)
     g.close()
+
+
+@pytest.mark.parametrize("nz", [17, 129, 385])
+def test_last_output_is_rounded_once(binding, nz):
+    """The output n = N, an alternating sum formed apart from the products, of rows whose terms cancel to a
+    thousandth: off by the rounding of the row's elements to 2^-63 of the power of two above the
+    largest (at most 2.11 of it) and by the roundings of the result, not of the row's scale."""
+    N = nz - 1
+    rng = np.random.Generator(np.random.PCG64(nz))
+    nx, ny = 12, 6
+    x = rng.standard_normal((1, nx // 2, ny, nz)) + 1j * rng.standard_normal((1, nx // 2, ny, nz))
+    x[..., 1::2] = x[..., 0:-1:2] * (1.0 + 1e-3 * rng.random((1, nx // 2, ny, N // 2)))
+    x[..., N] *= 1e-3
+    g = binding.Grid(nx, ny, nz)
+    g.set_chebyshev(binding.CHEB_TC)
+    F, B = matrices(N)
+    flat = x.reshape(-1, nz)
+    for direction, row in enumerate((F[N], B[N])):
+        got = g.chebyshev_lines(torch.from_numpy(x).cuda(), direction).cpu().numpy().reshape(-1, nz)[:, N]
+        for part in (np.real, np.imag):
+            xr = part(flat).astype(np.longdouble)
+            ref = xr @ row
+            bound = (2.0 ** -52 * np.abs(ref) + 1e-30
+                     + 2.0 ** -63 * 2.11 * np.max(np.abs(xr), axis=1) * float(np.sum(np.abs(row))))
+            assert np.all(np.abs(part(got).astype(np.longdouble) - ref) <= bound), direction
+    g.close()
