@@ -199,6 +199,31 @@ def cheb_issued_flops(w, nf):
     return 35 * 2.0 * (2 * nf * (w["nx"] // 2) * w["ny"]) * (2 * NT * nsl) * K
 
 
+def xy_issued_flops(w, kernel):
+    """Tensor-pipe flops that the launches of one float64 x or y stage issue on the tensor cores
+    (None for other stages): per field and tile (64 complex lines in y, 128 lines in x) a cosine and
+    a sine product, outputs in slices of at most 64 columns, inputs in stages of 16, 35 digit
+    products of 128 rows each."""
+    nx, ny, nz = w["nx"], w["ny"], w["nz"]
+    Mx, Px, Py = nx // 2, 3 * nx // 2, 3 * ny // 2
+    hx, hy, q = (Px + 1) // 2, (Py + 1) // 2, Py * nz
+    # (lines, lines per tile, fields, inputs, outputs) of the transforms a stage is made of
+    yb, yf = (Mx * nz, 64, ny // 2, hy), (Mx * nz, 64, hy, ny // 2)
+    xb, xf = (q, 128, Mx, hx), (q, 128, hx, Mx)
+    parts = {"ybwd": [(6, yb)], "yfwd": [(9, yf)], "xline": [(7, xb), (9, xf)],
+             "adj_ybwd": [(9, yb)], "adj_yfwd": [(6, yf)],
+             "adj_xline": [(7, xb), (9, xb), (7, xf)]}.get(kernel)
+    if parts is None:
+        return None
+    total = 0.0
+    for nf, (lines, rows, nk, nout) in parts:
+        nsl = -(-nout // 64)
+        NT = -(-(-(-nout // nsl)) // 16) * 16
+        tiles = nf * -(-lines // rows)
+        total += tiles * 2 * nsl * -(-nk // 16) * 35 * 2.0 * 128 * NT * 16
+    return total
+
+
 def cufft_transforms_ms(w, prec, reps=5, warmup=2, dev="cuda"):
     """Timed comparison only: the transforms of one step done with cuFFT through torch.fft, as a
     library user would write them (zero padding / truncation by copies, layouts as stored):
@@ -583,6 +608,10 @@ def run_ensemble(args):
     e2e_s = time.perf_counter() - t_e
     nbytes = sum(4 * m["nx"] * m["ny"] * m["nz"] * 8 for m in ms)
     names = list(binding.Ensemble.STAGES)
+    # launches per step: the grouped stages, two per member with its Chebyshev transforms on the
+    # tensor cores, six per float64 member with its x and y transforms there
+    own = sum(g.launches_per_step() > (8 if tc else 6) for g in ens.grids)
+    launches = 3 + (3 if own < len(ms) else 0) + 6 * own + (2 * len(ms) if tc else 0)
     out = {"metric": METRIC, "value": pts * args.steps / (tot_ms * 1e-3) / 1e6, "unit": UNIT,
            "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
            "ms_per_step": tot_ms / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -600,7 +629,7 @@ def run_ensemble(args):
                    "d2h_bytes_per_step": nbytes / args.steps,
                    "note": "set_fields_host of every member + K grouped steps + get_fields_host"},
            "stage_ms_per_step": {n: kms[i] / args.steps for i, n in enumerate(names)},
-           "tuning": tuning, "gpu_launches": (6 + (2 * len(ms) if tc else 0)) * args.steps,
+           "tuning": tuning, "gpu_launches": launches * args.steps,
            "clocks": clk.summary()}
     ens.close()
     print(json.dumps(out))
@@ -679,23 +708,35 @@ def run_adjoint(args):
     k = max(range(len(names)), key=lambda i: kms[i])
     per_launch_ms = kms[k] / nsteps
     fl, by = work[names[k]]
+    bound, peak = "alu", FP64_PEAK_TFLOPS
+    peak_kind = "float64 FMA pipe: 152 SMs x 2.07 GHz x 4 flop/clk (nominal)"
+    # launches of one step: six, five more with the z, x and y transforms on the tensor cores
+    tc = g.launches_per_step() == 11
+    if tc and xy_issued_flops(w, names[k]):
+        fl, bound = xy_issued_flops(w, names[k]), "tensor"
+        peak, peak_kind = tensor_peak()
     ach = fl / (per_launch_ms * 1e-3) / 1e12
-    roof = {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": ach / FP64_PEAK_TFLOPS,
+    roof = {"bound": bound, "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+            "frac": ach / peak,
             "traffic": traffic_bytes(args.workload, 0, names[k]), "kernel": names[k],
-            "peak_kind": "float64 FMA pipe: 152 SMs x 2.07 GHz x 4 flop/clk (nominal)",
+            "peak_kind": peak_kind,
             "kernel_share": {n: kms[i] / sum(kms) for i, n in enumerate(names)},
             "kernel_ms_per_reverse_step": {n: kms[i] / nsteps for i, n in enumerate(names)},
             "note": "kernel times from an instrumented step-by-step reverse sweep, which "
                     "recomputes each state's fields (zbwd, ybwd); the timed gradients reverse "
                     "whole segments that keep them"}
     nbytes = 4 * pts * 8
-    # launches of this library per gradient: set_fields 10 (4 x r2c, y pass, projection, four
-    # for the products), 6 per forward step, objective 2, restore of the final state 4,
-    # adjoint seed 2, per segment a restore (4) and 6 per recomputed step, 7 per reverse step
-    # (the segment keeps the y-padded fields), gradient 6 (projection transpose, y pass, 4 c2r)
+    # launches of this library per gradient: set_fields (into the spectrum, projection, the
+    # products), forward steps, objective 2, restore of the final state (the products), adjoint
+    # seed 2, per segment a restore and the recomputed steps, reverse steps (the segment keeps the
+    # y-padded fields), gradient.  By FFT: 4 x r2c, y pass, projection + 4 for the products; 6 a
+    # step, 7 a reverse step; projection transpose, y pass, 4 c2r.  On the tensor cores: x, y, z,
+    # projection + 8; 11 a step, 13 a reverse step; projection transpose, y, x
     nseg = -(-nsteps // 10)
-    launches = 10 + 6 * nsteps + 2 + 4 + 2 + 4 * nseg + 6 * (nsteps - nseg) + 7 * nsteps + 6
+    products, per_step, per_reverse = (8, 11, 13) if tc else (4, 6, 7)
+    launches = ((4 if tc else 6) + products + per_step * nsteps + 2 + products + 2
+                + products * nseg + per_step * (nsteps - nseg) + per_reverse * nsteps
+                + (3 if tc else 6))
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": 1, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": tot_ms / args.steps,
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
@@ -712,10 +753,11 @@ def run_adjoint(args):
     print(json.dumps(out))
 
 
-def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
+def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names, tx=False):
     """Roofline of the dominant kernel of a timed run (kms: summed ms per kernel over `steps`
     steps, in the order of `names`), the per-kernel times and shares, and the step-level HBM
-    fraction (the step's algorithmic bytes over its time, against the measured copy peak)."""
+    fraction (the step's algorithmic bytes over its time, against the measured copy peak).  tx: the
+    x and y stages ran on the tensor cores (float64 grids from 2^15 modes on)."""
     work = kernel_work(w, prec, cheb)
     # the FFT method launches no tensor-core transforms: their timed entries are empty gaps
     active = [i for i, n in enumerate(names) if cheb == "tc" or not n.startswith("cheb")]
@@ -727,8 +769,9 @@ def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
     fl, by = work[name]
     hbm, hbm_kind = peaks()
     traffic = traffic_bytes(workload, prec, name, cheb)
-    # float64 kernels (all of precision 0, the z kernels of every precision) are ALU-bound and
-    # measured against the float64 peak, the double-float x/y kernels (float64-accurate work on
+    # float64 kernels (those of precision 0, the z kernels of every precision) are ALU-bound and
+    # measured against the float64 peak (transforms on the tensor cores against the measured bf16
+    # peak, by the flops they issue there), the double-float x/y kernels (float64-accurate work on
     # the float32 pipe) against the double-float rate of the float32 pipe, float32 kernels
     # against HBM
     fp64_like = (prec != 1) or name.startswith("z")
@@ -738,9 +781,10 @@ def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
                 "frac": ach / DF_PEAK_TFLOPS, "traffic": traffic, "kernel": name,
                 "peak_kind": "double-float on the float32 pipe: 152 SMs x 128 lanes x 2.07 GHz / "
                              "9.67 float32 instructions per float64-equivalent flop (nominal)"}
-    elif name.startswith("cheb"):
+    elif name.startswith("cheb") or (tx and xy_issued_flops(w, name)):
         tpk, tpk_kind = tensor_peak()
-        fl = cheb_issued_flops(w, 7 if name == "cheb_fwd" else 5)
+        fl = (cheb_issued_flops(w, 7 if name == "cheb_fwd" else 5) if name.startswith("cheb")
+              else xy_issued_flops(w, name))
         ach = fl / (per_launch_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": tpk, "unit": "TFLOP/s",
                 "frac": ach / tpk, "traffic": traffic, "kernel": name, "peak_kind": tpk_kind}
@@ -754,9 +798,6 @@ def roofline_of(workload, w, prec, cheb, kms, steps, ms_step, names):
         roof = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
                 "traffic": traffic, "kernel": name, "peak_kind": f"{hbm_kind} copy bandwidth"}
     roof["algorithmic_per_launch"] = {"flops": fl, "bytes": by}
-    if prec == 0 and name in ("ybwd", "xline", "yfwd"):
-        roof["note"] = ("float64 FFT flops as the yardstick; from 2^15 modes on the transforms run "
-                        "on the tensor cores")
     if roof["bound"] == "alu" and roof["peak"] == FP64_PEAK_TFLOPS and MEASURED_FMA.get("tflops"):
         roof["fp64_fma_measured_tflops"] = MEASURED_FMA["tflops"]
         roof["frac_of_measured_fma_rate"] = roof["achieved"] / MEASURED_FMA["tflops"]
@@ -784,6 +825,10 @@ def precision_variants(binding, w, workload, fields, kw, steps, device, main):
     for pr, cheb, prune in combos:
         g = binding.Grid(w["nx"], w["ny"], w["nz"], precision=pr, device=device, **kw)
         g.set_chebyshev(cheb)
+        tx = g.launches_per_step() > (8 if cheb else 6)
+        if prune and tx:   # its x/y transforms are on the tensor cores: pruned schedules do not apply
+            g.close()
+            continue
         g.set_fft_pruning(prune)
         g.set_fields(*[torch.from_numpy(f) for f in fields])
         g.step(3)
@@ -803,7 +848,7 @@ def precision_variants(binding, w, workload, fields, kw, steps, device, main):
                  float((a - b).abs().max() / b.abs().max())
                  for a, b in zip(final[(pr, cheb, prune)], final[(0, 0, 0)]))}
         if (pr, cheb, prune) == (0, 0, 0):
-            v["roofline"] = roofline_of(workload, w, 0, "fft", kms, steps, tot / steps, names)
+            v["roofline"] = roofline_of(workload, w, 0, "fft", kms, steps, tot / steps, names, tx)
         out[name] = v
     return out
 
@@ -925,7 +970,10 @@ def main():
 
     # ---- roofline of the dominant kernel
     names = list(binding.Grid.KERNELS)
-    roof = roofline_of(args.workload, w, prec, cheb, kms, args.steps, ms_step, names)
+    tx = g.launches_per_step() > (8 if cheb == "tc" else 6)
+    if tx:   # pruned schedules do not apply to x/y transforms on the tensor cores
+        config["pruned_xy_transforms"] = False
+    roof = roofline_of(args.workload, w, prec, cheb, kms, args.steps, ms_step, names, tx)
 
     if rank != 0:
         g.close()
