@@ -147,7 +147,8 @@ int ch_step(ch_grid* g, int nsteps);
 
 /* Select the step's Chebyshev method; allocates the tensor-core tables, where the grid does not have
  * them yet, on the first CH_CHEB_TC (synchronous).  CH_ERR_ARG: bad method; CH_ERR_STATE: a reverse sweep is open;
- * CH_ERR_SIZE: nz > 496.
+ * CH_ERR_SIZE: nz > 496.  A selection stays: selecting CH_CHEB_FFT, as ch_get_chebyshev reports it
+ * while none was made, is a selection too and takes a large grid's transforms off the tensor cores.
  * The captured step graph is rebuilt at the next ch_step. */
 int ch_set_chebyshev(ch_grid* g, int method);
 int ch_get_chebyshev(const ch_grid* g);

@@ -525,7 +525,7 @@ int coef_to_rows(ch_grid* G, const double2* coef, int nf, const chf::YMap& ym, i
   CK(chf::launch_txy_rows(1, g, out, G->auxB, G->fs, nx_out, xsrc, xmask, G->tx, s));
   return CH_OK;
 }
-// nf physical rows -> coefficient fields `coef` (not auxA or auxB's first nf fields)
+// nf physical rows -> coefficient fields `coef` (auxA or elsewhere, but not auxB's first nf fields)
 int rows_to_coef(ch_grid* G, double* const* phys, int nf, double2* coef) {
   const GridDev& g = G->g;
   cudaStream_t s = G->stream;

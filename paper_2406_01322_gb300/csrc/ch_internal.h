@@ -290,7 +290,7 @@ struct ChebTc {
   char* keep = nullptr;            // device: fixed-point values of one tile per persistent CTA
   int NT = 0, nsl = 0, nst = 0, kc = 0, gst = 0;
   int dir = 0;                     // 0 forward (samples -> coefficients), 1 backward
-  int nmag = 0;                    // accumulators that stay within 2^22 in magnitude: 7, 3 or 0
+  int nmag = 0;                    // accumulators that stay within 2^22 in magnitude: 8 (all), 3 or 0
   int q = 0;                       // log2 of the matrix scale
   long long ymid = 0;              // weight of the middle element, times 2^q
   int ctas = 0;                    // persistent CTAs (keep holds ctas cheb_tc_keep_bytes)

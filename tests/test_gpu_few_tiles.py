@@ -63,13 +63,14 @@ def test_one_field_equals_the_same_field_among_four(binding, n):
     g.close()
 
 
-@pytest.mark.parametrize("n", [(512, 6, 33), (72, 72, 49), (256, 16, 17), (8, 648, 17), (96, 96, 65)],
+@pytest.mark.parametrize("n", [(512, 6, 33), (72, 72, 49), (256, 16, 17), (8, 648, 17), (96, 96, 65),
+                               (24, 1024, 33)],
                          ids=lambda n: "x".join(map(str, n)))
 def test_routes_of_one_and_four_fields_agree(binding, n):
     """A field that the grid holds exactly (three x, three y and five z modes): set_fields and get_fields (one
     by FFT, the other on the tensor cores for the first and third size), and the transforms of one field
     (forward by FFT and backward on the tensor cores for the second, both by FFT for the fourth, both on the
-    tensor cores for the last) give it back.  Bound: 1e-12 of the largest value, as above."""
+    tensor cores for the last two, in four K groups at 1024 points) give it back.  Bound: 1e-12 of the largest value, as above."""
     nx, ny, nz = n
     x = np.arange(nx) * (2 * np.pi / nx)
     y = (np.arange(ny) * (2 * np.pi / ny))[:, None]
