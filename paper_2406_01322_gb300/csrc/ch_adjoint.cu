@@ -268,10 +268,9 @@ int ch_adjoint_segment(ch_grid* G, const void* checkpoint, int nsteps) {
     G->seg_cap = nsteps;
   }
   char* seg = (char*)G->seg_block;
-  int r = ch_sync_status(G);                 // of the segments before this one
-  if (r != CH_OK) return r;
-  // recompute the segment from its checkpoint, keeping each state's y-padded fields
-  r = ch_set_state(G, checkpoint);           // also evaluates the fields of the first state
+  // recompute the segment from its checkpoint, keeping each state's y-padded fields (restoring also
+  // evaluates those of the first state; with the status of the segments before this one)
+  int r = ch_restore(G, checkpoint, true);
   if (r != CH_OK) return r;
   std::vector<int> first((size_t)nsteps);
   for (int k = 0; k < nsteps; ++k) {

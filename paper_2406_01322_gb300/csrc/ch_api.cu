@@ -1061,12 +1061,21 @@ int ch_get_state(ch_grid* G, void* buf) {
   return ch_sync_status(G);
 }
 
-int ch_set_state(ch_grid* G, const void* buf) {
+int ch_set_state(ch_grid* G, const void* buf) { return ch_restore(G, buf, false); }
+}  // extern "C"
+
+// status: CH_ERR_TIMEOUT before anything is restored while the flag of the device waits is set
+int ch_restore(ch_grid* G, const void* buf, bool status) {
   if (!G || !buf) return CH_ERR_ARG;
   StateHeader h;
   const char* b = (const char*)buf;
   CK(cudaMemcpyAsync(&h, b, sizeof(h), cudaMemcpyDeviceToHost, G->stream));
-  CK(cudaStreamSynchronize(G->stream));
+  if (status) {
+    const int r = ch_sync_status(G);
+    if (r != CH_OK) return r;
+  } else {
+    CK(cudaStreamSynchronize(G->stream));
+  }
   if (h.magic != chf::kStateMagic || h.nx != G->g.nx || h.ny != G->g.ny || h.nz != G->g.nz)
     return CH_ERR_ARG;
   const size_t sb = (size_t)G->fs * sizeof(double2);
@@ -1082,6 +1091,7 @@ int ch_set_state(ch_grid* G, const void* buf) {
   return eval_nonlinear_impl(G);
 }
 
+extern "C" {
 int ch_get_spectral(ch_grid* G, double* om, double* w, double* phi) {
   if (!G) return CH_ERR_ARG;
   const size_t sb = (size_t)G->fs * sizeof(double2);

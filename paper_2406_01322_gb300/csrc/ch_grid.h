@@ -122,6 +122,8 @@ int ch_eval_nonlinear(ch_grid* G);
 // synchronises the stream: CH_ERR_TIMEOUT while the flag of the bounded device waits is set (it stays
 // set until ch_device_status), else CH_OK
 int ch_sync_status(ch_grid* G);
+// ch_set_state; status: answering the flag as ch_sync_status does, with one wait for both
+int ch_restore(ch_grid* G, const void* state, bool status);
 // bw <- the five backward fields u v w phi D phi of the state, as the step itself forms them
 cudaError_t ch_launch_fields(ch_grid* G, cudaStream_t s);
 // the x/y stages of the step on stream s: 3 y backward (bw -> ya), 4 x line (ya -> yb), 5 y
