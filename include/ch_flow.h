@@ -311,9 +311,9 @@ int ch_render_interface(ch_grid* g, unsigned char* rgb, double* depth, int width
  * the three; CH_ERR_ARG if they differ).  One ensemble step advances every member by one time
  * step with six grouped persistent launches (one per stage; their CTAs walk a work list spanning
  * all members; two more per member whose Chebyshev transforms run on the tensor cores, and members
- * with and without get a zrhs and a zbwd launch of their own; members whose x and y transforms run
- * there, see ch_step, make the six launches of those stages themselves and leave the grouped ones to
- * the others), captured once into a CUDA graph and replayed.  Members are set, read and diagnosed through their ch_grid handles
+ * with and without get a zrhs and a zbwd launch of their own; members whose x or y transforms run
+ * there, see ch_step, launch those stages themselves, up to six launches, and leave the grouped ones
+ * to the others; an x line of few long lines stays grouped), captured once into a CUDA graph and replayed.  Members are set, read and diagnosed through their ch_grid handles
  * (ch_ensemble_member); ch_ensemble_step needs every member set.  ch_ensemble_autotune times the
  * transforms' radix schedules and the persistent CTAs per SM of each stage on the live members
  * (their states are saved and restored bit for bit) and keeps the fastest (a stage without grouped
